@@ -16,6 +16,7 @@ from __future__ import annotations
 
 import argparse
 import json
+import math
 import os
 import statistics
 import subprocess
@@ -67,7 +68,7 @@ def parse(argv=None):
     ap.add_argument("--groups", type=int, default=512, help="grouped: the first G of the 512 problems")
     ap.add_argument("--complex-form", choices=["auto", "gauss", "four_m"], default="auto",
                     help="split mode, full biquaternions: complex products as Gauss's three real products, as two "
-                         "over twice the inner dimension, or the library's default (four_m for k <= 512)")
+                         "over twice the inner dimension, or the library's default (the matrix form: fourteen products per modulus)")
     ap.add_argument("--tile-table", default=None,
                     help="tuned tables (tile width, FP64 split-k) JSON written by the autotuner")
     ap.add_argument("--results", default=None,
@@ -253,6 +254,29 @@ def measured_peaks():
     return {"hbm_gbs": 6800.0, "bf16_tflops": 1900.0, "bf16_tflops_sustained": 1700.0}, "fallback"
 
 
+# The matrix form of split-mode products (the library's default, csrc/split_mat2.cu): its moduli and, per pair of
+# component flags, the factor planes of each side and the products per modulus.
+MATRIX_FORM_MODULI = (241, 233, 229, 221, 205, 197, 193, 181, 173, 157, 149, 137, 113, 109, 101, 97, 89, 73)
+MATRIX_FORM_PLANES = {(0xFF, 0xFF): (14, 14, 14)}
+
+
+def matrix_form(hm, k, tol, fa, fb, algo="bilinear", complex_form="auto", planned=24):
+    """(moduli, left planes, right planes, products) of the matrix form when a split-mode product of inner dimension
+    k runs in it, else None: the default complex form, where its planes do not outnumber the plan's (`planned` per
+    modulus)."""
+    planes = MATRIX_FORM_PLANES.get((fa, fb))
+    if planes is None or algo != "bilinear" or complex_form != "auto":
+        return None
+    mods, bits = hm.split_info(k, tol)
+    need, acc, n = 2 * bits + math.log2(max(k, 1)) + 4.25, 0.0, 0
+    while acc <= need:
+        if n == len(MATRIX_FORM_MODULI):
+            return None
+        acc += math.log2(MATRIX_FORM_MODULI[n])
+        n += 1
+    return (n, *planes) if n * planes[2] <= len(mods) * planned else None
+
+
 def split_stage_work(hm, shapes, tol, opA="N", opB="N", fa=0xFF, fb=0xFF, algo="bilinear", complex_form="auto"):
     """Algorithmic work of one split-mode step per stage, summed over (m, n, k) shapes:
     bytes for the exponent, encode and CRT stages (what each stage must read and write:
@@ -261,8 +285,9 @@ def split_stage_work(hm, shapes, tol, opA="N", opB="N", fa=0xFF, fb=0xFF, algo="
     residue GEMM (moduli x product terms x 2 m n k); "split_residue_gemm_bytes" is the least
     DRAM traffic of the residue GEMM (every encoded factor tile read once, every int8
     residue written once), its bound on products too small to reuse their tiles.  Full
-    biquaternion products in the four-multiplication form (complex_form "four_m", or
-    "auto" at k <= 512) count its 16 factors per side, 16 products and 32 terms."""
+    biquaternion products in the four-multiplication form (complex_form "four_m") count its
+    16 factors per side, 16 products and 32 terms, those in the matrix form (complex_form
+    "auto") its own moduli and planes."""
     def form(a):
         T, U, V, _, _ = hm.plan_info(opA, opB, fa, fb, algo=a)
         P = T // 2 if a == "four_m" else T
@@ -275,6 +300,10 @@ def split_stage_work(hm, shapes, tol, opA="N", opB="N", fa=0xFF, fb=0xFF, algo="
     for m, n, k in shapes:
         T, P, nlf, nrf = four if complex_form == "four_m" or (complex_form == "auto" and k <= 512) else gauss
         L = len(hm.split_info(k, tol)[0])
+        mat = matrix_form(hm, k, tol, fa, fb, algo, complex_form, P)
+        if mat:
+            L, nlf, nrf, P = mat
+            T = P
         kp = -(-k // 64) * 64
         raw = 8.0 * (ca * m * k + cb * k * n)
         w["split_exponents"] += raw
@@ -486,7 +515,13 @@ def ours(args, rank, world, local):
         if (args.mode == "split" and args.algo == "bilinear" and fa == fb == 0xFF and
                 (args.complex_form == "four_m" or (args.complex_form == "auto" and k <= 512))):
             P = hm.plan_info(args.opA, "N", fa, fb, algo="four_m")[0]   # product terms (two per product)
+    P64 = P                               # products of FP64 mode
     mods, bits = hm.split_info(kin, args.tol)
+    nmods = len(mods)
+    if args.mode == "split":
+        mat = matrix_form(hm, kin, args.tol, fa, fb, args.algo, args.complex_form, 16 if k <= 512 else 24)
+        if mat:
+            nmods, P = mat[0], mat[3]
     if rank == 0:
         rng = np.random.default_rng(args.seed + 7)
         rows = np.sort(rng.choice(m, size=args.sample_rows, replace=False))
@@ -509,7 +544,7 @@ def ours(args, rank, world, local):
             torch.cuda.synchronize()
             fms = e0.elapsed_time(e1)
             got64 = C[:, torch.as_tensor(rows, device=dev), :].cpu().numpy()
-            ex64 = P * size * 2.0 * m * n * k / (fms * 1e-3) / 1e12
+            ex64 = P64 * size * 2.0 * m * n * k / (fms * 1e-3) / 1e12
             info["fp64_plain"] = {"ms": fms, "tflops_64equiv": flops64 / (fms * 1e-3) / 1e12,
                                   "tflops_executed": ex64,
                                   "rel_fro_err_sampled": float(np.linalg.norm(got64 - want) / np.linalg.norm(want)),
@@ -579,7 +614,7 @@ def ours(args, rank, world, local):
                   ("" if args.algo == "bilinear" else f" algo={args.algo}"))
         if args.mode == "split":
             # BF16 tensor flops of the GEMM launches of one step, per launch
-            alg = len(mods) * P * size * 2.0 * m * n * k * args.steps / max(gl, 1)
+            alg = nmods * P * size * 2.0 * m * n * k * args.steps / max(gl, 1)
             avg = gms / max(gl, 1)
             ach = alg / (avg * 1e-3) / 1e12
             peak = peaks.get("bf16_tflops_sustained", peaks.get("bf16_tflops"))
@@ -600,7 +635,7 @@ def ours(args, rank, world, local):
                 "warmup": args.warmup, "ms_per_step": ms, "higher_is_better": True, "scaling": "weak",
                 "vs_baseline": None, "dtype": "bf16" if args.mode == "split" else "f64", "data": "synthetic",
                 "config": dict(workload_config(args), parallelism=f"replicas x{world}",
-                               moduli=len(mods), bits=bits, products=P),
+                               moduli=nmods, bits=bits, products=P),
                 "roofline": roof, "cpu_baseline": info.get("cpu_baseline"), "e2e": info.get("e2e"),
                 "gpu_launches": launches, "clocks": clk,
                 "rel_fro_err_sampled": info.get("rel_fro_err_sampled"),
@@ -611,7 +646,7 @@ def ours(args, rank, world, local):
                            and info.get("freivalds_ratio") is not None
                            and info["freivalds_ratio"] <= args.tol + 1e-14),
                 "fp64_plain": info.get("fp64_plain"), "stages": stages,
-                "executed_tflops": value * size * (len(mods) * P if args.mode == "split" else P) / 64.0,
+                "executed_tflops": value * size * (nmods * P if args.mode == "split" else P) / 64.0,
                 "naive_equiv_tflops": value * naive / 64.0,
                 "naive_equiv_note": f"counted as {naive} component-wise real GEMMs of n^3"}
         emit(args, line)
@@ -887,9 +922,12 @@ def streamed_arm(args, rank, world, local):
         err = float(np.linalg.norm(got - want) / np.linalg.norm(want))
         h2d, d2h = hm.streamed_traffic(n, n, n, mode=args.mode, tol=args.tol, budget=budget, handle=h)
         mods, bits = hm.split_info(kb, args.tol)
-        P = hm.plan_info("N", "N", hm.HMAT_BQ, hm.HMAT_BQ)[0]
+        nmods, P = len(mods), hm.plan_info("N", "N", hm.HMAT_BQ, hm.HMAT_BQ)[0]
+        mat = matrix_form(hm, kb, args.tol, hm.HMAT_BQ, hm.HMAT_BQ)
+        if mat:
+            nmods, P = mat[0], mat[3]
         gl, gms = kernels["split_residue_gemm"]
-        alg = len(mods) * P * 2.0 * mb * nb * kb     # per launch (full blocks)
+        alg = nmods * P * 2.0 * mb * nb * kb         # per launch (full blocks)
         avg = gms / max(gl, 1)
         peaks, src = measured_peaks()
         peak = peaks.get("bf16_tflops_sustained", peaks.get("bf16_tflops"))

@@ -332,13 +332,23 @@ hmat_status hmat_set_algorithm(hmat_handle handle, int32_t algo);
  *                      and 16 factor planes per side, 4/3 of the
  *                      multiplications, 2/3 of the bytes of the encoded
  *                      planes and the product residues;
- *   HMAT_CFORM_AUTO:   (default) FOUR_M for inner dimensions up to 512,
- *                      where a product's two terms fit one exact FP32
- *                      accumulation chunk of the residue GEMM, GAUSS above.
- * Every residue is exact in both forms, so both give the same bits.
- * Other flag pairs, FP64 mode and streamed products always use Gauss's
- * form; hmat_bq_gemm_split_noalloc follows the setting.  hmat_workspace_size
- * and hmat_workspace_size_modes follow the setting (FOUR_M needs less).
+ *   HMAT_CFORM_AUTO:   (default) the matrix form: modulo p with a square root
+ *                      s of -1 the biquaternions are two copies of the 2 x 2
+ *                      matrices (i -> s, i -> -s), each product of which takes
+ *                      seven multiplications: 14 residue GEMMs per modulus and
+ *                      14 factor planes per side, over its own moduli (all prime
+ *                      factors 1 modulo 4).  Where those planes would outnumber
+ *                      the plan's (a few k below 16 at loose tolerances):
+ *                      FOUR_M for inner dimensions up to 512, where a product's
+ *                      two terms fit one exact FP32 accumulation chunk of the
+ *                      residue GEMM, GAUSS above.
+ * Every residue is exact in all forms, so all give the same bits.
+ * Other flag pairs and FP64 mode always use Gauss's form; streamed products
+ * take the matrix form under AUTO and Gauss's form otherwise;
+ * hmat_bq_gemm_split_noalloc follows the setting.  hmat_workspace_size and
+ * hmat_workspace_size_modes follow the setting: FOUR_M needs less than GAUSS,
+ * and AUTO reports FOUR_M's bytes for k up to 512 and GAUSS's above, inside
+ * which the matrix form runs.
  * Errors: NOT_INITIALIZED, INVALID_VALUE (unknown form). */
 HMAT_API
 hmat_status hmat_set_complex_form(hmat_handle handle, int32_t form);
@@ -366,8 +376,10 @@ hmat_status hmat_plan_info(int32_t algo, int32_t opA, int32_t opB, uint32_t flag
                            int8_t *V, double *W, int32_t *strategy);
 
 /* Split-mode parameters for inner dimension k and target tol — host only.
- * On return *n_moduli = L, moduli[0..L-1] the moduli (caller array of >= 32),
- * *bits = the integer width b of the scaled operands (|X| <= 2^b). */
+ * On return *n_moduli = L, moduli[0..L-1] the moduli (caller array of >= 32) of
+ * Gauss's and the four-multiplication form (the matrix form, which see
+ * hmat_set_complex_form, has its own), *bits = the integer width b of the
+ * scaled operands (|X| <= 2^b) in every form. */
 HMAT_API
 hmat_status hmat_split_info(int64_t k, double tol, int32_t *n_moduli,
                             int32_t *moduli, int32_t *bits);

@@ -109,8 +109,9 @@ struct SplitReuse {
   // FP64 mode: never split the inner dimension (the streamed blocks, so that
   // they compute exactly what the in-core product computes)
   bool fp64_whole_k = false;
-  // split mode: Gauss's three-product form whatever the handle's setting (the
-  // streamed blocks, whose workspace is planned without the handle)
+  // split mode: lay products out as Gauss's three-product form does whatever the
+  // handle's setting (the streamed blocks, whose workspace is planned without
+  // the handle); under AUTO the matrix form runs inside those bytes
   bool gauss = false;
 };
 

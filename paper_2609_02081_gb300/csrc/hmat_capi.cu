@@ -423,6 +423,12 @@ int split_plan_algo(int32_t cform, int palgo, uint32_t fa, uint32_t fb, int64_t 
   return palgo;
 }
 
+// Full biquaternion products may run in the matrix form: the default complex
+// form under the bilinear algorithm.  A form chosen by name is the one that runs.
+static bool mat2_allowed(const hmat_context* h) {
+  return h->cform == HMAT_CFORM_AUTO && h->algo == HMAT_ALGO_BILINEAR;
+}
+
 hmat_status prepare(hmat_context* h, int32_t count, const hmat_gemm_desc* descs, int32_t mode, double tol,
                     void* workspace, size_t ws_bytes, cudaStream_t stream, Prepared* out, bool allow_splitk = true,
                     const int32_t* modes = nullptr, bool gauss = false) {
@@ -503,7 +509,7 @@ hmat_status prepare(hmat_context* h, int32_t count, const hmat_gemm_desc* descs,
   out->ws_needed = out->split_offset;
   if (!split_jobs.empty()) {
     const size_t avail = ws_bytes > (size_t)out->split_offset ? ws_bytes - (size_t)out->split_offset : 0;
-    hmat_status st = split_prepare(split_jobs, h->h_plans, tol, avail, split_table(h), &out->sp);
+    hmat_status st = split_prepare(split_jobs, h->h_plans, tol, avail, split_table(h), mat2_allowed(h), &out->sp);
     if (st != HMAT_STATUS_SUCCESS) return st;
     out->has_split = true;
     out->ws_needed += out->sp.ws_needed;
@@ -1044,7 +1050,8 @@ hmat_status hmat_bq_gemm_split_noalloc(hmat_handle h, int32_t opA, int32_t opB, 
   if (j.k == 0 || h->h_plans[slot].np == 0) return HMAT_STATUS_UNSUPPORTED;
   SplitJob sj;
   SplitUnits u;
-  st = split_layout_single(j, h->h_plans[slot], tol, split_table(h), &sj, &u);
+  // (the entry point always runs the bilinear algorithm)
+  st = split_layout_single(j, h->h_plans[slot], tol, split_table(h), h->cform == HMAT_CFORM_AUTO, &sj, &u);
   if (st != HMAT_STATUS_SUCCESS) return st;
   if ((size_t)u.ws_bytes > kNoAllocScratchBytes) return HMAT_STATUS_WORKSPACE_TOO_SMALL;
   NoAllocAddrs a;
@@ -1053,13 +1060,20 @@ hmat_status hmat_bq_gemm_split_noalloc(hmat_handle h, int32_t opA, int32_t opB, 
   noalloc_store_job_kernel<<<1, 1, 0, stream>>>(sj);
   e = cudaGetLastError();
   if (e == cudaSuccess) e = launch_split_exponents(a.job, 1, u.exp, 0, stream, a.scratch);
-  if (e == cudaSuccess) e = launch_split_encode(a.job, 1, h->d_plans, 0, u.encA, stream, a.scratch, u.max_bits);
-  if (e == cudaSuccess) e = launch_split_encode(a.job, 1, h->d_plans, 1, u.encB, stream, a.scratch, u.max_bits);
+  if (sj.mat2) {
+    if (e == cudaSuccess) e = launch_mat2_encode(a.job, 1, u.encA + u.encB, 0, stream, a.scratch, u.max_bits);
+  } else {
+    if (e == cudaSuccess) e = launch_split_encode(a.job, 1, h->d_plans, 0, u.encA, stream, a.scratch, u.max_bits);
+    if (e == cudaSuccess) e = launch_split_encode(a.job, 1, h->d_plans, 1, u.encB, stream, a.scratch, u.max_bits);
+  }
   if (e == cudaSuccess)
     e = launch_split_gemm(a.job, 1, u.items, (int)std::min<int64_t>(u.items, h->sm_count), stream, a.scratch,
                           u.max_nkb);
-  if (e == cudaSuccess) e = launch_split_crt(a.job, 1, h->d_plans, u.crt, stream, a.scratch, u.max_nmod, u.max_np, u.all_full,
-                                                u.four_m ? 1 : 0, sj.crt_w == kCrtCols);
+  if (e == cudaSuccess && sj.mat2)
+    e = launch_mat2_crt(a.job, 1, u.crt, stream, a.scratch, u.max_nmod, sj.crt_w == kCrtCols);
+  else if (e == cudaSuccess)
+    e = launch_split_crt(a.job, 1, h->d_plans, u.crt, stream, a.scratch, u.max_nmod, u.max_np, u.all_full,
+                         u.four_m ? 1 : 0, sj.crt_w == kCrtCols);
   return cuda_status(e);
 }
 

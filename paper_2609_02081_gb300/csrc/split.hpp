@@ -20,6 +20,13 @@
 //                  the moduli (exact integer of up to ~140 bits), conversion to
 //                  FP64, the 2^-(s_i + t_j) rescaling and the complex alpha/beta
 //                  update (Sec. III scaling and addition).
+// Full biquaternion products run by default in the matrix form
+// (split_mat2.cu), which replaces the plan's products by fewer ones that exist
+// only modulo suitable p: with s^2 = -1 (mod p) the biquaternions modulo p are
+// two copies of the 2 x 2 matrices modulo p (i -> s and i -> -s), and each 2 x 2
+// product takes seven multiplications (Strassen's, in Winograd's variant): 14
+// residue GEMMs per modulus instead of 24.  The integers that the CRT recovers,
+// and so the results, are the same.
 // The only rounding is step 2's scaling to b-bit integers; b and the modulus
 // count follow from the requested tolerance and k.
 #pragma once
@@ -55,8 +62,17 @@ inline int crt_width(int64_t n) { return n >= 1024 ? kCrtCols : 32; }
 // residue sum satisfies |4Q| <= 36 * 127 = 4572, which the CRT's integer
 // residue step relies on.  Plans above it are refused.
 constexpr int kMaxWeightSum = 36;
-// Largest inner dimension for which HMAT_CFORM_AUTO takes the four-
-// multiplication form: its products (two terms of depth k) then fit one
+// Matrix form: residue planes per modulus (factors per side and products), and
+// the largest sum of product residues in one output: |sum| <= 16 (p - 1)/2.
+constexpr int kMat2Planes = 14;
+constexpr int kMat2WeightSum = 16;
+constexpr int kMat2HalfMax = 120;  // (p - 1)/2 of its largest modulus, 241
+// Most moduli whose sums S < 2 N P fit four 32-bit limbs (P < 2^111.1 and N =
+// 15 * 16 * 120 < 2^14.9; checked when the tables are built)
+constexpr int kMat2FourLimbs = 15;
+// Largest inner dimension for which HMAT_CFORM_AUTO falls back from the matrix
+// form to the four-multiplication form (and whose workspace it reports), not to
+// Gauss's: its products (two terms of depth k) then fit one
 // 1024-deep exact chunk of the residue GEMM.
 constexpr int64_t kFourMMaxK = kChunkK / 2;
 
@@ -69,6 +85,9 @@ struct SplitParams {
 
 // Moduli count and integer width for inner dimension k and target tolerance.
 hmat_status split_params(int64_t k, double tol, SplitParams* out);
+// Modulus count of the matrix form for inner dimension k and integer width
+// bits; 0 when its moduli do not reach far enough.
+int mat2_moduli(int64_t k, int bits);
 
 struct SplitShape {
   int64_t m, n, k;
@@ -112,9 +131,12 @@ struct SplitJob {
   int64_t off_res;                  // int8 product residues
   int64_t encA_plane, encB_plane;   // bytes between consecutive (modulus, factor) tile planes
   int64_t res_plane;                // bytes between consecutive (modulus, product) residue planes
+  int32_t mat2;                     // matrix form: its own moduli, encoder and CRT (np = nlf = nrf = kMat2Planes)
+  int32_t mod_base;                 // first modulus in the GEMM's table (kModTable: the matrix form's moduli)
   int64_t item_begin;               // residue-GEMM work items before this job
-  int64_t encA_begin, encB_begin;   // encode blocks before this job
-  int64_t crt_begin;                // CRT blocks before this job
+  int64_t encA_begin, encB_begin;   // encode blocks before this job (matrix-form jobs have none)
+  int64_t crt_begin;                // CRT blocks before this job (likewise)
+  int64_t enc2_begin, crt2_begin;   // matrix form: encode blocks (A side, then B side) and CRT blocks before this job
   int64_t exp_begin;                // exponent work units before this job
 };
 
@@ -158,10 +180,14 @@ void split_release(SplitState& s);
 struct SplitPrep {
   std::vector<SplitJob> jobs;
   int64_t exp_units = 0, encA_units = 0, encB_units = 0, items = 0, crt_units = 0;
+  int64_t enc2_units = 0, crt2_units = 0;   // matrix-form jobs
+  int max_bits2 = 0, max_nmod2 = 0;         // matrix-form jobs (max_bits, max_nmod, max_np: the others)
+  bool all_wide2 = true;                    // matrix-form jobs: every CRT block is one row of kCrtCols columns
   int64_t ws_needed = 0;
   int max_bits = 0, max_nmod = 0, max_np = 0, max_nkb = 0;
-  bool all_full = true;             // every job uses the paper's full plan (Gauss or four-multiplication form)
+  bool all_full = true;             // every job outside the matrix form uses the paper's full plan (either form)
   int n_four_m = 0;                 // jobs in the four-multiplication form
+  int n_plan = 0;                   // jobs outside the matrix form
   bool all_wide = true;             // every job's full-plan CRT blocks are one row of kCrtCols columns
   // one job whose A-side exponents and encoded factor tiles are already in the
   // workspace from the previous call with the same A block and the same shape
@@ -180,8 +206,11 @@ hmat_status split_b_region_bytes(const SplitShape& sh, double tol, const TileTab
 void split_place_b(SplitJob& sj, int64_t offset);
 
 // Lay the jobs out in a workspace of ws_bytes (WORKSPACE_TOO_SMALL if it does not fit).
+// mat2: full biquaternion products run in the matrix form inside the bytes that
+// their plan's form occupies (the workspace a caller must bring does not depend
+// on it); products for which it has no advantage keep the plan's form.
 hmat_status split_prepare(const std::vector<JobDesc>& jobs, const KPlan* h_plans, double tol, size_t ws_bytes,
-                          const TileTables& tables, SplitPrep* out);
+                          const TileTables& tables, bool mat2, SplitPrep* out);
 // Layout of one job at workspace offset 0 with its per-stage unit counts;
 // uses no heap memory (for the entry point that allocates nothing).
 struct SplitUnits {
@@ -190,8 +219,8 @@ struct SplitUnits {
   bool all_full = false;
   bool four_m = false;
 };
-hmat_status split_layout_single(const JobDesc& d, const KPlan& P, double tol, const TileTables& tables, SplitJob* out,
-                                SplitUnits* units);
+hmat_status split_layout_single(const JobDesc& d, const KPlan& P, double tol, const TileTables& tables, bool mat2,
+                                SplitJob* out, SplitUnits* units);
 // Launch the four stages reading the device job table d_jobs.
 hmat_status split_launch(hmat_context* h, const SplitPrep& sp, const SplitJob* d_jobs, const KPlan* d_plans,
                          unsigned char* ws, cudaStream_t stream);
@@ -239,6 +268,20 @@ cudaError_t launch_split_gemm(const SplitJob* d_jobs, int njobs, int64_t items, 
 cudaError_t launch_split_crt(const SplitJob* d_jobs, int njobs, const KPlan* d_plans, int64_t units,
                              cudaStream_t s, unsigned char* ws, int max_nmod, int max_np, bool all_full,
                              int full_form, bool all_wide);
+// Matrix form (split_mat2.cu).  Encode blocks [first, first + units) of the
+// A and B sides of its jobs; jobs of other forms have no blocks.
+cudaError_t launch_mat2_encode(const SplitJob* d_jobs, int njobs, int64_t units, int64_t first, cudaStream_t s,
+                               unsigned char* ws, int max_bits);
+cudaError_t launch_mat2_crt(const SplitJob* d_jobs, int njobs, int64_t units, cudaStream_t s, unsigned char* ws,
+                            int max_nmod, bool all_wide);
+// n (kMaxModuli) moduli, root[l]^2 = -1 mod moduli[l], and the CRT tables
+// [n + 1][2][n][kLimbs], [n + 1][kLimbs], [n + 1][kLimbs] by modulus count
+cudaError_t mat2_configure(const int* moduli, const int* root, int n, const int32_t* crt_d, const uint32_t* crt_P,
+                           const uint32_t* crt_off);
+// Constants of the CRT's quotient estimate for the modulus product P: pb the
+// limb below its top one, pinv = fl(2^(32 pb) / P).  False when the estimate's
+// error on sums below max_quotient P could miss the quotient with `limbs` limbs.
+bool crt_estimate_constants(const uint32_t* P, double max_quotient, int limbs, int* pb, float* pinv);
 cudaError_t split_upload_constants(const int* moduli, int nmod_table, const int32_t* crt_d, const uint32_t* crt_P,
                                    const uint32_t* crt_off);
 

@@ -166,7 +166,7 @@ struct Item {
   const uint8_t* b2;
   int8_t* out;        // residue tile origin (row 0, column 0 of the tile)
   int64_t ncols;      // residue row pitch
-  int nkb, bn, l;     // nkb: k-blocks of all terms
+  int nkb, bn, l;     // nkb: k-blocks of all terms; l: index into the modulus table
   int kb2;            // first k-block of the second term (nkb: one term)
   bool neg;           // the second term is subtracted
   int rows, cols;     // rows and columns of the tile inside the product (the rest is padding)
@@ -215,7 +215,7 @@ __device__ __forceinline__ Item decode_item(const SplitJob* jobs, int job, int64
   it.kb2 = sj.four_m ? sj.nkb : it.nkb;
   it.neg = sj.four_m && ((sj.neg2 >> p) & 1ull);
   it.bn = sj.bn;
-  it.l = l;
+  it.l = sj.mod_base + l;
   it.rows = min(kTileM, sj.d.m - tm * kTileM);
   it.cols = min(sj.bn, sj.d.n - tn * sj.bn);
   // padding rows hold whatever the workspace held: they meet only padding
@@ -267,7 +267,7 @@ struct GemmModConst {
   int p;
   float pf, inv;
 };
-__constant__ GemmModConst c_gmod[kModTable];
+__constant__ GemmModConst c_gmod[2 * kModTable];   // the plans' moduli, then the matrix form's
 
 // kOneChunk: every item of the launch has an inner dimension of one chunk
 // (k <= 1024), so the multi-chunk epilogue and its 128 running sums per
@@ -589,8 +589,8 @@ cudaError_t launch_wait_selftest(long long limit_cycles, cudaStream_t s) {
 size_t split_gemm_smem_bytes() { return sizeof(GemmSmem) + 1024; }
 
 cudaError_t split_gemm_configure(const int* moduli, int n) {
-  GemmModConst g[kModTable];
-  for (int l = 0; l < kModTable; ++l) {
+  GemmModConst g[2 * kModTable];
+  for (int l = 0; l < 2 * kModTable; ++l) {
     const int p = l < n ? moduli[l] : 255;
     g[l].p = p;
     g[l].pf = (float)p;

@@ -19,6 +19,13 @@ cudaError_t split_gemm_configure(const int* moduli, int n);
 static const int kModuli[kModTable] = {255, 253, 251, 247, 241, 239, 233, 229, 227, 223, 217, 211,
                                        199, 197, 193, 191, 181, 179, 173, 167, 163, 157, 151, 149};
 
+// Matrix form: odd, pairwise coprime moduli below 255 all of whose prime
+// factors are 1 modulo 4 (221 = 13*17, 205 = 5*41, the rest prime), so that -1
+// has a square root modulo each: the largest eighteen, 130.4 bits together.
+// 257 is left out: its centred residues do not fit int8.
+static const int kMat2Moduli[kMaxModuli] = {241, 233, 229, 221, 205, 197, 193, 181, 173,
+                                            157, 149, 137, 113, 109, 101, 97,  89,  73};
+
 // Margin (bits) between the requested tolerance and the integer width: the
 // scaling error of one operand element is <= 2^-b of its row/column maximum,
 // and sums over k of such errors relative to the result stay well below 2^6.
@@ -54,6 +61,64 @@ hmat_status split_params(int64_t k, double tol, SplitParams* out) {
   return HMAT_STATUS_SUCCESS;
 }
 
+static int centred_mod(long long v, int p) {
+  const int r = (int)(((v % p) + p) % p);
+  return r > (p - 1) / 2 ? r - p : r;
+}
+// sum of the magnitudes of the weights 2^0, 2^16, 2^32 and their multiples by s modulo p
+static long long mat2_digit_sum(int p, int s) {
+  long long sum = 0;
+  for (int d = 0; d < 3; ++d) {
+    const int c = centred_mod(1ll << (16 * d), p);
+    sum += std::abs(c) + std::abs(centred_mod((long long)c * s, p));
+  }
+  return sum;
+}
+// The square root of -1 modulo p with the smallest digit-weight sum (see
+// mat2_digit_sum), up to sign, in [1, p); 0 if p has none within the bound.
+static int mat2_root(int p) {
+  int best = 0;
+  long long best_sum = 0;
+  for (int s = 1; s < p; ++s) {
+    if ((s * s + 1) % p != 0) continue;
+    const long long sum = mat2_digit_sum(p, s);
+    if (best == 0 || sum < best_sum) {
+      best = s;
+      best_sum = sum;
+    }
+  }
+  // u = sum_d x_d c_d + s y_d c_d stays an exact float: digits |x_d|, |y_d| <=
+  // 2^15 + 1 (the fourth one <= 2^6) times the weights, below 2^24
+  return best_sum < 500 ? best : 0;
+}
+
+int mat2_moduli(int64_t k, int bits) {
+  // the same range as split_params: the recovered integers are the same
+  const double need = 2.0 * bits + std::log2((double)std::max<int64_t>(k, 1)) + 4.0 + 0.25;
+  double acc = 0.0;
+  int n = 0;
+  while (acc <= need) {
+    if (n >= kMaxModuli) return 0;
+    acc += std::log2((double)kMat2Moduli[n++]);
+  }
+  return n;
+}
+
+bool crt_estimate_constants(const uint32_t* P, double max_quotient, int limbs, int* pb, float* pinv) {
+  int top = 0;
+  for (int q = 0; q < kLimbs; ++q)
+    if (P[q]) top = q;
+  *pb = top > 0 ? top - 1 : 0;
+  double f = 0.0;                      // P / 2^(32 pb), then its float reciprocal
+  for (int q = kLimbs - 1; q >= *pb; --q) f = f * 4294967296.0 + (double)P[q];
+  *pinv = f > 0.0 ? (float)(1.0 / f) : 1.f;
+  // the sums fit the limbs, and 2 + 2 (limbs - 1 - pb) + 2 float roundings of
+  // relative size 2^-24 on S / P stay below the 0.0796 margin (1/2 - 2^-1.25)
+  if (std::log2(f) + 32.0 * *pb + std::log2(std::max(max_quotient, 1.0)) >= 32.0 * limbs) return false;
+  const double rounds = 4.0 + 2.0 * (limbs - 1 - *pb);
+  return rounds * std::ldexp(1.0, -24) * max_quotient < 0.5 - std::exp2(-1.25);
+}
+
 // ----------------------------------------------------------------- tiny big integers (32-bit limbs)
 namespace {
 
@@ -75,6 +140,57 @@ uint32_t inv_mod(uint32_t a, uint32_t m) {
     if ((unsigned long long)a * x % m == 1) return x;
   return 0;
 }
+// CRT basis element of moduli[l] among the first n: congruent to c modulo p_l
+// and to 0 modulo the others, below P, in signed 32-bit digits (each word above
+// 2^31 - 1 borrows from the next)
+bool crt_element(const int* moduli, int n, int l, uint32_t c, int32_t* digits) {
+  const uint32_t p = (uint32_t)moduli[l];
+  uint32_t Ml[kLimbs] = {1, 0, 0, 0, 0};
+  for (int j = 0; j < n; ++j)
+    if (j != l) big_mul_small(Ml, (uint32_t)moduli[j]);
+  const uint32_t inv = inv_mod(big_mod_small(Ml, p), p);
+  big_mul_small(Ml, (uint32_t)((unsigned long long)inv * (c % p) % p));
+  long long carry = 0;
+  for (int q = 0; q < kLimbs; ++q) {
+    long long w = (long long)Ml[q] + carry;
+    carry = 0;
+    if (w >= (1ll << 31)) {
+      w -= 1ll << 32;
+      carry = 1;
+    }
+    digits[q] = (int32_t)w;
+  }
+  return carry == 0;   // the element is below P < 2^(32 kLimbs - 1)
+}
+
+// Tables of the matrix form: s with s^2 = -1 (mod p) per modulus, the CRT
+// elements carrying 1/4 (outputs formed from the sums of the two matrix copies)
+// and 1/(4 s) (from their differences), the products P and the offsets.
+cudaError_t mat2_configure_tables() {
+  static int32_t crt[kMaxModuli + 1][2][kMaxModuli][kLimbs];
+  static uint32_t P[kMaxModuli + 1][kLimbs], off[kMaxModuli + 1][kLimbs];
+  std::memset(crt, 0, sizeof(crt));
+  std::memset(P, 0, sizeof(P));
+  std::memset(off, 0, sizeof(off));
+  int root[kMaxModuli];
+  for (int l = 0; l < kMaxModuli; ++l) {
+    root[l] = mat2_root(kMat2Moduli[l]);
+    if (root[l] == 0) return cudaErrorInvalidValue;
+  }
+  for (int n = 1; n <= kMaxModuli; ++n) {
+    P[n][0] = 1;
+    for (int l = 0; l < n; ++l) big_mul_small(P[n], (uint32_t)kMat2Moduli[l]);
+    std::memcpy(off[n], P[n], sizeof(off[n]));
+    big_mul_small(off[n], (uint32_t)(n * kMat2WeightSum * kMat2HalfMax));
+    for (int l = 0; l < n; ++l) {
+      const uint32_t p = (uint32_t)kMat2Moduli[l];
+      if (!crt_element(kMat2Moduli, n, l, inv_mod(4u, p), crt[n][0][l]) ||
+          !crt_element(kMat2Moduli, n, l, inv_mod(4u * (uint32_t)root[l] % p, p), crt[n][1][l]))
+        return cudaErrorInvalidValue;
+    }
+  }
+  return mat2_configure(kMat2Moduli, root, kMaxModuli, &crt[0][0][0][0], &P[0][0], &off[0][0]);
+}
 
 }  // namespace
 
@@ -94,30 +210,20 @@ cudaError_t split_configure() {
     for (int l = 0; l < n; ++l) {
       // d_l = (P / p_l) * ((P / p_l)^-1 4^-1 mod p_l): congruent to 4^-1 modulo
       // p_l and to 0 modulo the other moduli, below P
-      const uint32_t p = (uint32_t)kModuli[l];
-      uint32_t Ml[kLimbs] = {1, 0, 0, 0, 0};
-      for (int j = 0; j < n; ++j)
-        if (j != l) big_mul_small(Ml, (uint32_t)kModuli[j]);
-      const uint32_t inv = inv_mod(big_mod_small(Ml, p), p);
-      const uint32_t inv4 = inv_mod(4u, p);
-      big_mul_small(Ml, (uint32_t)((unsigned long long)inv * inv4 % p));
-      // signed 32-bit digits: each word above 2^31 - 1 borrows from the next
-      long long carry = 0;
-      for (int q = 0; q < kLimbs; ++q) {
-        long long w = (long long)Ml[q] + carry;
-        carry = 0;
-        if (w >= (1ll << 31)) {
-          w -= 1ll << 32;
-          carry = 1;
-        }
-        crt[n][l][q] = (int32_t)w;
-      }
-      if (carry != 0) return cudaErrorInvalidValue;   // d_l < P < 2^(32 kLimbs - 1)
+      if (!crt_element(kModuli, n, l, inv_mod(4u, (uint32_t)kModuli[l]), crt[n][l])) return cudaErrorInvalidValue;
     }
   }
   cudaError_t e = split_upload_constants(kModuli, kModTable, &crt[0][0][0], &P[0][0], &off[0][0]);
   if (e != cudaSuccess) return e;
-  return split_gemm_configure(kModuli, kModTable);
+  e = mat2_configure_tables();
+  if (e != cudaSuccess) return e;
+  // the GEMM's modulus table: the plans' moduli, then (from kModTable) the matrix form's
+  int moduli[2 * kModTable];
+  for (int l = 0; l < kModTable; ++l) {
+    moduli[l] = kModuli[l];
+    moduli[kModTable + l] = l < kMaxModuli ? kMat2Moduli[l] : kMat2Moduli[0];
+  }
+  return split_gemm_configure(moduli, 2 * kModTable);
 }
 
 void split_release(SplitState& s) {
@@ -165,6 +271,48 @@ static int choose_bn(const int8_t* table, int64_t m, int64_t n) {
 
 static inline int64_t align256(int64_t x) { return (x + 255) & ~(int64_t)255; }
 
+// Places the job's regions behind *offset (exponents, encoded factors, product residues).
+static void place_job(SplitJob* sj, int64_t m, int64_t n, int64_t* offset) {
+  int64_t off = *offset;
+  sj->off_sexp = off;
+  off = align256(off + 4 * m);
+  sj->off_texp = off;
+  off = align256(off + 4 * n);
+  sj->off_encA = off;
+  off = align256(off + (int64_t)sj->nmod * sj->nlf * sj->encA_plane);
+  sj->off_encB = off;
+  off = align256(off + (int64_t)sj->nmod * sj->nrf * sj->encB_plane);
+  sj->off_res = off;
+  off = align256(off + (int64_t)sj->nmod * sj->np * sj->res_plane);
+  *offset = off;
+}
+
+// Turns a full-plan job laid out at *offset0 into the matrix form, inside the
+// bytes its plan's form occupies.  The form wins wherever its planes (14 per
+// modulus, one or two moduli more) do not outnumber the plan's (24, or 16 in the
+// four-multiplication form), which also keeps it inside those bytes; that leaves
+// out a few tiny k at loose tolerances (k <= 15 at tol 1e-3: 6 x 14 planes
+// against 5 x 16).  Measured at tol 1e-12: m = n = k = 8192, 15 x 14 planes
+// against Gauss's 14 x 24: 226 -> 144 ms; the 512-product batch: 31.9 -> 23.5 ms.
+static void to_mat2(SplitJob* sj, int64_t offset0) {
+  const int nm = mat2_moduli(sj->d.k, sj->bits);
+  if (nm == 0 || nm * kMat2Planes > sj->nmod * sj->np || nm * kMat2Planes > sj->nmod * sj->nlf ||
+      nm * kMat2Planes > sj->nmod * sj->nrf)
+    return;
+  sj->mat2 = 1;
+  sj->mod_base = kModTable;
+  sj->four_m = 0;
+  sj->neg2 = 0;
+  sj->nmod = nm;
+  sj->np = sj->nlf = sj->nrf = kMat2Planes;
+  for (int p = 0; p < kMaxProducts; ++p) {
+    sj->pl[p] = sj->pr[p] = (int8_t)(p < kMat2Planes ? p : 0);
+    sj->pl2[p] = sj->pr2[p] = 0;
+  }
+  int64_t off = offset0;
+  place_job(sj, sj->d.m, sj->d.n, &off);
+}
+
 // plane skews: an odd multiple of 256 B (bulk copies need 16-byte alignment)
 static constexpr int64_t kPlaneSkewEnc = 3 * 256;
 static constexpr int64_t kPlaneSkewRes = 3 * 256;
@@ -177,11 +325,11 @@ static inline int64_t enc_blocks(int64_t rows, int64_t nkb) { return ((rows + 15
 static inline int64_t crt_blocks(int64_t m, int64_t n, int rows) {
   return ((m + rows - 1) / rows) * ((n + kCrtCols - 1) / kCrtCols);
 }
-// CRT blocks of a job and its block width: the full-plan kernel's blocks are
-// kCrtCols / crt_width(n) rows of crt_width(n) columns, the other kernels'
+// CRT blocks of a job and its block width: the full-plan and matrix-form kernels' blocks
+// are kCrtCols / crt_width(n) rows of crt_width(n) columns, the other kernels'
 // kCrtRows rows of kCrtCols columns
 static inline int64_t crt_job_blocks(SplitJob& sj, bool all_full) {
-  if (!all_full) {
+  if (!all_full && !sj.mat2) {
     sj.crt_w = kCrtCols;
     return crt_blocks(sj.d.m, sj.d.n, kCrtRows);
   }
@@ -238,18 +386,7 @@ static hmat_status layout_job(const SplitShape& sh, const KPlan* plan, double to
   // the encoder addresses a factor plane with a 32-bit stride (m k or k n below 2^31)
   if (sj->encA_plane >= ((int64_t)1 << 32) || sj->encB_plane >= ((int64_t)1 << 32)) return HMAT_STATUS_UNSUPPORTED;
   sj->res_plane = ((int64_t)sj->tiles_m * kTileM) * ((int64_t)sj->tiles_n * sj->bn) + kPlaneSkewRes;
-  int64_t off = *offset;
-  sj->off_sexp = off;
-  off = align256(off + 4 * sh.m);
-  sj->off_texp = off;
-  off = align256(off + 4 * sh.n);
-  sj->off_encA = off;
-  off = align256(off + (int64_t)sj->nmod * sj->nlf * sj->encA_plane);
-  sj->off_encB = off;
-  off = align256(off + (int64_t)sj->nmod * sj->nrf * sj->encB_plane);
-  sj->off_res = off;
-  off = align256(off + (int64_t)sj->nmod * sj->np * sj->res_plane);
-  *offset = off;
+  place_job(sj, sh.m, sh.n, offset);
   return HMAT_STATUS_SUCCESS;
 }
 
@@ -282,7 +419,7 @@ hmat_status split_workspace_bytes(const std::vector<SplitShape>& shapes, double 
 }
 
 hmat_status split_prepare(const std::vector<JobDesc>& jobs, const KPlan* h_plans, double tol, size_t ws_bytes,
-                          const TileTables& tables, SplitPrep* out) {
+                          const TileTables& tables, bool mat2, SplitPrep* out) {
   SplitPrep sp;
   int64_t off = 0;
   for (const JobDesc& d : jobs) {
@@ -291,32 +428,46 @@ hmat_status split_prepare(const std::vector<JobDesc>& jobs, const KPlan* h_plans
     std::memset(&sj, 0, sizeof(sj));
     sj.d = d;
     SplitShape sh{d.m, d.n, d.k, P.np, P.nlf, P.nrf, P.bilinear_full, d.fa, d.fb, P.four_m};
+    const int64_t off0 = off;
     hmat_status st = layout_job(sh, &P, tol, tables, &sj, &off);
     if (st != HMAT_STATUS_SUCCESS) return st;
+    // the residue GEMM decodes a job's items with 32-bit arithmetic
+    const int64_t plan_items = (int64_t)sj.nmod * sj.np * sj.tiles_m * sj.tiles_n;
+    if (plan_items >= ((int64_t)1 << 31)) return HMAT_STATUS_UNSUPPORTED;
+    if (mat2 && sj.full) to_mat2(&sj, off0);
     sj.exp_begin = sp.exp_units;
     sp.exp_units += (d.m + 31) / 32 + (d.n + 31) / 32;
+    const int64_t ea = enc_blocks(d.m, sj.nkb), eb = enc_blocks(d.n, sj.nkb);
     sj.encA_begin = sp.encA_units;
-    sp.encA_units += enc_blocks(d.m, sj.nkb);
     sj.encB_begin = sp.encB_units;
-    sp.encB_units += enc_blocks(d.n, sj.nkb);
+    sj.enc2_begin = sp.enc2_units;
+    if (sj.mat2) {
+      sp.enc2_units += ea + eb;
+      sp.max_bits2 = std::max(sp.max_bits2, sj.bits);
+      sp.max_nmod2 = std::max(sp.max_nmod2, sj.nmod);
+    } else {
+      sp.encA_units += ea;
+      sp.encB_units += eb;
+      sp.max_bits = std::max(sp.max_bits, sj.bits);
+      sp.max_nmod = std::max(sp.max_nmod, sj.nmod);
+      sp.max_np = std::max(sp.max_np, sj.np);
+      sp.all_full = sp.all_full && sj.full;
+      ++sp.n_plan;
+    }
     sj.item_begin = sp.items;
-    // the residue GEMM decodes a job's items with 32-bit arithmetic
-    const int64_t job_items = (int64_t)sj.nmod * sj.np * sj.tiles_m * sj.tiles_n;
-    if (job_items >= ((int64_t)1 << 31)) return HMAT_STATUS_UNSUPPORTED;
-    sp.items += job_items;
-    sp.max_bits = std::max(sp.max_bits, sj.bits);
-    sp.max_nmod = std::max(sp.max_nmod, sj.nmod);
-    sp.max_np = std::max(sp.max_np, sj.np);
+    sp.items += (int64_t)sj.nmod * sj.np * sj.tiles_m * sj.tiles_n;
     sp.max_nkb = std::max(sp.max_nkb, sj.four_m ? 2 * sj.nkb : sj.nkb);
-    sp.all_full = sp.all_full && sj.full;
     sp.n_four_m += sj.four_m ? 1 : 0;
     sp.jobs.push_back(sj);
   }
   // the CRT kernel, and with it the block shape, depends on every job's plan
   for (SplitJob& sj : sp.jobs) {
+    const int64_t blocks = crt_job_blocks(sj, sp.all_full);
     sj.crt_begin = sp.crt_units;
-    sp.crt_units += crt_job_blocks(sj, sp.all_full);
-    sp.all_wide = sp.all_wide && sj.crt_w == kCrtCols;
+    sj.crt2_begin = sp.crt2_units;
+    (sj.mat2 ? sp.crt2_units : sp.crt_units) += blocks;
+    bool& wide = sj.mat2 ? sp.all_wide2 : sp.all_wide;
+    wide = wide && sj.crt_w == kCrtCols;
   }
   if ((size_t)off > ws_bytes) return HMAT_STATUS_WORKSPACE_TOO_SMALL;
   sp.ws_needed = off;
@@ -324,8 +475,8 @@ hmat_status split_prepare(const std::vector<JobDesc>& jobs, const KPlan* h_plans
   return HMAT_STATUS_SUCCESS;
 }
 
-hmat_status split_layout_single(const JobDesc& d, const KPlan& P, double tol, const TileTables& tables, SplitJob* out,
-                                SplitUnits* units) {
+hmat_status split_layout_single(const JobDesc& d, const KPlan& P, double tol, const TileTables& tables, bool mat2,
+                                SplitJob* out, SplitUnits* units) {
   SplitJob sj;
   std::memset(&sj, 0, sizeof(sj));
   sj.d = d;
@@ -333,11 +484,12 @@ hmat_status split_layout_single(const JobDesc& d, const KPlan& P, double tol, co
   int64_t off = 0;
   hmat_status st = layout_job(sh, &P, tol, tables, &sj, &off);
   if (st != HMAT_STATUS_SUCCESS) return st;
+  if ((int64_t)sj.nmod * sj.np * sj.tiles_m * sj.tiles_n >= ((int64_t)1 << 31)) return HMAT_STATUS_UNSUPPORTED;
+  if (mat2 && sj.full) to_mat2(&sj, 0);
   units->exp = (d.m + 31) / 32 + (d.n + 31) / 32;
   units->encA = enc_blocks(d.m, sj.nkb);
   units->encB = enc_blocks(d.n, sj.nkb);
   units->items = (int64_t)sj.nmod * sj.np * sj.tiles_m * sj.tiles_n;
-  if (units->items >= ((int64_t)1 << 31)) return HMAT_STATUS_UNSUPPORTED;
   units->crt = crt_job_blocks(sj, sj.full != 0);
   units->max_bits = sj.bits;
   units->max_nmod = sj.nmod;
@@ -370,6 +522,11 @@ hmat_status split_launch(hmat_context* h, const SplitPrep& sp, const SplitJob* d
     if (!skip_a) e = launch_split_encode(d_jobs, njobs, d_plans, 0, sp.encA_units, stream, ws, sp.max_bits);
     if (e == cudaSuccess && !skip_b)
       e = launch_split_encode(d_jobs, njobs, d_plans, 1, sp.encB_units, stream, ws, sp.max_bits);
+    // the matrix form's blocks: A side first, then B side
+    const int64_t a_blocks = njobs == 1 ? enc_blocks(sp.jobs[0].d.m, sp.jobs[0].nkb) : 0;
+    const int64_t first = skip_a ? a_blocks : 0, end = skip_b ? std::min(a_blocks, sp.enc2_units) : sp.enc2_units;
+    if (e == cudaSuccess && end > first)
+      e = launch_mat2_encode(d_jobs, njobs, end - first, first, stream, ws, sp.max_bits2);
   }
   if (e != cudaSuccess) return split_cuda_error(e);
   {
@@ -380,9 +537,11 @@ hmat_status split_launch(hmat_context* h, const SplitPrep& sp, const SplitJob* d
   if (e != cudaSuccess) return split_cuda_error(e);
   {
     ProfScope ps(h, 4, stream);
-    const int full_form = sp.n_four_m == 0 ? 0 : (sp.n_four_m == njobs ? 1 : 2);
+    const int full_form = sp.n_four_m == 0 ? 0 : (sp.n_four_m == sp.n_plan ? 1 : 2);
     e = launch_split_crt(d_jobs, njobs, d_plans, sp.crt_units, stream, ws, sp.max_nmod, sp.max_np, sp.all_full,
                          full_form, sp.all_wide);
+    if (e == cudaSuccess && sp.crt2_units > 0)
+      e = launch_mat2_crt(d_jobs, njobs, sp.crt2_units, stream, ws, sp.max_nmod2, sp.all_wide2);
   }
   return e == cudaSuccess ? HMAT_STATUS_SUCCESS : split_cuda_error(e);
 }

@@ -1,0 +1,219 @@
+"""The matrix form of the split mode's full biquaternion products (split_mat2.cu).
+
+Modulo p with s^2 = -1 the biquaternions are two copies of the 2 x 2 matrices;
+each copy's product takes Winograd's seven multiplications.  The CPU tests
+restate that algebra and the kernels' exact arithmetic on integers; the GPU
+tests require the bits of Gauss's form, which computes the same exact integers
+through the paper's 24 products.
+"""
+import itertools
+import math
+import random
+
+import numpy as np
+import pytest
+import torch
+
+import bq_inputs as bi
+import paper_2609_02081_gb300 as hm
+
+MODULI = (241, 233, 229, 221, 205, 197, 193, 181, 173, 157, 149, 137, 113, 109, 101, 97, 89, 73)
+TOL = 1e-12
+
+
+def centred(v, p):
+    r = v % p
+    return r - p if r > (p - 1) // 2 else r
+
+
+def root(p):
+    """The root of -1 with the smallest sum of digit weights, up to sign."""
+    def weight(s):
+        return sum(abs(centred(1 << (16 * d), p)) + abs(centred(s << (16 * d), p)) for d in range(3))
+    return min((s for s in range(1, p) if (s * s + 1) % p == 0), key=weight)
+
+
+def quaternion_product(a, b):
+    """Eight real components (M_e + i M_{e+4} the coefficient of 1, i, j, k)."""
+    q, r = [complex(0)] * 4, None
+    A = [(a[e], a[e + 4]) for e in range(4)]
+    B = [(b[e], b[e + 4]) for e in range(4)]
+
+    def mul(x, y):
+        return x[0] * y[0] - x[1] * y[1], x[0] * y[1] + x[1] * y[0]
+    signs = [[(0, 0, 1), (1, 1, -1), (2, 2, -1), (3, 3, -1)], [(0, 1, 1), (1, 0, 1), (2, 3, 1), (3, 2, -1)],
+             [(0, 2, 1), (2, 0, 1), (3, 1, 1), (1, 3, -1)], [(0, 3, 1), (3, 0, 1), (1, 2, 1), (2, 1, -1)]]
+    out = [0] * 8
+    for e, terms in enumerate(signs):
+        for f, g, sg in terms:
+            re, im = mul(A[f], B[g])
+            out[e] += sg * re
+            out[e + 4] += sg * im
+    return out
+
+
+def entries(x):
+    """(Re, Im) of the matrix entries 11, 12, 21, 22 of a biquaternion with integer components."""
+    return [(x[0] - x[5], x[4] + x[1]), (x[2] - x[7], x[6] + x[3]), (-x[2] - x[7], x[3] - x[6]),
+            (x[0] + x[5], x[4] - x[1])]
+
+
+def left(x11, x12, x21, x22):
+    s1 = x21 + x22
+    s2 = s1 - x11
+    return [x11, x12, x12 - s2, x22, s1, s2, x11 - x21]
+
+
+def right(y11, y12, y21, y22):
+    t3 = y22 - y12
+    t2 = t3 + y11
+    return [y11, y21, y22, t2 - y21, y12 - y11, t2, t3]
+
+
+def outputs(u, v):
+    """The kernels' eight sums by (half, slot): 4 times (half 1: 4 s times) the component, modulo p."""
+    out = {}
+    for half, sg in ((0, 1), (1, -1)):
+        t = [a + sg * b for a, b in zip(u, v)]
+        u1 = t[0] + t[5]
+        u2 = u1 + t[6]
+        c11, c12, c21, c22 = t[0] + t[1], u1 + t[4] + t[2], u2 - t[3], u2 + t[4]
+        z = [c11 + c22, c22 - c11, c12 - c21, -(c12 + c21)]
+        for e in range(4):
+            out[(4 * half + e) ^ ((e & 1) << 2)] = -z[e] if half and e & 1 else z[e]
+    return out
+
+
+def test_moduli_and_digit_weights():
+    assert all(math.gcd(a, b) == 1 for a, b in itertools.combinations(MODULI, 2))
+    assert all(p <= 255 and p % 2 == 1 for p in MODULI)
+    for p in MODULI:
+        s = root(p)
+        assert (s * s + 1) % p == 0
+        # u = sum_d x_d w_d + y_d s w_d over balanced 16-bit digits (the fourth below 2^6) is an exact float
+        w = [abs(centred(1 << (16 * d), p)) + abs(centred(s << (16 * d), p)) for d in range(4)]
+        assert sum(w[:3]) * (2 ** 15 + 1) + w[3] * 2 ** 6 < 2 ** 24
+    # 1024-deep sums of products of residues up to 121 are exact in FP32
+    assert 1024 * 121 ** 2 < 2 ** 24
+
+
+def test_matrix_form_recombines_to_the_product():
+    rng = random.Random(3)
+    for p in MODULI:
+        s = root(p)
+        for _ in range(20):
+            a, b = ([rng.randrange(-(1 << 46), (1 << 46) + 1) for _ in range(8)] for _ in range(2))
+            copies = []
+            for sign in (1, -1):
+                x = [(re + sign * s * im) % p for re, im in entries(a)]
+                y = [(re + sign * s * im) % p for re, im in entries(b)]
+                copies.append([centred(f * g, p) for f, g in zip(left(*x), right(*y))])
+            got = outputs(*copies)
+            want = quaternion_product(a, b)
+            for c in range(8):
+                # half 1 (slots 0 and 2: imaginary parts of q1, q3; 1 and 3: real parts of q2, q4) carries s
+                scale = 4 * s if c in (4, 1, 6, 3) else 4
+                assert (got[c] - scale * want[c]) % p == 0, (p, c)
+                assert abs(got[c]) <= 16 * (p - 1) // 2
+
+
+def test_mat2_crt_quotient_is_exact():
+    """S = N P + sum_l x_l d_l with |x_l| <= 16 * 120 and N = nmod * 16 * 120: positive, within the limbs, and the
+    float32 estimate of S / P rounds to the quotient for outputs up to |X| = P / 2^1.25."""
+    W = 16 * 120
+    rng = random.Random(12)
+    for nm in range(1, len(MODULI) + 1):
+        mods = MODULI[:nm]
+        P = math.prod(mods)
+        L = 4 if nm <= 15 else 5
+        pb = max((P.bit_length() - 1) // 32 - 1, 0)
+        pinv = np.float32(1.0 / sum(float((P >> (32 * q)) & 0xFFFFFFFF) * 2.0 ** (32 * (q - pb)) for q in range(pb, L)))
+        assert 2 * nm * W * P < 2 ** (32 * L)
+        lim = int(P / 2 ** 1.25)
+        for carry in (4, None):
+            for trial in range(100):
+                X = rng.choice([lim, -lim, rng.randrange(-lim, lim + 1), rng.randrange(-min(lim, 99), min(lim, 99) + 1)])
+                S = nm * W * P
+                for p in mods:
+                    c = 4 if carry else 4 * root(p) % p
+                    d = P // p * (pow(P // p % p, -1, p) * pow(c, -1, p) % p)
+                    r = c * X % p
+                    lo, hi = -W + (r + W) % p, W - (W - r) % p
+                    S += rng.choice([lo, hi, lo + p * rng.randrange(0, (hi - lo) // p + 1)]) * d
+                assert 0 < S < 2 * nm * W * P
+                limbs = [(S >> (32 * q)) & 0xFFFFFFFF for q in range(L)]
+                sf = np.float32(limbs[L - 1])
+                for q in range(L - 2, pb - 1, -1):
+                    sf = np.float32(sf * np.float32(2.0 ** 32) + np.float32(limbs[q]))
+                assert S - int(np.rint(np.float32(sf * pinv))) * P == X, (nm, X)
+
+
+# ------------------------------------------------------------------ GPU
+@pytest.fixture(scope="module")
+def handles():
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    with hm.Handle() as default, hm.Handle() as gauss:
+        gauss.set_complex_form("gauss")
+        yield default, gauss
+        assert default.device_error() == 0 and gauss.device_error() == 0
+
+
+def stored(op, rows, cols):
+    return (cols, rows) if op in ("T", "H") else (rows, cols)
+
+
+# edges of the encoder's 16 x 32 tiles and the 64-deep k-blocks, of the GEMM's 128-row tiles, its output widths and its
+# 1024-deep chunks, of the CRT's 32- and 128-column blocks (n = 1024) and of the modulus counts (k = 290 / 291 at 1e-12)
+SHAPES = [(1, 1, 1), (16, 32, 64), (17, 33, 65), (128, 256, 290), (129, 257, 291), (40, 1023, 512), (35, 1024, 513),
+          (33, 1025, 1024), (130, 70, 1025), (5, 300, 2049)]
+OPS = ["N", "T", "C", "H", "QC"]
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("tol", [1e-3, 1e-9, 1e-12, 1e-13, 1e-14])
+@pytest.mark.parametrize("i", range(len(SHAPES)))
+def test_default_form_gives_gausss_bits(handles, i, tol):
+    """Both forms recover the same integers and round them once: equal bits, over the digit counts (bits <= 46 and
+    above), the limb counts (15 moduli and more), every op, strided operands, complex alpha / beta and plain stores."""
+    m, n, k = SHAPES[i]
+    opA, opB = OPS[i % 5], OPS[(i * 2 + 1) % 5]
+    dev = torch.device("cuda")
+    (ra, ca), (rb, cb) = stored(opA, m, k), stored(opB, k, n)
+    A = bi.fock_like(800 + i, ra, ca + 3, row_scale=True).to(dev)[:, :, :ca]
+    B = bi.uniform(820 + i, rb, cb + 2).to(dev)[:, :, 1:cb + 1]
+    C0 = bi.uniform(840 + i, m, n + 5).to(dev)
+    for alpha, beta in ((1.0, 0.0), (0.5 - 2j, 0.25 + 1j)):
+        outs = []
+        for h in handles:
+            C = C0.clone()
+            hm.hmat_bq_gemm(h, A, B, C[:, :, :n], opA, opB, alpha=alpha, beta=beta, mode="split", tol=tol)
+            outs.append(C)
+        torch.cuda.synchronize()
+        assert torch.equal(outs[0], outs[1])
+        assert torch.equal(outs[0][:, :, n:], C0[:, :, n:])
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("use_graph", [False, True])
+def test_grouped_matrix_form_beside_other_forms(handles, use_graph):
+    """One grouped call of full products (matrix form; k = 5 at tol 1e-3 keeps its plan's form, which then needs fewer
+    planes) and subalgebra products: the bits of an all-Gauss handle."""
+    dev = torch.device("cuda")
+    shapes = [(64, 64, 5, bi.BQ), (130, 70, 64, bi.BQ), (100, 90, 300, bi.TRS), (33, 1030, 200, bi.BQ), (7, 9, 12, bi.BQ)]
+    mats = [(bi.uniform(860 + i, m, k, flags=f).to(dev), bi.uniform(870 + i, k, n).to(dev), f)
+            for i, (m, n, k, f) in enumerate(shapes)]
+    for tol in (1e-3, TOL):
+        res = []
+        for h in handles:
+            Cs = [torch.full((8, m, n), float("nan"), dtype=torch.float64, device=dev) for m, n, _, _ in shapes]
+            descs = [hm.make_desc(A, B, C, flagsA=f) for (A, B, f), C in zip(mats, Cs)]
+            ws = torch.empty(hm.hmat_workspace_size(h, descs, "split", tol), dtype=torch.uint8, device=dev)
+            s = torch.cuda.Stream()
+            s.wait_stream(torch.cuda.current_stream())
+            for _ in range(2 if use_graph else 1):
+                hm.hmat_bq_gemm_grouped(h, descs, mode="split", tol=tol, workspace=ws, stream=s, use_graph=use_graph)
+            s.synchronize()
+            res.append(Cs)
+        for a, b in zip(*res):
+            assert torch.equal(a, b)
