@@ -256,7 +256,7 @@ def measured_peaks():
 
 # The matrix form of split-mode products (the library's default, csrc/split_mat2.cu): its moduli and, per pair of
 # component flags, the factor planes of each side and the products per modulus.
-MATRIX_FORM_MODULI = (241, 233, 229, 221, 205, 197, 193, 181, 173, 157, 149, 137, 113, 109, 101, 97, 89, 73)
+MATRIX_FORM_MODULI = (241, 233, 229, 221, 205, 197, 193, 181, 173, 157, 149, 137, 113, 109, 101, 97, 89)
 MATRIX_FORM_PLANES = {(0xFF, 0xFF): (14, 14, 14)}
 
 

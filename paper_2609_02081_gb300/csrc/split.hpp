@@ -70,6 +70,7 @@ constexpr int kMat2HalfMax = 120;  // (p - 1)/2 of its largest modulus, 241
 // Most moduli whose sums S < 2 N P fit four 32-bit limbs (P < 2^111.1 and N =
 // 15 * 16 * 120 < 2^14.9; checked when the tables are built)
 constexpr int kMat2FourLimbs = 15;
+constexpr int kMat2MaxModuli = 17; // whose CRT elements (P < 2^124.2) have sixteen 8-bit digits
 // Largest inner dimension for which HMAT_CFORM_AUTO falls back from the matrix
 // form to the four-multiplication form (and whose workspace it reports), not to
 // Gauss's: its products (two terms of depth k) then fit one
@@ -274,10 +275,11 @@ cudaError_t launch_mat2_encode(const SplitJob* d_jobs, int njobs, int64_t units,
                                unsigned char* ws, int max_bits);
 cudaError_t launch_mat2_crt(const SplitJob* d_jobs, int njobs, int64_t units, cudaStream_t s, unsigned char* ws,
                             int max_nmod, bool all_wide);
-// n (kMaxModuli) moduli, root[l]^2 = -1 mod moduli[l], and the CRT tables
-// [n + 1][2][n][kLimbs], [n + 1][kLimbs], [n + 1][kLimbs] by modulus count
+// n (kMat2MaxModuli) moduli, root[l]^2 = -1 mod moduli[l], and by modulus count
+// the CRT tables [n + 1][2][n][kLimbs], [n + 1][kLimbs], [n + 1][kLimbs], all
+// times 2^shift[count]
 cudaError_t mat2_configure(const int* moduli, const int* root, int n, const int32_t* crt_d, const uint32_t* crt_P,
-                           const uint32_t* crt_off);
+                           const uint32_t* crt_off, const int* shift);
 // Constants of the CRT's quotient estimate for the modulus product P: pb the
 // limb below its top one, pinv = fl(2^(32 pb) / P).  False when the estimate's
 // error on sums below max_quotient P could miss the quotient with `limbs` limbs.

@@ -3,7 +3,8 @@
 // Work item = (problem, modulus l, product p, 128 x bn output tile).  For the
 // item the kernel computes T = L_f R_g^T over the padded inner dimension, where
 // L_f / R_g are the BF16-encoded residues of the plan's left / right factors
-// (values in [-128, 128]), and stores T mod p_l (centred int8).  A two-term
+// (values in [-128, 128]), and stores T mod p_l (centred int8; the matrix
+// form's with 128 added).  A two-term
 // product (the four-multiplication form of a complex product) accumulates
 // L_f R_g^T +- L_f' R_g'^T in one accumulator: the k-blocks of the second
 // term follow those of the first, its sign through the negate-B bit.
@@ -252,10 +253,11 @@ __device__ __forceinline__ float2 fmod_centred2(float2 v, float2 npf, float2 inv
   return __ffma2_rn(q, npf, v);
 }
 
-// the int8 residues of four centred values (|t| <= 128) in one word: the low
-// byte of the bits of t + 1.5 * 2^23 is t mod 256 (two's complement)
-__device__ __forceinline__ uint32_t pack4_residues(float2 t01, float2 t23) {
-  const float2 m = make_float2(12582912.0f, 12582912.0f);
+// the residues of four centred values (|t| <= 128) as bytes of one word: the low
+// byte of the bits of t + magic is t mod 256 (two's complement) with magic = 1.5 *
+// 2^23, and t + 128 with 128 more (the matrix form's unsigned bytes)
+__device__ __forceinline__ uint32_t pack4_residues(float2 t01, float2 t23, float magic) {
+  const float2 m = make_float2(magic, magic);
   const float2 u01 = __fadd2_rn(t01, m), u23 = __fadd2_rn(t23, m);
   return __byte_perm(__byte_perm(__float_as_uint(u01.x), __float_as_uint(u01.y), 0x0040),
                      __byte_perm(__float_as_uint(u23.x), __float_as_uint(u23.y), 0x0040), 0x5410);
@@ -266,6 +268,7 @@ __device__ __forceinline__ uint32_t pack4_residues(float2 t01, float2 t23) {
 struct GemmModConst {
   int p;
   float pf, inv;
+  float magic;        // of the stored byte (pack4_residues)
 };
 __constant__ GemmModConst c_gmod[2 * kModTable];   // the plans' moduli, then the matrix form's
 
@@ -409,7 +412,7 @@ split_residue_gemm_kernel(const SplitJob* __restrict__ jobs, int njobs, int64_t 
       const int cols = it.bn >> 1;        // columns handled by this thread: a multiple of 16 up to 128
       const int col0 = half * cols;
       const int nchunks = (it.nkb + kKbPerChunk - 1) / kKbPerChunk;
-      const float pf = c_gmod[it.l].pf, pinv = c_gmod[it.l].inv;
+      const float pf = c_gmod[it.l].pf, pinv = c_gmod[it.l].inv, magic = c_gmod[it.l].magic;
       const float2 npf2 = make_float2(-pf, -pf), inv2 = make_float2(pinv, pinv);
       if (nchunks == 1) {
         // One chunk: each 32-column load is reduced and stored at once.
@@ -444,7 +447,7 @@ split_residue_gemm_kernel(const SplitJob* __restrict__ jobs, int njobs, int64_t 
                   t01 = fmod_centred2(t01, npf2, inv2);
                   t23 = fmod_centred2(t23, npf2, inv2);
                 }
-                w[v] = pack4_residues(t01, t23);
+                w[v] = pack4_residues(t01, t23, magic);
               }
               *reinterpret_cast<uint4*>(dst + c16) = make_uint4(w[0], w[1], w[2], w[3]);
             }
@@ -548,7 +551,7 @@ split_residue_gemm_kernel(const SplitJob* __restrict__ jobs, int njobs, int64_t 
             for (int v = 0; v < 4; ++v) {
               const int b = g * 16 + v * 4;
               w[v] = pack4_residues(fmod_centred2(make_float2(acc[b], acc[b + 1]), npf2, inv2),
-                                    fmod_centred2(make_float2(acc[b + 2], acc[b + 3]), npf2, inv2));
+                                    fmod_centred2(make_float2(acc[b + 2], acc[b + 3]), npf2, inv2), magic);
             }
             *reinterpret_cast<uint4*>(dst + g * 16) = make_uint4(w[0], w[1], w[2], w[3]);
           }
@@ -595,6 +598,7 @@ cudaError_t split_gemm_configure(const int* moduli, int n) {
     g[l].p = p;
     g[l].pf = (float)p;
     g[l].inv = 1.0f / (float)p;
+    g[l].magic = l < kModTable ? 12582912.0f : 12583040.0f;
   }
   cudaError_t e = cudaMemcpyToSymbol(c_gmod, g, sizeof(g));
   if (e != cudaSuccess) return e;

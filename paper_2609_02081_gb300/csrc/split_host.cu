@@ -21,10 +21,10 @@ static const int kModuli[kModTable] = {255, 253, 251, 247, 241, 239, 233, 229, 2
 
 // Matrix form: odd, pairwise coprime moduli below 255 all of whose prime
 // factors are 1 modulo 4 (221 = 13*17, 205 = 5*41, the rest prime), so that -1
-// has a square root modulo each: the largest eighteen, 130.4 bits together.
-// 257 is left out: its centred residues do not fit int8.
-static const int kMat2Moduli[kMaxModuli] = {241, 233, 229, 221, 205, 197, 193, 181, 173,
-                                            157, 149, 137, 113, 109, 101, 97,  89,  73};
+// has a square root modulo each: the largest seventeen, 124.2 bits together.
+// 257 is left out: its centred residues do not fit a byte.
+static const int kMat2Moduli[kMat2MaxModuli] = {241, 233, 229, 221, 205, 197, 193, 181, 173,
+                                                157, 149, 137, 113, 109, 101, 97,  89};
 
 // Margin (bits) between the requested tolerance and the integer width: the
 // scaling error of one operand element is <= 2^-b of its row/column maximum,
@@ -98,7 +98,7 @@ int mat2_moduli(int64_t k, int bits) {
   double acc = 0.0;
   int n = 0;
   while (acc <= need) {
-    if (n >= kMaxModuli) return 0;
+    if (n >= kMat2MaxModuli) return 0;
     acc += std::log2((double)kMat2Moduli[n++]);
   }
   return n;
@@ -142,14 +142,15 @@ uint32_t inv_mod(uint32_t a, uint32_t m) {
 }
 // CRT basis element of moduli[l] among the first n: congruent to c modulo p_l
 // and to 0 modulo the others, below P, in signed 32-bit digits (each word above
-// 2^31 - 1 borrows from the next)
-bool crt_element(const int* moduli, int n, int l, uint32_t c, int32_t* digits) {
+// 2^31 - 1 borrows from the next); times 2^shift
+bool crt_element(const int* moduli, int n, int l, uint32_t c, int32_t* digits, int shift = 0) {
   const uint32_t p = (uint32_t)moduli[l];
   uint32_t Ml[kLimbs] = {1, 0, 0, 0, 0};
   for (int j = 0; j < n; ++j)
     if (j != l) big_mul_small(Ml, (uint32_t)moduli[j]);
   const uint32_t inv = inv_mod(big_mod_small(Ml, p), p);
   big_mul_small(Ml, (uint32_t)((unsigned long long)inv * (c % p) % p));
+  for (int i = 0; i < shift; ++i) big_mul_small(Ml, 2u);
   long long carry = 0;
   for (int q = 0; q < kLimbs; ++q) {
     long long w = (long long)Ml[q] + carry;
@@ -167,29 +168,36 @@ bool crt_element(const int* moduli, int n, int l, uint32_t c, int32_t* digits) {
 // elements carrying 1/4 (outputs formed from the sums of the two matrix copies)
 // and 1/(4 s) (from their differences), the products P and the offsets.
 cudaError_t mat2_configure_tables() {
-  static int32_t crt[kMaxModuli + 1][2][kMaxModuli][kLimbs];
-  static uint32_t P[kMaxModuli + 1][kLimbs], off[kMaxModuli + 1][kLimbs];
+  static int32_t crt[kMat2MaxModuli + 1][2][kMat2MaxModuli][kLimbs];
+  static uint32_t P[kMat2MaxModuli + 1][kLimbs], off[kMat2MaxModuli + 1][kLimbs];
   std::memset(crt, 0, sizeof(crt));
   std::memset(P, 0, sizeof(P));
   std::memset(off, 0, sizeof(off));
-  int root[kMaxModuli];
-  for (int l = 0; l < kMaxModuli; ++l) {
+  int root[kMat2MaxModuli], shift[kMat2MaxModuli + 1] = {};
+  for (int l = 0; l < kMat2MaxModuli; ++l) {
     root[l] = mat2_root(kMat2Moduli[l]);
     if (root[l] == 0) return cudaErrorInvalidValue;
   }
-  for (int n = 1; n <= kMaxModuli; ++n) {
+  for (int n = 1; n <= kMat2MaxModuli; ++n) {
     P[n][0] = 1;
-    for (int l = 0; l < n; ++l) big_mul_small(P[n], (uint32_t)kMat2Moduli[l]);
+    double log2P = 0.0;
+    for (int l = 0; l < n; ++l) {
+      big_mul_small(P[n], (uint32_t)kMat2Moduli[l]);
+      log2P += std::log2((double)kMat2Moduli[l]);
+    }
+    if (n <= kMat2FourLimbs)                         // 2 N P in (2^126.9, 2^127.99)
+      shift[n] = (int)std::floor(127.99 - log2P - std::log2(2.0 * n * kMat2WeightSum * kMat2HalfMax));
+    for (int i = 0; i < shift[n]; ++i) big_mul_small(P[n], 2u);
     std::memcpy(off[n], P[n], sizeof(off[n]));
     big_mul_small(off[n], (uint32_t)(n * kMat2WeightSum * kMat2HalfMax));
     for (int l = 0; l < n; ++l) {
       const uint32_t p = (uint32_t)kMat2Moduli[l];
-      if (!crt_element(kMat2Moduli, n, l, inv_mod(4u, p), crt[n][0][l]) ||
-          !crt_element(kMat2Moduli, n, l, inv_mod(4u * (uint32_t)root[l] % p, p), crt[n][1][l]))
+      if (!crt_element(kMat2Moduli, n, l, inv_mod(4u, p), crt[n][0][l], shift[n]) ||
+          !crt_element(kMat2Moduli, n, l, inv_mod(4u * (uint32_t)root[l] % p, p), crt[n][1][l], shift[n]))
         return cudaErrorInvalidValue;
     }
   }
-  return mat2_configure(kMat2Moduli, root, kMaxModuli, &crt[0][0][0][0], &P[0][0], &off[0][0]);
+  return mat2_configure(kMat2Moduli, root, kMat2MaxModuli, &crt[0][0][0][0], &P[0][0], &off[0][0], shift);
 }
 
 }  // namespace
@@ -221,7 +229,7 @@ cudaError_t split_configure() {
   int moduli[2 * kModTable];
   for (int l = 0; l < kModTable; ++l) {
     moduli[l] = kModuli[l];
-    moduli[kModTable + l] = l < kMaxModuli ? kMat2Moduli[l] : kMat2Moduli[0];
+    moduli[kModTable + l] = l < kMat2MaxModuli ? kMat2Moduli[l] : kMat2Moduli[0];
   }
   return split_gemm_configure(moduli, 2 * kModTable);
 }

@@ -17,7 +17,7 @@ import torch
 import bq_inputs as bi
 import paper_2609_02081_gb300 as hm
 
-MODULI = (241, 233, 229, 221, 205, 197, 193, 181, 173, 157, 149, 137, 113, 109, 101, 97, 89, 73)
+MODULI = (241, 233, 229, 221, 205, 197, 193, 181, 173, 157, 149, 137, 113, 109, 101, 97, 89)
 TOL = 1e-12
 
 
@@ -117,35 +117,102 @@ def test_matrix_form_recombines_to_the_product():
                 assert abs(got[c]) <= 16 * (p - 1) // 2
 
 
+def shift_of(nm):
+    """Power of two by which the tables of up to 15 moduli are scaled: 2 N P just below 2^128."""
+    if nm > 15:
+        return 0
+    return math.floor(127.99 - sum(math.log2(p) for p in MODULI[:nm]) - math.log2(2 * nm * 16 * 120))
+
+
+def elements_of(nm, half):
+    mods, P = MODULI[:nm], math.prod(MODULI[:nm])
+    return [(P // p * (pow(P // p % p, -1, p) * pow(4 * root(p) if half else 4, -1, p) % p)) << shift_of(nm)
+            for p in mods]
+
+
 def test_mat2_crt_quotient_is_exact():
     """S = N P + sum_l x_l d_l with |x_l| <= 16 * 120 and N = nmod * 16 * 120: positive, within the limbs, and the
-    float32 estimate of S / P rounds to the quotient for outputs up to |X| = P / 2^1.25."""
+    float32 estimate of S / P rounds to the quotient for outputs up to |X| = P / 2^1.25: from the leading limb alone
+    (up to 15 moduli, scaled to fill 128 bits), or from the limbs from the one below P's top."""
     W = 16 * 120
     rng = random.Random(12)
     for nm in range(1, len(MODULI) + 1):
-        mods = MODULI[:nm]
-        P = math.prod(mods)
+        mods, sh = MODULI[:nm], shift_of(nm)
+        P = math.prod(mods) << sh
         L = 4 if nm <= 15 else 5
         pb = max((P.bit_length() - 1) // 32 - 1, 0)
         pinv = np.float32(1.0 / sum(float((P >> (32 * q)) & 0xFFFFFFFF) * 2.0 ** (32 * (q - pb)) for q in range(pb, L)))
         assert 2 * nm * W * P < 2 ** (32 * L)
-        lim = int(P / 2 ** 1.25)
-        for carry in (4, None):
+        lim = int((P >> sh) / 2 ** 1.25)
+        for half in (0, 1):
+            d = elements_of(nm, half)
             for trial in range(100):
                 X = rng.choice([lim, -lim, rng.randrange(-lim, lim + 1), rng.randrange(-min(lim, 99), min(lim, 99) + 1)])
                 S = nm * W * P
-                for p in mods:
-                    c = 4 if carry else 4 * root(p) % p
-                    d = P // p * (pow(P // p % p, -1, p) * pow(c, -1, p) % p)
+                for p, dl in zip(mods, d):
+                    c = 4 * root(p) % p if half else 4
                     r = c * X % p
                     lo, hi = -W + (r + W) % p, W - (W - r) % p
-                    S += rng.choice([lo, hi, lo + p * rng.randrange(0, (hi - lo) // p + 1)]) * d
+                    S += rng.choice([lo, hi, lo + p * rng.randrange(0, (hi - lo) // p + 1)]) * dl
                 assert 0 < S < 2 * nm * W * P
                 limbs = [(S >> (32 * q)) & 0xFFFFFFFF for q in range(L)]
                 sf = np.float32(limbs[L - 1])
                 for q in range(L - 2, pb - 1, -1):
                     sf = np.float32(sf * np.float32(2.0 ** 32) + np.float32(limbs[q]))
-                assert S - int(np.rint(np.float32(sf * pinv))) * P == X, (nm, X)
+                assert S - int(np.rint(np.float32(sf * pinv))) * P == X << sh, (nm, X)
+                if nm <= 15:
+                    q = int(np.rint(float(np.float32(limbs[3])) * float(np.float32(2.0 ** 96 / P))))
+                    assert S - q * P == X << sh, (nm, X)
+
+
+def test_mat2_crt_digit_sums():
+    """The CRT's contraction restated: residues stored with 128 added, the sums c11, c22, c12, c21 of both copies (at
+    most 2048, exact in FP16), u + v and u - v times the balanced 8-bit digits of the CRT elements, sums below 2^22,
+    packed in pairs below 2^31; together with an offset less 128 times the weights they give N P + sum_l x_l d_l."""
+    rng = random.Random(13)
+    weights = {0: (1536, 512, 512, -1536), 1: (0, 0, 0, 0)}
+    for nm in (1, 2, 14, 15, 16, 17):
+        mods = MODULI[:nm]
+        P = math.prod(mods) << shift_of(nm)
+        for half, sg in ((0, 1), (1, -1)):
+            elements, digits = elements_of(nm, half), []
+            for e in elements:
+                dl = []
+                for _ in range(17):
+                    v = (e + 128) % 256 - 128
+                    dl.append(v)
+                    e = (e - v) >> 8
+                assert e == 0 and dl[16] == 0
+                digits.append(dl[:16])
+            for i in range(16):
+                worst = sum(abs(dl[i]) * 8 * ((p - 1) // 2 + 128) for dl, p in zip(digits, mods))
+                assert worst < 2 ** 22
+            for trial in range(20):
+                ext = trial < 4                                    # extreme residues first
+                u, v = ([[(p - 1) // 2 * (1 if (trial ^ which) & 1 else -1) if ext else
+                          rng.randrange(-((p - 1) // 2), (p - 1) // 2 + 1) for _ in range(7)] for p in mods]
+                        for which in (0, 1))
+                true = [outputs(a, b) for a, b in zip(u, v)]
+
+                def sums(t):
+                    u1 = t[0] + t[5]
+                    return [t[0] + t[1], u1 + t[6] + t[4], u1 + t[4] + t[2], u1 + t[6] - t[3]]
+                cu, cv = ([sums([x + 128 for x in row]) for row in side] for side in (u, v))
+                assert all(0 <= abs(x) <= 2048 for side in (cu, cv) for row in side for x in row)
+                tt = [[a + sg * b for a, b in zip(x, y)] for x, y in zip(cu, cv)]
+                assert all(abs(x) <= 2048 for row in tt for x in row)
+                pairs = [[sum(row[e] * (dl[2 * i] + 256 * dl[2 * i + 1]) for row, dl in zip(tt, digits))
+                          for i in range(8)] for e in range(4)]
+                z = [[a + b for a, b in zip(pairs[0], pairs[1])], [b - a for a, b in zip(pairs[0], pairs[1])],
+                     [a - b for a, b in zip(pairs[2], pairs[3])], [-(a + b) for a, b in zip(pairs[2], pairs[3])]]
+                for slot in range(4):
+                    if half and slot & 1:
+                        z[slot] = [-x for x in z[slot]]
+                    assert all(abs(x) < 2 ** 31 for x in z[slot])
+                    off = nm * 16 * 120 * P - weights[half][slot] * sum(elements)
+                    S = off + sum(x << (16 * i) for i, x in enumerate(z[slot]))
+                    comp = (4 * half + slot) ^ ((slot & 1) << 2)
+                    assert S == nm * 16 * 120 * P + sum(t[comp] * e for t, e in zip(true, elements))
 
 
 # ------------------------------------------------------------------ GPU
