@@ -257,13 +257,14 @@ def measured_peaks():
 # The matrix form of split-mode products (the library's default, csrc/split_mat2.cu): its moduli and, per pair of
 # component flags, the factor planes of each side and the products per modulus.
 MATRIX_FORM_MODULI = (241, 233, 229, 221, 205, 197, 193, 181, 173, 157, 149, 137, 113, 109, 101, 97, 89)
-MATRIX_FORM_PLANES = {(0xFF, 0xFF): (14, 14, 14)}
+MATRIX_FORM_PLANES = {(0xFF, 0xFF): (14, 14, 14), (0x11, 0xFF): (2, 8, 8), (0xFF, 0x11): (8, 2, 8), (0x11, 0x11): (2, 2, 2),
+                      **{(q, 0xFF): (7, 14, 14) for q in (0x0F, 0xF0)}, **{(0xFF, q): (14, 7, 14) for q in (0x0F, 0xF0)},
+                      **{(p, q): (7, 7, 7) for p in (0x0F, 0xF0) for q in (0x0F, 0xF0)}}
 
 
-def matrix_form(hm, k, tol, fa, fb, algo="bilinear", complex_form="auto", planned=24):
+def matrix_form(hm, k, tol, fa, fb, algo="bilinear", complex_form="auto"):
     """(moduli, left planes, right planes, products) of the matrix form when a split-mode product of inner dimension
-    k runs in it, else None: the default complex form, where its planes do not outnumber the plan's (`planned` per
-    modulus)."""
+    k runs in it, else None: the default complex form, where its planes do not outnumber the plan's."""
     planes = MATRIX_FORM_PLANES.get((fa, fb))
     if planes is None or algo != "bilinear" or complex_form != "auto":
         return None
@@ -274,6 +275,7 @@ def matrix_form(hm, k, tol, fa, fb, algo="bilinear", complex_form="auto", planne
             return None
         acc += math.log2(MATRIX_FORM_MODULI[n])
         n += 1
+    planned = 16 if fa == fb == 0xFF and k <= 512 else hm.plan_info("N", "N", fa, fb)[0]
     return (n, *planes) if n * planes[2] <= len(mods) * planned else None
 
 
@@ -300,7 +302,7 @@ def split_stage_work(hm, shapes, tol, opA="N", opB="N", fa=0xFF, fb=0xFF, algo="
     for m, n, k in shapes:
         T, P, nlf, nrf = four if complex_form == "four_m" or (complex_form == "auto" and k <= 512) else gauss
         L = len(hm.split_info(k, tol)[0])
-        mat = matrix_form(hm, k, tol, fa, fb, algo, complex_form, P)
+        mat = matrix_form(hm, k, tol, fa, fb, algo, complex_form)
         if mat:
             L, nlf, nrf, P = mat
             T = P
@@ -519,7 +521,7 @@ def ours(args, rank, world, local):
     mods, bits = hm.split_info(kin, args.tol)
     nmods = len(mods)
     if args.mode == "split":
-        mat = matrix_form(hm, kin, args.tol, fa, fb, args.algo, args.complex_form, 16 if k <= 512 else 24)
+        mat = matrix_form(hm, kin, args.tol, fa, fb, args.algo, args.complex_form)
         if mat:
             nmods, P = mat[0], mat[3]
     if rank == 0:

@@ -319,13 +319,13 @@ int32_t hmat_last_bad_index(hmat_handle handle);
 HMAT_API
 hmat_status hmat_set_algorithm(hmat_handle handle, int32_t algo);
 
-/* Form of the complex products of split-mode products whose operands are
- * both full biquaternions (flags 0xFF) under the BILINEAR algorithm.
+/* Form of split-mode products under the BILINEAR algorithm.
  *   HMAT_CFORM_GAUSS:  each of the eight complex products P_r of Eq.
  *                      bilinearH as Gauss's three real products (Eq.
  *                      cmplx-3-real-mult), as in the paper: 24 residue
  *                      GEMMs per modulus, 24 encoded factor planes per side;
- *   HMAT_CFORM_FOUR_M: Re P_r = Re X Re Y - Im X Im Y and
+ *   HMAT_CFORM_FOUR_M: (full biquaternions, flags 0xFF; other pairs as GAUSS)
+ *                      Re P_r = Re X Re Y - Im X Im Y and
  *                      Im P_r = Re X Im Y + Im X Re Y, each one real GEMM
  *                      over twice the inner dimension (the second term's
  *                      sign through the MMA's negate bit): 16 residue GEMMs
@@ -333,22 +333,25 @@ hmat_status hmat_set_algorithm(hmat_handle handle, int32_t algo);
  *                      multiplications, 2/3 of the bytes of the encoded
  *                      planes and the product residues;
  *   HMAT_CFORM_AUTO:   (default) the matrix form: modulo p with a square root
- *                      s of -1 the biquaternions are two copies of the 2 x 2
- *                      matrices (i -> s, i -> -s), each product of which takes
- *                      seven multiplications: 14 residue GEMMs per modulus and
- *                      14 factor planes per side, over its own moduli (all prime
- *                      factors 1 modulo 4).  Where those planes would outnumber
- *                      the plan's (a few k below 16 at loose tolerances):
- *                      FOUR_M for inner dimensions up to 512, where a product's
- *                      two terms fit one exact FP32 accumulation chunk of the
- *                      residue GEMM, GAUSS above.
+ *                      s of -1 the complex numbers are two copies of the
+ *                      integers (i -> s, i -> -s) and the quaternions are the
+ *                      2 x 2 matrices, whose product takes seven
+ *                      multiplications.  Residue GEMMs per modulus: full x
+ *                      full and real (or i times real) quaternion x full 14
+ *                      (Gauss's form 24 and 16), quaternion x quaternion 7 (8),
+ *                      complex x full 8 (12), complex x complex 2 (3), over its
+ *                      own moduli (all prime factors 1 modulo 4).  Other flag
+ *                      pairs, and products whose plan then needs fewer planes
+ *                      (a few k below 16 at loose tolerances), keep their plan:
+ *                      for full operands FOUR_M for inner dimensions up to 512,
+ *                      where a product's two terms fit one exact FP32
+ *                      accumulation chunk of the residue GEMM, GAUSS above.
  * Every residue is exact in all forms, so all give the same bits.
- * Other flag pairs and FP64 mode always use Gauss's form; streamed products
- * take the matrix form under AUTO and Gauss's form otherwise;
- * hmat_bq_gemm_split_noalloc follows the setting.  hmat_workspace_size and
- * hmat_workspace_size_modes follow the setting: FOUR_M needs less than GAUSS,
- * and AUTO reports FOUR_M's bytes for k up to 512 and GAUSS's above, inside
- * which the matrix form runs.
+ * FP64 mode always uses the plan.  Streamed products take the matrix form under
+ * AUTO and Gauss's form otherwise; hmat_bq_gemm_split_noalloc follows the
+ * setting.  hmat_workspace_size and hmat_workspace_size_modes follow the
+ * setting: FOUR_M needs less than GAUSS, and AUTO reports FOUR_M's bytes for k up
+ * to 512 and GAUSS's above, inside which the matrix form runs.
  * Errors: NOT_INITIALIZED, INVALID_VALUE (unknown form). */
 HMAT_API
 hmat_status hmat_set_complex_form(hmat_handle handle, int32_t form);

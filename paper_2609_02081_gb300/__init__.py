@@ -252,9 +252,9 @@ class Handle:
         _check(lib().hmat_set_algorithm(self._h, a), "hmat_set_algorithm")
 
     def set_complex_form(self, form):
-        """Form of split-mode full-biquaternion products: 'auto' (default: two 2 x 2 matrix products
-        modulo suitable moduli, seven multiplications each), 'gauss' (three real products per complex
-        one, as in the paper) or 'four_m' (two real products over 2 k).  All give the same bits."""
+        """Form of split-mode products: 'auto' (default: 2 x 2 matrix products modulo suitable moduli,
+        seven multiplications each), 'gauss' (three real products per complex one, as in the paper) or
+        'four_m' (full biquaternions: two real products over 2 k).  All give the same bits."""
         f = CFORMS[form] if isinstance(form, str) else int(form)
         _check(lib().hmat_set_complex_form(self._h, f), "hmat_set_complex_form")
 

@@ -423,8 +423,8 @@ int split_plan_algo(int32_t cform, int palgo, uint32_t fa, uint32_t fb, int64_t 
   return palgo;
 }
 
-// Full biquaternion products may run in the matrix form: the default complex
-// form under the bilinear algorithm.  A form chosen by name is the one that runs.
+// Products may run in the matrix form: the default complex form under the
+// bilinear algorithm.  A form chosen by name is the one that runs.
 static bool mat2_allowed(const hmat_context* h) {
   return h->cform == HMAT_CFORM_AUTO && h->algo == HMAT_ALGO_BILINEAR;
 }
@@ -1070,7 +1070,7 @@ hmat_status hmat_bq_gemm_split_noalloc(hmat_handle h, int32_t opA, int32_t opB, 
     e = launch_split_gemm(a.job, 1, u.items, (int)std::min<int64_t>(u.items, h->sm_count), stream, a.scratch,
                           u.max_nkb);
   if (e == cudaSuccess && sj.mat2)
-    e = launch_mat2_crt(a.job, 1, u.crt, stream, a.scratch, u.max_nmod, sj.crt_w == kCrtCols);
+    e = launch_mat2_crt(a.job, 1, u.crt, stream, a.scratch, u.max_nmod);
   else if (e == cudaSuccess)
     e = launch_split_crt(a.job, 1, h->d_plans, u.crt, stream, a.scratch, u.max_nmod, u.max_np, u.all_full,
                          u.four_m ? 1 : 0, sj.crt_w == kCrtCols);

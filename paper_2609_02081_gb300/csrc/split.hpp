@@ -20,13 +20,13 @@
 //                  the moduli (exact integer of up to ~140 bits), conversion to
 //                  FP64, the 2^-(s_i + t_j) rescaling and the complex alpha/beta
 //                  update (Sec. III scaling and addition).
-// Full biquaternion products run by default in the matrix form
-// (split_mat2.cu), which replaces the plan's products by fewer ones that exist
-// only modulo suitable p: with s^2 = -1 (mod p) the biquaternions modulo p are
-// two copies of the 2 x 2 matrices modulo p (i -> s and i -> -s), and each 2 x 2
-// product takes seven multiplications (Strassen's, in Winograd's variant): 14
-// residue GEMMs per modulus instead of 24.  The integers that the CRT recovers,
-// and so the results, are the same.
+// Most products run by default in the matrix form (split_mat2.cu), which
+// replaces the plan's products by fewer ones that exist only modulo suitable p:
+// with s^2 = -1 (mod p) the biquaternions modulo p are two copies of the 2 x 2
+// matrices modulo p (i -> s and i -> -s), and each 2 x 2 product takes seven
+// multiplications (Strassen's, in Winograd's variant): 14 residue GEMMs per
+// modulus instead of 24.  The integers that the CRT recovers, and so the results,
+// are the same.
 // The only rounding is step 2's scaling to b-bit integers; b and the modulus
 // count follow from the requested tolerance and k.
 #pragma once
@@ -62,9 +62,20 @@ inline int crt_width(int64_t n) { return n >= 1024 ? kCrtCols : 32; }
 // residue sum satisfies |4Q| <= 36 * 127 = 4572, which the CRT's integer
 // residue step relies on.  Plans above it are refused.
 constexpr int kMaxWeightSum = 36;
-// Matrix form: residue planes per modulus (factors per side and products), and
-// the largest sum of product residues in one output: |sum| <= 16 (p - 1)/2.
-constexpr int kMat2Planes = 14;
+// Matrix form (split_mat2.cu).  What a job multiplies (SplitJob::mat2), by the
+// operands' component flags: a pair of 2 x 2 products (full biquaternions, or one of
+// them a real or i times a real quaternion), one 2 x 2 product (two such
+// quaternions), a complex operand times the four coefficients of a full one, two
+// complex operands.
+enum { kMat2None = 0, kMat2Full = 1, kMat2Quat = 2, kMat2Scaled = 3, kMat2Complex = 4 };
+struct Mat2Shape {
+  int kind = kMat2None;
+  int nlf = 0, nrf = 0, np = 0;      // factor planes per side and products per modulus
+  int rot = 0;                       // the product is i^rot times that of the operands as encoded
+};
+Mat2Shape mat2_shape(uint32_t fa, uint32_t fb);
+constexpr int kMat2MaxPlanes = 14;
+// the largest sum of product residues in one output: |sum| <= 16 (p - 1)/2
 constexpr int kMat2WeightSum = 16;
 constexpr int kMat2HalfMax = 120;  // (p - 1)/2 of its largest modulus, 241
 // Most moduli whose sums S < 2 N P fit four 32-bit limbs (P < 2^111.1 and N =
@@ -132,7 +143,7 @@ struct SplitJob {
   int64_t off_res;                  // int8 product residues
   int64_t encA_plane, encB_plane;   // bytes between consecutive (modulus, factor) tile planes
   int64_t res_plane;                // bytes between consecutive (modulus, product) residue planes
-  int32_t mat2;                     // matrix form: its own moduli, encoder and CRT (np = nlf = nrf = kMat2Planes)
+  int32_t mat2, rot;                // matrix form (kMat2None: a plan's products): kind, power of i of the result
   int32_t mod_base;                 // first modulus in the GEMM's table (kModTable: the matrix form's moduli)
   int64_t item_begin;               // residue-GEMM work items before this job
   int64_t encA_begin, encB_begin;   // encode blocks before this job (matrix-form jobs have none)
@@ -183,7 +194,6 @@ struct SplitPrep {
   int64_t exp_units = 0, encA_units = 0, encB_units = 0, items = 0, crt_units = 0;
   int64_t enc2_units = 0, crt2_units = 0;   // matrix-form jobs
   int max_bits2 = 0, max_nmod2 = 0;         // matrix-form jobs (max_bits, max_nmod, max_np: the others)
-  bool all_wide2 = true;                    // matrix-form jobs: every CRT block is one row of kCrtCols columns
   int64_t ws_needed = 0;
   int max_bits = 0, max_nmod = 0, max_np = 0, max_nkb = 0;
   bool all_full = true;             // every job outside the matrix form uses the paper's full plan (either form)
@@ -207,7 +217,7 @@ hmat_status split_b_region_bytes(const SplitShape& sh, double tol, const TileTab
 void split_place_b(SplitJob& sj, int64_t offset);
 
 // Lay the jobs out in a workspace of ws_bytes (WORKSPACE_TOO_SMALL if it does not fit).
-// mat2: full biquaternion products run in the matrix form inside the bytes that
+// mat2: products that have a matrix form run in it inside the bytes that
 // their plan's form occupies (the workspace a caller must bring does not depend
 // on it); products for which it has no advantage keep the plan's form.
 hmat_status split_prepare(const std::vector<JobDesc>& jobs, const KPlan* h_plans, double tol, size_t ws_bytes,
@@ -274,7 +284,7 @@ cudaError_t launch_split_crt(const SplitJob* d_jobs, int njobs, const KPlan* d_p
 cudaError_t launch_mat2_encode(const SplitJob* d_jobs, int njobs, int64_t units, int64_t first, cudaStream_t s,
                                unsigned char* ws, int max_bits);
 cudaError_t launch_mat2_crt(const SplitJob* d_jobs, int njobs, int64_t units, cudaStream_t s, unsigned char* ws,
-                            int max_nmod, bool all_wide);
+                            int max_nmod);
 // n (kMat2MaxModuli) moduli, root[l]^2 = -1 mod moduli[l], and by modulus count
 // the CRT tables [n + 1][2][n][kLimbs], [n + 1][kLimbs], [n + 1][kLimbs], all
 // times 2^shift[count]

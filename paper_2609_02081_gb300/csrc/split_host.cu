@@ -295,26 +295,54 @@ static void place_job(SplitJob* sj, int64_t m, int64_t n, int64_t* offset) {
   *offset = off;
 }
 
-// Turns a full-plan job laid out at *offset0 into the matrix form, inside the
-// bytes its plan's form occupies.  The form wins wherever its planes (14 per
-// modulus, one or two moduli more) do not outnumber the plan's (24, or 16 in the
-// four-multiplication form), which also keeps it inside those bytes; that leaves
-// out a few tiny k at loose tolerances (k <= 15 at tol 1e-3: 6 x 14 planes
-// against 5 x 16).  Measured at tol 1e-12: m = n = k = 8192, 15 x 14 planes
-// against Gauss's 14 x 24: 226 -> 144 ms; the 512-product batch: 31.9 -> 23.5 ms.
+Mat2Shape mat2_shape(uint32_t fa, uint32_t fb) {
+  enum { kNone, kFull, kReal, kImag, kCplx };
+  auto what = [](uint32_t f) {
+    return f == 0xFFu ? kFull : f == 0x0Fu ? kReal : f == 0xF0u ? kImag : f == 0x11u ? kCplx : kNone;
+  };
+  const int a = what(fa), b = what(fb);
+  const bool qa = a == kReal || a == kImag, qb = b == kReal || b == kImag;
+  const int rot = (a == kImag ? 1 : 0) + (b == kImag ? 1 : 0);
+  if ((a == kFull || qa) && (b == kFull || qb)) {
+    if (qa && qb) return Mat2Shape{kMat2Quat, 7, 7, 7, rot};
+    return Mat2Shape{kMat2Full, qa ? 7 : 14, qb ? 7 : 14, 14, rot};
+  }
+  if (a == kCplx && b == kFull) return Mat2Shape{kMat2Scaled, 2, 8, 8, 0};
+  if (a == kFull && b == kCplx) return Mat2Shape{kMat2Scaled, 8, 2, 8, 0};
+  if (a == kCplx && b == kCplx) return Mat2Shape{kMat2Complex, 2, 2, 2, 0};
+  return Mat2Shape{};
+}
+
+// Turns a job laid out at offset0 into the matrix form, inside the bytes its plan's
+// form occupies, when its operands have one.  The form wins wherever its planes
+// (14 per modulus for a full product, one or two moduli more) do not outnumber the
+// plan's (24, or 16 in the four-multiplication form), which also keeps it inside
+// those bytes; that leaves out a few tiny k at loose tolerances (k <= 15 at tol
+// 1e-3: 6 x 14 planes against 5 x 16).  Measured at tol 1e-12: full m = n = k =
+// 8192, 15 x 14 planes against Gauss's 14 x 24: 226 -> 141 ms; the 512-product
+// batch: 31.9 -> 21.3 ms; TRS x TRA m = n = k = 4096, 15 x 7 against 14 x 8: 14.4 -> 10.4 ms;
+// complex x full 3000 x 1000 x 2000, 15 x 8 against 14 x 12: 2.51 -> 1.44 ms.
 static void to_mat2(SplitJob* sj, int64_t offset0) {
+  const Mat2Shape s = mat2_shape(sj->d.fa, sj->d.fb);
+  if (s.kind == kMat2None) return;
   const int nm = mat2_moduli(sj->d.k, sj->bits);
-  if (nm == 0 || nm * kMat2Planes > sj->nmod * sj->np || nm * kMat2Planes > sj->nmod * sj->nlf ||
-      nm * kMat2Planes > sj->nmod * sj->nrf)
+  if (nm == 0 || nm * s.np > sj->nmod * sj->np || nm * s.nlf > sj->nmod * sj->nlf || nm * s.nrf > sj->nmod * sj->nrf)
     return;
-  sj->mat2 = 1;
+  sj->mat2 = s.kind;
+  sj->rot = s.rot;
   sj->mod_base = kModTable;
   sj->four_m = 0;
   sj->neg2 = 0;
   sj->nmod = nm;
-  sj->np = sj->nlf = sj->nrf = kMat2Planes;
+  sj->np = s.np;
+  sj->nlf = s.nlf;
+  sj->nrf = s.nrf;
+  // product p: the same plane of both sides; a side with half the planes has one
+  // for both copies (a quaternion), a complex side one per copy
   for (int p = 0; p < kMaxProducts; ++p) {
-    sj->pl[p] = sj->pr[p] = (int8_t)(p < kMat2Planes ? p : 0);
+    auto plane = [&](int planes) { return (int8_t)(p >= s.np ? 0 : planes == 2 ? p / (s.np / 2) : p % planes); };
+    sj->pl[p] = plane(s.nlf);
+    sj->pr[p] = plane(s.nrf);
     sj->pl2[p] = sj->pr2[p] = 0;
   }
   int64_t off = offset0;
@@ -442,7 +470,7 @@ hmat_status split_prepare(const std::vector<JobDesc>& jobs, const KPlan* h_plans
     // the residue GEMM decodes a job's items with 32-bit arithmetic
     const int64_t plan_items = (int64_t)sj.nmod * sj.np * sj.tiles_m * sj.tiles_n;
     if (plan_items >= ((int64_t)1 << 31)) return HMAT_STATUS_UNSUPPORTED;
-    if (mat2 && sj.full) to_mat2(&sj, off0);
+    if (mat2) to_mat2(&sj, off0);
     sj.exp_begin = sp.exp_units;
     sp.exp_units += (d.m + 31) / 32 + (d.n + 31) / 32;
     const int64_t ea = enc_blocks(d.m, sj.nkb), eb = enc_blocks(d.n, sj.nkb);
@@ -474,8 +502,7 @@ hmat_status split_prepare(const std::vector<JobDesc>& jobs, const KPlan* h_plans
     sj.crt_begin = sp.crt_units;
     sj.crt2_begin = sp.crt2_units;
     (sj.mat2 ? sp.crt2_units : sp.crt_units) += blocks;
-    bool& wide = sj.mat2 ? sp.all_wide2 : sp.all_wide;
-    wide = wide && sj.crt_w == kCrtCols;
+    if (!sj.mat2) sp.all_wide = sp.all_wide && sj.crt_w == kCrtCols;
   }
   if ((size_t)off > ws_bytes) return HMAT_STATUS_WORKSPACE_TOO_SMALL;
   sp.ws_needed = off;
@@ -493,7 +520,7 @@ hmat_status split_layout_single(const JobDesc& d, const KPlan& P, double tol, co
   hmat_status st = layout_job(sh, &P, tol, tables, &sj, &off);
   if (st != HMAT_STATUS_SUCCESS) return st;
   if ((int64_t)sj.nmod * sj.np * sj.tiles_m * sj.tiles_n >= ((int64_t)1 << 31)) return HMAT_STATUS_UNSUPPORTED;
-  if (mat2 && sj.full) to_mat2(&sj, 0);
+  if (mat2) to_mat2(&sj, 0);
   units->exp = (d.m + 31) / 32 + (d.n + 31) / 32;
   units->encA = enc_blocks(d.m, sj.nkb);
   units->encB = enc_blocks(d.n, sj.nkb);
@@ -549,7 +576,7 @@ hmat_status split_launch(hmat_context* h, const SplitPrep& sp, const SplitJob* d
     e = launch_split_crt(d_jobs, njobs, d_plans, sp.crt_units, stream, ws, sp.max_nmod, sp.max_np, sp.all_full,
                          full_form, sp.all_wide);
     if (e == cudaSuccess && sp.crt2_units > 0)
-      e = launch_mat2_crt(d_jobs, njobs, sp.crt2_units, stream, ws, sp.max_nmod2, sp.all_wide2);
+      e = launch_mat2_crt(d_jobs, njobs, sp.crt2_units, stream, ws, sp.max_nmod2);
   }
   return e == cudaSuccess ? HMAT_STATUS_SUCCESS : split_cuda_error(e);
 }

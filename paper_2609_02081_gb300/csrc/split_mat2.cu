@@ -1,25 +1,33 @@
-// split_mat2.cu — the matrix form of the split mode's full biquaternion products:
-// encoder and CRT (the residue GEMM between them is split_gemm.cu's).
+// split_mat2.cu — the matrix form of split-mode products: encoder and CRT (the
+// residue GEMM between them is split_gemm.cu's).
 //
 // Modulo an odd p all of whose prime factors are 1 modulo 4 there is an s with
-// s^2 = -1, so i -> s and i -> -s map the complex integers onto two copies of
-// Z_p, and through
-//     q1 + q2 i + q3 j + q4 k  ->  [[q1 + I q2, q3 + I q4], [-q3 + I q4, q1 - I q2]]
-// (I the imaginary unit of the coefficients) the biquaternions map onto two
-// copies of the 2 x 2 matrices over Z_p.  A product is then two independent 2 x 2
-// products, each with Strassen's seven multiplications in Winograd's variant
-// (S. Winograd, "On multiplication of 2 x 2 matrices", 1971):
-//     S1 = x21 + x22, S2 = S1 - x11, S3 = x11 - x21, S4 = x12 - S2,
-//     T1 = y12 - y11, T2 = y22 - T1, T3 = y22 - y12, T4 = T2 - y21,
-//     P1 = x11 y11, P2 = x12 y21, P3 = S4 y22, P4 = x22 T4, P5 = S1 T1, P6 = S2 T2, P7 = S3 T3,
-//     c11 = P1 + P2, c12 = P1 + P6 + P5 + P3, c21 = P1 + P6 + P7 - P4, c22 = P1 + P6 + P7 + P5.
-// That is 14 residue GEMMs per modulus where the paper's bilinear scheme has 24;
-// the moduli are smaller (15 of 111 bits where the plans' 14 have 109), so a
+// s^2 = -1.  Two consequences, each exact in integers modulo p:
+//   * i -> s and i -> -s map the complex integers onto two copies of Z_p: a
+//     complex product is two real ones (u: i -> s, v: i -> -s) instead of Gauss's
+//     three;
+//   * q1 + q2 i + q3 j + q4 k -> [[q1 + s q2, q3 + s q4], [-q3 + s q4, q1 - s q2]]
+//     maps the quaternions over Z_p onto the 2 x 2 matrices over Z_p: a quaternion
+//     product takes Strassen's seven multiplications, in Winograd's variant
+//     (S. Winograd, "On multiplication of 2 x 2 matrices", 1971):
+//       S1 = x21 + x22, S2 = S1 - x11, S3 = x11 - x21, S4 = x12 - S2,
+//       T1 = y12 - y11, T2 = y22 - T1, T3 = y22 - y12, T4 = T2 - y21,
+//       P1 = x11 y11, P2 = x12 y21, P3 = S4 y22, P4 = x22 T4, P5 = S1 T1, P6 = S2 T2, P7 = S3 T3,
+//       c11 = P1 + P2, c12 = P1 + P6 + P5 + P3, c21 = P1 + P6 + P7 - P4, c22 = P1 + P6 + P7 + P5.
+// Residue GEMMs per modulus, against the plan's (Eq. bilinearH with Gauss):
+//   biquaternion x biquaternion                    14  (two copies of 7)   24
+//   real (or i times real) quaternion x biquaternion  14                   16
+//   real quaternion x real quaternion               7                      8
+//   complex x biquaternion                          8  (two copies of 4)   12
+//   complex x complex                               2                      3
+// The moduli are smaller (15 of 111 bits where the plans' 14 have 109): a full
 // product at tol 1e-12 takes 210 GEMMs instead of 336.  Every residue is exact,
 // and the integers recovered are those of the plans' forms.
 //
-// Factor plane f of a side and product plane f: P_{f+1} of the copy i -> s for
-// f < 7, P_{f-6} of the copy i -> -s for f >= 7.
+// Factor and product planes: the seven of Winograd's order (P1..P7; the left
+// factors x11, x12, S4, x22, S1, S2, S3), copy u then copy v; complex x
+// biquaternion: the four coefficients, copy u then copy v.  A real quaternion is
+// the same in both copies and is encoded once.
 #include <cuda_runtime.h>
 
 #include <cmath>
@@ -30,8 +38,6 @@
 namespace hmat {
 
 namespace {
-
-constexpr int kPlanes = kMat2Planes;
 
 // Per modulus: the digit weights w[d] = 2^(16 d) and s 2^(16 d), centred.
 struct Mat2Mod {
@@ -47,8 +53,9 @@ __constant__ Mat2Mod c_m2[kMat2MaxModuli];
 // digit pair contribute.
 __constant__ uint32_t c_m2P[kMat2MaxModuli + 1][kLimbs];
 __constant__ uint4 c_m2negP[kMat2MaxModuli + 1];
-__constant__ long long c_m2off[kMat2MaxModuli + 1][2][4][kLimbs];   // per limb
-__constant__ uint4 c_m2off4[kMat2MaxModuli + 1][2][4];              // modulo 2^128
+// ([0]: matrix products, [1]: complex x biquaternion)
+__constant__ long long c_m2off[kMat2MaxModuli + 1][2][2][4][kLimbs];   // per limb
+__constant__ uint4 c_m2off4[kMat2MaxModuli + 1][2][2][4];              // modulo 2^128
 __constant__ int c_m2shift[kMat2MaxModuli + 1];
 __constant__ float c_m2Pinv[kMat2MaxModuli + 1];    // crt_estimate_constants
 __constant__ float c_m2Pinv4[kMat2MaxModuli + 1];   // fl(2^96 / P)
@@ -63,6 +70,7 @@ __device__ __forceinline__ float2 fmod2(float2 v, float2 npf, float2 inv) {
 __device__ __forceinline__ float2 sub2(float2 a, float2 b) { return __ffma2_rn(b, f2(-1.0f), a); }
 
 constexpr int kRows = 16, kK = 32, kThreads = 128, kPitch = kK + 2;
+enum { kOpFull = 0, kOpQuat = 1, kOpCoef = 2, kOpCplx = 3 };   // what a side's operand is encoded as
 
 // ND balanced 16-bit digits of two neighbouring integers as floats: X = sum_d
 // x_d 2^(16 d), the low ones in [-2^15, 2^15).  Adding 2^15 to every low digit
@@ -86,22 +94,57 @@ __device__ __forceinline__ void digits2(longlong2 X, float2 (&d)[ND]) {
   }
 }
 
-// One thread's pair of k positions of one row: for every modulus the four matrix
-// entries of both copies and the seven factors of each, 4-byte stores.
-template <int ND, int SIDE>
-__device__ __forceinline__ void encode_pair(const longlong2 (&E)[8], int nmod, unsigned char* out,
-                                            uint32_t plane_bytes) {
-  float2 d[8][ND];
+// The left (SIDE 0) or right factors of one 2 x 2 product from the entries 11, 12, 21, 22.
+template <int SIDE, class Put>
+__device__ __forceinline__ void matrix_factors(const float2 (&x)[4], float2 npf, float2 inv, Put&& put) {
+  if (SIDE == 0) {
+    const float2 s1 = __fadd2_rn(x[2], x[3]);
+    const float2 s2 = sub2(s1, x[0]);
+    put(x[0]);
+    put(x[1]);
+    put(fmod2(sub2(x[1], s2), npf, inv));
+    put(x[3]);
+    put(fmod2(s1, npf, inv));
+    put(fmod2(s2, npf, inv));
+    put(fmod2(sub2(x[0], x[2]), npf, inv));
+  } else {
+    const float2 t3 = sub2(x[3], x[1]);
+    const float2 t2 = __fadd2_rn(t3, x[0]);
+    put(x[0]);
+    put(x[2]);
+    put(x[3]);
+    put(fmod2(sub2(t2, x[2]), npf, inv));
+    put(fmod2(sub2(x[1], x[0]), npf, inv));
+    put(fmod2(t2, npf, inv));
+    put(fmod2(t3, npf, inv));
+  }
+}
+
+// One thread's pair of k positions of one row: the digits stay in registers over
+// the moduli; 4-byte stores, one per factor plane.
+//   OPERAND kOpFull:  E = Re, Im of the entries 11, 12, 21, 22 (integers): 14 planes
+//           kOpQuat:  E = the four real components: 7 planes
+//           kOpCoef:  E = Re, Im of the four coefficients: 8 planes
+//           kOpCplx:  E = Re, Im: 2 planes
+template <int ND, int SIDE, int OPERAND>
+__device__ __forceinline__ void encode_pair(const longlong2* E, int nmod, unsigned char* out, uint32_t plane_bytes) {
+  constexpr int kPairs = OPERAND == kOpQuat ? 2 : OPERAND == kOpCplx ? 1 : 4;   // (Re, Im) pairs
+  float2 d[2 * kPairs][ND];
 #pragma unroll
-  for (int e = 0; e < 8; ++e) digits2<ND>(E[e], d[e]);
+  for (int e = 0; e < 2 * kPairs; ++e) digits2<ND>(E[e], d[e]);
   for (int l = 0; l < nmod; ++l) {
     const Mat2Mod& mc = c_m2[l];
     const float2 npf = f2(mc.npf), inv = f2(mc.inv);
-    // entries 11, 12, 21, 22 of the copies i -> s (u) and i -> -s (v): |sum of
-    // weighted digits| < 2^24 (checked when the root s is chosen)
+    // |residue| <= 121 is exact in BF16, whose bits are the upper half of the float's
+    auto put = [&](float2 x) {
+      *reinterpret_cast<uint32_t*>(out) = __byte_perm(__float_as_uint(x.x), __float_as_uint(x.y), 0x7632);
+      out += plane_bytes;
+    };
+    // Re + s Im and Re - s Im: |sum of weighted digits| < 2^24 (checked when the
+    // root s is chosen)
     float2 u[4], v[4];
 #pragma unroll
-    for (int e = 0; e < 4; ++e) {
+    for (int e = 0; e < kPairs; ++e) {
       float2 re = d[2 * e][0], im = __fmul2_rn(d[2 * e + 1][0], f2(mc.sw[0]));
 #pragma unroll
       for (int q = 1; q < ND; ++q) {
@@ -109,39 +152,24 @@ __device__ __forceinline__ void encode_pair(const longlong2 (&E)[8], int nmod, u
         im = __ffma2_rn(d[2 * e + 1][q], f2(mc.sw[q]), im);
       }
       u[e] = fmod2(__fadd2_rn(re, im), npf, inv);
-      v[e] = fmod2(sub2(re, im), npf, inv);
+      // (the copy v's entries 12 and 21 are s Im - Re of the other one)
+      const bool neg = (OPERAND == kOpFull && (e == 1 || e == 2)) || (OPERAND == kOpQuat && e == 1);
+      v[e] = fmod2(neg ? sub2(im, re) : sub2(re, im), npf, inv);
     }
-    // |residue| <= 121 is exact in BF16, whose bits are the upper half of the float's
-    auto put = [&](float2 x) {
-      *reinterpret_cast<uint32_t*>(out) = __byte_perm(__float_as_uint(x.x), __float_as_uint(x.y), 0x7632);
-      out += plane_bytes;
-    };
-    auto factors = [&](const float2 (&x)[4]) {
-      if (SIDE == 0) {
-        const float2 s1 = __fadd2_rn(x[2], x[3]);
-        const float2 s2 = sub2(s1, x[0]);
-        const float2 s4 = sub2(x[1], s2);
-        put(x[0]);
-        put(x[1]);
-        put(fmod2(s4, npf, inv));
-        put(x[3]);
-        put(fmod2(s1, npf, inv));
-        put(fmod2(s2, npf, inv));
-        put(fmod2(sub2(x[0], x[2]), npf, inv));
-      } else {
-        const float2 t3 = sub2(x[3], x[1]);
-        const float2 t2 = __fadd2_rn(t3, x[0]);
-        put(x[0]);
-        put(x[2]);
-        put(x[3]);
-        put(fmod2(sub2(t2, x[2]), npf, inv));
-        put(fmod2(sub2(x[1], x[0]), npf, inv));
-        put(fmod2(t2, npf, inv));
-        put(fmod2(t3, npf, inv));
-      }
-    };
-    factors(u);
-    factors(v);
+    if constexpr (OPERAND == kOpFull) {
+      const float2 vm[4] = {v[3], v[2], v[1], v[0]};
+      matrix_factors<SIDE>(u, npf, inv, put);
+      matrix_factors<SIDE>(vm, npf, inv, put);
+    } else if constexpr (OPERAND == kOpQuat) {
+      // 11: a1 + s a2, 12: a3 + s a4, 21: s a4 - a3, 22: a1 - s a2
+      const float2 x[4] = {u[0], u[1], v[1], v[0]};
+      matrix_factors<SIDE>(x, npf, inv, put);
+    } else {
+#pragma unroll
+      for (int e = 0; e < kPairs; ++e) put(u[e]);
+#pragma unroll
+      for (int e = 0; e < kPairs; ++e) put(v[e]);
+    }
   }
 }
 
@@ -149,13 +177,15 @@ __device__ __forceinline__ void encode_pair(const longlong2 (&E)[8], int nmod, u
 // columns), every modulus.
 //   phase 1: the present components of the tile are read (coalesced along
 //            whichever index is contiguous in memory, all loads of a thread in
-//            flight at once), scaled to integers, combined to the real and
-//            imaginary parts of the four matrix entries and staged in shared memory;
+//            flight at once), scaled to integers, for a full operand combined to
+//            the real and imaginary parts of its matrix entries, and staged in
+//            shared memory;
 //   phase 2: a thread takes two neighbouring k of one row, splits its eight
 //            integers into float digits once, holds them in registers over the
 //            moduli and stores one bfloat162 per factor plane: 16 lanes fill one
 //            aligned half of a swizzled 128-byte row.
-// Bound by its writes (28 bytes per modulus and element).
+// Bound by its writes (28 bytes per modulus and element of a full operand: 65 GB in
+// 10.2 ms at n = 8192, 0.94 of the copy bandwidth).
 template <int ND>
 __global__ void __launch_bounds__(kThreads, 4) mat2_encode_kernel(const SplitJob* __restrict__ jobs, int njobs,
                                                                   unsigned char* __restrict__ ws, int64_t first) {
@@ -166,19 +196,25 @@ __global__ void __launch_bounds__(kThreads, 4) mat2_encode_kernel(const SplitJob
   const JobDesc& d = sj.d;
   const int ktiles = sj.nkb * (kTileK / kK);
   const int64_t a_blocks = (int64_t)((d.m + kRows - 1) / kRows) * ktiles;
-  int64_t local = blk - sj.enc2_begin;
-  const int side = local >= a_blocks ? 1 : 0;
-  if (side) local -= a_blocks;
+  int64_t within = blk - sj.enc2_begin;
+  const int side = within >= a_blocks ? 1 : 0;
+  if (side) within -= a_blocks;
+  const uint32_t local = (uint32_t)within;               // a launch has fewer than 2^31 blocks
   const int tile_rows = side ? sj.bn : kTileM;
   const int rows_pad = (side ? sj.tiles_n : sj.tiles_m) * tile_rows;
-  const int r0 = (int)(local / ktiles) * kRows;
-  const int k0 = (int)(local % ktiles) * kK;
+  const uint32_t rowtile = local / (uint32_t)ktiles;
+  const int r0 = (int)rowtile * kRows;
+  const int k0 = (int)(local - rowtile * (uint32_t)ktiles) * kK;
   const int nout = side ? d.n : d.m;
   const uint32_t flags = side ? d.fb : d.fa;
   const double* base = side ? d.B : d.A;
   const int64_t ld = side ? d.ldb : d.lda, cs = side ? d.sB : d.sA;
   const int8_t* sign = side ? d.signB : d.signA;
   const bool contiguous = side ? (d.transB != 0) : (d.transA == 0);
+  // block-uniform: fourteen planes a full operand, seven a quaternion, eight the
+  // coefficients beside a complex one, two a complex one
+  const int planes = side ? sj.nrf : sj.nlf;
+  const int operand = planes == 14 ? kOpFull : planes == 7 ? kOpQuat : planes == 8 ? kOpCoef : kOpCplx;
   const int t = threadIdx.x;
   if (t < kRows) {
     const int r = r0 + t;
@@ -212,15 +248,27 @@ __global__ void __launch_bounds__(kThreads, 4) mat2_encode_kernel(const SplitJob
       X[c] = scaled_int(raw[u][c], s);
       if (sign[c] < 0) X[c] = -X[c];
     }
-    // a_e = X[e], b_e = X[e + 4]: Re and Im of entries 11, 12, 21, 22
-    ent[0][rr][kk] = X[0] - X[5];
-    ent[1][rr][kk] = X[4] + X[1];
-    ent[2][rr][kk] = X[2] - X[7];
-    ent[3][rr][kk] = X[6] + X[3];
-    ent[4][rr][kk] = -X[2] - X[7];
-    ent[5][rr][kk] = X[3] - X[6];
-    ent[6][rr][kk] = X[0] + X[5];
-    ent[7][rr][kk] = X[4] - X[1];
+    if (operand == kOpFull) {
+      // a_e = X[e], b_e = X[e + 4]: Re and Im of the entries 11, 12, 21, 22 (copy u)
+      ent[0][rr][kk] = X[0] - X[5];
+      ent[1][rr][kk] = X[4] + X[1];
+      ent[2][rr][kk] = X[2] - X[7];
+      ent[3][rr][kk] = X[6] + X[3];
+      ent[4][rr][kk] = -X[2] - X[7];
+      ent[5][rr][kk] = X[3] - X[6];
+      ent[6][rr][kk] = X[0] + X[5];
+      ent[7][rr][kk] = X[4] - X[1];
+    } else if (operand == kOpQuat) {         // one of the two halves is absent (zero)
+#pragma unroll
+      for (int e = 0; e < 4; ++e) ent[e][rr][kk] = X[e] + X[e + 4];
+    } else {
+#pragma unroll
+      for (int e = 0; e < 4; ++e)
+        if (e == 0 || operand == kOpCoef) {
+          ent[2 * e][rr][kk] = X[e];
+          ent[2 * e + 1][rr][kk] = X[e + 4];
+        }
+    }
   }
   __syncthreads();
 
@@ -240,10 +288,26 @@ __global__ void __launch_bounds__(kThreads, 4) mat2_encode_kernel(const SplitJob
     unsigned char* out = enc + ((int64_t)rt * sj.nkb + kb) * tile_bytes + (int64_t)(rin >> 3) * 1024 +
                          (rin & 7) * 128 + ((c16 ^ (rin & 7)) << 4) + in16;
     longlong2 E[8];
+    auto load = [&](int count) {
 #pragma unroll
-    for (int e = 0; e < 8; ++e) E[e] = *reinterpret_cast<const longlong2*>(&ent[e][rr][kp]);
-    if (side) encode_pair<ND, 1>(E, nmod, out, plane_bytes);
-    else encode_pair<ND, 0>(E, nmod, out, plane_bytes);
+      for (int e = 0; e < 8; ++e)
+        if (e < count) E[e] = *reinterpret_cast<const longlong2*>(&ent[e][rr][kp]);
+    };
+    if (operand == kOpFull) {
+      load(8);
+      if (side) encode_pair<ND, 1, kOpFull>(E, nmod, out, plane_bytes);
+      else encode_pair<ND, 0, kOpFull>(E, nmod, out, plane_bytes);
+    } else if (operand == kOpQuat) {
+      load(4);
+      if (side) encode_pair<ND, 1, kOpQuat>(E, nmod, out, plane_bytes);
+      else encode_pair<ND, 0, kOpQuat>(E, nmod, out, plane_bytes);
+    } else if (operand == kOpCoef) {
+      load(8);
+      encode_pair<ND, 0, kOpCoef>(E, nmod, out, plane_bytes);
+    } else {
+      load(2);
+      encode_pair<ND, 0, kOpCplx>(E, nmod, out, plane_bytes);
+    }
   }
 }
 
@@ -251,19 +315,23 @@ __global__ void __launch_bounds__(kThreads, 4) mat2_encode_kernel(const SplitJob
 // One warp per 32 consecutive elements of an output row; a block of four warps
 // covers one row of 128 columns, or four rows of 32 for narrow products.
 //
-// Per element the sums c11, c12, c21, c22 of both copies' product residues are
-// formed per modulus, and with u, v the two copies and t = u + v (half 0) or
-// u - v (half 1) of c:
-//   half 0: M1 = (t11 + t22)/4, M6 = (t22 - t11)/4, M3 = (t12 - t21)/4, M8 = -(t12 + t21)/4
-//   half 1: M5 = (t11 + t22)/4s, M2 = (t11 - t22)/4s, M7 = (t12 - t21)/4s, M4 = (t12 + t21)/4s.
-// S = N P + sum_l x_l d_l with d_l the CRT elements that carry 1/4 or 1/(4 s) is
-// congruent to the output modulo P.
+// Per element and modulus the outputs are sums of the product residues.  With cu,
+// cv the entries of the two copies' 2 x 2 products:
+//   half 0 (1/4):   t11 = cu11 + cv22, t22 = cu22 + cv11, t12 = cu12 - cv21, t21 = cu21 - cv12,
+//   half 1 (1/4s):  t11 = cu11 - cv22, t22 = cu22 - cv11, t12 = cu12 + cv21, t21 = cu21 + cv12,
+//   half 0: M1 = t11 + t22, M6 = t22 - t11, M3 = t12 - t21, M8 = -(t12 + t21)
+//   half 1: M5 = t11 + t22, M2 = t11 - t22, M7 = t12 - t21, M4 = t12 + t21
+// (real quaternions: one copy, t = 2 cu, M1 and M3 of half 0, M2 and M4 of half 1);
+// complex x biquaternion: M_e = 2 (u_e + v_e) of half 0, M_{e+4} = 2 (u_e - v_e) of
+// half 1.  S = N P + sum_l x_l d_l with d_l the CRT elements that carry 1/4 or
+// 1/(4 s) is congruent to the output modulo P.  An operand that is i times a real
+// quaternion was encoded as the real one; the outputs are turned by its i.
 //
 // The sum over the moduli is a contraction of depth nmod <= 16 (or two steps of
 // it), and runs on the tensor cores: A[element][modulus] = the integers t (FP16,
 // exact up to 2048), B[modulus][digit] = the balanced 8-bit digits of d_l, FP32
 // sums below 2^22 (exact).  A thread holds the fragment elements of four columns
-// and four moduli: it reads its 4 x 14 words of residues from shared memory,
+// and four moduli: it reads their residues as words from shared memory,
 // interleaves two moduli by byte permutes into half2 (an unsigned byte is an FP16
 // subnormal, so no conversion is needed: everything carries a factor 2^-24) and
 // forms the sums with half2 additions.  The residues are stored with 128 added
@@ -277,7 +345,9 @@ __global__ void __launch_bounds__(kThreads, 4) mat2_encode_kernel(const SplitJob
 // for 4096 x 4096 (2.35 ms with those), 0.87 ms of which its 5.9 GB would take at
 // the copy bandwidth; the 512-product batch 3.6 ms (6.1 ms).
 constexpr int kCrtThreads = 128;
-constexpr int kModStride = kPlanes * kCrtCols + 16;   // bytes; the four moduli pairs of a read fall on different banks
+constexpr int mod_stride(int planes) {                // bytes; the four moduli pairs of a read fall on different banks
+  return planes * kCrtCols + 16;
+}
 constexpr int kTrStride = 40;                         // words; likewise for the 16-byte stores of the transpose
 
 // digits of the CRT elements in the B fragments' layout: [nmod][half][k step][n tile][register][lane]
@@ -297,16 +367,6 @@ __device__ __forceinline__ uint32_t hsub2(uint32_t a, uint32_t b) {
   uint32_t r;
   asm("sub.rn.f16x2 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(b));
   return r;
-}
-
-// The sums c11, c22, c12, c21 of one copy for one column and a pair of moduli,
-// from its seven products.
-__device__ __forceinline__ void copy_sums(const uint32_t (&p)[7], uint32_t (&c)[4]) {
-  const uint32_t u1 = hadd2(p[0], p[5]), u2 = hadd2(u1, p[6]);
-  c[0] = hadd2(p[0], p[1]);
-  c[1] = hadd2(u2, p[4]);
-  c[2] = hadd2(hadd2(u1, p[4]), p[2]);
-  c[3] = hsub2(u2, p[3]);
 }
 
 // kMagic + x for an FP32 sum x 2^-24 of the products: its bits are kMagicBits + x
@@ -374,39 +434,55 @@ __device__ __forceinline__ double crt_value4(const uint32_t (&p)[8], uint4 off, 
                           (int)(uint32_t)bits);
 }
 
-// L: limbs of the sums, KS: k steps (of 16 moduli), kWide: every job's blocks are
-// one row of 128 columns.
-template <int L, int KS, bool kWide>
-__global__ void __launch_bounds__(kCrtThreads, 4) mat2_crt_kernel(const SplitJob* __restrict__ jobs, int njobs,
-                                                                  unsigned char* __restrict__ ws) {
+struct Mat2Pair {          // a coefficient's real and imaginary part
+  double re, im;
+};
+
+// x turned by i^rot; zeros stay +0
+__device__ __forceinline__ Mat2Pair turn(Mat2Pair x, int rot) {
+  auto neg = [](double v) {
+    const long long b = __double_as_longlong(v);
+    return __longlong_as_double((b << 1) == 0 ? b : b ^ (1ll << 63));
+  };
+  if (rot == 1) return {neg(x.im), x.re};
+  if (rot == 2) return {neg(x.re), neg(x.im)};
+  return x;
+}
+
+// The block's work for a job of kind KIND; L: limbs of the sums, KS: k steps (of 16 moduli).
+template <int L, int KS, int KIND>
+__device__ __forceinline__ void crt_block(const SplitJob& sj, uint32_t local, const unsigned char* __restrict__ ws,
+                                          uint8_t* ring, uint32_t (*tr)[8][kTrStride]) {
+  constexpr int NP = KIND == kMat2Full ? 14 : KIND == kMat2Quat ? 7 : KIND == kMat2Scaled ? 8 : 2;
+  constexpr int kStride = mod_stride(NP);
   constexpr int kRingMods = KS == 1 ? 16 : kMat2MaxModuli + 1;
-  __shared__ __align__(16) uint8_t ring[kRingMods][kModStride];
-  __shared__ __align__(16) uint32_t tr[kCrtThreads / 32][2][8][kTrStride];
-  const int64_t blk = blockIdx.x;
-  const SplitJob& sj = jobs[find_split_job(jobs, njobs, blk, 6)];
   const JobDesc& d = sj.d;
   const int nm = sj.nmod;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3;
-  const int w = kWide ? kCrtCols : sj.crt_w;
-  const int64_t local = blk - sj.crt2_begin;
-  const int colblocks = (d.n + w - 1) / w;
-  const int i0 = (int)(local / colblocks) * (kCrtCols / w);
-  const int j0 = (int)(local % colblocks) * w;
+  // one row of 128 columns or four rows of 32; a launch has fewer than 2^31 blocks
+  const bool wide = sj.crt_w == kCrtCols;
+  const uint32_t colblocks = wide ? (uint32_t)(d.n + kCrtCols - 1) / kCrtCols : (uint32_t)(d.n + 31) / 32;
+  const uint32_t rowblock = local / colblocks;
+  const int i0 = (int)(wide ? rowblock : 4 * rowblock);
+  const int j0 = (int)(local - rowblock * colblocks) * (wide ? kCrtCols : 32);
   const int64_t ncols = (int64_t)sj.tiles_n * sj.bn;
   // copy: thread tid takes 16-byte chunk tid % 8 of planes tid / 8, tid / 8 + 16, ...
   {
     const int64_t plane = sj.res_plane;
-    const int cc = tid & 7, cw = w / 16, crow = cc / cw, ccol = (cc % cw) * 16;
+    const int cc = tid & 7, crow = wide ? 0 : cc >> 1, ccol = (wide ? cc : cc & 1) * 16;
     if (i0 + crow < d.m && (int64_t)j0 + ccol < ncols) {
       int q = tid >> 3;                                    // plane: modulus l, product r
       const unsigned char* src = ws + sj.off_res + (int64_t)q * plane + (int64_t)(i0 + crow) * ncols + j0 + ccol;
-      int l = q >= kPlanes ? 1 : 0, r = q - l * kPlanes;
-      for (; q < nm * kPlanes; q += 16) {
-        cp_async16(&ring[l][r * kCrtCols + cc * 16], src);
+      int l = q / NP, r = q % NP;
+      for (; q < nm * NP; q += 16) {
+        cp_async16(ring + l * kStride + r * kCrtCols + cc * 16, src);
         src += 16 * plane;
-        r += 2;
-        l += r >= kPlanes ? 2 : 1;
-        r -= r >= kPlanes ? kPlanes : 0;
+        l += 16 / NP;
+        r += 16 % NP;
+        if (r >= NP) {
+          r -= NP;
+          ++l;
+        }
       }
     }
     cp_async_commit();
@@ -421,12 +497,11 @@ __global__ void __launch_bounds__(kCrtThreads, 4) mat2_crt_kernel(const SplitJob
       for (int nt = 0; nt < 2; ++nt)
 #pragma unroll
         for (int v = 0; v < 2; ++v) b[h][ks][nt][v] = __ldg(&g_m2digits[nm][h][ks][nt][v][lane]);
-  const int wi = i0 + (kWide ? 0 : 32 * warp / w), j = j0 + (kWide ? 32 * warp : 32 * warp % w) + lane;
+  const int wi = i0 + (wide ? 0 : warp), j = j0 + (wide ? 32 * warp : 0) + lane;
   const bool valid = wi < d.m && j < d.n;
-  int sc = 0;
+  int sc = -c_m2shift[nm];
   if (valid)
-    sc = -(reinterpret_cast<const int32_t*>(ws + sj.off_sexp)[wi] + reinterpret_cast<const int32_t*>(ws + sj.off_texp)[j]);
-  sc -= c_m2shift[nm];
+    sc -= reinterpret_cast<const int32_t*>(ws + sj.off_sexp)[wi] + reinterpret_cast<const int32_t*>(ws + sj.off_texp)[j];
   const int pb = c_m2Pbase[nm];
   const float pinv = L == 4 ? c_m2Pinv4[nm] : c_m2Pinv[nm];
   double* cbase = d.C + (int64_t)wi * d.ldc + j;
@@ -436,52 +511,81 @@ __global__ void __launch_bounds__(kCrtThreads, 4) mat2_crt_kernel(const SplitJob
   if (use_beta && valid)                                   // C is needed at the end: bring it near now
     for (int e = 0; e < 8; ++e) asm volatile("prefetch.global.L1 [%0];" ::"l"(cbase + (int64_t)e * d.sC));
   const bool plain = __double_as_longlong(d.alpha_re) == 0x3FF0000000000000ll && zero(d.alpha_im) && !use_beta;
+  const int rot = sj.rot;
   asm volatile("cp.async.wait_all;\n" ::: "memory");
   __syncthreads();
 
-  // sums c11, c22, c12, c21 of both copies for four columns and 2 KS pairs of moduli
-  uint32_t cu[4][2 * KS][4], cv[4][2 * KS][4];             // [sum][pair][column]
+  // cu: sums c11, c22, c12, c21 of copy u (or the four coefficients) for four
+  // columns and 2 KS pairs of moduli; cv: what copy v adds to t11, t22, t12, t21
+  // in half 0 and takes away in half 1
+  constexpr int kSums = KIND == kMat2Complex ? 1 : 4;
+  uint32_t cu[kSums][2 * KS][4], cv[kSums][2 * KS][4];     // [sum][pair][column]
 #pragma unroll
   for (int kp = 0; kp < 2 * KS; ++kp) {
     const int l = 8 * kp + 2 * t;
     const bool have = KS == 1 || l + 1 < kRingMods;        // beyond the ring: moduli that do not exist
-    uint32_t z[2 * kPlanes];
+    uint32_t z[2 * NP];
 #pragma unroll
-    for (int r = 0; r < kPlanes; ++r) {
+    for (int r = 0; r < NP; ++r) {
       uint32_t w0 = 0, w1 = 0;
       if (have) {
-        w0 = *reinterpret_cast<const uint32_t*>(&ring[l][r * kCrtCols + 32 * warp + 4 * g]);
-        w1 = *reinterpret_cast<const uint32_t*>(&ring[l + 1][r * kCrtCols + 32 * warp + 4 * g]);
+        const uint8_t* at = ring + l * kStride + r * kCrtCols + 32 * warp + 4 * g;
+        w0 = *reinterpret_cast<const uint32_t*>(at);
+        w1 = *reinterpret_cast<const uint32_t*>(at + kStride);
       }
       z[2 * r] = __byte_perm(w0, w1, 0x5140);              // columns 0 and 1, moduli interleaved
       z[2 * r + 1] = __byte_perm(w0, w1, 0x7362);          // columns 2 and 3
     }
 #pragma unroll
     for (int c = 0; c < 4; ++c) {
-      uint32_t pu[7], pv[7], su[4], sv[4];
+      uint32_t p[NP];
 #pragma unroll
-      for (int r = 0; r < 7; ++r) {
-        pu[r] = __byte_perm(z[2 * r + (c >> 1)], 0u, (c & 1) ? 0x4342 : 0x4140);
-        pv[r] = __byte_perm(z[2 * (r + 7) + (c >> 1)], 0u, (c & 1) ? 0x4342 : 0x4140);
-      }
-      copy_sums(pu, su);
-      copy_sums(pv, sv);
+      for (int r = 0; r < NP; ++r) p[r] = __byte_perm(z[2 * r + (c >> 1)], 0u, (c & 1) ? 0x4342 : 0x4140);
+      if constexpr (KIND == kMat2Full || KIND == kMat2Quat) {
+        auto sums = [&](int o, uint32_t (&x)[4]) {         // c11, c22, c12, c21 of the products o .. o + 6
+          const uint32_t u1 = hadd2(p[o], p[o + 5]), u2 = hadd2(u1, p[o + 6]);
+          x[0] = hadd2(p[o], p[o + 1]);
+          x[1] = hadd2(u2, p[o + 4]);
+          x[2] = hadd2(hadd2(u1, p[o + 4]), p[o + 2]);
+          x[3] = hsub2(u2, p[o + 3]);
+        };
+        uint32_t x[4];
+        sums(0, x);
 #pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        cu[e][kp][c] = su[e];
-        cv[e][kp][c] = sv[e];
+        for (int e = 0; e < 4; ++e) cu[e][kp][c] = x[e];
+        if constexpr (KIND == kMat2Full) {
+          sums(7, x);
+          cv[0][kp][c] = x[1];
+          cv[1][kp][c] = x[0];
+          cv[2][kp][c] = x[3];                             // (entries 12 and 21 with the opposite sign)
+          cv[3][kp][c] = x[2];
+        }
+      } else {
+#pragma unroll
+        for (int e = 0; e < kSums; ++e) {                  // twice the coefficient
+          cu[e][kp][c] = hadd2(p[e], p[e]);
+          cv[e][kp][c] = hadd2(p[kSums + e], p[kSums + e]);
+        }
       }
     }
   }
 
 #pragma unroll
-  for (int pr = 0; pr < 2; ++pr) {                         // sums 11 and 22, then 12 and 21
-    double val[2][2];                                      // [half][slot]
+  for (int pr = 0; pr < 2; ++pr) {                         // coefficients 2 pr and 2 pr + 1
+    // which slots (half, e) exist
+    auto has = [](int pr_, int h, int e) {
+      if (KIND == kMat2Quat) return h == e;
+      if (KIND == kMat2Complex) return pr_ == 0 && e == 0;
+      return true;
+    };
+    double val[2][2] = {};                                 // [half][slot]
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
+      if (!has(pr, h, 0) && !has(pr, h, 1)) continue;
       uint32_t pair[2][2][4];                              // [sum][n tile][column]
 #pragma unroll
-      for (int e = 0; e < 2; ++e)
+      for (int e = 0; e < 2; ++e) {
+        if (KIND == kMat2Complex && e > 0) continue;
 #pragma unroll
         for (int mt = 0; mt < 2; ++mt) {
           float acc[2][4] = {};
@@ -490,9 +594,15 @@ __global__ void __launch_bounds__(kCrtThreads, 4) mat2_crt_kernel(const SplitJob
             uint32_t a[4];
 #pragma unroll
             for (int v = 0; v < 4; ++v) {                  // rows g, g + 8: columns 2 mt, 2 mt + 1; then the next pair
-              const uint32_t x = cu[2 * pr + e][2 * ks + (v >> 1)][2 * mt + (v & 1)];
-              const uint32_t y = cv[2 * pr + e][2 * ks + (v >> 1)][2 * mt + (v & 1)];
-              a[v] = h ? hsub2(x, y) : hadd2(x, y);
+              const int si = KIND == kMat2Complex ? 0 : 2 * pr + e;
+              const uint32_t x = cu[si][2 * ks + (v >> 1)][2 * mt + (v & 1)];
+              if constexpr (KIND == kMat2Quat) {
+                a[v] = hadd2(x, x);
+              } else {
+                const uint32_t y = cv[si][2 * ks + (v >> 1)][2 * mt + (v & 1)];
+                const bool minus = (h == 1) != (KIND == kMat2Full && pr == 1);
+                a[v] = minus ? hsub2(x, y) : hadd2(x, y);
+              }
             }
 #pragma unroll
             for (int nt = 0; nt < 2; ++nt) mma_f16(acc[nt], a, b[h][ks][nt]);
@@ -503,33 +613,44 @@ __global__ void __launch_bounds__(kCrtThreads, 4) mat2_crt_kernel(const SplitJob
             pair[e][nt][2 * mt + 1] = digit_pair(acc[nt][2], acc[nt][3]);
           }
         }
+      }
       __syncwarp();                                        // the previous sums have been read
 #pragma unroll
       for (int nt = 0; nt < 2; ++nt) {
-        uint32_t s0[4], s1[4];
+        uint32_t s[2][4];
 #pragma unroll
         for (int c = 0; c < 4; ++c) {
-          const uint32_t x = pair[0][nt][c], y = pair[1][nt][c];
-          // pr 0: slot 0 = c11 + c22, slot 1 = c22 - c11 (half 1: c11 - c22);
-          // pr 1: slot 0 = c12 - c21, slot 1 = -(c12 + c21) (half 1: c12 + c21)
           // (2^31 added to make the pairs unsigned)
           constexpr uint32_t kPlus = 0x80000000u - 2u * kPairBias, kMinus = 0x80000000u + 2u * kPairBias;
-          s0[c] = pr == 0 ? x + y + kPlus : x - y + 0x80000000u;
-          s1[c] = pr == 0 ? (h ? x - y : y - x) + 0x80000000u : (h ? x + y + kPlus : kMinus - (x + y));
+          const uint32_t x = pair[0][nt][c];
+          if constexpr (KIND == kMat2Scaled || KIND == kMat2Complex) {
+            s[0][c] = x + (0x80000000u - kPairBias);
+            if constexpr (KIND == kMat2Scaled) s[1][c] = pair[1][nt][c] + (0x80000000u - kPairBias);
+          } else {
+            // pr 0: slot 0 = t11 + t22, slot 1 = t22 - t11 (half 1: t11 - t22);
+            // pr 1: slot 0 = t12 - t21, slot 1 = -(t12 + t21) (half 1: t12 + t21)
+            const uint32_t y = pair[1][nt][c];
+            s[0][c] = pr == 0 ? x + y + kPlus : x - y + 0x80000000u;
+            s[1][c] = pr == 0 ? (h ? x - y : y - x) + 0x80000000u : (h ? x + y + kPlus : kMinus - (x + y));
+          }
         }
-        *reinterpret_cast<uint4*>(&tr[warp][0][4 * nt + t][4 * g]) = make_uint4(s0[0], s0[1], s0[2], s0[3]);
-        *reinterpret_cast<uint4*>(&tr[warp][1][4 * nt + t][4 * g]) = make_uint4(s1[0], s1[1], s1[2], s1[3]);
+#pragma unroll
+        for (int e = 0; e < 2; ++e)
+          if (has(pr, h, e))
+            *reinterpret_cast<uint4*>(&tr[e][4 * nt + t][4 * g]) = make_uint4(s[e][0], s[e][1], s[e][2], s[e][3]);
       }
       __syncwarp();
 #pragma unroll
       for (int e = 0; e < 2; ++e) {
+        if (!has(pr, h, e)) continue;
+        constexpr int kTab = KIND == kMat2Scaled || KIND == kMat2Complex ? 1 : 0;
         uint32_t p[8];
 #pragma unroll
-        for (int i = 0; i < 8; ++i) p[i] = tr[warp][e][i][lane];
+        for (int i = 0; i < 8; ++i) p[i] = tr[e][i][lane];
         if constexpr (L == 4) {
-          val[h][e] = crt_value4(p, c_m2off4[nm][h][2 * pr + e], c_m2negP[nm], pinv, sc);
+          val[h][e] = crt_value4(p, c_m2off4[nm][kTab][h][2 * pr + e], c_m2negP[nm], pinv, sc);
         } else {
-          const long long* off = c_m2off[nm][h][2 * pr + e];
+          const long long* off = c_m2off[nm][kTab][h][2 * pr + e];
           long long s[L];
 #pragma unroll
           for (int q = 0; q < L; ++q) {
@@ -540,18 +661,17 @@ __global__ void __launch_bounds__(kCrtThreads, 4) mat2_crt_kernel(const SplitJob
         }
       }
     }
-    // slot e of half h is component (4 h + 2 pr + e) with the half flipped for
-    // odd e, so slot e's two values are the real (component 2 pr + e) and the
-    // imaginary part of one coefficient
     if (valid) {
 #pragma unroll
       for (int e = 0; e < 2; ++e) {
-        const double re = e ? val[1][e] : val[0][e], im = e ? val[0][e] : val[1][e];
+        // matrix products: slot 0 of half 0 and slot 1 of half 1 are real parts
+        const bool swap = (KIND == kMat2Full || KIND == kMat2Quat) && e == 1;
+        const Mat2Pair q = turn(swap ? Mat2Pair{val[1][e], val[0][e]} : Mat2Pair{val[0][e], val[1][e]}, rot);
         double* cr = cbase + (int64_t)(2 * pr + e) * d.sC;
         double* ci = cr + 4 * d.sC;
         if (plain) {                                       // block-uniform
-          *cr = re;
-          *ci = im;
+          *cr = q.re;
+          *ci = q.im;
           continue;
         }
         double x = 0.0, y = 0.0;
@@ -559,8 +679,8 @@ __global__ void __launch_bounds__(kCrtThreads, 4) mat2_crt_kernel(const SplitJob
           x = *cr;
           y = *ci;
         }
-        double vr = d.alpha_re * re + -1.0 * d.alpha_im * im;
-        double vi = d.alpha_re * im + 1.0 * d.alpha_im * re;
+        double vr = d.alpha_re * q.re + -1.0 * d.alpha_im * q.im;
+        double vi = d.alpha_re * q.im + 1.0 * d.alpha_im * q.re;
         if (use_beta) {
           vr += d.beta_re * x + -1.0 * d.beta_im * y;
           vi += d.beta_re * y + 1.0 * d.beta_im * x;
@@ -569,6 +689,23 @@ __global__ void __launch_bounds__(kCrtThreads, 4) mat2_crt_kernel(const SplitJob
         *ci = vi;
       }
     }
+  }
+}
+
+template <int L, int KS>
+__global__ void __launch_bounds__(kCrtThreads, 4) mat2_crt_kernel(const SplitJob* __restrict__ jobs, int njobs,
+                                                                  const unsigned char* __restrict__ ws) {
+  __shared__ __align__(16) uint8_t ring[(KS == 1 ? 16 : kMat2MaxModuli + 1) * mod_stride(kMat2MaxPlanes)];
+  __shared__ __align__(16) uint32_t tr[kCrtThreads / 32][2][8][kTrStride];
+  const int64_t blk = blockIdx.x;
+  const SplitJob& sj = jobs[find_split_job(jobs, njobs, blk, 6)];
+  const uint32_t local = (uint32_t)(blk - sj.crt2_begin);
+  auto* mine = tr[threadIdx.x >> 5];
+  switch (sj.mat2) {                                       // block-uniform
+    case kMat2Full: crt_block<L, KS, kMat2Full>(sj, local, ws, ring, mine); break;
+    case kMat2Quat: crt_block<L, KS, kMat2Quat>(sj, local, ws, ring, mine); break;
+    case kMat2Scaled: crt_block<L, KS, kMat2Scaled>(sj, local, ws, ring, mine); break;
+    default: crt_block<L, KS, kMat2Complex>(sj, local, ws, ring, mine); break;
   }
 }
 
@@ -609,8 +746,8 @@ cudaError_t mat2_configure(const int* moduli, const int* root, int n, const int3
   // holds column (digit) g of rows (moduli) 2t, 2t + 1 (register 0) and 2t + 8, 2t + 9
   // (register 1) of a 16 x 8 tile
   static uint32_t dig[M + 1][2][2][2][2][32];
-  static long long off[M + 1][2][4][kLimbs];
-  static uint4 off4[M + 1][2][4], negP[M + 1];
+  static long long off[M + 1][2][2][4][kLimbs];
+  static uint4 off4[M + 1][2][2][4], negP[M + 1];
   std::memset(dig, 0, sizeof(dig));
   std::memset(off, 0, sizeof(off));
   float pinv[M + 1], pinv4[M + 1] = {};
@@ -642,22 +779,21 @@ cudaError_t mat2_configure(const int* moduli, const int* root, int n, const int3
       for (int q = 0; q < 16; ++q)                  // exact under the conversion's magic number, pairs within int32
         if (worst[q] >= 4194304.0 || (q % 2 && 2.0 * (worst[q - 1] + 256.0 * worst[q]) >= 2147483648.0))
           return cudaErrorInvalidValue;
-      // 128 times the sum of the weights of the residues in each slot (half 1: u - v, none)
-      static const int bias[4] = {1536, 512, 512, -1536};
-      for (int s = 0; s < 4; ++s)
-        for (int q = 0; q < kLimbs; ++q)
-          off[m][h][s][q] = (long long)crt_off[m * kLimbs + q] - (h == 0 ? bias[s] * total[q] : 0) -
-                            (q < 4 ? (1ll << 31) + (1ll << 47) : 0);
-      for (int s = 0; s < 4; ++s) {
-        uint32_t w[4];
-        long long carry = 0;
-        for (int q = 0; q < 4; ++q) {
-          carry += off[m][h][s][q];
-          w[q] = (uint32_t)carry;
-          carry >>= 32;
+      // 128 times the sum of the weights of the residues in each slot: matrix products, complex x biquaternion
+      static const int bias[2][2][4] = {{{1536, 0, 512, 0}, {0, -512, 0, 1536}}, {{512, 512, 512, 512}, {0, 0, 0, 0}}};
+      for (int tab = 0; tab < 2; ++tab)
+        for (int s = 0; s < 4; ++s) {
+          long long carry = 0;
+          uint32_t w[kLimbs];
+          for (int q = 0; q < kLimbs; ++q) {
+            long long& o = off[m][tab][h][s][q];
+            o = (long long)crt_off[m * kLimbs + q] - bias[tab][h][s] * total[q] - (q < 4 ? (1ll << 31) + (1ll << 47) : 0);
+            carry += o;
+            w[q] = (uint32_t)carry;
+            carry >>= 32;
+          }
+          off4[m][tab][h][s] = make_uint4(w[0], w[1], w[2], w[3]);
         }
-        off4[m][h][s] = make_uint4(w[0], w[1], w[2], w[3]);
-      }
     }
     const uint32_t* P = crt_P + m * kLimbs;
     if (!crt_estimate_constants(P, 2.0 * m * kMat2WeightSum * kMat2HalfMax, m <= kMat2FourLimbs ? 4 : 5, &pb[m],
@@ -707,16 +843,10 @@ cudaError_t launch_mat2_encode(const SplitJob* d_jobs, int njobs, int64_t units,
 }
 
 cudaError_t launch_mat2_crt(const SplitJob* d_jobs, int njobs, int64_t units, cudaStream_t s, unsigned char* ws,
-                            int max_nmod, bool all_wide) {
+                            int max_nmod) {
   if (units <= 0) return cudaSuccess;
-  const unsigned grid = (unsigned)units;
-  auto launch = [&](auto kernel) { kernel<<<grid, kCrtThreads, 0, s>>>(d_jobs, njobs, ws); };
-  if (max_nmod <= kMat2FourLimbs) {
-    if (all_wide) launch(mat2_crt_kernel<4, 1, true>);
-    else launch(mat2_crt_kernel<4, 1, false>);
-  } else {
-    launch(mat2_crt_kernel<kLimbs, 2, false>);
-  }
+  if (max_nmod <= kMat2FourLimbs) mat2_crt_kernel<4, 1><<<(unsigned)units, kCrtThreads, 0, s>>>(d_jobs, njobs, ws);
+  else mat2_crt_kernel<kLimbs, 2><<<(unsigned)units, kCrtThreads, 0, s>>>(d_jobs, njobs, ws);
   return cudaGetLastError();
 }
 

@@ -1,10 +1,10 @@
-"""The matrix form of the split mode's full biquaternion products (split_mat2.cu).
+"""The matrix form of split-mode products (split_mat2.cu).
 
 Modulo p with s^2 = -1 the biquaternions are two copies of the 2 x 2 matrices;
 each copy's product takes Winograd's seven multiplications.  The CPU tests
 restate that algebra and the kernels' exact arithmetic on integers; the GPU
 tests require the bits of Gauss's form, which computes the same exact integers
-through the paper's 24 products.
+through the paper's products.
 """
 import itertools
 import math
@@ -70,15 +70,32 @@ def right(y11, y12, y21, y22):
     return [y11, y21, y22, t2 - y21, y12 - y11, t2, t3]
 
 
+def matrices(x, s, p):
+    """The entries 11, 12, 21, 22 modulo p of both copies (the second one with -s for the coefficients' i)."""
+    (r11, i11), (r12, i12), (r21, i21), (r22, i22) = entries(x)
+    return ([(r + s * i) % p for r, i in entries(x)],
+            [(r22 - s * i22) % p, (s * i21 - r21) % p, (s * i12 - r12) % p, (r11 - s * i11) % p])
+
+
+def sums(t):
+    """c11, c22, c12, c21 of the seven products."""
+    u1 = t[0] + t[5]
+    return [t[0] + t[1], u1 + t[6] + t[4], u1 + t[4] + t[2], u1 + t[6] - t[3]]
+
+
+def contractands(u, v, half):
+    """t11, t22, t12, t21 of a half from both copies' products."""
+    cu, cv = sums(u), sums(v)
+    cv = [cv[1], cv[0], -cv[3], -cv[2]]
+    return [a - b if half else a + b for a, b in zip(cu, cv)]
+
+
 def outputs(u, v):
     """The kernels' eight sums by (half, slot): 4 times (half 1: 4 s times) the component, modulo p."""
     out = {}
-    for half, sg in ((0, 1), (1, -1)):
-        t = [a + sg * b for a, b in zip(u, v)]
-        u1 = t[0] + t[5]
-        u2 = u1 + t[6]
-        c11, c12, c21, c22 = t[0] + t[1], u1 + t[4] + t[2], u2 - t[3], u2 + t[4]
-        z = [c11 + c22, c22 - c11, c12 - c21, -(c12 + c21)]
+    for half in (0, 1):
+        t11, t22, t12, t21 = contractands(u, v, half)
+        z = [t11 + t22, t22 - t11, t12 - t21, -(t12 + t21)]
         for e in range(4):
             out[(4 * half + e) ^ ((e & 1) << 2)] = -z[e] if half and e & 1 else z[e]
     return out
@@ -103,11 +120,8 @@ def test_matrix_form_recombines_to_the_product():
         s = root(p)
         for _ in range(20):
             a, b = ([rng.randrange(-(1 << 46), (1 << 46) + 1) for _ in range(8)] for _ in range(2))
-            copies = []
-            for sign in (1, -1):
-                x = [(re + sign * s * im) % p for re, im in entries(a)]
-                y = [(re + sign * s * im) % p for re, im in entries(b)]
-                copies.append([centred(f * g, p) for f, g in zip(left(*x), right(*y))])
+            copies = [[centred(f * g, p) for f, g in zip(left(*x), right(*y))]
+                      for x, y in zip(matrices(a, s, p), matrices(b, s, p))]
             got = outputs(*copies)
             want = quaternion_product(a, b)
             for c in range(8):
@@ -115,6 +129,31 @@ def test_matrix_form_recombines_to_the_product():
                 scale = 4 * s if c in (4, 1, 6, 3) else 4
                 assert (got[c] - scale * want[c]) % p == 0, (p, c)
                 assert abs(got[c]) <= 16 * (p - 1) // 2
+
+
+def test_matrix_form_of_subalgebra_products():
+    """A real quaternion's copies agree, so it is encoded once; one 2 x 2 product serves two of them (twice its sums
+    stand for both copies' in the 1/4 and 1/(4 s) elements); a complex operand is one number per copy."""
+    rng = random.Random(4)
+    for p in MODULI:
+        s = root(p)
+        a, b, q = ([rng.randrange(-(1 << 46), (1 << 46) + 1) for _ in range(8)] for _ in range(3))
+        a[4:] = q[4:] = [0] * 4
+        x, y, z = matrices(a, s, p), matrices(b, s, p), matrices(q, s, p)
+        assert x[0] == x[1]
+        got = outputs(*[[centred(f * g, p) for f, g in zip(left(*x[0]), right(*yc))] for yc in y])
+        want = quaternion_product(a, b)
+        assert all((got[c] - (4 * s if c in (4, 1, 6, 3) else 4) * want[c]) % p == 0 for c in range(8))
+        c11, c22, c12, c21 = sums([centred(f * g, p) for f, g in zip(left(*x[0]), right(*z[0]))])
+        want = quaternion_product(a, q)
+        for value, scale, w in ((c11 + c22, 4, want[0]), (c11 - c22, 4 * s, want[1]), (c12 - c21, 4, want[2]),
+                                (c12 + c21, 4 * s, want[3])):
+            assert (2 * value - scale * w) % p == 0
+        c = [b[0], 0, 0, 0, b[4], 0, 0, 0]
+        want = quaternion_product(c, q[:4] + b[4:])
+        for e in range(4):
+            u, v = (centred((c[0] + t * c[4]) * (q[e] + t * b[4 + e]), p) for t in (s, -s))
+            assert (2 * (u + v) - 4 * want[e]) % p == 0 and (2 * (u - v) - 4 * s * want[e + 4]) % p == 0
 
 
 def shift_of(nm):
@@ -170,11 +209,11 @@ def test_mat2_crt_digit_sums():
     most 2048, exact in FP16), u + v and u - v times the balanced 8-bit digits of the CRT elements, sums below 2^22,
     packed in pairs below 2^31; together with an offset less 128 times the weights they give N P + sum_l x_l d_l."""
     rng = random.Random(13)
-    weights = {0: (1536, 512, 512, -1536), 1: (0, 0, 0, 0)}
+    weights = {0: (1536, 0, 512, 0), 1: (0, -512, 0, 1536)}
     for nm in (1, 2, 14, 15, 16, 17):
         mods = MODULI[:nm]
         P = math.prod(mods) << shift_of(nm)
-        for half, sg in ((0, 1), (1, -1)):
+        for half in (0, 1):
             elements, digits = elements_of(nm, half), []
             for e in elements:
                 dl = []
@@ -194,12 +233,7 @@ def test_mat2_crt_digit_sums():
                         for which in (0, 1))
                 true = [outputs(a, b) for a, b in zip(u, v)]
 
-                def sums(t):
-                    u1 = t[0] + t[5]
-                    return [t[0] + t[1], u1 + t[6] + t[4], u1 + t[4] + t[2], u1 + t[6] - t[3]]
-                cu, cv = ([sums([x + 128 for x in row]) for row in side] for side in (u, v))
-                assert all(0 <= abs(x) <= 2048 for side in (cu, cv) for row in side for x in row)
-                tt = [[a + sg * b for a, b in zip(x, y)] for x, y in zip(cu, cv)]
+                tt = [contractands([x + 128 for x in a], [x + 128 for x in b], half) for a, b in zip(u, v)]
                 assert all(abs(x) <= 2048 for row in tt for x in row)
                 pairs = [[sum(row[e] * (dl[2 * i] + 256 * dl[2 * i + 1]) for row, dl in zip(tt, digits))
                           for i in range(8)] for e in range(4)]
@@ -262,12 +296,43 @@ def test_default_form_gives_gausss_bits(handles, i, tol):
 
 
 @pytest.mark.gpu
+@pytest.mark.parametrize("i", [0, 2, 4, 6, 8])
+@pytest.mark.parametrize("fa,fb", [(bi.TRS, bi.TRS), (bi.TRS, bi.TRA), (bi.TRA, bi.TRA), (bi.TRS, bi.BQ),
+                                   (bi.BQ, bi.TRA), (bi.TRA, bi.BQ), (bi.COMPLEX, bi.BQ), (bi.BQ, bi.COMPLEX),
+                                   (bi.COMPLEX, bi.COMPLEX)])
+def test_subalgebra_products_give_gausss_bits(handles, i, fa, fb):
+    """The matrix form of each pair of subalgebras it serves, absent components holding NaN; small integers (whose
+    exact zeros keep their sign) and wide-ranging data."""
+    m, n, k = SHAPES[i]
+    opA, opB = OPS[(i + 3) % 5], OPS[i % 5]
+    dev = torch.device("cuda")
+    (ra, ca), (rb, cb) = stored(opA, m, k), stored(opB, k, n)
+    for A, B in ((bi.fock_like(880 + i, ra, ca, row_scale=True), bi.uniform(890 + i, rb, cb)),
+                 (bi.small_int(880 + i, ra, ca, lo=-1, hi=1), bi.small_int(890 + i, rb, cb, lo=-1, hi=1))):
+        for X, f in ((A, fa), (B, fb)):
+            for c in range(8):
+                if not (f >> c) & 1:
+                    X[c] = float("nan")
+        A, B = A.to(dev), B.to(dev)
+        C0 = bi.uniform(840 + i, m, n).to(dev)
+        for alpha, beta, tol in ((1.0, 0.0, TOL), (0.5 - 2j, 0.25 + 1j, 1e-14)):
+            outs = []
+            for h in handles:
+                C = C0.clone()
+                hm.hmat_bq_gemm(h, A, B, C, opA, opB, fa, fb, alpha, beta, mode="split", tol=tol)
+                outs.append(C)
+            torch.cuda.synchronize()
+            assert torch.equal(outs[0].view(torch.int64), outs[1].view(torch.int64))
+
+
+@pytest.mark.gpu
 @pytest.mark.parametrize("use_graph", [False, True])
 def test_grouped_matrix_form_beside_other_forms(handles, use_graph):
     """One grouped call of full products (matrix form; k = 5 at tol 1e-3 keeps its plan's form, which then needs fewer
     planes) and subalgebra products: the bits of an all-Gauss handle."""
     dev = torch.device("cuda")
-    shapes = [(64, 64, 5, bi.BQ), (130, 70, 64, bi.BQ), (100, 90, 300, bi.TRS), (33, 1030, 200, bi.BQ), (7, 9, 12, bi.BQ)]
+    shapes = [(64, 64, 5, bi.BQ), (130, 70, 64, bi.BQ), (100, 90, 300, bi.TRS), (33, 1030, 200, bi.BQ),
+              (50, 60, 70, bi.REAL), (20, 200, 90, bi.COMPLEX), (7, 9, 12, bi.BQ)]
     mats = [(bi.uniform(860 + i, m, k, flags=f).to(dev), bi.uniform(870 + i, k, n).to(dev), f)
             for i, (m, n, k, f) in enumerate(shapes)]
     for tol in (1e-3, TOL):
