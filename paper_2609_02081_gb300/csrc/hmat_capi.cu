@@ -1059,20 +1059,21 @@ hmat_status hmat_bq_gemm_split_noalloc(hmat_handle h, int32_t opA, int32_t opB, 
   if (e != cudaSuccess) return cuda_status(e);
   noalloc_store_job_kernel<<<1, 1, 0, stream>>>(sj);
   e = cudaGetLastError();
-  if (e == cudaSuccess) e = launch_split_exponents(a.job, 1, u.exp, 0, stream, a.scratch);
+  const SplitJobs jobs{a.job, 1, nullptr};
+  if (e == cudaSuccess) e = launch_split_exponents(jobs, u.exp, 0, stream, a.scratch);
   if (sj.mat2) {
-    if (e == cudaSuccess) e = launch_mat2_encode(a.job, 1, u.encA + u.encB, 0, stream, a.scratch, u.max_bits);
+    if (e == cudaSuccess) e = launch_mat2_encode(jobs, u.encA + u.encB, 0, stream, a.scratch, u.max_bits);
   } else {
-    if (e == cudaSuccess) e = launch_split_encode(a.job, 1, h->d_plans, 0, u.encA, stream, a.scratch, u.max_bits);
-    if (e == cudaSuccess) e = launch_split_encode(a.job, 1, h->d_plans, 1, u.encB, stream, a.scratch, u.max_bits);
+    if (e == cudaSuccess) e = launch_split_encode(jobs, h->d_plans, 0, u.encA, stream, a.scratch, u.max_bits);
+    if (e == cudaSuccess) e = launch_split_encode(jobs, h->d_plans, 1, u.encB, stream, a.scratch, u.max_bits);
   }
   if (e == cudaSuccess)
-    e = launch_split_gemm(a.job, 1, u.items, (int)std::min<int64_t>(u.items, h->sm_count), stream, a.scratch,
+    e = launch_split_gemm(jobs, u.items, (int)std::min<int64_t>(u.items, h->sm_count), stream, a.scratch,
                           u.max_nkb);
   if (e == cudaSuccess && sj.mat2)
-    e = launch_mat2_crt(a.job, 1, u.crt, stream, a.scratch, u.max_nmod);
+    e = launch_mat2_crt(jobs, u.crt, stream, a.scratch, u.max_nmod);
   else if (e == cudaSuccess)
-    e = launch_split_crt(a.job, 1, h->d_plans, u.crt, stream, a.scratch, u.max_nmod, u.max_np, u.all_full,
+    e = launch_split_crt(jobs, h->d_plans, u.crt, stream, a.scratch, u.max_nmod, u.max_np, u.all_full,
                          u.four_m ? 1 : 0, sj.crt_w == kCrtCols);
   return cuda_status(e);
 }

@@ -33,6 +33,7 @@
 #include <cuda_runtime.h>
 
 #include <cstdint>
+#include <utility>
 #include <vector>
 
 #include "../../include/hmat.h"
@@ -152,6 +153,23 @@ struct SplitJob {
   int64_t exp_begin;                // exponent work units before this job
 };
 
+// The job table as the launchers take it: a device array of n jobs, or one
+// matrix-form job in host memory that travels in the kernels' arguments (table
+// null), with nothing to stage, copy or wait for before the launch.
+struct SplitJobs {
+  const SplitJob* table = nullptr;
+  int32_t n = 0;
+  const SplitJob* one = nullptr;
+};
+// Kernel argument of the kernels that come in both versions.
+template <bool kOne>
+struct JobParam {};
+template <>
+struct JobParam<true> {
+  SplitJob job;
+};
+static_assert(sizeof(SplitJob) <= 3800, "a job must fit the kernel argument space");
+
 // Workspace bytes for a set of problems (sum of the per-problem layouts).
 hmat_status split_workspace_bytes(const std::vector<SplitShape>& shapes, double tol, const TileTables& tables,
                                   size_t* bytes);
@@ -232,10 +250,12 @@ struct SplitUnits {
 };
 hmat_status split_layout_single(const JobDesc& d, const KPlan& P, double tol, const TileTables& tables, bool mat2,
                                 SplitJob* out, SplitUnits* units);
-// Launch the four stages reading the device job table d_jobs.
+// Launch the four stages reading the device job table d_jobs (null: sp's one
+// matrix-form job, in the kernel arguments).
 hmat_status split_launch(hmat_context* h, const SplitPrep& sp, const SplitJob* d_jobs, const KPlan* d_plans,
                          unsigned char* ws, cudaStream_t stream);
-// Upload the job table through the handle's staging buffer, then split_launch.
+// Upload the job table through the handle's staging buffer (unless it is one
+// matrix-form job), then split_launch.
 hmat_status run_split(hmat_context* h, const SplitPrep& sp, const KPlan* d_plans, void* workspace,
                       cudaStream_t stream);
 
@@ -258,17 +278,35 @@ hmat_status split_cuda_error(cudaError_t e);
 SplitState& handle_split(hmat_context* h);
 
 
+// Launch on `s` that may begin while the previous kernel of the stream still runs
+// (programmatic dependent launch): only for kernels that call
+// wait_for_previous_kernel() before they touch what it writes.
+template <class... Params, class... Args>
+cudaError_t launch_dependent(void (*kernel)(Params...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
+                             Args&&... args) {
+  cudaLaunchAttribute attr{};
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
+}
+
 // Device-side kernel launchers (split_kernels.cu).
-struct SplitConsts;
-cudaError_t launch_split_exponents(const SplitJob* d_jobs, int njobs, int64_t units, int64_t first_unit,
+cudaError_t launch_split_exponents(const SplitJobs& jobs, int64_t units, int64_t first_unit,
                                    cudaStream_t s, unsigned char* ws);
 // units are blocks: encode tiles of 32 rows x 32 k, CRT blocks of 256 elements
-cudaError_t launch_split_encode(const SplitJob* d_jobs, int njobs, const KPlan* d_plans, int side, int64_t units,
+cudaError_t launch_split_encode(const SplitJobs& jobs, const KPlan* d_plans, int side, int64_t units,
                                 cudaStream_t s, unsigned char* ws, int max_bits);
 // max_nkb: the most 64-deep k-blocks of any job's products (two-term products
 // count both terms; the one-chunk kernel form serves launches whose jobs all
 // have at most 16)
-cudaError_t launch_split_gemm(const SplitJob* d_jobs, int njobs, int64_t items, int grid, cudaStream_t s,
+cudaError_t launch_split_gemm(const SplitJobs& jobs, int64_t items, int grid, cudaStream_t s,
                               unsigned char* ws, int max_nkb);
 // all_full: every job uses the paper's full plan (structured recombination),
 // full_form: 0 all in Gauss's form, 1 all in the four-multiplication form, 2
@@ -276,14 +314,14 @@ cudaError_t launch_split_gemm(const SplitJob* d_jobs, int njobs, int64_t items, 
 // columns; else plans of at most 24 products take the packed-weight kernel with
 // the same layout, larger ones (the component-wise comparison plan) the
 // generic one
-cudaError_t launch_split_crt(const SplitJob* d_jobs, int njobs, const KPlan* d_plans, int64_t units,
+cudaError_t launch_split_crt(const SplitJobs& jobs, const KPlan* d_plans, int64_t units,
                              cudaStream_t s, unsigned char* ws, int max_nmod, int max_np, bool all_full,
                              int full_form, bool all_wide);
 // Matrix form (split_mat2.cu).  Encode blocks [first, first + units) of the
 // A and B sides of its jobs; jobs of other forms have no blocks.
-cudaError_t launch_mat2_encode(const SplitJob* d_jobs, int njobs, int64_t units, int64_t first, cudaStream_t s,
+cudaError_t launch_mat2_encode(const SplitJobs& jobs, int64_t units, int64_t first, cudaStream_t s,
                                unsigned char* ws, int max_bits);
-cudaError_t launch_mat2_crt(const SplitJob* d_jobs, int njobs, int64_t units, cudaStream_t s, unsigned char* ws,
+cudaError_t launch_mat2_crt(const SplitJobs& jobs, int64_t units, cudaStream_t s, unsigned char* ws,
                             int max_nmod);
 // n (kMat2MaxModuli) moduli, root[l]^2 = -1 mod moduli[l], and by modulus count
 // the CRT tables [n + 1][2][n][kLimbs], [n + 1][kLimbs], [n + 1][kLimbs], all

@@ -34,7 +34,9 @@
 // error word, stops, waits (bounded) for its own copies and MMAs and frees TMEM.
 #include <cuda_runtime.h>
 
-#include "split.hpp"
+#include <type_traits>
+
+#include "split_device.cuh"
 
 namespace hmat {
 
@@ -192,8 +194,14 @@ __device__ __forceinline__ int advance_job(const SplitJob* jobs, int njobs, int6
   return cur;
 }
 
-__device__ __forceinline__ Item decode_item(const SplitJob* jobs, int job, int64_t item, uint8_t* ws) {
-  const SplitJob& sj = jobs[job];
+template <bool kOne>
+__device__ __forceinline__ const SplitJob& item_job(const JobParam<kOne>& one, const SplitJob* __restrict__ jobs,
+                                                    int job) {
+  if constexpr (kOne) return one.job;
+  else return jobs[job];
+}
+
+__device__ __forceinline__ Item decode_item(const SplitJob& sj, int64_t item, uint8_t* ws) {
   // 32-bit arithmetic: a job has fewer than 2^31 items (checked on the host);
   // every role decodes every item, so the divisions are a per-item cost
   const uint32_t local = (uint32_t)(item - sj.item_begin);
@@ -276,10 +284,11 @@ __constant__ GemmModConst c_gmod[2 * kModTable];   // the plans' moduli, then th
 // (k <= 1024), so the multi-chunk epilogue and its 128 running sums per
 // thread are compiled out (the register budget then holds the single-chunk
 // drain without spills).
-template <bool kOneChunk>
+// kOne: one job, in the arguments, instead of the table.
+template <bool kOneChunk, bool kOne>
 __global__ void __launch_bounds__(kThreads, 1)
-split_residue_gemm_kernel(const SplitJob* __restrict__ jobs, int njobs, int64_t total_items, uint8_t* ws,
-                          uint32_t* err) {
+split_residue_gemm_kernel(const __grid_constant__ JobParam<kOne> one, const SplitJob* __restrict__ jobs, int njobs,
+                          int64_t total_items, uint8_t* ws, uint32_t* err) {
   extern __shared__ uint8_t smem_dyn[];
   // 1024-byte alignment for the swizzled operand tiles
   const uint32_t raw = smem_u32(smem_dyn);
@@ -312,6 +321,8 @@ split_residue_gemm_kernel(const SplitJob* __restrict__ jobs, int njobs, int64_t 
   tc_fence_after();
   const uint32_t tmem = s.tmem_base;
 
+  wait_for_previous_kernel();           // the encoded factors
+
   if (warp == 0) {
     // ------------------------------------------------------------ producer
     int armed[kStages];
@@ -321,10 +332,10 @@ split_residue_gemm_kernel(const SplitJob* __restrict__ jobs, int njobs, int64_t 
       int stage = 0;
       uint32_t phase = 0;
       bool ok = true;
-      int job = find_item_job(jobs, njobs, blockIdx.x);
+      int job = kOne ? 0 : find_item_job(jobs, njobs, blockIdx.x);
       for (int64_t item = blockIdx.x; ok && item < total_items; item += gridDim.x) {
-        job = advance_job(jobs, njobs, item, job);
-        const Item it = decode_item(jobs, job, item, ws);
+        if constexpr (!kOne) job = advance_job(jobs, njobs, item, job);
+        const Item it = decode_item(item_job(one, jobs, job), item, ws);
         const uint32_t bstride = (uint32_t)it.bn * kTileK * 2;
         for (int kb = 0; kb < it.nkb; ++kb) {
           if (!mbar_wait(smem_u32(&s.empty[stage]), phase ^ 1u, abort_flag, err, kErrWaitProducer)) { ok = false; break; }
@@ -356,10 +367,10 @@ split_residue_gemm_kernel(const SplitJob* __restrict__ jobs, int njobs, int64_t 
       uint32_t chunk_ctr = 0;
       bool ok = true;
       bool issued = false;
-      int job = find_item_job(jobs, njobs, blockIdx.x);
+      int job = kOne ? 0 : find_item_job(jobs, njobs, blockIdx.x);
       for (int64_t item = blockIdx.x; ok && item < total_items; item += gridDim.x) {
-        job = advance_job(jobs, njobs, item, job);
-        const Item it = decode_item(jobs, job, item, ws);
+        if constexpr (!kOne) job = advance_job(jobs, njobs, item, job);
+        const Item it = decode_item(item_job(one, jobs, job), item, ws);
         const uint32_t idesc = instr_desc(it.bn);
         // the subtracted second term of a two-term product: negate B
         const uint32_t idesc2 = it.neg ? (idesc | kNegateB) : idesc;
@@ -405,10 +416,10 @@ split_residue_gemm_kernel(const SplitJob* __restrict__ jobs, int njobs, int64_t 
     const int row = q * 32 + lane;
     uint32_t chunk_ctr = 0;
     bool ok = true;
-    int job = find_item_job(jobs, njobs, blockIdx.x);
+    int job = kOne ? 0 : find_item_job(jobs, njobs, blockIdx.x);
     for (int64_t item = blockIdx.x; ok && item < total_items; item += gridDim.x) {
-      job = advance_job(jobs, njobs, item, job);
-      const Item it = decode_item(jobs, job, item, ws);
+      if constexpr (!kOne) job = advance_job(jobs, njobs, item, job);
+      const Item it = decode_item(item_job(one, jobs, job), item, ws);
       const int cols = it.bn >> 1;        // columns handled by this thread: a multiple of 16 up to 128
       const int col0 = half * cols;
       const int nchunks = (it.nkb + kKbPerChunk - 1) / kKbPerChunk;
@@ -602,23 +613,26 @@ cudaError_t split_gemm_configure(const int* moduli, int n) {
   }
   cudaError_t e = cudaMemcpyToSymbol(c_gmod, g, sizeof(g));
   if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(split_residue_gemm_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)split_gemm_smem_bytes());
-  if (e != cudaSuccess) return e;
-  return cudaFuncSetAttribute(split_residue_gemm_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              (int)split_gemm_smem_bytes());
+  auto allow = [](auto kernel) {
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)split_gemm_smem_bytes());
+  };
+  for (auto kernel : {split_residue_gemm_kernel<false, false>, split_residue_gemm_kernel<true, false>})
+    if (e == cudaSuccess) e = allow(kernel);
+  for (auto kernel : {split_residue_gemm_kernel<false, true>, split_residue_gemm_kernel<true, true>})
+    if (e == cudaSuccess) e = allow(kernel);
+  return e;
 }
 
-cudaError_t launch_split_gemm(const SplitJob* d_jobs, int njobs, int64_t items, int grid, cudaStream_t s,
+cudaError_t launch_split_gemm(const SplitJobs& jobs, int64_t items, int grid, cudaStream_t s,
                               unsigned char* ws, int max_nkb) {
   if (items <= 0) return cudaSuccess;
-  if (max_nkb <= kKbPerChunk)
-    split_residue_gemm_kernel<true><<<grid, kThreads, split_gemm_smem_bytes(), s>>>(d_jobs, njobs, items, ws,
-                                                                                   device_error_ptr());
-  else
-    split_residue_gemm_kernel<false><<<grid, kThreads, split_gemm_smem_bytes(), s>>>(d_jobs, njobs, items, ws,
-                                                                                    device_error_ptr());
-  return cudaGetLastError();
+  return with_jobs(jobs, [&](const auto& one) {
+    constexpr bool kOne = std::is_same_v<std::decay_t<decltype(one)>, JobParam<true>>;
+    return launch_dependent(max_nkb <= kKbPerChunk ? split_residue_gemm_kernel<true, kOne>
+                                                   : split_residue_gemm_kernel<false, kOne>,
+                            dim3(grid), dim3(kThreads), split_gemm_smem_bytes(), s, one, jobs.table, jobs.n, items, ws,
+                            device_error_ptr());
+  });
 }
 
 }  // namespace hmat

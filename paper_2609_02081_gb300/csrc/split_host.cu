@@ -540,6 +540,10 @@ hmat_status split_layout_single(const JobDesc& d, const KPlan& P, double tol, co
 hmat_status split_launch(hmat_context* h, const SplitPrep& sp, const SplitJob* d_jobs, const KPlan* d_plans,
                          unsigned char* ws, cudaStream_t stream) {
   const int njobs = (int)sp.jobs.size();
+  SplitJobs jobs;
+  jobs.table = d_jobs;
+  jobs.n = njobs;
+  jobs.one = &sp.jobs[0];
   cudaError_t e;
   // with reuse_a / reuse_b (one job) the A units, which come first in the
   // exponent stage, or the B units after them, are skipped, and so is that
@@ -549,34 +553,34 @@ hmat_status split_launch(hmat_context* h, const SplitPrep& sp, const SplitJob* d
     ProfScope ps(h, 1, stream);
     const int64_t a_units = njobs == 1 ? (sp.jobs[0].d.m + 31) / 32 : 0;
     const int64_t first = skip_a ? a_units : 0, end = skip_b ? a_units : sp.exp_units;
-    e = launch_split_exponents(d_jobs, njobs, end, first, stream, ws);
+    e = launch_split_exponents(jobs, end, first, stream, ws);
   }
   if (e != cudaSuccess) return split_cuda_error(e);
   {
     ProfScope ps(h, 2, stream);
-    if (!skip_a) e = launch_split_encode(d_jobs, njobs, d_plans, 0, sp.encA_units, stream, ws, sp.max_bits);
+    if (!skip_a) e = launch_split_encode(jobs, d_plans, 0, sp.encA_units, stream, ws, sp.max_bits);
     if (e == cudaSuccess && !skip_b)
-      e = launch_split_encode(d_jobs, njobs, d_plans, 1, sp.encB_units, stream, ws, sp.max_bits);
+      e = launch_split_encode(jobs, d_plans, 1, sp.encB_units, stream, ws, sp.max_bits);
     // the matrix form's blocks: A side first, then B side
     const int64_t a_blocks = njobs == 1 ? enc_blocks(sp.jobs[0].d.m, sp.jobs[0].nkb) : 0;
     const int64_t first = skip_a ? a_blocks : 0, end = skip_b ? std::min(a_blocks, sp.enc2_units) : sp.enc2_units;
     if (e == cudaSuccess && end > first)
-      e = launch_mat2_encode(d_jobs, njobs, end - first, first, stream, ws, sp.max_bits2);
+      e = launch_mat2_encode(jobs, end - first, first, stream, ws, sp.max_bits2);
   }
   if (e != cudaSuccess) return split_cuda_error(e);
   {
     ProfScope ps(h, 3, stream);
     const int grid = (int)std::min<int64_t>(sp.items, handle_sm_count(h));
-    e = launch_split_gemm(d_jobs, njobs, sp.items, grid, stream, ws, sp.max_nkb);
+    e = launch_split_gemm(jobs, sp.items, grid, stream, ws, sp.max_nkb);
   }
   if (e != cudaSuccess) return split_cuda_error(e);
   {
     ProfScope ps(h, 4, stream);
     const int full_form = sp.n_four_m == 0 ? 0 : (sp.n_four_m == sp.n_plan ? 1 : 2);
-    e = launch_split_crt(d_jobs, njobs, d_plans, sp.crt_units, stream, ws, sp.max_nmod, sp.max_np, sp.all_full,
+    e = launch_split_crt(jobs, d_plans, sp.crt_units, stream, ws, sp.max_nmod, sp.max_np, sp.all_full,
                          full_form, sp.all_wide);
     if (e == cudaSuccess && sp.crt2_units > 0)
-      e = launch_mat2_crt(d_jobs, njobs, sp.crt2_units, stream, ws, sp.max_nmod2);
+      e = launch_mat2_crt(jobs, sp.crt2_units, stream, ws, sp.max_nmod2);
   }
   return e == cudaSuccess ? HMAT_STATUS_SUCCESS : split_cuda_error(e);
 }
@@ -584,6 +588,9 @@ hmat_status split_launch(hmat_context* h, const SplitPrep& sp, const SplitJob* d
 // Upload the job table through the handle's staging buffer and launch.
 hmat_status run_split(hmat_context* h, const SplitPrep& sp, const KPlan* d_plans, void* workspace,
                       cudaStream_t stream) {
+  // one matrix-form job travels in the kernel arguments: nothing to stage, copy or wait for
+  if (sp.jobs.size() == 1 && sp.jobs[0].mat2)
+    return split_launch(h, sp, nullptr, d_plans, static_cast<unsigned char*>(workspace), stream);
   SplitState& st_all = handle_split(h);
   SplitSlot& s = st_all.slots[st_all.next];
   st_all.next = (st_all.next + 1) % kSplitSlots;

@@ -7,10 +7,10 @@
 //         swizzled K-major rows: the tcgen05 shared-memory operand layout)
 //   encB  [nmod][nrf][tiles_n][nkb] tiles of bn x 64 BF16
 //   res   [nmod][np][tiles_m*128][tiles_n*bn] int8 centred product residues
-#include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
 #include <cmath>
+#include <type_traits>
 
 #include "split_device.cuh"
 
@@ -73,9 +73,9 @@ __device__ __forceinline__ float residue_i64(long long X, const ModConst& mc) {
 }
 
 // ------------------------------------------------------------------ 1. exponents
-// One block (256 threads) per group of 32 outputs: rows of op(A) or columns of op(B).
+// One block per group of 32 outputs: rows of op(A) or columns of op(B).
 // s = b - 1 - floor(log2 max|x|) over the eight present components and k.
-constexpr int kExpThreads = 1024;   // 32 warps per 32 outputs: k is split over the warps (or lanes)
+constexpr int kExpThreads = 1024;   // 32 warps: k is split over the warps (or lanes)
 
 // biased exponent field of x; inf / NaN set `bad`
 __device__ __forceinline__ int exp_field(double x, bool& bad) {
@@ -84,18 +84,21 @@ __device__ __forceinline__ int exp_field(double x, bool& bad) {
   return ef;
 }
 
-__global__ void __launch_bounds__(kExpThreads) split_exponents_kernel(const SplitJob* __restrict__ jobs, int njobs,
-                                                                      unsigned char* __restrict__ ws,
-                                                                      uint32_t* err, int64_t first_unit) {
+// kSub: blocks per group of 32 outputs (1 or 4, each 32 / kSub of them).
+template <bool kOne, int kSub>
+__global__ void __launch_bounds__(kExpThreads)
+    split_exponents_kernel(const __grid_constant__ JobParam<kOne> one, const SplitJob* __restrict__ jobs, int njobs,
+                           unsigned char* __restrict__ ws, uint32_t* err, int64_t first_unit) {
   __shared__ int red[32][33];
-  const int64_t unit = first_unit + blockIdx.x;
-  const int g = find_split_job(jobs, njobs, unit, 0);
-  const SplitJob& sj = jobs[g];
+  allow_next_kernel();
+  constexpr int kOut = 32 / kSub;       // outputs of this block
+  const int64_t unit = first_unit + blockIdx.x / kSub;
+  const SplitJob& sj = unit_job(one, jobs, njobs, unit, 0);
   const JobDesc& d = sj.d;
   const int64_t local = unit - sj.exp_begin;
   const int64_t a_units = (d.m + 31) / 32;
   const bool sideB = local >= a_units;
-  const int grp = (int)(sideB ? local - a_units : local);
+  const int r0 = (int)(sideB ? local - a_units : local) * 32 + (int)(blockIdx.x % kSub) * kOut;
   const double* base = sideB ? d.B : d.A;
   const int64_t ld = sideB ? d.ldb : d.lda, cs = sideB ? d.sB : d.sA;
   const uint32_t flags = sideB ? d.fb : d.fa;
@@ -107,55 +110,77 @@ __global__ void __launch_bounds__(kExpThreads) split_exponents_kernel(const Spli
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   int best = 0;
   bool bad = false;
-  if (contiguous) {
-    // warp w handles output grp*32 + w; lanes stride k, four loads in flight
-    const int r = grp * 32 + warp;
+  // k positions k0, k0 + st, ... of every present component.  Long rows: one
+  // component after the other, four loads in flight (sequential DRAM streams:
+  // 1.21 ms at n = 8192, the copy bandwidth).  Short ones are bound by the chain of
+  // round trips: two positions of all eight components at a time, sixteen loads in
+  // flight.
+  constexpr int st = 32 * kSub;
+  auto scan = [&](const double* src, int64_t k0, int64_t step) {
     int mx = 0;
-    if (r < nout) {
+    if (K > 1024) {
       for (int c = 0; c < 8; ++c) {
         if (!((flags >> c) & 1u)) continue;
-        const double* row = base + (int64_t)c * cs + (int64_t)r * ld;
-        int64_t kk = lane;
-        for (; kk + 96 < K; kk += 128) {
-          const double x0 = __ldg(row + kk), x1 = __ldg(row + kk + 32);
-          const double x2 = __ldg(row + kk + 64), x3 = __ldg(row + kk + 96);
+        const double* p = src + (int64_t)c * cs;
+        int64_t kk = k0;
+        for (; kk + 3 * st < K; kk += 4 * st) {
+          const double x0 = __ldg(p + kk * step), x1 = __ldg(p + (kk + st) * step);
+          const double x2 = __ldg(p + (kk + 2 * st) * step), x3 = __ldg(p + (kk + 3 * st) * step);
           mx = max(mx, max(max(exp_field(x0, bad), exp_field(x1, bad)), max(exp_field(x2, bad), exp_field(x3, bad))));
         }
-        for (; kk < K; kk += 32) mx = max(mx, exp_field(__ldg(row + kk), bad));
+        for (; kk < K; kk += st) mx = max(mx, exp_field(__ldg(p + kk * step), bad));
       }
+      return mx;
     }
+    for (int64_t kk = k0; kk < K; kk += 2 * st) {
+      double x[2][8];
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-    if (lane == 0) red[0][warp] = mx;
-    __syncthreads();
-    if (threadIdx.x < 32) best = red[0][threadIdx.x];
-  } else {
-    // lanes over the 32 outputs (consecutive addresses), the 32 warps split k, four loads in flight
-    const int r = grp * 32 + lane;
-    int mx = 0;
-    if (r < nout) {
-      for (int c = 0; c < 8; ++c) {
-        if (!((flags >> c) & 1u)) continue;
-        const double* col = base + (int64_t)c * cs + r;
-        int64_t kk = warp;
-        for (; kk + 96 < K; kk += 128) {
-          const double x0 = __ldg(col + kk * ld), x1 = __ldg(col + (kk + 32) * ld);
-          const double x2 = __ldg(col + (kk + 64) * ld), x3 = __ldg(col + (kk + 96) * ld);
-          mx = max(mx, max(max(exp_field(x0, bad), exp_field(x1, bad)), max(exp_field(x2, bad), exp_field(x3, bad))));
+      for (int u = 0; u < 2; ++u)
+#pragma unroll
+        for (int c = 0; c < 8; ++c) {
+          const bool in = ((flags >> c) & 1u) != 0 && kk + st * u < K;
+          x[u][c] = in ? __ldg(src + (int64_t)c * cs + (kk + st * u) * step) : 0.0;
         }
-        for (; kk < K; kk += 32) mx = max(mx, exp_field(__ldg(col + kk * ld), bad));
-      }
+#pragma unroll
+      for (int u = 0; u < 2; ++u)
+#pragma unroll
+        for (int c = 0; c < 8; ++c) mx = max(mx, exp_field(x[u][c], bad));
     }
-    red[warp][lane] = mx;
+    return mx;
+  };
+  // red[part][output]: partial maxima of the block's outputs
+  constexpr int kParts = kExpThreads / 32;
+  if (contiguous) {
+    // kSub warps to an output; lanes stride k
+    const int o = warp / kSub, r = r0 + o;
+    int mx = r < nout ? scan(base + (int64_t)r * ld, (warp % kSub) * 32 + lane, 1) : 0;
+#pragma unroll
+    for (int x = 16; x > 0; x >>= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, x));
+    if (lane == 0) red[warp % kSub][o] = mx;
     __syncthreads();
-    if (threadIdx.x < 32) {
-      best = red[0][lane];
-      for (int w = 1; w < 32; ++w) best = max(best, red[w][lane]);
+    if (threadIdx.x < kOut) {
+      best = red[0][threadIdx.x];
+#pragma unroll
+      for (int w = 1; w < kSub; ++w) best = max(best, red[w][threadIdx.x]);
+    }
+  } else {
+    // lanes over the outputs (consecutive addresses; kSub k positions beside each
+    // other), the 32 warps split k
+    const int o = lane % kOut, r = r0 + o;
+    int mx = r < nout ? scan(base + r, warp * kSub + lane / kOut, ld) : 0;
+#pragma unroll
+    for (int x = kOut; x < 32; x <<= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, x));
+    if (lane < kOut) red[warp][o] = mx;
+    __syncthreads();
+    if (threadIdx.x < kOut) {
+      best = red[0][threadIdx.x];
+#pragma unroll 8
+      for (int w = 1; w < kParts; ++w) best = max(best, red[w][threadIdx.x]);
     }
   }
   if (bad) atomicOr(err, kErrNonFinite);
-  if (threadIdx.x < 32) {
-    const int r = grp * 32 + threadIdx.x;
+  if (threadIdx.x < kOut) {
+    const int r = r0 + threadIdx.x;
     if (r < nout) {
       int32_t* out = reinterpret_cast<int32_t*>(ws + (sideB ? sj.off_texp : sj.off_sexp));
       // max |x| < 2^(best - 1023 + 1): scale so that |x| 2^s < 2^b
@@ -973,23 +998,33 @@ cudaError_t split_upload_constants(const int* moduli, int nmod_table, const int3
   return cudaMemcpyToSymbol(c_Pinv, pinv, sizeof(pinv));
 }
 
-cudaError_t launch_split_exponents(const SplitJob* d_jobs, int njobs, int64_t units, int64_t first_unit,
+cudaError_t launch_split_exponents(const SplitJobs& jobs, int64_t units, int64_t first_unit,
                                    cudaStream_t s, unsigned char* ws) {
   if (units <= first_unit) return cudaSuccess;
-  split_exponents_kernel<<<(unsigned)(units - first_unit), kExpThreads, 0, s>>>(d_jobs, njobs, ws,
-                                                                                 device_error_ptr(), first_unit);
-  return cudaGetLastError();
+  return with_jobs(jobs, [&](const auto& one) {
+    constexpr bool kOne = std::is_same_v<std::decay_t<decltype(one)>, JobParam<true>>;
+    // few groups: four blocks to each, so that more SMs share the reads (n = 256,
+    // 16 groups: 14.3 us -> 8; a whole product 46.9 -> 41.1)
+    const int64_t blocks = units - first_unit;
+    if (blocks < 152)
+      split_exponents_kernel<kOne, 4><<<(unsigned)(4 * blocks), kExpThreads, 0, s>>>(one, jobs.table, jobs.n, ws,
+                                                                                     device_error_ptr(), first_unit);
+    else
+      split_exponents_kernel<kOne, 1><<<(unsigned)blocks, kExpThreads, 0, s>>>(one, jobs.table, jobs.n, ws,
+                                                                               device_error_ptr(), first_unit);
+    return cudaGetLastError();
+  });
 }
 
-cudaError_t launch_split_encode(const SplitJob* d_jobs, int njobs, const KPlan* d_plans, int side, int64_t units,
+cudaError_t launch_split_encode(const SplitJobs& jobs, const KPlan* d_plans, int side, int64_t units,
                                 cudaStream_t s, unsigned char* ws, int max_bits) {
   if (units <= 0) return cudaSuccess;
-  if (max_bits <= 47) split_encode_kernel<2><<<(unsigned)units, kEncThreads, 0, s>>>(d_jobs, njobs, d_plans, side, ws);
-  else split_encode_kernel<3><<<(unsigned)units, kEncThreads, 0, s>>>(d_jobs, njobs, d_plans, side, ws);
+  if (max_bits <= 47) split_encode_kernel<2><<<(unsigned)units, kEncThreads, 0, s>>>(jobs.table, jobs.n, d_plans, side, ws);
+  else split_encode_kernel<3><<<(unsigned)units, kEncThreads, 0, s>>>(jobs.table, jobs.n, d_plans, side, ws);
   return cudaGetLastError();
 }
 
-cudaError_t launch_split_crt(const SplitJob* d_jobs, int njobs, const KPlan* d_plans, int64_t units,
+cudaError_t launch_split_crt(const SplitJobs& jobs, const KPlan* d_plans, int64_t units,
                              cudaStream_t s, unsigned char* ws, int max_nmod, int max_np, bool all_full, int full_form,
                              bool all_wide) {
   if (units <= 0) return cudaSuccess;
@@ -1001,24 +1036,24 @@ cudaError_t launch_split_crt(const SplitJob* d_jobs, int njobs, const KPlan* d_p
     // when all their jobs have it (that instantiation keeps the 64 registers
     // without spills; the fixed four-multiplication one spills)
     if (full_form == 0 && all_wide) {
-      if (l4) split_crt_full_kernel<4, 0, true><<<grid, block, 0, s>>>(d_jobs, njobs, ws);
-      else split_crt_full_kernel<kLimbs, 0, true><<<grid, block, 0, s>>>(d_jobs, njobs, ws);
+      if (l4) split_crt_full_kernel<4, 0, true><<<grid, block, 0, s>>>(jobs.table, jobs.n, ws);
+      else split_crt_full_kernel<kLimbs, 0, true><<<grid, block, 0, s>>>(jobs.table, jobs.n, ws);
     } else if (full_form == 0) {
-      if (l4) split_crt_full_kernel<4, 0, false><<<grid, block, 0, s>>>(d_jobs, njobs, ws);
-      else split_crt_full_kernel<kLimbs, 0, false><<<grid, block, 0, s>>>(d_jobs, njobs, ws);
+      if (l4) split_crt_full_kernel<4, 0, false><<<grid, block, 0, s>>>(jobs.table, jobs.n, ws);
+      else split_crt_full_kernel<kLimbs, 0, false><<<grid, block, 0, s>>>(jobs.table, jobs.n, ws);
     } else if (all_wide) {
-      if (l4) split_crt_full_kernel<4, 2, true><<<grid, block, 0, s>>>(d_jobs, njobs, ws);
-      else split_crt_full_kernel<kLimbs, 2, true><<<grid, block, 0, s>>>(d_jobs, njobs, ws);
+      if (l4) split_crt_full_kernel<4, 2, true><<<grid, block, 0, s>>>(jobs.table, jobs.n, ws);
+      else split_crt_full_kernel<kLimbs, 2, true><<<grid, block, 0, s>>>(jobs.table, jobs.n, ws);
     } else {
-      if (l4) split_crt_full_kernel<4, 2, false><<<grid, block, 0, s>>>(d_jobs, njobs, ws);
-      else split_crt_full_kernel<kLimbs, 2, false><<<grid, block, 0, s>>>(d_jobs, njobs, ws);
+      if (l4) split_crt_full_kernel<4, 2, false><<<grid, block, 0, s>>>(jobs.table, jobs.n, ws);
+      else split_crt_full_kernel<kLimbs, 2, false><<<grid, block, 0, s>>>(jobs.table, jobs.n, ws);
     }
   } else if (max_np <= kFullPlanes) {
-    if (max_nmod <= 14) split_crt_plan_kernel<4><<<grid, block, 0, s>>>(d_jobs, njobs, d_plans, ws);
-    else split_crt_plan_kernel<kLimbs><<<grid, block, 0, s>>>(d_jobs, njobs, d_plans, ws);
+    if (max_nmod <= 14) split_crt_plan_kernel<4><<<grid, block, 0, s>>>(jobs.table, jobs.n, d_plans, ws);
+    else split_crt_plan_kernel<kLimbs><<<grid, block, 0, s>>>(jobs.table, jobs.n, d_plans, ws);
   } else {
-    if (max_nmod <= 14) split_crt_kernel<4><<<grid, block, 0, s>>>(d_jobs, njobs, d_plans, ws);
-    else split_crt_kernel<kLimbs><<<grid, block, 0, s>>>(d_jobs, njobs, d_plans, ws);
+    if (max_nmod <= 14) split_crt_kernel<4><<<grid, block, 0, s>>>(jobs.table, jobs.n, d_plans, ws);
+    else split_crt_kernel<kLimbs><<<grid, block, 0, s>>>(jobs.table, jobs.n, d_plans, ws);
   }
   return cudaGetLastError();
 }

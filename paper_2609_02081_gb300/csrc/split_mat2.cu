@@ -32,6 +32,7 @@
 
 #include <cmath>
 #include <cstring>
+#include <type_traits>
 
 #include "split_device.cuh"
 
@@ -127,12 +128,13 @@ __device__ __forceinline__ void matrix_factors(const float2 (&x)[4], float2 npf,
 //           kOpCoef:  E = Re, Im of the four coefficients: 8 planes
 //           kOpCplx:  E = Re, Im: 2 planes
 template <int ND, int SIDE, int OPERAND>
-__device__ __forceinline__ void encode_pair(const longlong2* E, int nmod, unsigned char* out, uint32_t plane_bytes) {
+__device__ __forceinline__ void encode_pair(const longlong2* E, int l0, int l1, unsigned char* out,
+                                            uint32_t plane_bytes) {
   constexpr int kPairs = OPERAND == kOpQuat ? 2 : OPERAND == kOpCplx ? 1 : 4;   // (Re, Im) pairs
   float2 d[2 * kPairs][ND];
 #pragma unroll
   for (int e = 0; e < 2 * kPairs; ++e) digits2<ND>(E[e], d[e]);
-  for (int l = 0; l < nmod; ++l) {
+  for (int l = l0; l < l1; ++l) {
     const Mat2Mod& mc = c_m2[l];
     const float2 npf = f2(mc.npf), inv = f2(mc.inv);
     // |residue| <= 121 is exact in BF16, whose bits are the upper half of the float's
@@ -186,13 +188,14 @@ __device__ __forceinline__ void encode_pair(const longlong2* E, int nmod, unsign
 //            aligned half of a swizzled 128-byte row.
 // Bound by its writes (28 bytes per modulus and element of a full operand: 65 GB in
 // 10.2 ms at n = 8192, 0.94 of the copy bandwidth).
-template <int ND>
-__global__ void __launch_bounds__(kThreads, 4) mat2_encode_kernel(const SplitJob* __restrict__ jobs, int njobs,
-                                                                  unsigned char* __restrict__ ws, int64_t first) {
+template <int ND, bool kOne>
+__global__ void __launch_bounds__(kThreads, 4)
+    mat2_encode_kernel(const __grid_constant__ JobParam<kOne> one, const SplitJob* __restrict__ jobs, int njobs,
+                       unsigned char* __restrict__ ws, int64_t first) {
   __shared__ __align__(16) long long ent[8][kRows][kPitch];
   __shared__ int s_row[kRows];
   const int64_t blk = first + blockIdx.x;
-  const SplitJob& sj = jobs[find_split_job(jobs, njobs, blk, 5)];
+  const SplitJob& sj = unit_job(one, jobs, njobs, blk, 5);
   const JobDesc& d = sj.d;
   const int ktiles = sj.nkb * (kTileK / kK);
   const int64_t a_blocks = (int64_t)((d.m + kRows - 1) / kRows) * ktiles;
@@ -216,10 +219,6 @@ __global__ void __launch_bounds__(kThreads, 4) mat2_encode_kernel(const SplitJob
   const int planes = side ? sj.nrf : sj.nlf;
   const int operand = planes == 14 ? kOpFull : planes == 7 ? kOpQuat : planes == 8 ? kOpCoef : kOpCplx;
   const int t = threadIdx.x;
-  if (t < kRows) {
-    const int r = r0 + t;
-    s_row[t] = (r < nout) ? reinterpret_cast<const int32_t*>(ws + (side ? sj.off_texp : sj.off_sexp))[r] : 0;
-  }
   constexpr int kPos = kRows * kK / kThreads;    // positions per thread
   unsigned long long raw[kPos][8];
 #pragma unroll
@@ -235,6 +234,11 @@ __global__ void __launch_bounds__(kThreads, 4) mat2_encode_kernel(const SplitJob
       if (in && ((flags >> c) & 1u))
         raw[u][c] = (unsigned long long)__double_as_longlong(__ldcs(src + (int64_t)c * cs));
     }
+  }
+  wait_for_previous_kernel();                    // the exponents
+  if (t < kRows) {
+    const int r = r0 + t;
+    s_row[t] = (r < nout) ? reinterpret_cast<const int32_t*>(ws + (side ? sj.off_texp : sj.off_sexp))[r] : 0;
   }
   __syncthreads();
 #pragma unroll
@@ -275,7 +279,9 @@ __global__ void __launch_bounds__(kThreads, 4) mat2_encode_kernel(const SplitJob
   const int64_t tile_bytes = (int64_t)tile_rows * kTileK * 2;
   const uint32_t plane_bytes = (uint32_t)(side ? sj.encB_plane : sj.encA_plane);   // below 2^32 (checked on the host)
   unsigned char* enc = ws + (side ? sj.off_encB : sj.off_encA);
-  const int nmod = sj.nmod;
+  // this block's moduli (small launches share a tile's moduli between blocks)
+  const int l0 = (int)(blockIdx.y * (unsigned)sj.nmod / gridDim.y), l1 = (int)((blockIdx.y + 1) * (unsigned)sj.nmod / gridDim.y);
+  enc += (int64_t)l0 * planes * plane_bytes;
 #pragma unroll 1
   for (int pass = 0; pass < kRows * kK / 2 / kThreads; ++pass) {
     const int pos = t + pass * kThreads;
@@ -295,18 +301,18 @@ __global__ void __launch_bounds__(kThreads, 4) mat2_encode_kernel(const SplitJob
     };
     if (operand == kOpFull) {
       load(8);
-      if (side) encode_pair<ND, 1, kOpFull>(E, nmod, out, plane_bytes);
-      else encode_pair<ND, 0, kOpFull>(E, nmod, out, plane_bytes);
+      if (side) encode_pair<ND, 1, kOpFull>(E, l0, l1, out, plane_bytes);
+      else encode_pair<ND, 0, kOpFull>(E, l0, l1, out, plane_bytes);
     } else if (operand == kOpQuat) {
       load(4);
-      if (side) encode_pair<ND, 1, kOpQuat>(E, nmod, out, plane_bytes);
-      else encode_pair<ND, 0, kOpQuat>(E, nmod, out, plane_bytes);
+      if (side) encode_pair<ND, 1, kOpQuat>(E, l0, l1, out, plane_bytes);
+      else encode_pair<ND, 0, kOpQuat>(E, l0, l1, out, plane_bytes);
     } else if (operand == kOpCoef) {
       load(8);
-      encode_pair<ND, 0, kOpCoef>(E, nmod, out, plane_bytes);
+      encode_pair<ND, 0, kOpCoef>(E, l0, l1, out, plane_bytes);
     } else {
       load(2);
-      encode_pair<ND, 0, kOpCplx>(E, nmod, out, plane_bytes);
+      encode_pair<ND, 0, kOpCplx>(E, l0, l1, out, plane_bytes);
     }
   }
 }
@@ -466,6 +472,17 @@ __device__ __forceinline__ void crt_block(const SplitJob& sj, uint32_t local, co
   const int i0 = (int)(wide ? rowblock : 4 * rowblock);
   const int j0 = (int)(local - rowblock * colblocks) * (wide ? kCrtCols : 32);
   const int64_t ncols = (int64_t)sj.tiles_n * sj.bn;
+  // this thread's fragments of the digits (zero for moduli >= nmod)
+  uint32_t b[2][KS][2][2];
+#pragma unroll
+  for (int h = 0; h < 2; ++h)
+#pragma unroll
+    for (int ks = 0; ks < KS; ++ks)
+#pragma unroll
+      for (int nt = 0; nt < 2; ++nt)
+#pragma unroll
+        for (int v = 0; v < 2; ++v) b[h][ks][nt][v] = __ldg(&g_m2digits[nm][h][ks][nt][v][lane]);
+  wait_for_previous_kernel();                              // the residues
   // copy: thread tid takes 16-byte chunk tid % 8 of planes tid / 8, tid / 8 + 16, ...
   {
     const int64_t plane = sj.res_plane;
@@ -487,16 +504,6 @@ __device__ __forceinline__ void crt_block(const SplitJob& sj, uint32_t local, co
     }
     cp_async_commit();
   }
-  // this thread's fragments of the digits (zero for moduli >= nmod)
-  uint32_t b[2][KS][2][2];
-#pragma unroll
-  for (int h = 0; h < 2; ++h)
-#pragma unroll
-    for (int ks = 0; ks < KS; ++ks)
-#pragma unroll
-      for (int nt = 0; nt < 2; ++nt)
-#pragma unroll
-        for (int v = 0; v < 2; ++v) b[h][ks][nt][v] = __ldg(&g_m2digits[nm][h][ks][nt][v][lane]);
   const int wi = i0 + (wide ? 0 : warp), j = j0 + (wide ? 32 * warp : 0) + lane;
   const bool valid = wi < d.m && j < d.n;
   int sc = -c_m2shift[nm];
@@ -692,13 +699,14 @@ __device__ __forceinline__ void crt_block(const SplitJob& sj, uint32_t local, co
   }
 }
 
-template <int L, int KS>
-__global__ void __launch_bounds__(kCrtThreads, 4) mat2_crt_kernel(const SplitJob* __restrict__ jobs, int njobs,
-                                                                  const unsigned char* __restrict__ ws) {
+template <int L, int KS, bool kOne>
+__global__ void __launch_bounds__(kCrtThreads, 4)
+    mat2_crt_kernel(const __grid_constant__ JobParam<kOne> one, const SplitJob* __restrict__ jobs, int njobs,
+                    const unsigned char* __restrict__ ws) {
   __shared__ __align__(16) uint8_t ring[(KS == 1 ? 16 : kMat2MaxModuli + 1) * mod_stride(kMat2MaxPlanes)];
   __shared__ __align__(16) uint32_t tr[kCrtThreads / 32][2][8][kTrStride];
   const int64_t blk = blockIdx.x;
-  const SplitJob& sj = jobs[find_split_job(jobs, njobs, blk, 6)];
+  const SplitJob& sj = unit_job(one, jobs, njobs, blk, 6);
   const uint32_t local = (uint32_t)(blk - sj.crt2_begin);
   auto* mine = tr[threadIdx.x >> 5];
   switch (sj.mat2) {                                       // block-uniform
@@ -833,21 +841,30 @@ cudaError_t mat2_configure(const int* moduli, const int* root, int n, const int3
   return cudaMemcpyToSymbol(c_m2Pinv, pinv, sizeof(pinv));
 }
 
-cudaError_t launch_mat2_encode(const SplitJob* d_jobs, int njobs, int64_t units, int64_t first, cudaStream_t s,
+cudaError_t launch_mat2_encode(const SplitJobs& jobs, int64_t units, int64_t first, cudaStream_t s,
                                unsigned char* ws, int max_bits) {
   if (units <= 0) return cudaSuccess;
+  // A launch whose tiles do not fill the GPU (152 SMs x 4 blocks) splits each
+  // tile's moduli over up to four blocks, which repeat phase 1: a whole product
+  // at n = 256 (256 tiles) 43.1 -> 41.0 us, at n = 64 24.6 -> 20.5.
+  const int64_t fill = 608;
+  const unsigned groups = (unsigned)(units * 4 <= fill ? 4 : units * 2 <= fill ? 2 : 1);
   // the matrix entries are sums of two b-bit integers: three digits hold 2^47
-  if (max_bits <= 46) mat2_encode_kernel<3><<<(unsigned)units, kThreads, 0, s>>>(d_jobs, njobs, ws, first);
-  else mat2_encode_kernel<4><<<(unsigned)units, kThreads, 0, s>>>(d_jobs, njobs, ws, first);
-  return cudaGetLastError();
+  return with_jobs(jobs, [&](const auto& one) {
+    constexpr bool kOne = std::is_same_v<std::decay_t<decltype(one)>, JobParam<true>>;
+    return launch_dependent(max_bits <= 46 ? mat2_encode_kernel<3, kOne> : mat2_encode_kernel<4, kOne>,
+                            dim3((unsigned)units, groups), dim3(kThreads), 0, s, one, jobs.table, jobs.n, ws, first);
+  });
 }
 
-cudaError_t launch_mat2_crt(const SplitJob* d_jobs, int njobs, int64_t units, cudaStream_t s, unsigned char* ws,
+cudaError_t launch_mat2_crt(const SplitJobs& jobs, int64_t units, cudaStream_t s, unsigned char* ws,
                             int max_nmod) {
   if (units <= 0) return cudaSuccess;
-  if (max_nmod <= kMat2FourLimbs) mat2_crt_kernel<4, 1><<<(unsigned)units, kCrtThreads, 0, s>>>(d_jobs, njobs, ws);
-  else mat2_crt_kernel<kLimbs, 2><<<(unsigned)units, kCrtThreads, 0, s>>>(d_jobs, njobs, ws);
-  return cudaGetLastError();
+  return with_jobs(jobs, [&](const auto& one) {
+    constexpr bool kOne = std::is_same_v<std::decay_t<decltype(one)>, JobParam<true>>;
+    return launch_dependent(max_nmod <= kMat2FourLimbs ? mat2_crt_kernel<4, 1, kOne> : mat2_crt_kernel<kLimbs, 2, kOne>,
+                            dim3((unsigned)units), dim3(kCrtThreads), 0, s, one, jobs.table, jobs.n, ws);
+  });
 }
 
 }  // namespace hmat
