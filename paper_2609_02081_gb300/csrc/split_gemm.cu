@@ -25,9 +25,10 @@
 //               (kind::f16, BF16 in, FP32 accumulate, M=128, N=bn, K=16) into
 //               one of two accumulator buffers, commits stages and chunks;
 //   warps 2..9  epilogue: tcgen05.ld of finished chunks (each warp its 32-lane
-//               quadrant and half the columns), mod p, int8 stores of the rows
-//               and columns inside the product.  Two accumulator buffers let
-//               chunk c+1 run on the tensor core while chunk c is drained.
+//               quadrant and half the columns, or every other item), mod p, int8
+//               stores of the rows and columns inside the product.  Two
+//               accumulator buffers let chunk c+1 run on the tensor core while
+//               chunk c is drained.
 // Each role walks its items in increasing order with a forward cursor over the
 // job table (no search per item).
 // Every mbarrier wait is bounded (~2 s); on timeout the CTA raises the device
@@ -304,7 +305,7 @@ split_residue_gemm_kernel(const __grid_constant__ JobParam<kOne> one, const Spli
     }
     for (int i = 0; i < 2; ++i) {
       mbar_init(smem_u32(&s.tfull[i]), 1);
-      mbar_init(smem_u32(&s.tempty[i]), kEpiWarps);
+      mbar_init(smem_u32(&s.tempty[i]), kOneChunk ? kEpiWarps / 2 : kEpiWarps);
     }
     mbar_init(smem_u32(&s.final_bar), 1);
     s.abort_flag = 0;
@@ -320,7 +321,6 @@ split_residue_gemm_kernel(const __grid_constant__ JobParam<kOne> one, const Spli
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = s.tmem_base;
-
   wait_for_previous_kernel();           // the encoded factors
 
   if (warp == 0) {
@@ -414,14 +414,21 @@ split_residue_gemm_kernel(const __grid_constant__ JobParam<kOne> one, const Spli
     const int q = warp & 3;               // TMEM lane quadrant of this warp
     const int half = (warp - 2) >> 2;     // which half of the tile's columns
     const int row = q * 32 + lane;
-    uint32_t chunk_ctr = 0;
+    // One-chunk launches: the two halves of the epilogue warps take alternate items
+    // (each its own accumulator buffer, all columns), so that one item's decode,
+    // TMEM loads and stores overlap the other's (the 512-product batch: GEMM 10.2
+    // -> 8.9 ms; 64 small products 220 -> 200 us).  Otherwise every warp takes half
+    // the columns of every item.
+    const uint32_t first = kOneChunk ? (uint32_t)half : 0u, stride = kOneChunk ? 2u : 1u;
+    uint32_t chunk_ctr = first;
     bool ok = true;
-    int job = kOne ? 0 : find_item_job(jobs, njobs, blockIdx.x);
-    for (int64_t item = blockIdx.x; ok && item < total_items; item += gridDim.x) {
+    const int64_t item0 = blockIdx.x + (int64_t)first * gridDim.x;
+    int job = kOne || item0 >= total_items ? 0 : find_item_job(jobs, njobs, item0);
+    for (int64_t item = item0; ok && item < total_items; item += (int64_t)stride * gridDim.x) {
       if constexpr (!kOne) job = advance_job(jobs, njobs, item, job);
       const Item it = decode_item(item_job(one, jobs, job), item, ws);
-      const int cols = it.bn >> 1;        // columns handled by this thread: a multiple of 16 up to 128
-      const int col0 = half * cols;
+      const int cols = kOneChunk ? it.bn : it.bn >> 1;   // columns handled by this thread: a multiple of 16
+      const int col0 = kOneChunk ? 0 : half * cols;
       const int nchunks = (it.nkb + kKbPerChunk - 1) / kKbPerChunk;
       const float pf = c_gmod[it.l].pf, pinv = c_gmod[it.l].inv, magic = c_gmod[it.l].magic;
       const float2 npf2 = make_float2(-pf, -pf), inv2 = make_float2(pinv, pinv);
@@ -474,7 +481,7 @@ split_residue_gemm_kernel(const __grid_constant__ JobParam<kOne> one, const Spli
         if constexpr (kOneChunk) {
           // two 32-column loads per wait (registers this form leaves free)
 #pragma unroll
-          for (int g = 0; g < kBnMax / 2 / 32; g += 2) {
+          for (int g = 0; g < kBnMax / 32; g += 2) {
             if (g * 32 >= cols) break;
             const bool two = (g + 1) * 32 < cols;
             uint32_t r[64];
@@ -499,7 +506,7 @@ split_residue_gemm_kernel(const __grid_constant__ JobParam<kOne> one, const Spli
             if (row < it.rows) drain32(g, r);
           }
         }
-        ++chunk_ctr;
+        chunk_ctr += stride;
         continue;
       }
       if constexpr (kOneChunk) {
