@@ -74,8 +74,8 @@ hmat_status hmat_bq_add(hmat_handle h, int32_t opA, int32_t opB, uint32_t flagsA
   if (flagsA == 0) p.a.X = nullptr;
   if (!p.a.X) p.a.flags = 0;
   p.alpha_re = alpha_re; p.alpha_im = alpha_im; p.beta_re = beta_re; p.beta_im = beta_im;
-  p.kind_a = scalar_kind(alpha_re, alpha_im);
-  p.kind_b = p.b.X ? scalar_kind(beta_re, beta_im) : kScalarZero;
+  p.kind_a = p.b.X ? as_axpby_kind(alpha_re, alpha_im) : scalar_kind(alpha_re, alpha_im);
+  p.kind_b = p.b.X ? as_axpby_kind(beta_re, beta_im) : kScalarZero;
   p.C = C; p.ldc = ldc; p.sC = strideC; p.m = (int32_t)m; p.n = (int32_t)n;
   std::lock_guard<std::mutex> lock(h->mu);
   ProfScope ps(h, 8, static_cast<cudaStream_t>(stream));

@@ -20,9 +20,9 @@
 // element.  Everything that is not arithmetic stays in the integer pipes: the
 // op signs and negations flip the sign bit, maxima compare bit patterns,
 // halving decrements the exponent (falling back to a multiply only for zero,
-// subnormal and the smallest normal numbers), and scalars 0, +-1, +-i permute
-// and negate instead of multiplying.  Each result is still the correctly
-// rounded value of the formula's steps in order, bit for bit.
+// subnormal and the smallest normal numbers), scalars 0, +-1, +-i permute and
+// negate instead of multiplying, and +-2^k adds to the exponent.  Each result is
+// still the correctly rounded value of the formula's steps in order, bit for bit.
 //
 // Layout: operands read without transposition stream along their rows (RT
 // threads cover RT * V consecutive columns of one row; V = 2 uses 16-byte
@@ -83,6 +83,21 @@ __device__ __forceinline__ double half_fast(double x, bool& bad) {
   return zero ? x : __hiloint2double(hi - (1 << 20), lo);
 }
 
+// x times the +-2^k whose sign bit and exponent step (k << 20) are given, for
+// zeros and values whose biased exponent and the result's lie in 1..2046; `bad` is
+// set for anything else (subnormals, inf, NaN, overflow), which a multiply must redo.
+__device__ __forceinline__ double pow2_fast(double x, int step, unsigned flip, bool& bad) {
+  const int hi = __double2hiint(x), lo = __double2loint(x);
+  const int e = (int)(((unsigned)hi >> 20) & 0x7FFu), r = e + (step >> 20);
+  const bool zero = ((hi & 0x7FFFFFFF) | lo) == 0;
+  bad |= !zero && ((unsigned)(e - 1) > 2045u || (unsigned)(r - 1) > 2045u);
+  return __hiloint2double((zero ? hi : hi + step) ^ (int)flip, lo);
+}
+// Not inlined: reached through a warp-uniform branch, which keeps the multiplies behind it.
+__device__ __noinline__ double2 scaled_slow(double a, double x0, double x1) {
+  return make_double2(__dmul_rn(a, x0), __dmul_rn(a, x1));
+}
+
 // (x0 + i x1) times the scalar of kind k (ScalarKind), step by step as
 // (a_R x0 - a_I x1) + i (a_R x1 + a_I x0).
 __device__ __forceinline__ void scale_pair(int k, double ar, double ai, double x0, double x1, double* re,
@@ -99,6 +114,28 @@ __device__ __forceinline__ void scale_pair(int k, double ar, double ai, double x
       break;
     default: *re = 0.0; *im = 0.0; break;
   }
+}
+
+// scale_pair where, with kPow2, kScalarPow2 may occur (launches without it keep the
+// smaller code: with it 2.5 X at n = 8192 took 1.40 ms, 1.23 without).
+template <bool kPow2>
+__device__ __forceinline__ void scale_any(int k, double ar, double ai, double x0, double x1, double* re, double* im) {
+  if constexpr (kPow2) {
+    if (k == kScalarPow2) {
+      const int step = (int)(((unsigned)__double2hiint(ar) & 0x7FF00000u) - (1023u << 20));
+      const unsigned flip = (unsigned)__double2hiint(ar) & 0x80000000u;
+      bool bad = false;
+      *re = pow2_fast(x0, step, flip, bad);
+      *im = pow2_fast(x1, step, flip, bad);
+      if (__any_sync(__activemask(), bad)) {
+        const double2 z = scaled_slow(ar, x0, x1);
+        *re = z.x;
+        *im = z.y;
+      }
+      return;
+    }
+  }
+  scale_pair(k, ar, ai, x0, x1, re, im);
 }
 
 // max |a_k - b_k| (as bit patterns) over the k whose bit is set in `mask`.
@@ -183,6 +220,7 @@ __device__ __forceinline__ void tile_origin(int64_t tile, int cols, int64_t* r0,
 // Four resident blocks per SM (64 registers a thread, no spills): at two
 // (110 registers, the inlined general scalar path) A^dagger + B ran at 0.63 of
 // the HBM peak, at four at 0.83.
+template <bool kPow2>
 __global__ void __launch_bounds__(TT * TY, 4) axpby_tiles_kernel(AxpbyParams p) {
   __shared__ Tile sa0, sa1, sb0, sb1;
   int64_t r0, q0;
@@ -208,10 +246,10 @@ __global__ void __launch_bounds__(TT * TY, 4) axpby_tiles_kernel(AxpbyParams p) 
       const int r = threadIdx.y + k, q = threadIdx.x;
       if (r0 + r < p.m && q0 + q < p.n) {
         double re, im;
-        scale_pair(p.kind_a, p.alpha_re, p.alpha_im, sa0[r][q], sa1[r][q], &re, &im);
+        scale_any<kPow2>(p.kind_a, p.alpha_re, p.alpha_im, sa0[r][q], sa1[r][q], &re, &im);
         if (has_b) {
           double bre, bim;
-          scale_pair(p.kind_b, p.beta_re, p.beta_im, sb0[r][q], sb1[r][q], &bre, &bim);
+          scale_any<kPow2>(p.kind_b, p.beta_re, p.beta_im, sb0[r][q], sb1[r][q], &bre, &bim);
           re = __dadd_rn(re, bre);
           im = __dadd_rn(im, bim);
         }
@@ -221,6 +259,156 @@ __global__ void __launch_bounds__(TT * TY, 4) axpby_tiles_kernel(AxpbyParams p) 
       }
     }
     __syncthreads();
+  }
+}
+
+__device__ __forceinline__ void tri_index(int64_t b, int64_t* I, int64_t* J);
+
+// axpby of one square matrix with itself, one operand transposed and the other
+// not (alpha X + beta X^dagger): one block per tile pair (I <= J) reads tiles
+// (I, J) and (J, I) once and writes both outputs, where the general kernel reads
+// every entry twice.  Each thread keeps the entries of its own outputs in
+// registers; only the transposed ones go through shared memory.
+__global__ void __launch_bounds__(TT * TY, 3) axpby_pair_kernel(AxpbyParams p) {
+  __shared__ Tile s1[2], s2[2];
+  int64_t I, J;
+  tri_index(blockIdx.x, &I, &J);
+  const int64_t r0 = I * TT, q0 = J * TT;
+  const uint32_t both = p.a.flags | p.b.flags;
+  const BqView &a = p.a, &b = p.b;
+  for (int e = 0; e < 4; ++e) {
+    TileRegs t1[2], t2[2];                     // tiles (I, J) and (J, I) of components e, e + 4
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int c = e + 4 * h;
+      const double* base = a.X + (int64_t)c * a.cs;
+      const bool present = (both >> c) & 1u;
+      fetch_tile(base, a.ld, present, false, false, r0, q0, p.n, p.n, t1[h]);
+      fetch_tile(base, a.ld, present, false, false, q0, r0, p.n, p.n, t2[h]);
+    }
+    if (e > 0) __syncthreads();                // the previous components' tiles have been read
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      put_tile(t1[h], true, s1[h]);            // s1[q][r] = X[r0 + r][q0 + q]
+      put_tile(t2[h], true, s2[h]);
+    }
+    __syncthreads();
+    auto out = [&](const TileRegs (&own)[2], const Tile (&other)[2], int64_t ro, int64_t qo) {
+#pragma unroll
+      for (int k = 0; k < TT / TY; ++k) {
+        const int r = threadIdx.y + k * TY, q = threadIdx.x;
+        if (ro + r < p.n && qo + q < p.n) {
+          double x[2], y[2];                   // op(A), op(B) entries
+#pragma unroll
+          for (int h = 0; h < 2; ++h) {
+            const int c = e + 4 * h;
+            // the transposed operand's entry (r, q) is the other tile's (q, r)
+            const double d = own[h].v[k], t = other[h][r][q];
+            x[h] = flip_if(((a.flags >> c) & 1u) ? (a.trans ? t : d) : 0.0, a.sign[c] < 0);
+            y[h] = flip_if(((b.flags >> c) & 1u) ? (a.trans ? d : t) : 0.0, b.sign[c] < 0);
+          }
+          double re, im, bre, bim;
+          scale_any<true>(p.kind_a, p.alpha_re, p.alpha_im, x[0], x[1], &re, &im);
+          scale_any<true>(p.kind_b, p.beta_re, p.beta_im, y[0], y[1], &bre, &bim);
+          double* c = p.C + (ro + r) * p.ldc + (qo + q);
+          c[(int64_t)e * p.sC] = __dadd_rn(re, bre);
+          c[(int64_t)(e + 4) * p.sC] = __dadd_rn(im, bim);
+        }
+      }
+    };
+    out(t1, s2, r0, q0);
+    if (I != J) out(t2, s1, q0, r0);
+  }
+}
+
+// The same for |alpha| = |beta| = 2^k, -32 <= k <= 0 (the Hermitian part: 1/2, 1/2)
+// and equal component flags: +-a +- b in one FP64 addition, then k added to the
+// exponent of the sum.  For a sum of biased exponent 128..1900 that is the rounded
+// sum of the exactly scaled terms: a term whose scaling would round is below 2^-960
+// and too small to reach the other one's last bit.  Every other sum but zero takes
+// the formula's steps one by one, behind a warp-uniform branch.  Instructions per
+// entry decide here: with the general kernel's scalar switch 0.5 X + 0.5 X^dagger at
+// n = 4096 took 546 us, issue-bound (873 us in the general kernel); this one 405 us,
+// 5.3 TB/s.
+__device__ __noinline__ double scaled_sum_slow(double sa, double x, double sb, double y) {
+  return __dadd_rn(__dmul_rn(sa, x), __dmul_rn(sb, y));
+}
+
+__global__ void __launch_bounds__(TT * TY, 3) axpby_pair_scaled_kernel(AxpbyParams p) {
+  __shared__ Tile s1[2], s2[2];
+  int64_t I, J;
+  tri_index(blockIdx.x, &I, &J);
+  const int r0 = (int)I * TT, q0 = (int)J * TT, n = p.n;
+  const bool inside = q0 + TT <= n;              // both tiles (r0 <= q0)
+  const BqView& a = p.a;
+  const int64_t ld = a.ld;
+  const int tx = threadIdx.x, ty = threadIdx.y;
+  const int step = (int)(((unsigned)__double2hiint(p.alpha_re) & 0x7FF00000u) - (1023u << 20));
+  const double* const own1 = a.X + (int64_t)(r0 + ty) * ld + q0 + tx;
+  const double* const own2 = a.X + (int64_t)(q0 + ty) * ld + r0 + tx;
+  double* const out1 = p.C + (int64_t)(r0 + ty) * p.ldc + q0 + tx;
+  double* const out2 = p.C + (int64_t)(q0 + ty) * p.ldc + r0 + tx;
+  constexpr int kPer = TT / TY;
+#pragma unroll 1
+  for (int e = 0; e < 4; ++e) {
+    double t1[2][kPer], t2[2][kPer];             // tiles (I, J) and (J, I) of components e, e + 4
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int c = e + 4 * h;
+      const bool present = (a.flags >> c) & 1u;
+#pragma unroll
+      for (int k = 0; k < kPer; ++k) {
+        const int64_t at = (int64_t)c * a.cs + (int64_t)(k * TY) * ld;
+        const bool in1 = present && (inside || (r0 + ty + k * TY < n && q0 + tx < n));
+        const bool in2 = present && (inside || (q0 + ty + k * TY < n && r0 + tx < n));
+        t1[h][k] = in1 ? __ldcs(own1 + at) : 0.0;
+        t2[h][k] = in2 ? __ldcs(own2 + at) : 0.0;
+      }
+    }
+    if (e > 0) __syncthreads();                  // the previous components' tiles have been read
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+#pragma unroll
+      for (int k = 0; k < kPer; ++k) {
+        s1[h][tx][ty + k * TY] = t1[h][k];
+        s2[h][tx][ty + k * TY] = t2[h][k];
+      }
+    __syncthreads();
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int c = e + 4 * h;
+      // sign bits of the scaled own (not transposed) and other (transposed) entry
+      const unsigned fa = ((unsigned)__double2hiint(p.alpha_re) ^ (a.sign[c] < 0 ? 0x80000000u : 0u)) & 0x80000000u;
+      const unsigned fb = ((unsigned)__double2hiint(p.beta_re) ^ (p.b.sign[c] < 0 ? 0x80000000u : 0u)) & 0x80000000u;
+      const unsigned fo = a.trans ? fb : fa, ft = a.trans ? fa : fb;
+      const double so = __hiloint2double((int)(0x3FF00000u + (unsigned)step | fo), 0);
+      const double st = __hiloint2double((int)(0x3FF00000u + (unsigned)step | ft), 0);
+      auto emit = [&](const double (&own)[kPer], const Tile& other, double* out, int ro, int qo) {
+        double y[kPer], v[kPer];
+        bool bad = false;
+#pragma unroll
+        for (int k = 0; k < kPer; ++k) {
+          y[k] = other[ty + k * TY][tx];
+          const double x = __hiloint2double(__double2hiint(own[k]) ^ (int)fo, __double2loint(own[k]));
+          const double z = __hiloint2double(__double2hiint(y[k]) ^ (int)ft, __double2loint(y[k]));
+          const double sum = __dadd_rn(x, z);
+          const int hi = __double2hiint(sum), lo = __double2loint(sum);
+          const unsigned mag = (unsigned)hi & 0x7FFFFFFFu;
+          const bool zero = (mag | (unsigned)lo) == 0u;
+          bad |= !zero && mag - (128u << 20) >= (1773u << 20);
+          v[k] = __hiloint2double(zero ? hi : hi + step, lo);
+        }
+        if (step != 0 && __any_sync(0xffffffffu, bad)) {
+#pragma unroll
+          for (int k = 0; k < kPer; ++k) v[k] = scaled_sum_slow(so, own[k], st, y[k]);
+        }
+#pragma unroll
+        for (int k = 0; k < kPer; ++k)
+          if (inside || (ro + ty + k * TY < n && qo + tx < n)) out[(int64_t)c * p.sC + (int64_t)(k * TY) * p.ldc] = v[k];
+      };
+      emit(t1[h], s2[h], out1, r0, q0);
+      if (I != J) emit(t2[h], s1[h], out2, q0, r0);
+    }
   }
 }
 
@@ -425,7 +613,7 @@ __device__ __forceinline__ int valid_count(int64_t q, int32_t n, int V) {
   return r >= V ? V : (r > 0 ? (int)r : 0);
 }
 
-template <int V>
+template <int V, bool kPow2>
 __global__ void __launch_bounds__(RT) axpby_rows_kernel(AxpbyParams p) {
   int64_t row, q;
   row_origin(p.n, V, &row, &q);
@@ -441,10 +629,10 @@ __global__ void __launch_bounds__(RT) axpby_rows_kernel(AxpbyParams p) {
     double re[V], im[V];
 #pragma unroll
     for (int u = 0; u < V; ++u) {
-      scale_pair(p.kind_a, p.alpha_re, p.alpha_im, a[e][u], a[e + 4][u], &re[u], &im[u]);
+      scale_any<kPow2>(p.kind_a, p.alpha_re, p.alpha_im, a[e][u], a[e + 4][u], &re[u], &im[u]);
       if (has_b) {
         double bre, bim;
-        scale_pair(p.kind_b, p.beta_re, p.beta_im, b[e][u], b[e + 4][u], &bre, &bim);
+        scale_any<kPow2>(p.kind_b, p.beta_re, p.beta_im, b[e][u], b[e + 4][u], &bre, &bim);
         re[u] = __dadd_rn(re[u], bre);
         im[u] = __dadd_rn(im[u], bim);
       }
@@ -686,14 +874,41 @@ int scalar_kind(double re, double im) {
   return kScalarGeneral;
 }
 
+int as_axpby_kind(double re, double im) {
+  const int k = scalar_kind(re, im);
+  if (k != kScalarReal) return k;
+  int e = 0;
+  const double f = std::frexp(std::fabs(re), &e);   // |re| = f 2^e, f in [0.5, 1)
+  return f == 0.5 && std::abs(e - 1) <= 64 ? (int)kScalarPow2 : k;
+}
+
 cudaError_t launch_axpby(const AxpbyParams& p, cudaStream_t s) {
   if (p.m <= 0 || p.n <= 0) return cudaSuccess;
-  if (p.a.trans || (p.b.trans && p.kind_b != kScalarZero)) {
-    axpby_tiles_kernel<<<tiles_grid(p.m, p.n), dim3(TT, TY), 0, s>>>(p);
+  const bool pow2 = p.kind_a == kScalarPow2 || p.kind_b == kScalarPow2;
+  const bool same = p.kind_a != kScalarZero && p.kind_b != kScalarZero && p.a.X == p.b.X && p.a.ld == p.b.ld &&
+                    p.a.cs == p.b.cs && p.m == p.n && p.a.trans != p.b.trans;
+  if (same) {
+    const int64_t t = (p.n + TT - 1) / TT;
+    const unsigned grid = (unsigned)(t * (t + 1) / 2);
+    auto real = [](int k) { return k == kScalarOne || k == kScalarMinusOne || k == kScalarPow2; };
+    const double al = std::fabs(p.alpha_re);
+    if (real(p.kind_a) && real(p.kind_b) && al == std::fabs(p.beta_re) && al <= 1.0 && al >= std::ldexp(1.0, -32) &&
+        p.a.flags == p.b.flags)
+      axpby_pair_scaled_kernel<<<grid, dim3(TT, TY), 0, s>>>(p);
+    else
+      axpby_pair_kernel<<<grid, dim3(TT, TY), 0, s>>>(p);
+  } else if (p.a.trans || (p.b.trans && p.kind_b != kScalarZero)) {
+    const unsigned grid = tiles_grid(p.m, p.n);
+    if (pow2) axpby_tiles_kernel<true><<<grid, dim3(TT, TY), 0, s>>>(p);
+    else axpby_tiles_kernel<false><<<grid, dim3(TT, TY), 0, s>>>(p);
   } else if (vec2_ok(p.a.X, p.a.ld, p.a.cs) && vec2_ok(p.b.X, p.b.ld, p.b.cs) && vec2_ok(p.C, p.ldc, p.sC)) {
-    axpby_rows_kernel<2><<<rows_grid(p.m, p.n, 2), RT, 0, s>>>(p);
+    const unsigned grid = rows_grid(p.m, p.n, 2);
+    if (pow2) axpby_rows_kernel<2, true><<<grid, RT, 0, s>>>(p);
+    else axpby_rows_kernel<2, false><<<grid, RT, 0, s>>>(p);
   } else {
-    axpby_rows_kernel<1><<<rows_grid(p.m, p.n, 1), RT, 0, s>>>(p);
+    const unsigned grid = rows_grid(p.m, p.n, 1);
+    if (pow2) axpby_rows_kernel<1, true><<<grid, RT, 0, s>>>(p);
+    else axpby_rows_kernel<1, false><<<grid, RT, 0, s>>>(p);
   }
   return cudaGetLastError();
 }
