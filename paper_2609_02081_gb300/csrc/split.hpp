@@ -135,7 +135,7 @@ struct SplitJob {
   int32_t np, nlf, nrf;
   int32_t full;                     // the plan is the paper's full plan (KPlan::bilinear_full), either form
   int32_t four_m;                   // two-term products: p is pl pr + (-1 if bit p of neg2) pl2 pr2
-  int32_t crt_w;                    // full-plan CRT: columns per block row (kCrtCols / crt_w rows)
+  int32_t crt_w;                    // full-plan and matrix-form CRT: columns per block row (kCrtCols / crt_w rows)
   int8_t pl[kMaxProducts], pr[kMaxProducts];
   int8_t pl2[kMaxProducts], pr2[kMaxProducts];
   uint64_t neg2;

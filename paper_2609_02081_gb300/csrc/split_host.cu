@@ -361,15 +361,23 @@ static inline int64_t enc_blocks(int64_t rows, int64_t nkb) { return ((rows + 15
 static inline int64_t crt_blocks(int64_t m, int64_t n, int rows) {
   return ((m + rows - 1) / rows) * ((n + kCrtCols - 1) / kCrtCols);
 }
-// CRT blocks of a job and its block width: the full-plan and matrix-form kernels' blocks
-// are kCrtCols / crt_width(n) rows of crt_width(n) columns, the other kernels'
-// kCrtRows rows of kCrtCols columns
+// CRT blocks of a job and its block width: the full-plan kernel's blocks are
+// kCrtCols / crt_width(n) rows of crt_width(n) columns, the matrix form's likewise
+// with mat2_crt_width, the other kernels' kCrtRows rows of kCrtCols columns
+// Matrix form: the widest block (longest contiguous residue reads) that pads the
+// columns by at most 6 % more than 32-wide ones would.  The 512-product batch's CRT:
+// 3.59 ms with 32 columns for all n < 1024, 3.45 with this, 3.56 at 30 %.
+static int mat2_crt_width(int64_t n) {
+  for (int w = kCrtCols; w > 32; w /= 2)
+    if (100 * ((n + w - 1) / w * w) <= 106 * ((n + 31) / 32 * 32)) return w;
+  return 32;
+}
 static inline int64_t crt_job_blocks(SplitJob& sj, bool all_full) {
   if (!all_full && !sj.mat2) {
     sj.crt_w = kCrtCols;
     return crt_blocks(sj.d.m, sj.d.n, kCrtRows);
   }
-  sj.crt_w = crt_width(sj.d.n);
+  sj.crt_w = sj.mat2 ? mat2_crt_width(sj.d.n) : crt_width(sj.d.n);
   const int64_t rows = kCrtCols / sj.crt_w;
   return ((sj.d.m + rows - 1) / rows) * ((sj.d.n + sj.crt_w - 1) / sj.crt_w);
 }

@@ -319,7 +319,7 @@ __global__ void __launch_bounds__(kThreads, 4)
 
 // ------------------------------------------------------------------ CRT
 // One warp per 32 consecutive elements of an output row; a block of four warps
-// covers one row of 128 columns, or four rows of 32 for narrow products.
+// covers one row of 128 columns, two of 64 or four of 32.
 //
 // Per element and modulus the outputs are sums of the product residues.  With cu,
 // cv the entries of the two copies' 2 x 2 products:
@@ -346,10 +346,10 @@ __global__ void __launch_bounds__(kThreads, 4)
 // 2^(16 i), transposed through shared memory so that a lane owns one column, and
 // finished there.
 //
-// Bound by instruction issue (2.7 of 4 per cycle, 57 instructions per element and
-// warp lane; 64-bit multiply-adds per modulus, output and limb took 113): 1.25 ms
-// for 4096 x 4096 (2.35 ms with those), 0.87 ms of which its 5.9 GB would take at
-// the copy bandwidth; the 512-product batch 3.6 ms (6.1 ms).
+// Bound by instruction issue (2.6 of 4 per cycle, 54 instructions per element and
+// warp lane; 64-bit multiply-adds per modulus, output and limb took 113): 1.2 ms
+// for 4096 x 4096 (2.35 ms with those), 0.68 ms of which its 4.6 GB would take at
+// the copy bandwidth; the 512-product batch 3.45 ms (6.1 ms).
 constexpr int kCrtThreads = 128;
 constexpr int mod_stride(int planes) {                // bytes; the four moduli pairs of a read fall on different banks
   return planes * kCrtCols + 16;
@@ -359,10 +359,11 @@ constexpr int kTrStride = 40;                         // words; likewise for the
 // digits of the CRT elements in the B fragments' layout: [nmod][half][k step][n tile][register][lane]
 __device__ uint32_t g_m2digits[kMat2MaxModuli + 1][2][2][2][2][32];
 
-__device__ __forceinline__ void mma_f16(float (&c)[4], const uint32_t (&a)[4], const uint32_t (&b)[2]) {
-  asm("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
-      : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
-      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[0]), "r"(b[1]));
+__device__ __forceinline__ void mma_f16(float (&d)[4], const uint32_t (&a)[4], const uint32_t (&b)[2],
+                                        const float (&c)[4]) {
+  asm("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%10,%11,%12,%13};"
+      : "=f"(d[0]), "=f"(d[1]), "=f"(d[2]), "=f"(d[3])
+      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[0]), "r"(b[1]), "f"(c[0]), "f"(c[1]), "f"(c[2]), "f"(c[3]));
 }
 __device__ __forceinline__ uint32_t hadd2(uint32_t a, uint32_t b) {
   uint32_t r;
@@ -375,14 +376,15 @@ __device__ __forceinline__ uint32_t hsub2(uint32_t a, uint32_t b) {
   return r;
 }
 
-// kMagic + x for an FP32 sum x 2^-24 of the products: its bits are kMagicBits + x
-constexpr float kMagic = 12582912.0f;
-constexpr uint32_t kMagicBits = 0x4B400000u;
+// The accumulators start at kMagic: with an integer sum x, |x| < 2^22, the result
+// kMagic + x 2^-24 lies in (0.5, 1), where a float's last bit is 2^-24, so its bits
+// are kMagicBits + x and no conversion is needed.
+constexpr float kMagic = 0.75f;
+constexpr uint32_t kMagicBits = 0x3F400000u;
 // the packed pair of digit sums x0 + 256 x1, plus this constant
 constexpr uint32_t kPairBias = kMagicBits * 257u;
 __device__ __forceinline__ uint32_t digit_pair(float x0, float x1) {
-  const float2 v = __ffma2_rn(make_float2(x0, x1), f2(16777216.0f), f2(kMagic));
-  return __float_as_uint(v.x) + 256u * __float_as_uint(v.y);
+  return __float_as_uint(x0) + 256u * __float_as_uint(x1);
 }
 
 // A double's bits rounded from |X| = [x3 x2 x1 x0] 2^scale_exp for values the fast
@@ -465,12 +467,12 @@ __device__ __forceinline__ void crt_block(const SplitJob& sj, uint32_t local, co
   const JobDesc& d = sj.d;
   const int nm = sj.nmod;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3;
-  // one row of 128 columns or four rows of 32; a launch has fewer than 2^31 blocks
-  const bool wide = sj.crt_w == kCrtCols;
-  const uint32_t colblocks = wide ? (uint32_t)(d.n + kCrtCols - 1) / kCrtCols : (uint32_t)(d.n + 31) / 32;
+  // 128 / w rows of w columns, w = 128, 64 or 32; a launch has fewer than 2^31 blocks
+  const int w = sj.crt_w, lw = 31 - __clz(w);
+  const uint32_t colblocks = (uint32_t)(d.n + w - 1) >> lw;
   const uint32_t rowblock = local / colblocks;
-  const int i0 = (int)(wide ? rowblock : 4 * rowblock);
-  const int j0 = (int)(local - rowblock * colblocks) * (wide ? kCrtCols : 32);
+  const int i0 = (int)rowblock * (kCrtCols >> lw);
+  const int j0 = (int)(local - rowblock * colblocks) << lw;
   const int64_t ncols = (int64_t)sj.tiles_n * sj.bn;
   // this thread's fragments of the digits (zero for moduli >= nmod)
   uint32_t b[2][KS][2][2];
@@ -486,7 +488,7 @@ __device__ __forceinline__ void crt_block(const SplitJob& sj, uint32_t local, co
   // copy: thread tid takes 16-byte chunk tid % 8 of planes tid / 8, tid / 8 + 16, ...
   {
     const int64_t plane = sj.res_plane;
-    const int cc = tid & 7, crow = wide ? 0 : cc >> 1, ccol = (wide ? cc : cc & 1) * 16;
+    const int cc = tid & 7, crow = cc >> (lw - 4), ccol = (cc & ((w >> 4) - 1)) * 16;
     if (i0 + crow < d.m && (int64_t)j0 + ccol < ncols) {
       int q = tid >> 3;                                    // plane: modulus l, product r
       const unsigned char* src = ws + sj.off_res + (int64_t)q * plane + (int64_t)(i0 + crow) * ncols + j0 + ccol;
@@ -504,7 +506,7 @@ __device__ __forceinline__ void crt_block(const SplitJob& sj, uint32_t local, co
     }
     cp_async_commit();
   }
-  const int wi = i0 + (wide ? 0 : warp), j = j0 + (wide ? 32 * warp : 0) + lane;
+  const int wi = i0 + (32 * warp >> lw), j = j0 + (32 * warp & (w - 1)) + lane;
   const bool valid = wi < d.m && j < d.n;
   int sc = -c_m2shift[nm];
   if (valid)
@@ -519,6 +521,7 @@ __device__ __forceinline__ void crt_block(const SplitJob& sj, uint32_t local, co
     for (int e = 0; e < 8; ++e) asm volatile("prefetch.global.L1 [%0];" ::"l"(cbase + (int64_t)e * d.sC));
   const bool plain = __double_as_longlong(d.alpha_re) == 0x3FF0000000000000ll && zero(d.alpha_im) && !use_beta;
   const int rot = sj.rot;
+  const float start[4] = {kMagic, kMagic, kMagic, kMagic};
   asm volatile("cp.async.wait_all;\n" ::: "memory");
   __syncthreads();
 
@@ -595,7 +598,7 @@ __device__ __forceinline__ void crt_block(const SplitJob& sj, uint32_t local, co
         if (KIND == kMat2Complex && e > 0) continue;
 #pragma unroll
         for (int mt = 0; mt < 2; ++mt) {
-          float acc[2][4] = {};
+          float acc[2][4];
 #pragma unroll
           for (int ks = 0; ks < KS; ++ks) {
             uint32_t a[4];
@@ -612,7 +615,10 @@ __device__ __forceinline__ void crt_block(const SplitJob& sj, uint32_t local, co
               }
             }
 #pragma unroll
-            for (int nt = 0; nt < 2; ++nt) mma_f16(acc[nt], a, b[h][ks][nt]);
+            for (int nt = 0; nt < 2; ++nt) {
+              if (ks == 0) mma_f16(acc[nt], a, b[h][ks][nt], start);
+              else mma_f16(acc[nt], a, b[h][ks][nt], acc[nt]);
+            }
           }
 #pragma unroll
           for (int nt = 0; nt < 2; ++nt) {
