@@ -13,20 +13,28 @@
 //              complex alpha / beta update (Sec. III scaling and addition) and
 //              stores C.
 //
-// GB300 note: FP64 FMA throughput is 2 per clock per SM (1.2 TFLOP/s measured),
-// so a warp-wide DFMA occupies an SM sub-partition's FP64 pipe for 64 clocks;
-// the kernel is bound by that pipe alone.  What matters is the count of FP64
-// operations that are not product FMAs (pre-additions and recombination: 17%
-// of the FP64 instructions at 32x32 tiles, measured) and keeping the pipe fed:
-// 24 accumulators per output point cap the tile at 32x32 per SM
-// (24 x 1024 doubles = 192 KB of registers).
+// GB300 note: FP64 FMA throughput is 2 per clock per SM (1.06 to 1.2 TFLOP/s
+// measured), so a warp-wide DFMA occupies an SM sub-partition's FP64 pipe for 64
+// clocks; the kernel is bound by that pipe alone.  24 accumulators per output point
+// cap the tile at 32x32 per SM (24 x 1024 doubles = 192 KB of registers).  What is
+// left to gain is the count of FP64 instructions that are not product FMAs, and a
+// pipe that never waits:
+//  - signs (of op and of the +-1 sums) are flips of the sign bit on the integer pipe;
+//    a select between x + y and x - y costs both.  With the Hadamard sums as a
+//    butterfly a point of a side takes 24 FP64 additions (80 before): 6 % of the
+//    FP64 instructions at 32x32 tiles instead of 17 %;
+//  - the factors of the next k-block are formed while this one's products run, one
+//    barrier a block, the two warps of a sub-partition at different times.
+// n = 2048: 434 -> 370 ms; products alone at 2 per clock would take 352.
 #include <cuda_runtime.h>
 
 #include "common.cuh"
 
 namespace hmat {
 
-constexpr int F_BM = 32, F_BN = 32, F_BK = 8, F_THREADS = 256;
+constexpr int F_BM = 32, F_BN = 32, F_BK = 4, F_THREADS = 256;
+constexpr int F_KALIGN = 8;         // slices of a split inner dimension are multiples of this
+static_assert(F_BM == 32 && F_BN == 32 && F_THREADS == 2 * F_BK * 32, "one factor point of one side per thread");
 // products per pass: 24 accumulators per output point fill the register file;
 // plans with more products run as several passes (host side)
 constexpr int F_MAXP = 24;
@@ -34,8 +42,8 @@ constexpr int F_MAXP = 24;
 struct Fp64Smem {
   double araw[2][8][F_BK][F_BM];    // staged op(A) components (double buffer)
   double braw[2][8][F_BK][F_BN];    // staged op(B) components
-  double xs[kMaxFactors][F_BK][F_BM];   // left factors
-  double ys[kMaxFactors][F_BK][F_BN];   // right factors
+  double xs[2][kMaxFactors][F_BK][F_BM];   // left factors (double buffer)
+  double ys[2][kMaxFactors][F_BK][F_BN];   // right factors
   double wd[8][F_MAXP];                 // recombination weights w4 / 4 of the loaded plan
   KPlan plan;
   int plan_id;
@@ -50,93 +58,107 @@ __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commi
 template <int N>
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;\n" ::"n"(N)); }
 
-// Stage k-block kb of the present components of op(A) (BM x BK) and op(B) (BK x BN);
-// inner indices at or beyond kend read as zero.
+// Stage the k-block at k0 of the present components of op(A) (BM x BK, warps 0-3) and
+// op(B) (BK x BN, warps 4-7); inner indices at or beyond kend read as zero.
 __device__ __forceinline__ void stage_raw(Fp64Smem& s, int buf, const JobDesc& jb, int i0, int j0, int k0, int kend) {
-  const int t = threadIdx.x;
-  // op(A)[i, kk]: non-transposed reads run along k, transposed along i
-  int r, kk;
-  if (jb.transA) { r = t % F_BM; kk = t / F_BM; }
-  else { r = t / F_BK; kk = t % F_BK; }
-  {
-    const int i = i0 + r, kg = k0 + kk;
-    const bool valid = (i < jb.m) && (kg < kend);
-    const int64_t off = jb.transA ? (int64_t)kg * jb.lda + i : (int64_t)i * jb.lda + kg;
+  const bool left = threadIdx.x < F_THREADS / 2;
+  const int t = threadIdx.x & (F_THREADS / 2 - 1);
+  // reads run along the operand's stored rows: along k for op(A) and transposed op(B)
+  const bool along_k = left ? !jb.transA : jb.transB;
+  const int r = along_k ? t / F_BK : t % 32, kk = along_k ? t % F_BK : t / 32;
+  const int at = (left ? i0 : j0) + r, kg = k0 + kk;
+  const bool valid = at < (left ? jb.m : jb.n) && kg < kend;
+  const int64_t ld = left ? jb.lda : jb.ldb;
+  const int64_t off = !valid ? 0 : along_k ? (int64_t)at * ld + kg : (int64_t)kg * ld + at;
+  const double* src = (left ? jb.A : jb.B) + off;
+  const int64_t stride = left ? jb.sA : jb.sB;
+  const uint32_t present = left ? jb.fa : jb.fb;
+  double* dst = left ? &s.araw[buf][0][kk][r] : &s.braw[buf][0][kk][r];
 #pragma unroll
-    for (int c = 0; c < 8; ++c) {
-      if (!((jb.fa >> c) & 1u)) continue;
-      const double* src = jb.A + (int64_t)c * jb.sA + (valid ? off : 0);
-      cp_async8(&s.araw[buf][c][kk][r], src, valid);
-    }
-  }
-  // op(B)[kk, j]: non-transposed reads run along j, transposed along k
-  int cj;
-  if (jb.transB) { kk = t % F_BK; cj = t / F_BK; }
-  else { cj = t % F_BN; kk = t / F_BN; }
-  {
-    const int j = j0 + cj, kg = k0 + kk;
-    const bool valid = (j < jb.n) && (kg < kend);
-    const int64_t off = jb.transB ? (int64_t)j * jb.ldb + kg : (int64_t)kg * jb.ldb + j;
-#pragma unroll
-    for (int c = 0; c < 8; ++c) {
-      if (!((jb.fb >> c) & 1u)) continue;
-      const double* src = jb.B + (int64_t)c * jb.sB + (valid ? off : 0);
-      cp_async8(&s.braw[buf][c][kk][cj], src, valid);
-    }
+  for (int c = 0; c < 8; ++c) {
+    if (!((present >> c) & 1u)) continue;
+    cp_async8(dst + c * F_BK * 32, src + (int64_t)c * stride, valid);
   }
 }
 
-// Signed +-1 sum of the staged components selected by coef (with op signs):
-// returns false when no component contributes.
-__device__ __forceinline__ bool signed_sum(const int8_t* coef, const int8_t* sign, const double* v,
-                                           int base, double& out) {
+// x with its sign bit flipped when bit 31 of mask is set: sign changes on the integer
+// pipe, none of them an FP64 instruction
+__device__ __forceinline__ double flip(double x, uint32_t mask) {
+  return __hiloint2double(__double2hiint(x) ^ (int)(mask & 0x80000000u), __double2loint(x));
+}
+
+// The components of staged point (kk, r) with their op signs (bit c of neg), zeros
+// where a component is absent.
+__device__ __forceinline__ void load_point(const double (*raw)[F_BK][F_BM], int kk, int r, uint32_t present,
+                                           uint32_t neg, double v[8]) {
+#pragma unroll
+  for (int c = 0; c < 8; ++c) v[c] = ((present >> c) & 1u) ? flip(raw[c][kk][r], neg << (31 - c)) : 0.0;
+}
+
+// Signed +-1 sum of v[0..3] with the four coefficients of a group (0, 1 or -1), in order.
+__device__ __forceinline__ double signed_sum(const int8_t* coef, const double* v) {
+  const uint32_t w = *reinterpret_cast<const uint32_t*>(coef);
   bool any = false;
   double acc = 0.0;
 #pragma unroll
   for (int e = 0; e < 4; ++e) {
-    const int cf = coef[e] * sign[base + e];
-    if (cf == 0) continue;
-    const double x = v[base + e];
-    if (!any) { acc = cf > 0 ? x : -x; any = true; }
-    else acc = cf > 0 ? acc + x : acc - x;
+    if (!(w >> (8 * e) & 0xFFu)) continue;
+    const double x = flip(v[e], w << (24 - 8 * e));
+    acc = any ? acc + x : x;
+    any = true;
   }
-  out = acc;
-  return any;
+  return acc;
 }
 
-// Prologue: left and right factors of k-block buf into xs / ys.
-__device__ __forceinline__ void form_factors(Fp64Smem& s, int buf, const JobDesc& jb) {
-  const KPlan& p = s.plan;
-  const int t = threadIdx.x;
-  {
-    const int kk = t / F_BM, r = t % F_BM;
-    double v[8];
+// One side's factors of staged point v into f[slot][kk][r].  The eight groups of the
+// full plan are the four components and their Hadamard sums, formed as a butterfly
+// (8 additions for the four sums instead of 12); other plans sum term by term.
+__device__ __forceinline__ void form_point(const double v[8], double (*f)[F_BK][F_BM], int kk, int r, int ngroups,
+                                           bool hadamard, const int8_t (*cre)[4], const int8_t (*cim)[4],
+                                           const int8_t (*slot)[3]) {
+  auto emit = [&](int g, double re, double im) {
+    const int sr = slot[g][0], si = slot[g][1], ss = slot[g][2];
+    if (sr >= 0) f[sr][kk][r] = re;
+    if (si >= 0) f[si][kk][r] = im;
+    if (ss >= 0) f[ss][kk][r] = re + im;
+  };
+  if (hadamard) {
 #pragma unroll
-    for (int c = 0; c < 8; ++c) v[c] = ((jb.fa >> c) & 1u) ? s.araw[buf][c][kk][r] : 0.0;
-    for (int g = 0; g < p.nlg; ++g) {
-      const int sr = p.lslot[g][0], si = p.lslot[g][1], ss = p.lslot[g][2];
-      double re = 0.0, im = 0.0;
-      if (sr >= 0 || ss >= 0) signed_sum(p.lre[g], jb.signA, v, 0, re);
-      if (si >= 0 || ss >= 0) signed_sum(p.lim[g], jb.signA, v, 4, im);
-      if (sr >= 0) s.xs[sr][kk][r] = re;
-      if (si >= 0) s.xs[si][kk][r] = im;
-      if (ss >= 0) s.xs[ss][kk][r] = re + im;
+    for (int g = 0; g < 4; ++g) {
+      int e = 0;                        // the group's component
+#pragma unroll
+      for (int i = 1; i < 4; ++i) e = cre[g][i] ? i : e;
+      const double re = e == 0 ? v[0] : e == 1 ? v[1] : e == 2 ? v[2] : v[3];
+      const double im = e == 0 ? v[4] : e == 1 ? v[5] : e == 2 ? v[6] : v[7];
+      emit(g, re, im);
     }
+    const double p01 = v[0] + v[1], m01 = v[0] - v[1], p23 = v[2] + v[3], m23 = v[2] - v[3];
+    const double q01 = v[4] + v[5], n01 = v[4] - v[5], q23 = v[6] + v[7], n23 = v[6] - v[7];
+    emit(4, p01 + p23, q01 + q23);
+    emit(5, p01 - p23, q01 - q23);
+    emit(6, m01 + m23, n01 + n23);
+    emit(7, m01 - m23, n01 - n23);
+    return;
   }
-  {
-    const int kk = t / F_BN, cj = t % F_BN;
-    double v[8];
-#pragma unroll
-    for (int c = 0; c < 8; ++c) v[c] = ((jb.fb >> c) & 1u) ? s.braw[buf][c][kk][cj] : 0.0;
-    for (int g = 0; g < p.nrg; ++g) {
-      const int sr = p.rslot[g][0], si = p.rslot[g][1], ss = p.rslot[g][2];
-      double re = 0.0, im = 0.0;
-      if (sr >= 0 || ss >= 0) signed_sum(p.rre[g], jb.signB, v, 0, re);
-      if (si >= 0 || ss >= 0) signed_sum(p.rim[g], jb.signB, v, 4, im);
-      if (sr >= 0) s.ys[sr][kk][cj] = re;
-      if (si >= 0) s.ys[si][kk][cj] = im;
-      if (ss >= 0) s.ys[ss][kk][cj] = re + im;
-    }
+  for (int g = 0; g < ngroups; ++g) {
+    const double re = signed_sum(cre[g], v), im = signed_sum(cim[g], v + 4);
+    emit(g, re, im);
+  }
+}
+
+// Prologue: the left factors of the k-block staged in raw (warps 0-3, one point a
+// thread) or its right factors (warps 4-7) into factor buffer fbuf.
+__device__ __forceinline__ void form_factors(Fp64Smem& s, int rbuf, int fbuf, const JobDesc& jb, uint32_t negA,
+                                             uint32_t negB) {
+  const KPlan& p = s.plan;
+  const int kk = (threadIdx.x >> 5) & (F_BK - 1), r = threadIdx.x & 31;
+  double v[8];
+  if (threadIdx.x < F_THREADS / 2) {
+    load_point(s.araw[rbuf], kk, r, jb.fa, negA, v);
+    form_point(v, s.xs[fbuf], kk, r, p.nlg, p.bilinear_left != 0, p.lre, p.lim, p.lslot);
+  } else {
+    load_point(s.braw[rbuf], kk, r, jb.fb, negB, v);
+    form_point(v, s.ys[fbuf], kk, r, p.nrg, p.bilinear_right != 0, p.rre, p.rim, p.rslot);
   }
 }
 
@@ -174,23 +196,41 @@ fp64_bilinear_kernel(const JobDesc* __restrict__ jobs, int njobs, const KPlan* _
 #pragma unroll
     for (int q = 0; q < F_MAXP; ++q) acc[q][0] = acc[q][1] = acc[q][2] = acc[q][3] = 0.0;
 
+    // One barrier per k-block.  While the products of block kb run, block kb + 1's
+    // factors are formed from its staged components and block kb + 2's components are
+    // copied; the left side's warps form before their products and the right side's
+    // after, so that one of a sub-partition's two warps feeds the FP64 pipe throughout.
+    uint32_t negA = 0, negB = 0;
+#pragma unroll
+    for (int c = 0; c < 8; ++c) {
+      negA |= jb.signA[c] < 0 ? 1u << c : 0u;
+      negB |= jb.signB[c] < 0 ? 1u << c : 0u;
+    }
     const int nkb = (kend - kbeg + F_BK - 1) / F_BK;
-    if (nkb > 0) stage_raw(s, 0, jb, i0, j0, kbeg, kend);
-    cp_async_commit();
-    for (int kb = 0; kb < nkb; ++kb) {
-      if (kb + 1 < nkb) stage_raw(s, (kb + 1) & 1, jb, i0, j0, kbeg + (kb + 1) * F_BK, kend);
+    if (nkb > 0) {
+      stage_raw(s, 0, jb, i0, j0, kbeg, kend);
+      cp_async_commit();
+      if (nkb > 1) stage_raw(s, 1, jb, i0, j0, kbeg + F_BK, kend);
       cp_async_commit();
       cp_async_wait<1>();
-      __syncthreads();                // staged block kb visible; previous compute finished
-      form_factors(s, kb & 1, jb);
-      __syncthreads();                // factors visible
+      __syncthreads();                // block 0 staged; the previous tile's products finished
+      form_factors(s, 0, 0, jb, negA, negB);
+    }
+    for (int kb = 0; kb < nkb; ++kb) {
+      cp_async_wait<0>();
+      __syncthreads();                // block kb's factors and block kb + 1's components visible
+      if (kb + 2 < nkb) stage_raw(s, kb & 1, jb, i0, j0, kbeg + (kb + 2) * F_BK, kend);
+      cp_async_commit();
+      const int cur = kb & 1;
+      const bool more = kb + 1 < nkb;
+      if (more && t < F_THREADS / 2) form_factors(s, cur ^ 1, cur ^ 1, jb, negA, negB);
 #pragma unroll 2
       for (int kk = 0; kk < F_BK; ++kk) {
 #pragma unroll
         for (int q = 0; q < F_MAXP; ++q) {
           if (q < np) {
-            const double2 x = *reinterpret_cast<const double2*>(&s.xs[s.plan.pl[q]][kk][2 * ty]);
-            const double2 y = *reinterpret_cast<const double2*>(&s.ys[s.plan.pr[q]][kk][2 * tx]);
+            const double2 x = *reinterpret_cast<const double2*>(&s.xs[cur][s.plan.pl[q]][kk][2 * ty]);
+            const double2 y = *reinterpret_cast<const double2*>(&s.ys[cur][s.plan.pr[q]][kk][2 * tx]);
             acc[q][0] = fma(x.x, y.x, acc[q][0]);
             acc[q][1] = fma(x.x, y.y, acc[q][1]);
             acc[q][2] = fma(x.y, y.x, acc[q][2]);
@@ -198,6 +238,7 @@ fp64_bilinear_kernel(const JobDesc* __restrict__ jobs, int njobs, const KPlan* _
           }
         }
       }
+      if (more && t >= F_THREADS / 2) form_factors(s, cur ^ 1, cur ^ 1, jb, negA, negB);
     }
     cp_async_wait<0>();
 
@@ -321,6 +362,6 @@ cudaError_t launch_fp64_bilinear(const JobDesc* d_jobs, int njobs, const KPlan* 
 int fp64_tile_m() { return F_BM; }
 int fp64_max_products() { return F_MAXP; }
 int fp64_tile_n() { return F_BN; }
-int fp64_tile_k() { return F_BK; }
+int fp64_tile_k() { return F_KALIGN; }
 
 }  // namespace hmat
