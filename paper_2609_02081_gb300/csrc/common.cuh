@@ -42,6 +42,18 @@ struct JobDesc {
   // reduction adds the slices in order, then applies alpha / beta
   int32_t kslices, kchunk;
   double* part;
+  // FP64 ranges (Fp64Ranges): tile_begin counts k-blocks, per_tile of them a tile
+  // (its own and padding), and tile0 is the job's first tile
+  int64_t tile0;
+  int32_t per_tile;
+};
+
+// FP64 calls whose tiles leave SMs idle, cut into equal ranges of k-blocks, one per CTA
+// (fp64_layout): width k-blocks each (0: not cut), ctas ranges over tiles output tiles;
+// part holds ctas + tiles partial tiles.
+struct Fp64Ranges {
+  int64_t width = 0, ctas = 0, tiles = 0;
+  double* part = nullptr;
 };
 
 // Complex-isomorph route (isomorph.cu): image of op(X) as two planes (real,

@@ -24,8 +24,11 @@
 //    butterfly a point of a side takes 24 FP64 additions (80 before): 6 % of the
 //    FP64 instructions at 32x32 tiles instead of 17 %;
 //  - the factors of the next k-block are formed while this one's products run, one
-//    barrier a block, the two warps of a sub-partition at different times.
-// n = 2048: 434 -> 370 ms; products alone at 2 per clock would take 352.
+//    barrier a block, the two warps of a sub-partition at different times;
+//  - components are copied four k-blocks ahead: plans of few products spend less time
+//    on a block than one copy takes (1 product, n = 1024: 5.99 ms with two blocks
+//    ahead, 3.06 with four).
+// n = 2048: 434 -> 367 ms; products alone at 2 per clock would take 352.
 #include <cuda_runtime.h>
 
 #include "common.cuh"
@@ -33,6 +36,7 @@
 namespace hmat {
 
 constexpr int F_BM = 32, F_BN = 32, F_BK = 4, F_THREADS = 256;
+constexpr int F_RING = 4;           // k-blocks of staged components: the copies run this far ahead
 constexpr int F_KALIGN = 8;         // slices of a split inner dimension are multiples of this
 static_assert(F_BM == 32 && F_BN == 32 && F_THREADS == 2 * F_BK * 32, "one factor point of one side per thread");
 // products per pass: 24 accumulators per output point fill the register file;
@@ -40,8 +44,8 @@ static_assert(F_BM == 32 && F_BN == 32 && F_THREADS == 2 * F_BK * 32, "one facto
 constexpr int F_MAXP = 24;
 
 struct Fp64Smem {
-  double araw[2][8][F_BK][F_BM];    // staged op(A) components (double buffer)
-  double braw[2][8][F_BK][F_BN];    // staged op(B) components
+  double araw[F_RING][8][F_BK][F_BM];   // staged op(A) components
+  double braw[F_RING][8][F_BK][F_BN];   // staged op(B) components
   double xs[2][kMaxFactors][F_BK][F_BM];   // left factors (double buffer)
   double ys[2][kMaxFactors][F_BK][F_BN];   // right factors
   double wd[8][F_MAXP];                 // recombination weights w4 / 4 of the loaded plan
@@ -162,9 +166,59 @@ __device__ __forceinline__ void form_factors(Fp64Smem& s, int rbuf, int fbuf, co
   }
 }
 
+// Recombination of point pt's 24 products of the paper's full plan (T1, T2, T3 of
+// P1, ..., P8): Gauss's differences, then the sums of P5..P8 as a butterfly; 56 FP64
+// instructions where the weights' table takes 100.
+__device__ __forceinline__ void recombine_full(const double acc[F_MAXP][4], int pt, double q[8]) {
+#pragma unroll
+  for (int part = 0; part < 2; ++part) {
+    double P[8];
+#pragma unroll
+    for (int r = 0; r < 8; ++r) {
+      const double t1 = acc[3 * r][pt], t2 = acc[3 * r + 1][pt];
+      P[r] = part ? acc[3 * r + 2][pt] - t1 - t2 : t1 - t2;
+    }
+    const double s56 = P[4] + P[5], d56 = P[4] - P[5], s78 = P[6] + P[7], d78 = P[6] - P[7];
+    q[4 * part] = fma(-0.25, s56 + s78, 2.0 * P[0]);
+    q[4 * part + 1] = fma(0.25, s56 - s78, -2.0 * P[1]);
+    q[4 * part + 2] = fma(0.25, d56 + d78, -2.0 * P[2]);
+    q[4 * part + 3] = fma(0.25, d56 - d78, -2.0 * P[3]);
+  }
+}
+
+// C[i][jj] <- alpha q + beta C[i][jj]
+__device__ __forceinline__ void store_point(const JobDesc& jb, int i, int jj, const double q[8]) {
+  double* cbase = jb.C + (int64_t)i * jb.ldc + jj;
+  if (jb.alpha_re == 1.0 && jb.alpha_im == 0.0 && jb.beta_re == 0.0 && jb.beta_im == 0.0) {
+#pragma unroll
+    for (int e = 0; e < 8; ++e) cbase[(int64_t)e * jb.sC] = q[e];
+    return;
+  }
+  const bool use_beta = (jb.beta_re != 0.0 || jb.beta_im != 0.0);
+#pragma unroll
+  for (int e = 0; e < 4; ++e) {
+    double re = jb.alpha_re * q[e] - jb.alpha_im * q[e + 4];
+    double im = jb.alpha_re * q[e + 4] + jb.alpha_im * q[e];
+    if (use_beta) {
+      const double cre = cbase[(int64_t)e * jb.sC];
+      const double cim = cbase[(int64_t)(e + 4) * jb.sC];
+      re += jb.beta_re * cre - jb.beta_im * cim;
+      im += jb.beta_re * cim + jb.beta_im * cre;
+    }
+    cbase[(int64_t)e * jb.sC] = re;
+    cbase[(int64_t)(e + 4) * jb.sC] = im;
+  }
+}
+
+// kRanges: the call's tiles, laid end to end in k-blocks (each job's tiles
+// ranges.per_tile of them apart), are cut into one range of ranges.width k-blocks per
+// CTA, whatever tiles it crosses.  Each piece of a tile goes to slot (CTA + tile) of
+// the partial outputs: along the ranges either number increases, so no two pieces
+// share one.
+template <bool kRanges>
 __global__ void __launch_bounds__(F_THREADS, 1)
 fp64_bilinear_kernel(const JobDesc* __restrict__ jobs, int njobs, const KPlan* __restrict__ plans,
-                     int64_t total_tiles) {
+                     int64_t total_tiles, Fp64Ranges ranges) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   Fp64Smem& s = *reinterpret_cast<Fp64Smem*>(smem_raw);
   const int t = threadIdx.x;
@@ -172,16 +226,36 @@ fp64_bilinear_kernel(const JobDesc* __restrict__ jobs, int njobs, const KPlan* _
   if (t == 0) s.plan_id = -1;
   __syncthreads();
 
-  for (int64_t tile = blockIdx.x; tile < total_tiles; tile += gridDim.x) {
-    const int j = find_job(jobs, njobs, tile);
-    const JobDesc& jb = jobs[j];
-    const int64_t ntile = (int64_t)jb.tiles_m * jb.tiles_n;
-    const int64_t local = (tile - jb.tile_begin) % ntile;
-    const int slice = (int)((tile - jb.tile_begin) / ntile);   // 0 unless the inner dimension is split
+  // pos: an output tile (or tile-slice) of the call, or a k-block of this CTA's range
+  const int64_t end = kRanges ? min(total_tiles, (int64_t)(blockIdx.x + 1) * ranges.width) : total_tiles;
+  int64_t pos = kRanges ? (int64_t)blockIdx.x * ranges.width : blockIdx.x;
+  while (pos < end) {
+    const JobDesc& jb = jobs[find_job(jobs, njobs, pos)];
+    int64_t local;
+    int kbeg, kend;
+    double* part = nullptr;             // this piece's partial result, or null: C itself
+    if constexpr (kRanges) {
+      const int64_t within = pos - jb.tile_begin;
+      local = within / jb.per_tile;
+      const int64_t tile_end = jb.tile_begin + (local + 1) * jb.per_tile;
+      const int kb = (int)(within - local * jb.per_tile);
+      const int blocks = (int)(min(end, tile_end) - pos);
+      kbeg = kb * F_BK;
+      kend = min(jb.k, kbeg + blocks * F_BK);
+      pos = min(end, tile_end);
+      if (kbeg >= jb.k) continue;       // the padding behind the tile's last k-block
+      part = ranges.part + (blockIdx.x + jb.tile0 + local) * (8 * F_BM * F_BN);
+    } else {
+      const int64_t ntile = (int64_t)jb.tiles_m * jb.tiles_n;
+      local = (pos - jb.tile_begin) % ntile;
+      const int64_t slice = (pos - jb.tile_begin) / ntile;   // 0 unless the inner dimension is split
+      kbeg = (int)slice * jb.kchunk;
+      kend = min(jb.k, kbeg + jb.kchunk);
+      pos += gridDim.x;
+      if (jb.kslices > 1) part = jb.part + (slice * ntile + local) * (8 * F_BM * F_BN);
+    }
     const int i0 = (int)(local / jb.tiles_n) * F_BM;
     const int j0 = (int)(local % jb.tiles_n) * F_BN;
-    const int kbeg = slice * jb.kchunk;
-    const int kend = min(jb.k, kbeg + jb.kchunk);
     if (s.plan_id != jb.plan) {
       __syncthreads();
       if (t == 0) { s.plan = plans[jb.plan]; s.plan_id = jb.plan; }
@@ -197,8 +271,8 @@ fp64_bilinear_kernel(const JobDesc* __restrict__ jobs, int njobs, const KPlan* _
     for (int q = 0; q < F_MAXP; ++q) acc[q][0] = acc[q][1] = acc[q][2] = acc[q][3] = 0.0;
 
     // One barrier per k-block.  While the products of block kb run, block kb + 1's
-    // factors are formed from its staged components and block kb + 2's components are
-    // copied; the left side's warps form before their products and the right side's
+    // factors are formed from its staged components and block kb + F_RING's components
+    // are copied; the left side's warps form before their products and the right side's
     // after, so that one of a sub-partition's two warps feeds the FP64 pipe throughout.
     uint32_t negA = 0, negB = 0;
 #pragma unroll
@@ -208,27 +282,30 @@ fp64_bilinear_kernel(const JobDesc* __restrict__ jobs, int njobs, const KPlan* _
     }
     const int nkb = (kend - kbeg + F_BK - 1) / F_BK;
     if (nkb > 0) {
-      stage_raw(s, 0, jb, i0, j0, kbeg, kend);
-      cp_async_commit();
-      if (nkb > 1) stage_raw(s, 1, jb, i0, j0, kbeg + F_BK, kend);
-      cp_async_commit();
-      cp_async_wait<1>();
+#pragma unroll
+      for (int i = 0; i < F_RING; ++i) {
+        if (i < nkb) stage_raw(s, i, jb, i0, j0, kbeg + i * F_BK, kend);
+        cp_async_commit();
+      }
+      cp_async_wait<F_RING - 1>();
       __syncthreads();                // block 0 staged; the previous tile's products finished
       form_factors(s, 0, 0, jb, negA, negB);
     }
     for (int kb = 0; kb < nkb; ++kb) {
-      cp_async_wait<0>();
+      cp_async_wait<F_RING - 2>();
       __syncthreads();                // block kb's factors and block kb + 1's components visible
-      if (kb + 2 < nkb) stage_raw(s, kb & 1, jb, i0, j0, kbeg + (kb + 2) * F_BK, kend);
+      const int cur = kb & 1, ahead = kb + F_RING;
+      // into the buffer whose factors are formed
+      if (ahead < nkb) stage_raw(s, ahead % F_RING, jb, i0, j0, kbeg + ahead * F_BK, kend);
       cp_async_commit();
-      const int cur = kb & 1;
       const bool more = kb + 1 < nkb;
-      if (more && t < F_THREADS / 2) form_factors(s, cur ^ 1, cur ^ 1, jb, negA, negB);
+      if (more && t < F_THREADS / 2) form_factors(s, (kb + 1) % F_RING, cur ^ 1, jb, negA, negB);
 #pragma unroll 2
       for (int kk = 0; kk < F_BK; ++kk) {
 #pragma unroll
         for (int q = 0; q < F_MAXP; ++q) {
-          if (q < np) {
+          if (q >= np) break;
+          {
             const double2 x = *reinterpret_cast<const double2*>(&s.xs[cur][s.plan.pl[q]][kk][2 * ty]);
             const double2 y = *reinterpret_cast<const double2*>(&s.ys[cur][s.plan.pr[q]][kk][2 * tx]);
             acc[q][0] = fma(x.x, y.x, acc[q][0]);
@@ -238,56 +315,36 @@ fp64_bilinear_kernel(const JobDesc* __restrict__ jobs, int njobs, const KPlan* _
           }
         }
       }
-      if (more && t >= F_THREADS / 2) form_factors(s, cur ^ 1, cur ^ 1, jb, negA, negB);
+      if (more && t >= F_THREADS / 2) form_factors(s, (kb + 1) % F_RING, cur ^ 1, jb, negA, negB);
     }
     cp_async_wait<0>();
 
     // Epilogue: recombination (weights w4/4, exact), then alpha / beta.
-    const bool plain = (jb.alpha_re == 1.0 && jb.alpha_im == 0.0 && jb.beta_re == 0.0 && jb.beta_im == 0.0);
-    const bool use_beta = (jb.beta_re != 0.0 || jb.beta_im != 0.0);
 #pragma unroll
     for (int pt = 0; pt < 4; ++pt) {
-      const int i = i0 + 2 * ty + (pt >> 1);
-      const int jj = j0 + 2 * tx + (pt & 1);
+      const int ti = 2 * ty + (pt >> 1), tj = 2 * tx + (pt & 1);
       double q[8];
+      if (s.plan.bilinear_full) {
+        recombine_full(acc, pt, q);
+      } else {
 #pragma unroll
-      for (int e = 0; e < 8; ++e) {
-        double o = 0.0;
+        for (int e = 0; e < 8; ++e) {
+          double o = 0.0;
 #pragma unroll
-        for (int pp = 0; pp < F_MAXP; ++pp) {
-          if (pp < np) {
-            if (s.plan.w4[e][pp] != 0) o = fma(acc[pp][pt], s.wd[e][pp], o);
+          for (int pp = 0; pp < F_MAXP; ++pp) {
+            if (pp < np) {
+              if (s.plan.w4[e][pp] != 0) o = fma(acc[pp][pt], s.wd[e][pp], o);
+            }
           }
+          q[e] = o;
         }
-        q[e] = o;
       }
-      if (jb.kslices > 1) {            // partial result of this slice, reduced later
-        double* dst = jb.part + ((int64_t)slice * ntile + local) * 8 * (F_BM * F_BN) +
-                      (2 * ty + (pt >> 1)) * F_BN + 2 * tx + (pt & 1);
+      if (part) {                      // reduced later
+        double* dst = part + ti * F_BN + tj;
 #pragma unroll
         for (int e = 0; e < 8; ++e) dst[(int64_t)e * (F_BM * F_BN)] = q[e];
-        continue;
-      }
-      if (i < jb.m && jj < jb.n) {
-        double* cbase = jb.C + (int64_t)i * jb.ldc + jj;
-        if (plain) {
-#pragma unroll
-          for (int e = 0; e < 8; ++e) cbase[(int64_t)e * jb.sC] = q[e];
-        } else {
-#pragma unroll
-          for (int e = 0; e < 4; ++e) {
-            double re = jb.alpha_re * q[e] - jb.alpha_im * q[e + 4];
-            double im = jb.alpha_re * q[e + 4] + jb.alpha_im * q[e];
-            if (use_beta) {
-              const double cre = cbase[(int64_t)e * jb.sC];
-              const double cim = cbase[(int64_t)(e + 4) * jb.sC];
-              re += jb.beta_re * cre - jb.beta_im * cim;
-              im += jb.beta_re * cim + jb.beta_im * cre;
-            }
-            cbase[(int64_t)e * jb.sC] = re;
-            cbase[(int64_t)(e + 4) * jb.sC] = im;
-          }
-        }
+      } else if (i0 + ti < jb.m && j0 + tj < jb.n) {
+        store_point(jb, i0 + ti, j0 + tj, q);
       }
     }
   }
@@ -310,27 +367,43 @@ __global__ void __launch_bounds__(256) fp64_splitk_reduce_kernel(JobDesc jb) {
 #pragma unroll
     for (int e = 0; e < 8; ++e) q[e] += src[(int64_t)e * (F_BM * F_BN)];
   }
-  double* cbase = jb.C + (int64_t)i * jb.ldc + jj;
-  const bool plain = (jb.alpha_re == 1.0 && jb.alpha_im == 0.0 && jb.beta_re == 0.0 && jb.beta_im == 0.0);
-  if (plain) {
-#pragma unroll
-    for (int e = 0; e < 8; ++e) cbase[(int64_t)e * jb.sC] = q[e];
-    return;
+  store_point(jb, i, jj, q);
+}
+
+// Reduction behind the ranges: C <- alpha (sum of the tile's pieces, in k order) +
+// beta C, four blocks a tile, one thread per output element.
+__global__ void __launch_bounds__(256)
+fp64_ranges_reduce_kernel(const JobDesc* __restrict__ jobs, int njobs, Fp64Ranges ranges) {
+  const int64_t tile = blockIdx.x >> 2;
+  int lo = 0, hi = njobs - 1;
+  while (lo < hi) {
+    const int mid = (lo + hi + 1) >> 1;
+    if (jobs[mid].tile0 <= tile) lo = mid;
+    else hi = mid - 1;
   }
-  const bool use_beta = (jb.beta_re != 0.0 || jb.beta_im != 0.0);
+  const JobDesc& jb = jobs[lo];
+  const int64_t local = tile - jb.tile0;
+  const int within = (int)(blockIdx.x & 3) * 256 + threadIdx.x;
+  const int i = (int)(local / jb.tiles_n) * F_BM + within / F_BN;
+  const int jj = (int)(local % jb.tiles_n) * F_BN + within % F_BN;
+  if (i >= jb.m || jj >= jb.n) return;
+  double q[8];
 #pragma unroll
-  for (int e = 0; e < 4; ++e) {
-    double re = jb.alpha_re * q[e] - jb.alpha_im * q[e + 4];
-    double im = jb.alpha_re * q[e + 4] + jb.alpha_im * q[e];
-    if (use_beta) {
-      const double cre = cbase[(int64_t)e * jb.sC];
-      const double cim = cbase[(int64_t)(e + 4) * jb.sC];
-      re += jb.beta_re * cre - jb.beta_im * cim;
-      im += jb.beta_re * cim + jb.beta_im * cre;
-    }
-    cbase[(int64_t)e * jb.sC] = re;
-    cbase[(int64_t)(e + 4) * jb.sC] = im;
+  for (int e = 0; e < 8; ++e) q[e] = 0.0;
+  const int64_t begin = jb.tile_begin + local * jb.per_tile;
+  const int64_t last = begin + (jb.k + F_BK - 1) / F_BK - 1;   // before begin: k = 0, no pieces
+  for (int64_t c = begin / ranges.width; c * ranges.width <= last; ++c) {
+    const double* src = ranges.part + (c + tile) * (8 * F_BM * F_BN) + within;
+#pragma unroll
+    for (int e = 0; e < 8; ++e) q[e] += src[(int64_t)e * (F_BM * F_BN)];
   }
+  store_point(jb, i, jj, q);
+}
+
+cudaError_t launch_fp64_ranges_reduce(const JobDesc* d_jobs, int njobs, const Fp64Ranges& ranges,
+                                      cudaStream_t stream) {
+  fp64_ranges_reduce_kernel<<<(unsigned)(4 * ranges.tiles), 256, 0, stream>>>(d_jobs, njobs, ranges);
+  return cudaGetLastError();
 }
 
 cudaError_t launch_fp64_splitk_reduce(const JobDesc& jb, cudaStream_t stream) {
@@ -349,16 +422,29 @@ int64_t fp64_splitk_bytes(int64_t m, int64_t n, int kslices) {
 size_t fp64_smem_bytes() { return sizeof(Fp64Smem); }
 
 cudaError_t fp64_configure() {
-  return cudaFuncSetAttribute(fp64_bilinear_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  const cudaError_t e = cudaFuncSetAttribute(fp64_bilinear_kernel<false>,
+                                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(Fp64Smem));
+  if (e != cudaSuccess) return e;
+  return cudaFuncSetAttribute(fp64_bilinear_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                               (int)sizeof(Fp64Smem));
 }
 
 cudaError_t launch_fp64_bilinear(const JobDesc* d_jobs, int njobs, const KPlan* d_plans, int64_t total_tiles,
-                                 int grid, cudaStream_t stream) {
-  fp64_bilinear_kernel<<<grid, F_THREADS, sizeof(Fp64Smem), stream>>>(d_jobs, njobs, d_plans, total_tiles);
+                                 int grid, const Fp64Ranges& ranges, cudaStream_t stream) {
+  if (ranges.width > 0)
+    fp64_bilinear_kernel<true>
+        <<<grid, F_THREADS, sizeof(Fp64Smem), stream>>>(d_jobs, njobs, d_plans, total_tiles, ranges);
+  else
+    fp64_bilinear_kernel<false>
+        <<<grid, F_THREADS, sizeof(Fp64Smem), stream>>>(d_jobs, njobs, d_plans, total_tiles, ranges);
   return cudaGetLastError();
 }
 
+int64_t fp64_ranges_bytes(const Fp64Ranges& r) {
+  return (r.ctas + r.tiles) * (int64_t)(8 * F_BM * F_BN * sizeof(double));
+}
+
+int fp64_block_k() { return F_BK; }
 int fp64_tile_m() { return F_BM; }
 int fp64_max_products() { return F_MAXP; }
 int fp64_tile_n() { return F_BN; }

@@ -77,7 +77,11 @@ size_t fp64_smem_bytes();
 cudaError_t fp64_configure();
 cudaError_t launch_wait_selftest(long long limit_cycles, cudaStream_t s);
 cudaError_t launch_fp64_bilinear(const JobDesc* d_jobs, int njobs, const KPlan* d_plans, int64_t total_tiles,
-                                 int grid, cudaStream_t stream);
+                                 int grid, const Fp64Ranges& ranges, cudaStream_t stream);
+int fp64_block_k();
+int64_t fp64_ranges_bytes(const Fp64Ranges& r);
+cudaError_t launch_fp64_ranges_reduce(const JobDesc* d_jobs, int njobs, const Fp64Ranges& ranges,
+                                      cudaStream_t stream);
 int fp64_tile_m();
 int fp64_tile_n();
 int fp64_tile_k();
@@ -323,6 +327,7 @@ struct IsoJob {
 struct Prepared {
   std::vector<std::vector<JobDesc>> f;
   std::vector<int64_t> f_tiles;
+  Fp64Ranges ranges;                   // of f[0]
   SplitPrep sp;
   bool has_split = false;
   int64_t split_offset = 0;            // split workspace starts here (after isomorph buffers)
@@ -369,10 +374,71 @@ int fp64_kslices(const hmat_context* h, int64_t tiles, int64_t k) {
   return s;
 }
 
+// One FP64 product as the ranges' rule sees it: output tiles, inner dimension and
+// products of its plan.
+struct Fp64Shape {
+  int64_t tiles, k;
+  int np;
+};
+
+// Equal ranges of the call's k-blocks, one per CTA, for calls that the built-in rule
+// of fp64_kslices splits (no tuned entry, twice the tiles fit the SMs, k of 128 or
+// more).  Two ways to cut: pieces of `width` k-blocks that never cross a tile (a tile's
+// last piece may be short), or every SM the same number of k-blocks, whose piece of a
+// second tile costs another epilogue.  In us, a k-block of np products takes about
+// 4 + np, an epilogue and the pipeline's fill 12 + np / 2; pieces below two k-blocks of
+// the full plan are not worth their partial result.  n = 256, 64 tiles of 64
+// k-blocks: 2 slices each on 128 SMs 32 + 1, equal ranges on 152 SMs 27 + 2:
+// 935 -> 788 us; 64 x 64 x 1024, 4 tiles: 936 -> 259 us (the rule stops at 8 slices).
+Fp64Ranges fp64_ranges(const hmat_context* h, const std::vector<Fp64Shape>& shapes, std::vector<int32_t>* per_tile) {
+  Fp64Ranges r;
+  int64_t units = 0, kmax = 0, shortest = INT64_MAX;
+  int np = 1;
+  for (const Fp64Shape& p : shapes) {
+    const int64_t nkb = (p.k + fp64_block_k() - 1) / fp64_block_k();
+    r.tiles += p.tiles;
+    units += p.tiles * nkb;
+    kmax = std::max(kmax, p.k);
+    if (nkb > 0) shortest = std::min(shortest, nkb);
+    np = std::max(np, p.np);
+  }
+  const int64_t sms = h->sm_count;
+  if (2 * r.tiles > sms || kmax < 128) return Fp64Ranges{};
+  for (const Fp64Shape& p : shapes)
+    if (h->has_fp64_splitk && h->fp64_splitk[ceil_log2_bin(r.tiles) * kTileBins + ceil_log2_bin(p.k)] != 0)
+      return Fp64Ranges{};
+  const int64_t least = (56 + 4 + np - 1) / (4 + np);
+  const double epilogue = (12 + 0.5 * np) / (4 + np);
+  auto pieces = [&](int64_t w) {
+    int64_t n = 0;
+    for (const Fp64Shape& p : shapes) {
+      const int64_t nkb = (p.k + fp64_block_k() - 1) / fp64_block_k();
+      n += p.tiles * ((nkb + w - 1) / w);
+    }
+    return n;
+  };
+  int64_t whole = std::max(least, (units + sms - 1) / sms);      // width of pieces within a tile
+  while (pieces(whole) > sms) ++whole;
+  const int64_t even = std::max(least, (units + sms - 1) / sms);
+  const bool cross = even + epilogue * (double)(even / shortest + 2) < whole + epilogue;
+  r.width = cross ? even : whole;
+  per_tile->clear();
+  int64_t total = 0;
+  for (const Fp64Shape& p : shapes) {
+    const int64_t nkb = (p.k + fp64_block_k() - 1) / fp64_block_k();
+    per_tile->push_back((int32_t)(cross ? nkb : (nkb + r.width - 1) / r.width * r.width));
+    total += p.tiles * per_tile->back();
+  }
+  r.ctas = (total + r.width - 1) / r.width;
+  if (r.ctas <= r.tiles) return Fp64Ranges{};                     // nothing would be cut
+  return r;
+}
+
 // FP64 tile counts of the prepared launch groups; with `allow_splitk`, a
 // single-pass call whose tiles leave SMs idle splits the inner dimension of
 // its products (fp64_kslices) when the workspace holds the partial outputs
-// behind everything else (otherwise k is not split).
+// behind everything else (otherwise k is not split): in equal ranges (fp64_ranges), or
+// in the slices of fp64_kslices with a tuned entry or a workspace too small for those.
 void fp64_layout(hmat_context* h, Prepared* out, unsigned char* ws, size_t ws_bytes, bool allow_splitk) {
   const int tm = fp64_tile_m(), tn = fp64_tile_n(), tk = fp64_tile_k();
   int64_t call_tiles = 0;
@@ -387,6 +453,27 @@ void fp64_layout(hmat_context* h, Prepared* out, unsigned char* ws, size_t ws_by
     }
   if (allow_splitk && out->f.size() == 1 && ws) {
     int64_t off = align_up256(out->ws_needed);
+    std::vector<Fp64Shape> shapes;
+    for (const auto& j : out->f[0])
+      shapes.push_back({(int64_t)j.tiles_m * j.tiles_n, j.k, h->h_plans[j.plan].np});
+    std::vector<int32_t> per_tile;
+    Fp64Ranges r = fp64_ranges(h, shapes, &per_tile);
+    if (r.width > 0 && (size_t)(off + fp64_ranges_bytes(r)) <= ws_bytes) {
+      r.part = reinterpret_cast<double*>(ws + off);
+      out->ranges = r;
+      out->ws_needed = std::max(out->ws_needed, align_up256(off + fp64_ranges_bytes(r)));
+      int64_t begin = 0, tile0 = 0;
+      for (size_t i = 0; i < shapes.size(); ++i) {
+        JobDesc& j = out->f[0][i];
+        j.tile_begin = begin;
+        j.tile0 = tile0;
+        j.per_tile = per_tile[i];
+        begin += shapes[i].tiles * per_tile[i];
+        tile0 += shapes[i].tiles;
+      }
+      out->f_tiles.push_back(begin);
+      return;
+    }
     bool fits = true;
     for (auto& j : out->f[0]) {
       const int s = fp64_kslices(h, call_tiles, j.k);
@@ -520,11 +607,18 @@ hmat_status prepare(hmat_context* h, int32_t count, const hmat_gemm_desc* descs,
 
 hmat_status launch_fp64_group(hmat_context* h, const Prepared& pr, int g, const JobDesc* d_jobs,
                               cudaStream_t stream) {
-  const int grid = (int)std::min<int64_t>(pr.f_tiles[g], h->sm_count);
+  const Fp64Ranges ranges = g == 0 ? pr.ranges : Fp64Ranges{};
+  const int grid = (int)(ranges.width > 0 ? ranges.ctas : std::min<int64_t>(pr.f_tiles[g], h->sm_count));
   {
     ProfScope ps(h, 0, stream);
-    cudaError_t e = launch_fp64_bilinear(d_jobs, (int)pr.f[g].size(), h->d_plans, pr.f_tiles[g], grid, stream);
+    cudaError_t e =
+        launch_fp64_bilinear(d_jobs, (int)pr.f[g].size(), h->d_plans, pr.f_tiles[g], grid, ranges, stream);
     if (e != cudaSuccess) return cuda_status(e);
+  }
+  if (ranges.width > 0) {
+    ProfScope ps(h, 14, stream);
+    cudaError_t e = launch_fp64_ranges_reduce(d_jobs, (int)pr.f[g].size(), ranges, stream);
+    return e == cudaSuccess ? HMAT_STATUS_SUCCESS : cuda_status(e);
   }
   // split-k: the slices of each split product added in order, then alpha / beta
   for (const JobDesc& j : pr.f[g]) {
@@ -941,6 +1035,22 @@ hmat_status workspace_bytes(int algo, const TileTables& tables, int32_t count, c
       tiles += ((m + tm - 1) / tm) * ((n + tn - 1) / tn);
     }
     int64_t off = (int64_t)align_up256((int64_t)*bytes);
+    std::vector<Fp64Shape> fshapes;
+    for (int32_t i = 0; i < count && 2 * tiles <= h->sm_count; ++i) {
+      if (!fp64[i]) continue;
+      const int64_t m = sc * descs[i].m, n = sc * descs[i].n;
+      KPlan p;
+      const bool iso_job = algo == HMAT_ALGO_ISOMORPH;
+      if (!build_plan(iso_job ? HMAT_COMPLEX : descs[i].flagsA, iso_job ? HMAT_COMPLEX : descs[i].flagsB, &p))
+        return HMAT_STATUS_INTERNAL;
+      fshapes.push_back({((m + tm - 1) / tm) * ((n + tn - 1) / tn), sc * descs[i].k, p.np});
+    }
+    std::vector<int32_t> per_tile;
+    const Fp64Ranges ranges = fshapes.empty() ? Fp64Ranges{} : fp64_ranges(h, fshapes, &per_tile);
+    if (ranges.width > 0) {
+      *bytes = (size_t)align_up256(off + fp64_ranges_bytes(ranges));
+      return HMAT_STATUS_SUCCESS;
+    }
     for (int32_t i = 0; i < count; ++i) {
       if (!fp64[i]) continue;
       const int64_t m = sc * descs[i].m, n = sc * descs[i].n, k = sc * descs[i].k;

@@ -27,3 +27,39 @@ def test_fp64_k_blocks(m, n, opA, opB, fa, fb):
             torch.cuda.synchronize()
             np.testing.assert_array_equal(C.cpu().numpy(), oracle.bq_gemm(A.numpy(), B.numpy(), opA, opB))
         assert h.device_error() == 0
+
+
+@pytest.mark.parametrize("use_graph", [False, True])
+@pytest.mark.parametrize("shapes", [
+    [(256, 256, 256)],                                       # ranges that cross tiles
+    [(64, 64, 131)],                                         # pieces within a tile, a ragged last one
+    [(32, 32, 2001)],                                        # one tile on every SM
+    [(250, 200, 300), (64, 40, 0), (33, 40, 1000), (10, 9, 50)]])
+def test_fp64_ranges(shapes, use_graph):
+    """Calls of few tiles are cut into equal ranges of the inner dimension when the workspace
+    holds the partial tiles, into fewer slices or none when it is smaller: the same exact result
+    with complex alpha and beta, also for a product without an inner dimension."""
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    alpha, beta = 1 - 2j, 2 + 1j
+    with hm.Handle() as h:
+        probs = []
+        for i, (m, n, k) in enumerate(shapes):
+            fb = bi.TRA if i == 2 else bi.BQ
+            A, B, C0 = bi.small_int(700 + i, m, k), bi.small_int(710 + i, k, n, flags=fb), bi.small_int(720 + i, m, n)
+            probs.append((A.cuda(), B.cuda(), torch.empty_like(C0, device="cuda"), C0, fb,
+                          oracle.bq_gemm(A.numpy(), B.numpy(), alpha=alpha, beta=beta, C=C0.numpy())))
+        descs = [hm.make_desc(a, b, c, flagsB=fb, alpha=alpha, beta=beta) for a, b, c, _, fb, _ in probs]
+        need = hm.hmat_workspace_size(h, descs, "fp64")
+        assert need > 0
+        s = torch.cuda.Stream()
+        for size in (need, need - 1, 4 << 20, 256):
+            ws = torch.empty(size, dtype=torch.uint8, device="cuda")
+            for _, _, c, c0, _, _ in probs:
+                c.copy_(c0)
+            torch.cuda.synchronize()
+            hm.hmat_bq_gemm_grouped(h, descs, "fp64", workspace=ws, use_graph=use_graph, stream=s)
+            torch.cuda.synchronize()
+            for _, _, c, _, _, want in probs:
+                np.testing.assert_array_equal(c.cpu().numpy(), want)
+        assert h.device_error() == 0
