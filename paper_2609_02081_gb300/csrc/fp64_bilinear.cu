@@ -258,7 +258,10 @@ fp64_bilinear_kernel(const JobDesc* __restrict__ jobs, int njobs, const KPlan* _
     const int j0 = (int)(local % jb.tiles_n) * F_BN;
     if (s.plan_id != jb.plan) {
       __syncthreads();
-      if (t == 0) { s.plan = plans[jb.plan]; s.plan_id = jb.plan; }
+      static_assert(sizeof(KPlan) % 8 == 0, "copied in 8-byte words");
+      for (int w = t; w < (int)(sizeof(KPlan) / 8); w += F_THREADS)
+        reinterpret_cast<uint64_t*>(&s.plan)[w] = reinterpret_cast<const uint64_t*>(plans + jb.plan)[w];
+      if (t == 0) s.plan_id = jb.plan;
       __syncthreads();
       for (int w = t; w < 8 * F_MAXP; w += F_THREADS)
         s.wd[w / F_MAXP][w % F_MAXP] = 0.25 * (double)s.plan.w4[w / F_MAXP][w % F_MAXP];

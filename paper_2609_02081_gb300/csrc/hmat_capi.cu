@@ -381,15 +381,15 @@ struct Fp64Shape {
   int np;
 };
 
-// Equal ranges of the call's k-blocks, one per CTA, for calls that the built-in rule
-// of fp64_kslices splits (no tuned entry, twice the tiles fit the SMs, k of 128 or
-// more).  Two ways to cut: pieces of `width` k-blocks that never cross a tile (a tile's
+// Equal ranges of the call's k-blocks, one per CTA, for calls without a tuned entry
+// whose tiles fit half the SMs and whose k is 32 or more.  Two ways to cut: pieces of `width` k-blocks that never cross a tile (a tile's
 // last piece may be short), or every SM the same number of k-blocks, whose piece of a
 // second tile costs another epilogue.  In us, a k-block of np products takes about
-// 4 + np, an epilogue and the pipeline's fill 12 + np / 2; pieces below two k-blocks of
-// the full plan are not worth their partial result.  n = 256, 64 tiles of 64
+// 4 + np, an epilogue and the pipeline's fill 12 + np / 2; a piece is not worth its
+// partial result below one k-block of the full plan (64 x 64 x 64: two at least 91 us,
+// one 74, uncut 504).  n = 256, 64 tiles of 64
 // k-blocks: 2 slices each on 128 SMs 32 + 1, equal ranges on 152 SMs 27 + 2:
-// 935 -> 788 us; 64 x 64 x 1024, 4 tiles: 936 -> 259 us (the rule stops at 8 slices).
+// 935 -> 776 us; 64 x 64 x 1024, 4 tiles: 936 -> 247 us (the rule stops at 8 slices).
 Fp64Ranges fp64_ranges(const hmat_context* h, const std::vector<Fp64Shape>& shapes, std::vector<int32_t>* per_tile) {
   Fp64Ranges r;
   int64_t units = 0, kmax = 0, shortest = INT64_MAX;
@@ -403,11 +403,11 @@ Fp64Ranges fp64_ranges(const hmat_context* h, const std::vector<Fp64Shape>& shap
     np = std::max(np, p.np);
   }
   const int64_t sms = h->sm_count;
-  if (2 * r.tiles > sms || kmax < 128) return Fp64Ranges{};
+  if (2 * r.tiles > sms || kmax < 32) return Fp64Ranges{};
   for (const Fp64Shape& p : shapes)
     if (h->has_fp64_splitk && h->fp64_splitk[ceil_log2_bin(r.tiles) * kTileBins + ceil_log2_bin(p.k)] != 0)
       return Fp64Ranges{};
-  const int64_t least = (56 + 4 + np - 1) / (4 + np);
+  const int64_t least = (28 + 4 + np - 1) / (4 + np);
   const double epilogue = (12 + 0.5 * np) / (4 + np);
   auto pieces = [&](int64_t w) {
     int64_t n = 0;

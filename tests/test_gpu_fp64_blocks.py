@@ -32,6 +32,7 @@ def test_fp64_k_blocks(m, n, opA, opB, fa, fb):
 @pytest.mark.parametrize("use_graph", [False, True])
 @pytest.mark.parametrize("shapes", [
     [(256, 256, 256)],                                       # ranges that cross tiles
+    [(33, 32, 32)],                                          # the shortest k that is cut
     [(64, 64, 131)],                                         # pieces within a tile, a ragged last one
     [(32, 32, 2001)],                                        # one tile on every SM
     [(250, 200, 300), (64, 40, 0), (33, 40, 1000), (10, 9, 50)]])
