@@ -127,6 +127,12 @@ struct TileTables {
   }
 };
 
+// A matrix-form operand whose last k-block holds at most 32 of k keeps it as a half
+// block: rows of 64 bytes in the 64-byte swizzle instead of 128, at the start of the
+// block's place, so that neither the encoder nor the GEMM moves the other half's zeros
+// (64 products of 32 to 160: 307 -> 296 us, 512 of 32 to 1024: 20.2 -> 19.6 ms).
+__host__ __device__ constexpr bool half_last_block(int k) { return ((k - 1) & 63) < 32; }
+
 // Per-problem layout inside the caller's workspace.
 struct SplitJob {
   JobDesc d;

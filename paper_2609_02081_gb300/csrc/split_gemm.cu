@@ -134,6 +134,17 @@ __device__ __forceinline__ uint64_t smem_desc(uint32_t addr) {
   d |= (uint64_t)2u << 61;                      // 128-byte swizzle
   return d;
 }
+// The same for a half k-block (half_last_block): rows of 64 bytes, 64-byte swizzle,
+// 512 bytes between groups of eight rows.
+__device__ __forceinline__ uint64_t smem_desc_half(uint32_t addr) {
+  uint64_t d = 0;
+  d |= (uint64_t)((addr >> 4) & 0x3FFFu);
+  d |= (uint64_t)1u << 16;
+  d |= (uint64_t)(512u >> 4) << 32;
+  d |= (uint64_t)1u << 46;
+  d |= (uint64_t)4u << 61;                      // 64-byte swizzle
+  return d;
+}
 // Instruction descriptor bit that negates the B operand (bit 14 of the
 // kind::f16 descriptor; bit 13 negates A, bits 15 / 16 select their majorness).
 constexpr uint32_t kNegateB = 1u << 14;
@@ -173,6 +184,7 @@ struct Item {
   int nkb, bn, l;     // nkb: k-blocks of all terms; l: index into the modulus table
   int kb2;            // first k-block of the second term (nkb: one term)
   bool neg;           // the second term is subtracted
+  bool half;          // the last k-block is a half block
   int rows, cols;     // rows and columns of the tile inside the product (the rest is padding)
   uint32_t a_bytes, b_bytes;   // bytes copied per k-block: the 8-row groups holding those rows / columns
 };
@@ -224,6 +236,7 @@ __device__ __forceinline__ Item decode_item(const SplitJob& sj, int64_t item, ui
   it.nkb = sj.four_m ? 2 * sj.nkb : sj.nkb;
   it.kb2 = sj.four_m ? sj.nkb : it.nkb;
   it.neg = sj.four_m && ((sj.neg2 >> p) & 1ull);
+  it.half = sj.mat2 != 0 && half_last_block(sj.d.k);
   it.bn = sj.bn;
   it.l = sj.mod_base + l;
   it.rows = min(kTileM, sj.d.m - tm * kTileM);
@@ -342,9 +355,10 @@ split_residue_gemm_kernel(const __grid_constant__ JobParam<kOne> one, const Spli
           const uint32_t fb = smem_u32(&s.full[stage]);
           const bool second = kb >= it.kb2;
           const int kt = second ? kb - it.kb2 : kb;
-          mbar_arrive_tx(fb, it.a_bytes + it.b_bytes);
-          bulk_g2s(smem_u32(s.a[stage]), (second ? it.a2 : it.a) + (int64_t)kt * kATileBytes, it.a_bytes, fb);
-          bulk_g2s(smem_u32(s.b[stage]), (second ? it.b2 : it.b) + (int64_t)kt * bstride, it.b_bytes, fb);
+          const uint32_t sh = it.half && kb + 1 == it.nkb ? 1u : 0u;   // half of the bytes
+          mbar_arrive_tx(fb, (it.a_bytes + it.b_bytes) >> sh);
+          bulk_g2s(smem_u32(s.a[stage]), (second ? it.a2 : it.a) + (int64_t)kt * kATileBytes, it.a_bytes >> sh, fb);
+          bulk_g2s(smem_u32(s.b[stage]), (second ? it.b2 : it.b) + (int64_t)kt * bstride, it.b_bytes >> sh, fb);
           armed[stage] = (int)phase;
           if (++stage == kStages) { stage = 0; phase ^= 1u; }
         }
@@ -381,7 +395,8 @@ split_residue_gemm_kernel(const __grid_constant__ JobParam<kOne> one, const Spli
           tc_fence_after();
           const uint32_t d_tmem = tmem + buf * kBnMax;
           const int kb0 = c * kKbPerChunk, kb1 = min(it.nkb, kb0 + kKbPerChunk);
-          for (int kb = kb0; kb < kb1; ++kb) {
+          const int full1 = kb1 - (it.half && kb1 == it.nkb ? 1 : 0);
+          for (int kb = kb0; kb < full1; ++kb) {
             if (!mbar_wait(smem_u32(&s.full[stage]), phase, abort_flag, err, kErrWaitMma)) { ok = false; break; }
             tc_fence_after();
             const uint64_t ad = smem_desc(smem_u32(s.a[stage]));
@@ -397,6 +412,18 @@ split_residue_gemm_kernel(const __grid_constant__ JobParam<kOne> one, const Spli
             if (++stage == kStages) { stage = 0; phase ^= 1u; }
           }
           if (!ok) break;
+          if (full1 < kb1) {
+            // the half block, outside the loop (a test inside it costs 20 % of long products)
+            if (!mbar_wait(smem_u32(&s.full[stage]), phase, abort_flag, err, kErrWaitMma)) { ok = false; break; }
+            tc_fence_after();
+            const uint64_t ad = smem_desc_half(smem_u32(s.a[stage]));
+            const uint64_t bd = smem_desc_half(smem_u32(s.b[stage]));
+            tc_mma(d_tmem, ad, bd, idesc, full1 > kb0 ? 1u : 0u);
+            tc_mma(d_tmem, ad + 2ull, bd + 2ull, idesc, 1u);
+            issued = true;
+            tc_commit(smem_u32(&s.empty[stage]));
+            if (++stage == kStages) { stage = 0; phase ^= 1u; }
+          }
           tc_commit(smem_u32(&s.tfull[buf]));
           ++chunk_ctr;
         }

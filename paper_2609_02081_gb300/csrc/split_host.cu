@@ -357,6 +357,11 @@ static constexpr int64_t kPlaneSkewRes = 3 * 256;
 // 16 (the residue GEMM copies whole 8-row groups of a tile and never reads the
 // rows beyond them) and the inner dimension padded to whole k-blocks (zeros)
 static inline int64_t enc_blocks(int64_t rows, int64_t nkb) { return ((rows + 15) / 16) * (nkb * kTileK / 32); }
+// the matrix form's: the last k-block may be a half one
+static inline int64_t mat2_enc_blocks(int64_t rows, int64_t k) { return ((rows + 15) / 16) * ((k + 31) / 32); }
+static inline int64_t job_enc_blocks(const SplitJob& sj, int64_t rows) {
+  return sj.mat2 ? mat2_enc_blocks(rows, sj.d.k) : enc_blocks(rows, sj.nkb);
+}
 // CRT blocks: one per `rows` output rows and kCrtCols consecutive columns
 static inline int64_t crt_blocks(int64_t m, int64_t n, int rows) {
   return ((m + rows - 1) / rows) * ((n + kCrtCols - 1) / kCrtCols);
@@ -481,7 +486,7 @@ hmat_status split_prepare(const std::vector<JobDesc>& jobs, const KPlan* h_plans
     if (mat2) to_mat2(&sj, off0);
     sj.exp_begin = sp.exp_units;
     sp.exp_units += (d.m + 31) / 32 + (d.n + 31) / 32;
-    const int64_t ea = enc_blocks(d.m, sj.nkb), eb = enc_blocks(d.n, sj.nkb);
+    const int64_t ea = job_enc_blocks(sj, d.m), eb = job_enc_blocks(sj, d.n);
     sj.encA_begin = sp.encA_units;
     sj.encB_begin = sp.encB_units;
     sj.enc2_begin = sp.enc2_units;
@@ -530,8 +535,8 @@ hmat_status split_layout_single(const JobDesc& d, const KPlan& P, double tol, co
   if ((int64_t)sj.nmod * sj.np * sj.tiles_m * sj.tiles_n >= ((int64_t)1 << 31)) return HMAT_STATUS_UNSUPPORTED;
   if (mat2) to_mat2(&sj, 0);
   units->exp = (d.m + 31) / 32 + (d.n + 31) / 32;
-  units->encA = enc_blocks(d.m, sj.nkb);
-  units->encB = enc_blocks(d.n, sj.nkb);
+  units->encA = job_enc_blocks(sj, d.m);
+  units->encB = job_enc_blocks(sj, d.n);
   units->items = (int64_t)sj.nmod * sj.np * sj.tiles_m * sj.tiles_n;
   units->crt = crt_job_blocks(sj, sj.full != 0);
   units->max_bits = sj.bits;
@@ -570,7 +575,7 @@ hmat_status split_launch(hmat_context* h, const SplitPrep& sp, const SplitJob* d
     if (e == cudaSuccess && !skip_b)
       e = launch_split_encode(jobs, d_plans, 1, sp.encB_units, stream, ws, sp.max_bits);
     // the matrix form's blocks: A side first, then B side
-    const int64_t a_blocks = njobs == 1 ? enc_blocks(sp.jobs[0].d.m, sp.jobs[0].nkb) : 0;
+    const int64_t a_blocks = njobs == 1 ? mat2_enc_blocks(sp.jobs[0].d.m, sp.jobs[0].d.k) : 0;
     const int64_t first = skip_a ? a_blocks : 0, end = skip_b ? std::min(a_blocks, sp.enc2_units) : sp.enc2_units;
     if (e == cudaSuccess && end > first)
       e = launch_mat2_encode(jobs, end - first, first, stream, ws, sp.max_bits2);

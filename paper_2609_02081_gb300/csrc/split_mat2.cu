@@ -185,7 +185,7 @@ __device__ __forceinline__ void encode_pair(const longlong2* E, int l0, int l1, 
 //   phase 2: a thread takes two neighbouring k of one row, splits its eight
 //            integers into float digits once, holds them in registers over the
 //            moduli and stores one bfloat162 per factor plane: 16 lanes fill one
-//            aligned half of a swizzled 128-byte row.
+//            aligned half of a swizzled 128-byte row (or a row of a half block).
 // Bound by its writes (28 bytes per modulus and element of a full operand: 65 GB in
 // 10.2 ms at n = 8192, 0.94 of the copy bandwidth).
 template <int ND, bool kOne>
@@ -197,7 +197,7 @@ __global__ void __launch_bounds__(kThreads, 4)
   const int64_t blk = first + blockIdx.x;
   const SplitJob& sj = unit_job(one, jobs, njobs, blk, 5);
   const JobDesc& d = sj.d;
-  const int ktiles = sj.nkb * (kTileK / kK);
+  const int ktiles = (d.k + kK - 1) / kK;
   const int64_t a_blocks = (int64_t)((d.m + kRows - 1) / kRows) * ktiles;
   int64_t within = blk - sj.enc2_begin;
   const int side = within >= a_blocks ? 1 : 0;
@@ -291,8 +291,9 @@ __global__ void __launch_bounds__(kThreads, 4)
     const int kg = k0 + kp;
     const int kb = kg / kTileK, c16 = (kg % kTileK) / 8, in16 = (kg % 8) * 2;
     const int rt = r / tile_rows, rin = r % tile_rows;
-    unsigned char* out = enc + ((int64_t)rt * sj.nkb + kb) * tile_bytes + (int64_t)(rin >> 3) * 1024 +
-                         (rin & 7) * 128 + ((c16 ^ (rin & 7)) << 4) + in16;
+    const bool half = kb + 1 == sj.nkb && half_last_block(d.k);
+    const int in_tile = half ? rin * 64 + ((c16 ^ ((rin >> 1) & 3)) << 4) : rin * 128 + ((c16 ^ (rin & 7)) << 4);
+    unsigned char* out = enc + ((int64_t)rt * sj.nkb + kb) * tile_bytes + in_tile + in16;
     longlong2 E[8];
     auto load = [&](int count) {
 #pragma unroll

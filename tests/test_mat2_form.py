@@ -349,3 +349,23 @@ def test_grouped_matrix_form_beside_other_forms(handles, use_graph):
             res.append(Cs)
         for a, b in zip(*res):
             assert torch.equal(a, b)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("fa,fb", [(bi.BQ, bi.BQ), (bi.TRS, bi.BQ), (bi.TRS, bi.TRA), (bi.COMPLEX, bi.BQ)])
+@pytest.mark.parametrize("m,n", [(5, 9), (130, 70), (300, 257)])
+def test_half_last_k_block(m, n, fa, fb):
+    """The last 64-deep k-block is kept as a half block when it holds at most 32 of k: exact on small
+    integers on both sides of every boundary, one chunk (k <= 1024) and more."""
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    with hm.Handle() as h:
+        for k in (1, 16, 31, 32, 33, 63, 64, 65, 80, 96, 97, 128, 150, 1024, 1025, 1056, 1057, 2090):
+            A, B = bi.small_int(800 + k, m, k, flags=fa), bi.small_int(801 + k, k, n, flags=fb)
+            want = torch.full((8, m, n), float("nan"), dtype=torch.float64, device="cuda")
+            got = want.clone()
+            Ad, Bd = A.cuda(), B.cuda()
+            hm.hmat_bq_gemm(h, Ad, Bd, want, flagsA=fa, flagsB=fb, mode="fp64")      # exact on small integers
+            hm.hmat_bq_gemm(h, Ad, Bd, got, flagsA=fa, flagsB=fb, mode="split", tol=TOL)
+            assert torch.equal(got, want), k
+        assert h.device_error() == 0
