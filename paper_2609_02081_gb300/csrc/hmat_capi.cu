@@ -1179,7 +1179,7 @@ hmat_status hmat_bq_gemm_split_noalloc(hmat_handle h, int32_t opA, int32_t opB, 
   }
   if (e == cudaSuccess)
     e = launch_split_gemm(jobs, u.items, (int)std::min<int64_t>(u.items, h->sm_count), stream, a.scratch,
-                          u.max_nkb);
+                          u.one_chunk);
   if (e == cudaSuccess && sj.mat2)
     e = launch_mat2_crt(jobs, u.crt, stream, a.scratch, u.max_nmod);
   else if (e == cudaSuccess)

@@ -78,6 +78,7 @@ Mat2Shape mat2_shape(uint32_t fa, uint32_t fb);
 constexpr int kMat2MaxPlanes = 14;
 // the largest sum of product residues in one output: |sum| <= 16 (p - 1)/2
 constexpr int kMat2WeightSum = 16;
+constexpr int kMat2ChunkK = 1088;  // its chunk (set_per_chunk)
 constexpr int kMat2HalfMax = 120;  // (p - 1)/2 of its largest modulus, 241
 // Most moduli whose sums S < 2 N P fit four 32-bit limbs (P < 2^111.1 and N =
 // 15 * 16 * 120 < 2^14.9; checked when the tables are built)
@@ -138,6 +139,7 @@ struct SplitJob {
   JobDesc d;
   int32_t nmod, bits, bn;           // moduli, integer width, tile N
   int32_t tiles_m, tiles_n, nkb;    // 128-row tiles, bn-column tiles, 64-wide k blocks
+  int32_t per_chunk;                // k-blocks of an accumulation chunk (set_per_chunk)
   int32_t np, nlf, nrf;
   int32_t full;                     // the plan is the paper's full plan (KPlan::bilinear_full), either form
   int32_t four_m;                   // two-term products: p is pl pr + (-1 if bit p of neg2) pl2 pr2
@@ -219,7 +221,8 @@ struct SplitPrep {
   int64_t enc2_units = 0, crt2_units = 0;   // matrix-form jobs
   int max_bits2 = 0, max_nmod2 = 0;         // matrix-form jobs (max_bits, max_nmod, max_np: the others)
   int64_t ws_needed = 0;
-  int max_bits = 0, max_nmod = 0, max_np = 0, max_nkb = 0;
+  int max_bits = 0, max_nmod = 0, max_np = 0;
+  bool one_chunk = true;              // every job's products fit one accumulation chunk
   bool all_full = true;             // every job outside the matrix form uses the paper's full plan (either form)
   int n_four_m = 0;                 // jobs in the four-multiplication form
   int n_plan = 0;                   // jobs outside the matrix form
@@ -250,7 +253,8 @@ hmat_status split_prepare(const std::vector<JobDesc>& jobs, const KPlan* h_plans
 // uses no heap memory (for the entry point that allocates nothing).
 struct SplitUnits {
   int64_t exp = 0, encA = 0, encB = 0, items = 0, crt = 0, ws_bytes = 0;
-  int max_bits = 0, max_nmod = 0, max_np = 0, max_nkb = 0;
+  int max_bits = 0, max_nmod = 0, max_np = 0;
+  bool one_chunk = true;              // every job's products fit one accumulation chunk
   bool all_full = false;
   bool four_m = false;
 };
@@ -309,11 +313,9 @@ cudaError_t launch_split_exponents(const SplitJobs& jobs, int64_t units, int64_t
 // units are blocks: encode tiles of 32 rows x 32 k, CRT blocks of 256 elements
 cudaError_t launch_split_encode(const SplitJobs& jobs, const KPlan* d_plans, int side, int64_t units,
                                 cudaStream_t s, unsigned char* ws, int max_bits);
-// max_nkb: the most 64-deep k-blocks of any job's products (two-term products
-// count both terms; the one-chunk kernel form serves launches whose jobs all
-// have at most 16)
+// one_chunk: every job's products fit one accumulation chunk (the one-chunk kernel form)
 cudaError_t launch_split_gemm(const SplitJobs& jobs, int64_t items, int grid, cudaStream_t s,
-                              unsigned char* ws, int max_nkb);
+                              unsigned char* ws, bool one_chunk);
 // all_full: every job uses the paper's full plan (structured recombination),
 // full_form: 0 all in Gauss's form, 1 all in the four-multiplication form, 2
 // both; all_wide: every job's full-plan CRT blocks are one row of kCrtCols

@@ -10,8 +10,8 @@
 // term follow those of the first, its sign through the negate-B bit.
 //
 // Exactness: every BF16 product is an integer of magnitude <= 2^14 and FP32
-// partial sums of at most 1024 of them stay <= 2^24, so the tensor-memory
-// accumulator is exact chunk by chunk; each 1024-deep chunk is drained, its
+// partial sums of at most 1024 of them stay <= 2^24 (1088 of the matrix form's), so
+// the tensor-memory accumulator is exact chunk by chunk; each chunk is drained, its
 // residue mod p added to a float running sum (exact), and the sum is reduced
 // mod p at the end of the item.
 //
@@ -50,7 +50,6 @@ constexpr int kBTileBytesMax = kBnMax * kTileK * 2;    // 32 KB
 constexpr int kThreads = 320;
 constexpr int kEpiWarps = 8;
 constexpr int kTmemCols = 2 * kBnMax;
-constexpr int kKbPerChunk = kChunkK / kTileK;          // 16
 constexpr long long kWaitCycles = 4000000000ll;        // ~2 s at 2 GHz
 constexpr int kRasterGroup = 16;                        // tile rows per raster group
 
@@ -185,6 +184,7 @@ struct Item {
   int kb2;            // first k-block of the second term (nkb: one term)
   bool neg;           // the second term is subtracted
   bool half;          // the last k-block is a half block
+  int per_chunk;      // k-blocks of an accumulation chunk
   int rows, cols;     // rows and columns of the tile inside the product (the rest is padding)
   uint32_t a_bytes, b_bytes;   // bytes copied per k-block: the 8-row groups holding those rows / columns
 };
@@ -236,6 +236,7 @@ __device__ __forceinline__ Item decode_item(const SplitJob& sj, int64_t item, ui
   it.nkb = sj.four_m ? 2 * sj.nkb : sj.nkb;
   it.kb2 = sj.four_m ? sj.nkb : it.nkb;
   it.neg = sj.four_m && ((sj.neg2 >> p) & 1ull);
+  it.per_chunk = sj.per_chunk;
   it.half = sj.mat2 != 0 && half_last_block(sj.d.k);
   it.bn = sj.bn;
   it.l = sj.mod_base + l;
@@ -295,7 +296,7 @@ struct GemmModConst {
 __constant__ GemmModConst c_gmod[2 * kModTable];   // the plans' moduli, then the matrix form's
 
 // kOneChunk: every item of the launch has an inner dimension of one chunk
-// (k <= 1024), so the multi-chunk epilogue and its 128 running sums per
+// (k <= 1024, the matrix form's k <= 1088), so the multi-chunk epilogue and its 128 running sums per
 // thread are compiled out (the register budget then holds the single-chunk
 // drain without spills).
 // kOne: one job, in the arguments, instead of the table.
@@ -388,13 +389,12 @@ split_residue_gemm_kernel(const __grid_constant__ JobParam<kOne> one, const Spli
         const uint32_t idesc = instr_desc(it.bn);
         // the subtracted second term of a two-term product: negate B
         const uint32_t idesc2 = it.neg ? (idesc | kNegateB) : idesc;
-        const int nchunks = (it.nkb + kKbPerChunk - 1) / kKbPerChunk;
-        for (int c = 0; ok && c < nchunks; ++c) {
+        for (int kb0 = 0; ok && kb0 < it.nkb; kb0 += it.per_chunk) {
           const uint32_t buf = chunk_ctr & 1u, aph = (chunk_ctr >> 1) & 1u;
           if (!mbar_wait(smem_u32(&s.tempty[buf]), aph ^ 1u, abort_flag, err, kErrWaitMma)) { ok = false; break; }
           tc_fence_after();
           const uint32_t d_tmem = tmem + buf * kBnMax;
-          const int kb0 = c * kKbPerChunk, kb1 = min(it.nkb, kb0 + kKbPerChunk);
+          const int kb1 = min(it.nkb, kb0 + it.per_chunk);
           const int full1 = kb1 - (it.half && kb1 == it.nkb ? 1 : 0);
           for (int kb = kb0; kb < full1; ++kb) {
             if (!mbar_wait(smem_u32(&s.full[stage]), phase, abort_flag, err, kErrWaitMma)) { ok = false; break; }
@@ -456,10 +456,9 @@ split_residue_gemm_kernel(const __grid_constant__ JobParam<kOne> one, const Spli
       const Item it = decode_item(item_job(one, jobs, job), item, ws);
       const int cols = kOneChunk ? it.bn : it.bn >> 1;   // columns handled by this thread: a multiple of 16
       const int col0 = kOneChunk ? 0 : half * cols;
-      const int nchunks = (it.nkb + kKbPerChunk - 1) / kKbPerChunk;
       const float pf = c_gmod[it.l].pf, pinv = c_gmod[it.l].inv, magic = c_gmod[it.l].magic;
       const float2 npf2 = make_float2(-pf, -pf), inv2 = make_float2(pinv, pinv);
-      if (nchunks == 1) {
+      if (it.nkb <= it.per_chunk) {
         // One chunk: each 32-column load is reduced and stored at once.
         // fmod_centred2 rounds the exact product v * fl(1/p), which is within
         // |v| 2^-24 / p of v / p, while v / p is at least 1/(2p) from a
@@ -550,7 +549,7 @@ split_residue_gemm_kernel(const __grid_constant__ JobParam<kOne> one, const Spli
       float acc[kBnMax / 2];
 #pragma unroll
       for (int i = 0; i < kBnMax / 2; ++i) acc[i] = 0.f;
-      for (int c = 0; c < nchunks; ++c) {
+      for (int kb0 = 0; kb0 < it.nkb; kb0 += it.per_chunk) {
         const uint32_t buf = chunk_ctr & 1u, aph = (chunk_ctr >> 1) & 1u;
         // one lane waits, the warp follows (tcgen05.ld is warp-collective)
         int got = 0;
@@ -658,11 +657,11 @@ cudaError_t split_gemm_configure(const int* moduli, int n) {
 }
 
 cudaError_t launch_split_gemm(const SplitJobs& jobs, int64_t items, int grid, cudaStream_t s,
-                              unsigned char* ws, int max_nkb) {
+                              unsigned char* ws, bool one_chunk) {
   if (items <= 0) return cudaSuccess;
   return with_jobs(jobs, [&](const auto& one) {
     constexpr bool kOne = std::is_same_v<std::decay_t<decltype(one)>, JobParam<true>>;
-    return launch_dependent(max_nkb <= kKbPerChunk ? split_residue_gemm_kernel<true, kOne>
+    return launch_dependent(one_chunk ? split_residue_gemm_kernel<true, kOne>
                                                    : split_residue_gemm_kernel<false, kOne>,
                             dim3(grid), dim3(kThreads), split_gemm_smem_bytes(), s, one, jobs.table, jobs.n, items, ws,
                             device_error_ptr());

@@ -349,6 +349,21 @@ static void to_mat2(SplitJob* sj, int64_t offset0) {
   place_job(sj, sj->d.m, sj->d.n, &off);
 }
 
+// Accumulation chunks of the job's products: FP32 sums are exact up to 2^24, which is
+// 1024 of k for residues up to 128 and 1088 for the matrix form's, up to 121.  Each
+// chunk's drain runs beside the next chunk's MMAs, so the k-blocks are spread evenly: a
+// short last chunk would leave the issuer waiting for the drain before it (1537 x 771 x
+// 2049, three chunks of 16 + 16 + 1 k-blocks against two of 17 + 16: 867 -> 828 us).
+static bool set_per_chunk(SplitJob* sj) {      // true when one chunk holds them all
+  const int total = sj->four_m ? 2 * sj->nkb : sj->nkb;
+  const int most = (sj->mat2 ? kMat2ChunkK : kChunkK) / kTileK;
+  const int chunks = std::max(1, (total + most - 1) / most);
+  sj->per_chunk = (total + chunks - 1) / chunks;
+  return chunks == 1;
+}
+static_assert(kChunkK * 128 * 128 <= (1 << 24) && kMat2ChunkK * (kMat2HalfMax + 1) * (kMat2HalfMax + 1) <= (1 << 24),
+              "exact FP32 accumulation of a chunk");
+
 // plane skews: an odd multiple of 256 B (bulk copies need 16-byte alignment)
 static constexpr int64_t kPlaneSkewEnc = 3 * 256;
 static constexpr int64_t kPlaneSkewRes = 3 * 256;
@@ -505,7 +520,7 @@ hmat_status split_prepare(const std::vector<JobDesc>& jobs, const KPlan* h_plans
     }
     sj.item_begin = sp.items;
     sp.items += (int64_t)sj.nmod * sj.np * sj.tiles_m * sj.tiles_n;
-    sp.max_nkb = std::max(sp.max_nkb, sj.four_m ? 2 * sj.nkb : sj.nkb);
+    if (!set_per_chunk(&sj)) sp.one_chunk = false;
     sp.n_four_m += sj.four_m ? 1 : 0;
     sp.jobs.push_back(sj);
   }
@@ -542,7 +557,7 @@ hmat_status split_layout_single(const JobDesc& d, const KPlan& P, double tol, co
   units->max_bits = sj.bits;
   units->max_nmod = sj.nmod;
   units->max_np = sj.np;
-  units->max_nkb = sj.four_m ? 2 * sj.nkb : sj.nkb;
+  units->one_chunk = set_per_chunk(&sj);
   units->all_full = sj.full != 0;
   units->four_m = sj.four_m != 0;
   units->ws_bytes = off;
@@ -584,7 +599,7 @@ hmat_status split_launch(hmat_context* h, const SplitPrep& sp, const SplitJob* d
   {
     ProfScope ps(h, 3, stream);
     const int grid = (int)std::min<int64_t>(sp.items, handle_sm_count(h));
-    e = launch_split_gemm(jobs, sp.items, grid, stream, ws, sp.max_nkb);
+    e = launch_split_gemm(jobs, sp.items, grid, stream, ws, sp.one_chunk);
   }
   if (e != cudaSuccess) return split_cuda_error(e);
   {

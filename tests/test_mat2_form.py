@@ -356,11 +356,11 @@ def test_grouped_matrix_form_beside_other_forms(handles, use_graph):
 @pytest.mark.parametrize("m,n", [(5, 9), (130, 70), (300, 257)])
 def test_half_last_k_block(m, n, fa, fb):
     """The last 64-deep k-block is kept as a half block when it holds at most 32 of k: exact on small
-    integers on both sides of every boundary, one chunk (k <= 1024) and more."""
+    integers on both sides of every boundary, and of the accumulation chunks (up to 1088 deep, spread evenly)."""
     if not torch.cuda.is_available():
         pytest.skip("no GPU")
     with hm.Handle() as h:
-        for k in (1, 16, 31, 32, 33, 63, 64, 65, 80, 96, 97, 128, 150, 1024, 1025, 1056, 1057, 2090):
+        for k in (1, 16, 31, 32, 33, 63, 64, 65, 80, 96, 97, 128, 150, 1024, 1025, 1057, 1088, 1089, 2090, 2177):
             A, B = bi.small_int(800 + k, m, k, flags=fa), bi.small_int(801 + k, k, n, flags=fb)
             want = torch.full((8, m, n), float("nan"), dtype=torch.float64, device="cuda")
             got = want.clone()
