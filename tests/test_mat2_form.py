@@ -369,3 +369,29 @@ def test_half_last_k_block(m, n, fa, fb):
             hm.hmat_bq_gemm(h, Ad, Bd, got, flagsA=fa, flagsB=fb, mode="split", tol=TOL)
             assert torch.equal(got, want), k
         assert h.device_error() == 0
+
+
+@pytest.mark.gpu
+def test_narrow_products_beside_deep_ones():
+    """Products of one accumulation chunk in a launch with deeper ones, over output widths whose halves
+    the epilogue splits unevenly (32: one half only; 96, 160, 224): exact on small integers."""
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    shapes = [(40, 20, 100), (70, 33, 1500), (10, 32, 64), (140, 32, 1300), (200, 224, 2100), (33, 90, 700), (150, 160, 1090),
+              (129, 100, 3000)]
+    with hm.Handle() as h:
+        descs, outs = [], []
+        for i, (m, n, k) in enumerate(shapes):
+            A, B = bi.small_int(830 + i, m, k).cuda(), bi.small_int(840 + i, k, n).cuda()
+            C, want = (torch.full((8, m, n), float("nan"), dtype=torch.float64, device="cuda") for _ in range(2))
+            hm.hmat_bq_gemm(h, A, B, want, mode="fp64")
+            descs.append(hm.make_desc(A, B, C))
+            outs.append((C, want, A, B))
+        hm.hmat_bq_gemm_grouped(h, descs, "split", TOL)
+        for i, (C, want, _, _) in enumerate(outs):
+            assert torch.equal(C, want), shapes[i]
+            C.fill_(float("nan"))
+        for d, (C, want, A, B) in zip(descs, outs):
+            hm.hmat_bq_gemm(h, A, B, C, mode="split", tol=TOL)
+            assert torch.equal(C, want)
+        assert h.device_error() == 0
