@@ -151,7 +151,9 @@ struct SplitJob {
   int64_t off_encA, off_encB;       // BF16 factor tiles
   int64_t off_res;                  // int8 product residues
   int64_t encA_plane, encB_plane;   // bytes between consecutive (modulus, factor) tile planes
-  int64_t res_plane;                // bytes between consecutive (modulus, product) residue planes
+  // bytes between consecutive (modulus, product) residue planes: rows of tiles_n bn bytes, in
+  // the matrix form groups of 32 columns, each the tiles_m * 128 rows of 32 bytes
+  int64_t res_plane;
   int32_t mat2, rot;                // matrix form (kMat2None: a plan's products): kind, power of i of the result
   int32_t mod_base;                 // first modulus in the GEMM's table (kModTable: the matrix form's moduli)
   int64_t item_begin;               // residue-GEMM work items before this job

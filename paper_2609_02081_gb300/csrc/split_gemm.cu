@@ -179,7 +179,7 @@ struct Item {
   const uint8_t* a2;  // two-term products: the second term's factors (k-blocks kb2 .. nkb - 1)
   const uint8_t* b2;
   int8_t* out;        // residue tile origin (row 0, column 0 of the tile)
-  int64_t ncols;      // residue row pitch
+  int64_t row_bytes, group_bytes;   // of the residues: between rows, between groups of 32 columns
   int nkb, bn, l;     // nkb: k-blocks of all terms; l: index into the modulus table
   int kb2;            // first k-block of the second term (nkb: one term)
   bool neg;           // the second term is subtracted
@@ -257,10 +257,10 @@ __device__ __forceinline__ Item decode_item(const SplitJob& sj, int64_t item, ui
     it.a2 = ws + sj.off_encA + ((int64_t)l * sj.nlf + sj.pl2[p]) * sj.encA_plane + ((int64_t)tm * sj.nkb) * a_tile;
     it.b2 = ws + sj.off_encB + ((int64_t)l * sj.nrf + sj.pr2[p]) * sj.encB_plane + ((int64_t)tn * sj.nkb) * b_tile;
   }
-  it.ncols = (int64_t)sj.tiles_n * sj.bn;
-  const int64_t plane = sj.res_plane;
-  it.out = reinterpret_cast<int8_t*>(ws + sj.off_res) + ((int64_t)l * sj.np + p) * plane +
-           (int64_t)tm * kTileM * it.ncols + (int64_t)tn * sj.bn;
+  it.row_bytes = sj.mat2 ? 32 : (int64_t)sj.tiles_n * sj.bn;
+  it.group_bytes = sj.mat2 ? (int64_t)sj.tiles_m * (kTileM * 32) : 32;
+  it.out = reinterpret_cast<int8_t*>(ws + sj.off_res) + ((int64_t)l * sj.np + p) * sj.res_plane +
+           (int64_t)tm * kTileM * it.row_bytes + (int64_t)((tn * sj.bn) >> 5) * it.group_bytes;
   return it;
 }
 
@@ -483,7 +483,7 @@ split_residue_gemm_kernel(const __grid_constant__ JobParam<kOne> one, const Spli
         tc_fence_after();
         const uint32_t taddr = tmem + ((uint32_t)(q * 32) << 16) + buf * kBnMax + (uint32_t)col0;
         const bool twice = it.nkb > 8;
-        int8_t* dst = it.out + (int64_t)row * it.ncols + col0;
+        int8_t* dst = it.out + (int64_t)row * it.row_bytes + (int64_t)(col0 >> 5) * it.group_bytes;
         // reduce and store the 32 columns of group g held in rr
         auto drain32 = [&](int g, const uint32_t* rr) {
           const int c32 = g * 32;
@@ -500,7 +500,7 @@ split_residue_gemm_kernel(const __grid_constant__ JobParam<kOne> one, const Spli
             }
             w[v] = pack4_residues(t01, t23, magic);
           }
-          store32(dst + c32, w);
+          store32(dst + g * it.group_bytes, w);
         };
         auto release = [&]() {
           tc_fence_before();
@@ -592,7 +592,7 @@ split_residue_gemm_kernel(const __grid_constant__ JobParam<kOne> one, const Spli
       // 129 * 127 < 2^14, where acc * (1/p) is within 2^-9 of acc / p, which
       // is at least 1/(2p) from a half-integer: the rounding is exact.
       if (row < it.rows) {
-        int8_t* dst = it.out + (int64_t)row * it.ncols + col0;
+        int8_t* dst = it.out + (int64_t)row * it.row_bytes + (int64_t)(col0 >> 5) * it.group_bytes;
 #pragma unroll
         for (int g = 0; g < kBnMax / 2 / 32; ++g) {
           if (g * 32 < cols && col0 + g * 32 < it.cols) {
@@ -603,7 +603,7 @@ split_residue_gemm_kernel(const __grid_constant__ JobParam<kOne> one, const Spli
               w[v] = pack4_residues(fmod_centred2(make_float2(acc[b], acc[b + 1]), npf2, inv2),
                                     fmod_centred2(make_float2(acc[b + 2], acc[b + 3]), npf2, inv2), magic);
             }
-            store32(dst + g * 32, w);
+            store32(dst + g * it.group_bytes, w);
           }
         }
       }

@@ -250,7 +250,7 @@ void split_release(SplitState& s) {
 // ----------------------------------------------------------------- layout
 // Built-in tile width: the fewest tiles of at most 256 columns, each as
 // narrow as a multiple of 32 allows (tcgen05 takes any N that is a multiple of
-// 16 with M = 128; the epilogue stores 16-column groups per half tile), so
+// 16 with M = 128; the epilogue stores 32-column groups), so
 // that padding columns stay below 32 per tile (n = 96: one tile of 96; n = 300:
 // two of 160).
 static int pick_bn(int64_t n) {
@@ -384,20 +384,28 @@ static inline int64_t crt_blocks(int64_t m, int64_t n, int rows) {
 // CRT blocks of a job and its block width: the full-plan kernel's blocks are
 // kCrtCols / crt_width(n) rows of crt_width(n) columns, the matrix form's likewise
 // with mat2_crt_width, the other kernels' kCrtRows rows of kCrtCols columns
-// Matrix form: the widest block (longest contiguous residue reads) that pads the
-// columns by at most 6 % more than 32-wide ones would.  The 512-product batch's CRT:
-// 3.59 ms with 32 columns for all n < 1024, 3.45 with this, 3.56 at 30 %.
-static int mat2_crt_width(int64_t n) {
-  for (int w = kCrtCols; w > 32; w /= 2)
-    if (100 * ((n + w - 1) / w * w) <= 106 * ((n + 31) / 32 * 32)) return w;
-  return 32;
+// Matrix form: 4 rows of 32 columns, which read 128 contiguous bytes of the residues (kept
+// in groups of 32 columns), unless a wider block pads the output by 6 % less (few rows).
+// The 512-product batch's CRT: 3.44 -> 3.27 ms against rows of residues with blocks of 32
+// to 128 columns; rows of 128 columns here: 4.08 ms.
+static int mat2_crt_width(int64_t m, int64_t n) {
+  int best = 32;
+  int64_t least = 0;
+  for (int w = 32; w <= kCrtCols; w *= 2) {
+    const int64_t rows = kCrtCols / w, elems = ((m + rows - 1) / rows * rows) * ((n + w - 1) / w * w);
+    if (w == 32 || 106 * elems < 100 * least) {
+      best = w;
+      least = elems;
+    }
+  }
+  return best;
 }
 static inline int64_t crt_job_blocks(SplitJob& sj, bool all_full) {
   if (!all_full && !sj.mat2) {
     sj.crt_w = kCrtCols;
     return crt_blocks(sj.d.m, sj.d.n, kCrtRows);
   }
-  sj.crt_w = sj.mat2 ? mat2_crt_width(sj.d.n) : crt_width(sj.d.n);
+  sj.crt_w = sj.mat2 ? mat2_crt_width(sj.d.m, sj.d.n) : crt_width(sj.d.n);
   const int64_t rows = kCrtCols / sj.crt_w;
   return ((sj.d.m + rows - 1) / rows) * ((sj.d.n + sj.crt_w - 1) / sj.crt_w);
 }

@@ -320,7 +320,7 @@ __global__ void __launch_bounds__(kThreads, 4)
 
 // ------------------------------------------------------------------ CRT
 // One warp per 32 consecutive elements of an output row; a block of four warps
-// covers one row of 128 columns, two of 64 or four of 32.
+// covers four rows of 32 columns, two of 64 or one of 128 (mat2_crt_width).
 //
 // Per element and modulus the outputs are sums of the product residues.  With cu,
 // cv the entries of the two copies' 2 x 2 products:
@@ -350,7 +350,7 @@ __global__ void __launch_bounds__(kThreads, 4)
 // Bound by instruction issue (2.6 of 4 per cycle, 54 instructions per element and
 // warp lane; 64-bit multiply-adds per modulus, output and limb took 113): 1.2 ms
 // for 4096 x 4096 (2.35 ms with those), 0.68 ms of which its 4.6 GB would take at
-// the copy bandwidth; the 512-product batch 3.45 ms (6.1 ms).
+// the copy bandwidth; the 512-product batch 3.27 ms (6.1 ms).
 constexpr int kCrtThreads = 128;
 constexpr int mod_stride(int planes) {                // bytes; the four moduli pairs of a read fall on different banks
   return planes * kCrtCols + 16;
@@ -474,7 +474,7 @@ __device__ __forceinline__ void crt_block(const SplitJob& sj, uint32_t local, co
   const uint32_t rowblock = local / colblocks;
   const int i0 = (int)rowblock * (kCrtCols >> lw);
   const int j0 = (int)(local - rowblock * colblocks) << lw;
-  const int64_t ncols = (int64_t)sj.tiles_n * sj.bn;
+  const int64_t group = (int64_t)sj.tiles_m * (kTileM * 32);   // bytes of 32 columns of residues
   // this thread's fragments of the digits (zero for moduli >= nmod)
   uint32_t b[2][KS][2][2];
 #pragma unroll
@@ -489,10 +489,11 @@ __device__ __forceinline__ void crt_block(const SplitJob& sj, uint32_t local, co
   // copy: thread tid takes 16-byte chunk tid % 8 of planes tid / 8, tid / 8 + 16, ...
   {
     const int64_t plane = sj.res_plane;
-    const int cc = tid & 7, crow = cc >> (lw - 4), ccol = (cc & ((w >> 4) - 1)) * 16;
-    if (i0 + crow < d.m && (int64_t)j0 + ccol < ncols) {
+    const int cc = tid & 7, crow = cc >> (lw - 4), col = j0 + (cc & ((w >> 4) - 1)) * 16;
+    if (i0 + crow < d.m && col < d.n) {
       int q = tid >> 3;                                    // plane: modulus l, product r
-      const unsigned char* src = ws + sj.off_res + (int64_t)q * plane + (int64_t)(i0 + crow) * ncols + j0 + ccol;
+      const unsigned char* src = ws + sj.off_res + (int64_t)q * plane + (int64_t)(col >> 5) * group +
+                                 (int64_t)(i0 + crow) * 32 + (col & 16);
       int l = q / NP, r = q % NP;
       for (; q < nm * NP; q += 16) {
         cp_async16(ring + l * kStride + r * kCrtCols + cc * 16, src);
