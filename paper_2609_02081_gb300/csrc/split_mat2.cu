@@ -486,24 +486,22 @@ __device__ __forceinline__ void crt_block(const SplitJob& sj, uint32_t local, co
 #pragma unroll
         for (int v = 0; v < 2; ++v) b[h][ks][nt][v] = __ldg(&g_m2digits[nm][h][ks][nt][v][lane]);
   wait_for_previous_kernel();                              // the residues
-  // copy: thread tid takes 16-byte chunk tid % 8 of planes tid / 8, tid / 8 + 16, ...
+  // copy: thread tid takes 16-byte chunk tid % 8 of one product's planes, of every
+  // 16 / NP-th modulus (constant steps in both addresses)
   {
-    const int64_t plane = sj.res_plane;
+    constexpr int kStep = 16 / NP;
     const int cc = tid & 7, crow = cc >> (lw - 4), col = j0 + (cc & ((w >> 4) - 1)) * 16;
-    if (i0 + crow < d.m && col < d.n) {
-      int q = tid >> 3;                                    // plane: modulus l, product r
-      const unsigned char* src = ws + sj.off_res + (int64_t)q * plane + (int64_t)(col >> 5) * group +
+    const int r = (tid >> 3) % NP, l0 = (tid >> 3) / NP;
+    if (l0 < kStep && i0 + crow < d.m && col < d.n) {
+      const int64_t step = (int64_t)(kStep * NP) * sj.res_plane;
+      const unsigned char* src = ws + sj.off_res + (int64_t)(l0 * NP + r) * sj.res_plane + (int64_t)(col >> 5) * group +
                                  (int64_t)(i0 + crow) * 32 + (col & 16);
-      int l = q / NP, r = q % NP;
-      for (; q < nm * NP; q += 16) {
-        cp_async16(ring + l * kStride + r * kCrtCols + cc * 16, src);
-        src += 16 * plane;
-        l += 16 / NP;
-        r += 16 % NP;
-        if (r >= NP) {
-          r -= NP;
-          ++l;
-        }
+      uint8_t* dst = ring + l0 * kStride + r * kCrtCols + cc * 16;
+#pragma unroll
+      for (int l = 0; l < kRingMods; l += kStep) {
+        if (l0 + l >= nm) break;
+        cp_async16(dst + l * kStride, src);
+        src += step;
       }
     }
     cp_async_commit();
