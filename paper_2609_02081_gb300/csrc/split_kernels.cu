@@ -90,6 +90,10 @@ __global__ void __launch_bounds__(kExpThreads)
     split_exponents_kernel(const __grid_constant__ JobParam<kOne> one, const SplitJob* __restrict__ jobs, int njobs,
                            unsigned char* __restrict__ ws, uint32_t* err, int64_t first_unit) {
   __shared__ int red[32][33];
+  // launched while the previous call's last kernel still runs; the next kernel reads the
+  // operands before its own wait, so it is let in only once everything before this call
+  // has finished
+  wait_for_previous_kernel();
   allow_next_kernel();
   constexpr int kOut = 32 / kSub;       // outputs of this block
   const int64_t unit = first_unit + blockIdx.x / kSub;
@@ -1003,16 +1007,16 @@ cudaError_t launch_split_exponents(const SplitJobs& jobs, int64_t units, int64_t
   if (units <= first_unit) return cudaSuccess;
   return with_jobs(jobs, [&](const auto& one) {
     constexpr bool kOne = std::is_same_v<std::decay_t<decltype(one)>, JobParam<true>>;
+    // A launch that depends on the end of a kernel starts on a 2.05 us grid on this GPU,
+    // one with programmatic serialisation at once: n = 64 20.5 -> 18.6 us, n = 256 39.0 -> 36.2.
     // few groups: four blocks to each, so that more SMs share the reads (n = 256,
     // 16 groups: 14.3 us -> 8; a whole product 46.9 -> 41.1)
     const int64_t blocks = units - first_unit;
     if (blocks < 152)
-      split_exponents_kernel<kOne, 4><<<(unsigned)(4 * blocks), kExpThreads, 0, s>>>(one, jobs.table, jobs.n, ws,
-                                                                                     device_error_ptr(), first_unit);
-    else
-      split_exponents_kernel<kOne, 1><<<(unsigned)blocks, kExpThreads, 0, s>>>(one, jobs.table, jobs.n, ws,
-                                                                               device_error_ptr(), first_unit);
-    return cudaGetLastError();
+      return launch_dependent(split_exponents_kernel<kOne, 4>, dim3((unsigned)(4 * blocks)), dim3(kExpThreads), 0, s, one,
+                              jobs.table, jobs.n, ws, device_error_ptr(), first_unit);
+    return launch_dependent(split_exponents_kernel<kOne, 1>, dim3((unsigned)blocks), dim3(kExpThreads), 0, s, one,
+                            jobs.table, jobs.n, ws, device_error_ptr(), first_unit);
   });
 }
 
