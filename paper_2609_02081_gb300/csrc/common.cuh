@@ -76,6 +76,25 @@ struct IsoMapOut {
   int64_t ldc, sC;
 };
 
+// Launch on `s` that may begin while the previous kernel of the stream still runs
+// (programmatic dependent launch): only for kernels that call
+// wait_for_previous_kernel() before they touch what it writes.
+template <class... Params, class... Args>
+cudaError_t launch_dependent(void (*kernel)(Params...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
+                             Args&&... args) {
+  cudaLaunchAttribute attr{};
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
+}
+
 // Locate the job owning global tile t (jobs sorted by tile_begin).
 __device__ __forceinline__ int find_job(const JobDesc* jobs, int njobs, int64_t t) {
   int lo = 0, hi = njobs - 1;

@@ -27,8 +27,8 @@
 //    barrier a block, the two warps of a sub-partition at different times;
 //  - components are copied four k-blocks ahead: plans of few products spend less time
 //    on a block than one copy takes (1 product, n = 1024: 5.99 ms with two blocks
-//    ahead, 3.06 with four).
-// n = 2048: 434 -> 367 ms; products alone at 2 per clock would take 352.
+//    ahead, 3.05 with four).
+// n = 2048: 434 -> 365 ms; products alone at 2 per clock would take 352.
 #include <cuda_runtime.h>
 
 #include "common.cuh"
@@ -50,6 +50,7 @@ struct Fp64Smem {
   double ys[2][kMaxFactors][F_BK][F_BN];   // right factors
   double wd[8][F_MAXP];                 // recombination weights w4 / 4 of the loaded plan
   KPlan plan;
+  JobDesc job;                          // the only job of a call (kOne)
   int plan_id;
 };
 
@@ -210,19 +211,39 @@ __device__ __forceinline__ void store_point(const JobDesc& jb, int i, int jj, co
   }
 }
 
+template <bool kOne>
+struct Fp64One {
+  JobDesc job;
+};
+template <>
+struct Fp64One<false> {};
+
 // kRanges: the call's tiles, laid end to end in k-blocks (each job's tiles
 // ranges.per_tile of them apart), are cut into one range of ranges.width k-blocks per
 // CTA, whatever tiles it crosses.  Each piece of a tile goes to slot (CTA + tile) of
 // the partial outputs: along the ranges either number increases, so no two pieces
 // share one.
-template <bool kRanges>
+// kOne: the call's only job, in the arguments: nothing to copy to the device first, and
+// the launch need not wait for the 2.05 us grid on which dependent launches start
+// (64 x 64 x 64: 74 -> 59 us, n = 256: 776 -> 756).
+// kFull: every job runs the paper's full plan, whose product q multiplies left and right
+// factor q: no plan look-ups between the products (n = 1024: 47.8 -> 47.4 ms).
+template <bool kRanges, bool kOne, bool kFull>
 __global__ void __launch_bounds__(F_THREADS, 1)
-fp64_bilinear_kernel(const JobDesc* __restrict__ jobs, int njobs, const KPlan* __restrict__ plans,
+fp64_bilinear_kernel(const __grid_constant__ Fp64One<kOne> one, const JobDesc* __restrict__ jobs, int njobs, const KPlan* __restrict__ plans,
                      int64_t total_tiles, Fp64Ranges ranges) {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
   extern __shared__ __align__(16) unsigned char smem_raw[];
   Fp64Smem& s = *reinterpret_cast<Fp64Smem*>(smem_raw);
   const int t = threadIdx.x;
   const int ty = t / 16, tx = t % 16;   // output rows 2ty, 2ty+1; cols 2tx, 2tx+1
+  // (a copy in shared memory: with the fields in constant memory the compiler spends
+  // the registers that the products' operands are prefetched in)
+  if constexpr (kOne) {
+    static_assert(sizeof(JobDesc) % 8 == 0 && sizeof(JobDesc) / 8 <= F_THREADS, "copied in 8-byte words");
+    if (t < (int)(sizeof(JobDesc) / 8))
+      reinterpret_cast<uint64_t*>(&s.job)[t] = reinterpret_cast<const uint64_t*>(&one.job)[t];
+  }
   if (t == 0) s.plan_id = -1;
   __syncthreads();
 
@@ -230,7 +251,7 @@ fp64_bilinear_kernel(const JobDesc* __restrict__ jobs, int njobs, const KPlan* _
   const int64_t end = kRanges ? min(total_tiles, (int64_t)(blockIdx.x + 1) * ranges.width) : total_tiles;
   int64_t pos = kRanges ? (int64_t)blockIdx.x * ranges.width : blockIdx.x;
   while (pos < end) {
-    const JobDesc& jb = jobs[find_job(jobs, njobs, pos)];
+    const JobDesc& jb = kOne ? s.job : jobs[find_job(jobs, njobs, pos)];
     int64_t local;
     int kbeg, kend;
     double* part = nullptr;             // this piece's partial result, or null: C itself
@@ -267,7 +288,7 @@ fp64_bilinear_kernel(const JobDesc* __restrict__ jobs, int njobs, const KPlan* _
         s.wd[w / F_MAXP][w % F_MAXP] = 0.25 * (double)s.plan.w4[w / F_MAXP][w % F_MAXP];
       __syncthreads();
     }
-    const int np = s.plan.np;
+    const int np = kFull ? F_MAXP : s.plan.np;
 
     double acc[F_MAXP][4];
 #pragma unroll
@@ -309,8 +330,9 @@ fp64_bilinear_kernel(const JobDesc* __restrict__ jobs, int njobs, const KPlan* _
         for (int q = 0; q < F_MAXP; ++q) {
           if (q >= np) break;
           {
-            const double2 x = *reinterpret_cast<const double2*>(&s.xs[cur][s.plan.pl[q]][kk][2 * ty]);
-            const double2 y = *reinterpret_cast<const double2*>(&s.ys[cur][s.plan.pr[q]][kk][2 * tx]);
+            const int fl = kFull ? q : s.plan.pl[q], fr = kFull ? q : s.plan.pr[q];
+            const double2 x = *reinterpret_cast<const double2*>(&s.xs[cur][fl][kk][2 * ty]);
+            const double2 y = *reinterpret_cast<const double2*>(&s.ys[cur][fr][kk][2 * tx]);
             acc[q][0] = fma(x.x, y.x, acc[q][0]);
             acc[q][1] = fma(x.x, y.y, acc[q][1]);
             acc[q][2] = fma(x.y, y.x, acc[q][2]);
@@ -327,7 +349,7 @@ fp64_bilinear_kernel(const JobDesc* __restrict__ jobs, int njobs, const KPlan* _
     for (int pt = 0; pt < 4; ++pt) {
       const int ti = 2 * ty + (pt >> 1), tj = 2 * tx + (pt & 1);
       double q[8];
-      if (s.plan.bilinear_full) {
+      if (kFull || s.plan.bilinear_full) {
         recombine_full(acc, pt, q);
       } else {
 #pragma unroll
@@ -375,16 +397,22 @@ __global__ void __launch_bounds__(256) fp64_splitk_reduce_kernel(JobDesc jb) {
 
 // Reduction behind the ranges: C <- alpha (sum of the tile's pieces, in k order) +
 // beta C, four blocks a tile, one thread per output element.
+template <bool kOne>
 __global__ void __launch_bounds__(256)
-fp64_ranges_reduce_kernel(const JobDesc* __restrict__ jobs, int njobs, Fp64Ranges ranges) {
+fp64_ranges_reduce_kernel(const __grid_constant__ Fp64One<kOne> one, const JobDesc* __restrict__ jobs, int njobs,
+                          Fp64Ranges ranges) {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
   const int64_t tile = blockIdx.x >> 2;
-  int lo = 0, hi = njobs - 1;
+  int lo = 0, hi = kOne ? 0 : njobs - 1;
   while (lo < hi) {
     const int mid = (lo + hi + 1) >> 1;
     if (jobs[mid].tile0 <= tile) lo = mid;
     else hi = mid - 1;
   }
-  const JobDesc& jb = jobs[lo];
+  const JobDesc& jb = [&]() -> const JobDesc& {
+    if constexpr (kOne) return one.job;
+    else return jobs[lo];
+  }();
   const int64_t local = tile - jb.tile0;
   const int within = (int)(blockIdx.x & 3) * 256 + threadIdx.x;
   const int i = (int)(local / jb.tiles_n) * F_BM + within / F_BN;
@@ -395,18 +423,28 @@ fp64_ranges_reduce_kernel(const JobDesc* __restrict__ jobs, int njobs, Fp64Range
   for (int e = 0; e < 8; ++e) q[e] = 0.0;
   const int64_t begin = jb.tile_begin + local * jb.per_tile;
   const int64_t last = begin + (jb.k + F_BK - 1) / F_BK - 1;   // before begin: k = 0, no pieces
-  for (int64_t c = begin / ranges.width; c * ranges.width <= last; ++c) {
-    const double* src = ranges.part + (c + tile) * (8 * F_BM * F_BN) + within;
+  if (last >= begin) {
+    const int64_t c0 = begin / ranges.width;
+    const int pieces = (int)(last / ranges.width - c0) + 1;
+    const double* src = ranges.part + (c0 + tile) * (8 * F_BM * F_BN) + within;
+    // four pieces' loads in flight (a tile that every SM shares has a hundred or more)
+#pragma unroll 4
+    for (int c = 0; c < pieces; ++c, src += 8 * F_BM * F_BN) {
 #pragma unroll
-    for (int e = 0; e < 8; ++e) q[e] += src[(int64_t)e * (F_BM * F_BN)];
+      for (int e = 0; e < 8; ++e) q[e] += src[(int64_t)e * (F_BM * F_BN)];
+    }
   }
   store_point(jb, i, jj, q);
 }
 
-cudaError_t launch_fp64_ranges_reduce(const JobDesc* d_jobs, int njobs, const Fp64Ranges& ranges,
+cudaError_t launch_fp64_ranges_reduce(const JobDesc* one, const JobDesc* d_jobs, int njobs, const Fp64Ranges& ranges,
                                       cudaStream_t stream) {
-  fp64_ranges_reduce_kernel<<<(unsigned)(4 * ranges.tiles), 256, 0, stream>>>(d_jobs, njobs, ranges);
-  return cudaGetLastError();
+  const dim3 grid((unsigned)(4 * ranges.tiles));
+  if (one)
+    return launch_dependent(fp64_ranges_reduce_kernel<true>, grid, dim3(256), 0, stream, Fp64One<true>{*one}, d_jobs,
+                            njobs, ranges);
+  return launch_dependent(fp64_ranges_reduce_kernel<false>, grid, dim3(256), 0, stream, Fp64One<false>{}, d_jobs,
+                          njobs, ranges);
 }
 
 cudaError_t launch_fp64_splitk_reduce(const JobDesc& jb, cudaStream_t stream) {
@@ -425,22 +463,42 @@ int64_t fp64_splitk_bytes(int64_t m, int64_t n, int kslices) {
 size_t fp64_smem_bytes() { return sizeof(Fp64Smem); }
 
 cudaError_t fp64_configure() {
-  const cudaError_t e = cudaFuncSetAttribute(fp64_bilinear_kernel<false>,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(Fp64Smem));
-  if (e != cudaSuccess) return e;
-  return cudaFuncSetAttribute(fp64_bilinear_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              (int)sizeof(Fp64Smem));
+  cudaError_t e = cudaSuccess;
+  auto set = [&e](auto kernel) {
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(Fp64Smem));
+  };
+  set(fp64_bilinear_kernel<false, false, false>);
+  set(fp64_bilinear_kernel<false, false, true>);
+  set(fp64_bilinear_kernel<true, false, false>);
+  set(fp64_bilinear_kernel<true, true, false>);
+  set(fp64_bilinear_kernel<true, true, true>);
+  return e;
 }
 
-cudaError_t launch_fp64_bilinear(const JobDesc* d_jobs, int njobs, const KPlan* d_plans, int64_t total_tiles,
-                                 int grid, const Fp64Ranges& ranges, cudaStream_t stream) {
-  if (ranges.width > 0)
-    fp64_bilinear_kernel<true>
-        <<<grid, F_THREADS, sizeof(Fp64Smem), stream>>>(d_jobs, njobs, d_plans, total_tiles, ranges);
-  else
-    fp64_bilinear_kernel<false>
-        <<<grid, F_THREADS, sizeof(Fp64Smem), stream>>>(d_jobs, njobs, d_plans, total_tiles, ranges);
-  return cudaGetLastError();
+// True when product q of the plan multiplies factors q and its products recombine as the
+// paper's full plan (kFull).
+bool fp64_full_plan(const KPlan& p) {
+  for (int q = 0; q < F_MAXP; ++q)
+    if (p.pl[q] != q || p.pr[q] != q) return false;
+  return p.bilinear_full != 0 && p.np == F_MAXP && !p.four_m;
+}
+
+// d_jobs: njobs of them; one: the only job of a call cut into ranges, or null; full:
+// every plan is fp64_full_plan
+cudaError_t launch_fp64_bilinear(const JobDesc* one, const JobDesc* d_jobs, int njobs, const KPlan* d_plans,
+                                 int64_t total_tiles, int grid, const Fp64Ranges& ranges, bool full,
+                                 cudaStream_t stream) {
+  auto go = [&](auto kernel, const auto& job) {
+    return launch_dependent(kernel, dim3((unsigned)grid), dim3(F_THREADS), sizeof(Fp64Smem), stream, job, d_jobs,
+                            njobs, d_plans, total_tiles, ranges);
+  };
+  if (one)
+    return full ? go(fp64_bilinear_kernel<true, true, true>, Fp64One<true>{*one})
+                : go(fp64_bilinear_kernel<true, true, false>, Fp64One<true>{*one});
+  if (ranges.width > 0) return go(fp64_bilinear_kernel<true, false, false>, Fp64One<false>{});
+  return full ? go(fp64_bilinear_kernel<false, false, true>, Fp64One<false>{})
+              : go(fp64_bilinear_kernel<false, false, false>, Fp64One<false>{});
 }
 
 int64_t fp64_ranges_bytes(const Fp64Ranges& r) {

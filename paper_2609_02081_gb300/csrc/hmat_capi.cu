@@ -76,11 +76,13 @@ static cudaError_t noalloc_setup(int device, NoAllocAddrs* out) {
 size_t fp64_smem_bytes();
 cudaError_t fp64_configure();
 cudaError_t launch_wait_selftest(long long limit_cycles, cudaStream_t s);
-cudaError_t launch_fp64_bilinear(const JobDesc* d_jobs, int njobs, const KPlan* d_plans, int64_t total_tiles,
-                                 int grid, const Fp64Ranges& ranges, cudaStream_t stream);
+cudaError_t launch_fp64_bilinear(const JobDesc* one, const JobDesc* d_jobs, int njobs, const KPlan* d_plans,
+                                 int64_t total_tiles, int grid, const Fp64Ranges& ranges, bool full,
+                                 cudaStream_t stream);
+bool fp64_full_plan(const KPlan& p);
 int fp64_block_k();
 int64_t fp64_ranges_bytes(const Fp64Ranges& r);
-cudaError_t launch_fp64_ranges_reduce(const JobDesc* d_jobs, int njobs, const Fp64Ranges& ranges,
+cudaError_t launch_fp64_ranges_reduce(const JobDesc* one, const JobDesc* d_jobs, int njobs, const Fp64Ranges& ranges,
                                       cudaStream_t stream);
 int fp64_tile_m();
 int fp64_tile_n();
@@ -386,10 +388,10 @@ struct Fp64Shape {
 // last piece may be short), or every SM the same number of k-blocks, whose piece of a
 // second tile costs another epilogue.  In us, a k-block of np products takes about
 // 4 + np, an epilogue and the pipeline's fill 12 + np / 2; a piece is not worth its
-// partial result below one k-block of the full plan (64 x 64 x 64: two at least 91 us,
-// one 74, uncut 504).  n = 256, 64 tiles of 64
+// partial result below one k-block of the full plan (64 x 64 x 64: two at least 76 us,
+// one 59, uncut 504).  n = 256, 64 tiles of 64
 // k-blocks: 2 slices each on 128 SMs 32 + 1, equal ranges on 152 SMs 27 + 2:
-// 935 -> 776 us; 64 x 64 x 1024, 4 tiles: 936 -> 247 us (the rule stops at 8 slices).
+// 935 -> 756 us; 64 x 64 x 1024, 4 tiles: 936 -> 232 us (the rule stops at 8 slices).
 Fp64Ranges fp64_ranges(const hmat_context* h, const std::vector<Fp64Shape>& shapes, std::vector<int32_t>* per_tile) {
   Fp64Ranges r;
   int64_t units = 0, kmax = 0, shortest = INT64_MAX;
@@ -605,19 +607,29 @@ hmat_status prepare(hmat_context* h, int32_t count, const hmat_gemm_desc* descs,
   return HMAT_STATUS_SUCCESS;
 }
 
+// One job cut into ranges travels in the kernel arguments; others, whose products run for
+// longer, in a table on the device.
+bool fp64_one_job(const Prepared& pr, size_t g) {
+  return g == 0 && pr.ranges.width > 0 && pr.f[g].size() == 1;
+}
+
 hmat_status launch_fp64_group(hmat_context* h, const Prepared& pr, int g, const JobDesc* d_jobs,
                               cudaStream_t stream) {
   const Fp64Ranges ranges = g == 0 ? pr.ranges : Fp64Ranges{};
+  const JobDesc* one = fp64_one_job(pr, g) ? &pr.f[g][0] : nullptr;
+  bool full = true;
+  for (const JobDesc& j : pr.f[g]) full = full && fp64_full_plan(h->h_plans[j.plan]);
   const int grid = (int)(ranges.width > 0 ? ranges.ctas : std::min<int64_t>(pr.f_tiles[g], h->sm_count));
   {
     ProfScope ps(h, 0, stream);
     cudaError_t e =
-        launch_fp64_bilinear(d_jobs, (int)pr.f[g].size(), h->d_plans, pr.f_tiles[g], grid, ranges, stream);
+        launch_fp64_bilinear(one, d_jobs, (int)pr.f[g].size(), h->d_plans, pr.f_tiles[g], grid, ranges, full,
+                             stream);
     if (e != cudaSuccess) return cuda_status(e);
   }
   if (ranges.width > 0) {
     ProfScope ps(h, 14, stream);
-    cudaError_t e = launch_fp64_ranges_reduce(d_jobs, (int)pr.f[g].size(), ranges, stream);
+    cudaError_t e = launch_fp64_ranges_reduce(one, d_jobs, (int)pr.f[g].size(), ranges, stream);
     return e == cudaSuccess ? HMAT_STATUS_SUCCESS : cuda_status(e);
   }
   // split-k: the slices of each split product added in order, then alpha / beta
@@ -677,12 +689,13 @@ hmat_status run(hmat_context* h, int32_t count, const hmat_gemm_desc* descs, int
   for (size_t g = 0; g < pr.f.size(); ++g) {
     if (pr.f_tiles[g] == 0) continue;
     JobDesc* d_jobs = nullptr;
-    int slot = 0;
-    st = upload_jobs(h, pr.f[g], stream, &d_jobs, &slot);
-    if (st != HMAT_STATUS_SUCCESS) return st;
+    int slot = -1;
+    if (!fp64_one_job(pr, g)) {
+      st = upload_jobs(h, pr.f[g], stream, &d_jobs, &slot);
+      if (st != HMAT_STATUS_SUCCESS) return st;
+    }
     st = launch_fp64_group(h, pr, (int)g, d_jobs, stream);
-    if (st != HMAT_STATUS_SUCCESS) return st;
-    st = finish_slot(h, slot, stream);
+    if (st == HMAT_STATUS_SUCCESS && slot >= 0) st = finish_slot(h, slot, stream);
     if (st != HMAT_STATUS_SUCCESS) return st;
   }
   return launch_iso_out(h, pr, stream);

@@ -290,25 +290,6 @@ hmat_status split_cuda_error(cudaError_t e);
 SplitState& handle_split(hmat_context* h);
 
 
-// Launch on `s` that may begin while the previous kernel of the stream still runs
-// (programmatic dependent launch): only for kernels that call
-// wait_for_previous_kernel() before they touch what it writes.
-template <class... Params, class... Args>
-cudaError_t launch_dependent(void (*kernel)(Params...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
-                             Args&&... args) {
-  cudaLaunchAttribute attr{};
-  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr.val.programmaticStreamSerializationAllowed = 1;
-  cudaLaunchConfig_t cfg{};
-  cfg.gridDim = grid;
-  cfg.blockDim = block;
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = s;
-  cfg.attrs = &attr;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
-}
-
 // Device-side kernel launchers (split_kernels.cu).
 cudaError_t launch_split_exponents(const SplitJobs& jobs, int64_t units, int64_t first_unit,
                                    cudaStream_t s, unsigned char* ws);
