@@ -319,9 +319,9 @@ Mat2Shape mat2_shape(uint32_t fa, uint32_t fb) {
 // plan's (24, or 16 in the four-multiplication form), which also keeps it inside
 // those bytes; that leaves out a few tiny k at loose tolerances (k <= 15 at tol
 // 1e-3: 6 x 14 planes against 5 x 16).  Measured at tol 1e-12: full m = n = k =
-// 8192, 15 x 14 planes against Gauss's 14 x 24: 226 -> 141 ms; the 512-product
-// batch: 31.9 -> 21.3 ms; TRS x TRA m = n = k = 4096, 15 x 7 against 14 x 8: 14.4 -> 10.4 ms;
-// complex x full 3000 x 1000 x 2000, 15 x 8 against 14 x 12: 2.51 -> 1.44 ms.
+// 8192, 15 x 14 planes against Gauss's 14 x 24: 226 -> 140 ms; the 512-product
+// batch: 31.7 -> 18.7 ms; TRS x TRA m = n = k = 4096, 15 x 7 against 14 x 8: 14.4 -> 10.0 ms;
+// complex x full 3000 x 1000 x 2000, 15 x 8 against 14 x 12: 2.49 -> 1.33 ms.
 static void to_mat2(SplitJob* sj, int64_t offset0) {
   const Mat2Shape s = mat2_shape(sj->d.fa, sj->d.fb);
   if (s.kind == kMat2None) return;
