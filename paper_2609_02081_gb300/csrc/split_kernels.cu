@@ -73,9 +73,8 @@ __device__ __forceinline__ float residue_i64(long long X, const ModConst& mc) {
 }
 
 // ------------------------------------------------------------------ 1. exponents
-// One block per group of 32 outputs: rows of op(A) or columns of op(B).
+// Blocks of outputs: rows of op(A) or columns of op(B).
 // s = b - 1 - floor(log2 max|x|) over the eight present components and k.
-constexpr int kExpThreads = 1024;   // 32 warps: k is split over the warps (or lanes)
 
 // biased exponent field of x; inf / NaN set `bad`
 __device__ __forceinline__ int exp_field(double x, bool& bad) {
@@ -84,9 +83,12 @@ __device__ __forceinline__ int exp_field(double x, bool& bad) {
   return ef;
 }
 
-// kSub: blocks per group of 32 outputs (1 or 4, each 32 / kSub of them).
-template <bool kOne, int kSub>
-__global__ void __launch_bounds__(kExpThreads)
+// kSub: blocks per group of 32 outputs (2 or 4, each 32 / kSub of them); kThr: threads of
+// a block.  The registers allow 1024 threads an SM: as two blocks of 512, so that one's
+// reduction and start run beside the other's loads (one block of 1024 and 32 outputs: the
+// 512-product batch 1.09 ms, now 1.00; n = 4096 374 -> 349 us; n = 8192 1.34 -> 1.30 ms).
+template <bool kOne, int kSub, int kThr>
+__global__ void __launch_bounds__(kThr)
     split_exponents_kernel(const __grid_constant__ JobParam<kOne> one, const SplitJob* __restrict__ jobs, int njobs,
                            unsigned char* __restrict__ ws, uint32_t* err, int64_t first_unit) {
   __shared__ int red[32][33];
@@ -115,11 +117,11 @@ __global__ void __launch_bounds__(kExpThreads)
   int best = 0;
   bool bad = false;
   // k positions k0, k0 + st, ... of every present component.  Long rows: one
-  // component after the other, four loads in flight (sequential DRAM streams:
-  // 1.21 ms at n = 8192, the copy bandwidth).  Short ones are bound by the chain of
+  // component after the other, four loads in flight (sequential DRAM streams).  Short ones are bound by the chain of
   // round trips: two positions of all eight components at a time, sixteen loads in
   // flight.
-  constexpr int st = 32 * kSub;
+  constexpr int kPer = kThr / 32 / kOut;       // warps to an output
+  constexpr int st = 32 * kPer;
   auto scan = [&](const double* src, int64_t k0, int64_t step) {
     int mx = 0;
     if (K > 1024) {
@@ -153,23 +155,23 @@ __global__ void __launch_bounds__(kExpThreads)
     return mx;
   };
   // red[part][output]: partial maxima of the block's outputs
-  constexpr int kParts = kExpThreads / 32;
+  constexpr int kParts = kThr / 32;
   if (contiguous) {
-    // kSub warps to an output; lanes stride k
-    const int o = warp / kSub, r = r0 + o;
-    int mx = r < nout ? scan(base + (int64_t)r * ld, (warp % kSub) * 32 + lane, 1) : 0;
+    // kPer warps to an output; lanes stride k
+    const int o = warp / kPer, r = r0 + o;
+    int mx = r < nout ? scan(base + (int64_t)r * ld, (warp % kPer) * 32 + lane, 1) : 0;
 #pragma unroll
     for (int x = 16; x > 0; x >>= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, x));
-    if (lane == 0) red[warp % kSub][o] = mx;
+    if (lane == 0) red[warp % kPer][o] = mx;
     __syncthreads();
     if (threadIdx.x < kOut) {
       best = red[0][threadIdx.x];
 #pragma unroll
-      for (int w = 1; w < kSub; ++w) best = max(best, red[w][threadIdx.x]);
+      for (int w = 1; w < kPer; ++w) best = max(best, red[w][threadIdx.x]);
     }
   } else {
     // lanes over the outputs (consecutive addresses; kSub k positions beside each
-    // other), the 32 warps split k
+    // other), the warps split k
     const int o = lane % kOut, r = r0 + o;
     int mx = r < nout ? scan(base + r, warp * kSub + lane / kOut, ld) : 0;
 #pragma unroll
@@ -1013,9 +1015,9 @@ cudaError_t launch_split_exponents(const SplitJobs& jobs, int64_t units, int64_t
     // 16 groups: 14.3 us -> 8; a whole product 46.9 -> 41.1)
     const int64_t blocks = units - first_unit;
     if (blocks < 152)
-      return launch_dependent(split_exponents_kernel<kOne, 4>, dim3((unsigned)(4 * blocks)), dim3(kExpThreads), 0, s, one,
-                              jobs.table, jobs.n, ws, device_error_ptr(), first_unit);
-    return launch_dependent(split_exponents_kernel<kOne, 1>, dim3((unsigned)blocks), dim3(kExpThreads), 0, s, one,
+      return launch_dependent(split_exponents_kernel<kOne, 4, 1024>, dim3((unsigned)(4 * blocks)), dim3(1024), 0, s,
+                              one, jobs.table, jobs.n, ws, device_error_ptr(), first_unit);
+    return launch_dependent(split_exponents_kernel<kOne, 2, 512>, dim3((unsigned)(2 * blocks)), dim3(512), 0, s, one,
                             jobs.table, jobs.n, ws, device_error_ptr(), first_unit);
   });
 }
