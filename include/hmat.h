@@ -93,8 +93,8 @@ typedef enum {
      * the GEMM prologue and the recombination in its epilogue.  Runs without
      * workspace.  Given the workspace hmat_workspace_size reports, a call
      * whose output tiles leave SMs idle splits the inner dimension of its
-     * products into slices (split-k, hmat_set_fp64_splitk_table) and adds the
-     * slices' partial outputs in slice order before alpha / beta: the result
+     * products into ranges or slices (split-k, hmat_set_fp64_splitk_table) and
+     * adds their partial outputs in the order of k before alpha / beta: the result
      * is deterministic but its rounding differs from the unsplit one. */
     HMAT_MODE_FP64 = 0,
     /* Split precision (Ozaki-type, integer modular): op(A), op(B) scaled by
@@ -434,9 +434,11 @@ hmat_status hmat_measure_fp64_peak(int32_t kind, int64_t iterations, double *tfl
 
 /* FP64 split-k table: 16 x 16 int8 codes indexed [min(15, ceil(log2 T))]
  * [min(15, ceil(log2 k))], T = output tiles (32 x 32) of the call, k = the
- * product's inner dimension: 0 = built-in rule (double the slices, up to 8,
- * while twice the tile-slices fit the SMs once and each slice keeps at least
- * 64 of k), 1/2/3/4 = 1/2/4/8 slices.  Written by the autotuner
+ * product's inner dimension: 0 = built-in rule (a call whose tiles fit half
+ * the SMs and whose largest k is 32 or more is cut into equal ranges of its
+ * inner dimensions, one per SM; with a workspace too small for their partial
+ * results into up to 8 slices while twice the tile-slices fit the SMs once and
+ * each slice keeps at least 64 of k), 1/2/3/4 = 1/2/4/8 slices.  Written by the autotuner
  * (paper_2609_02081_gb300/autotune.py --fp64); NULL restores the rule.
  * Applies to single-pass FP64 calls (every BILINEAR plan) made with
  * workspace; hmat_workspace_size accounts for it.  Streamed products never
