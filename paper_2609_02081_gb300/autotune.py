@@ -9,9 +9,9 @@ multiple of 32 wide) and with each fixed tile width (128 x 64, 128 x 128,
 64/128/256 columns) that :meth:`Handle.set_tile_table` installs.
 
 Split-k (--fp64): for every (ceil(log2 tiles), ceil(log2 k)) bin of the FP64
-shapes, one representative product is timed in FP64 mode with its inner
-dimension in 1, 2, 4 and 8 slices; the fastest code (1..4) goes into a second
-16 x 16 table that :meth:`Handle.set_fp64_splitk_table` installs.
+shapes, one representative product is timed in FP64 mode with the built-in rule
+and with its inner dimension in 1, 2, 4 and 8 slices; the fastest code (0 = the
+rule, 1..4) goes into a second 16 x 16 table that :meth:`Handle.set_fp64_splitk_table` installs.
 
 Grouped (--grouped): per-bin timing alone does not predict a grouped call,
 whose residue-GEMM items of all products share the SMs; this mode times
@@ -214,13 +214,13 @@ def tune_fp64(shapes, reps: int = 5, seed: int = 0):
             B = torch.rand((8, k, n), generator=g, device=dev, dtype=torch.float64) * 2 - 1
             C = torch.empty((8, m, n), dtype=torch.float64, device=dev)
             times = {}
-            for code in (1, 2, 3, 4):
+            for code, name in enumerate(("rule", 1, 2, 4, 8)):
                 t = np.zeros((BINS, BINS), dtype=np.int8)
                 t[bt, bk] = code
                 h.set_fp64_splitk_table(t)
-                times[1 << (code - 1)] = _time_fp64(h, A, B, C, reps)
+                times[name] = _time_fp64(h, A, B, C, reps)
             best = min(times, key=times.get)
-            table[bt, bk] = int(math.log2(best)) + 1
+            table[bt, bk] = list(times).index(best)
             report[f"{bt},{bk}"] = {"shape": [m, n, k], "ms": times, "best_slices": best, "members": len(members)}
     return table, report
 
