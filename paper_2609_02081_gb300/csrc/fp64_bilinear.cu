@@ -230,7 +230,7 @@ struct Fp64One<false> {};
 // factor q: no plan look-ups between the products (n = 1024: 47.8 -> 47.4 ms).
 template <bool kRanges, bool kOne, bool kFull>
 __global__ void __launch_bounds__(F_THREADS, 1)
-fp64_bilinear_kernel(const __grid_constant__ Fp64One<kOne> one, const JobDesc* __restrict__ jobs, int njobs, const KPlan* __restrict__ plans,
+fp64_bilinear_kernel(const __grid_constant__ Fp64One<kOne> one, const JobDesc* jobs, int njobs, const KPlan* plans,
                      int64_t total_tiles, Fp64Ranges ranges) {
   asm volatile("griddepcontrol.wait;" ::: "memory");
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -399,7 +399,7 @@ __global__ void __launch_bounds__(256) fp64_splitk_reduce_kernel(JobDesc jb) {
 // beta C, four blocks a tile, one thread per output element.
 template <bool kOne>
 __global__ void __launch_bounds__(256)
-fp64_ranges_reduce_kernel(const __grid_constant__ Fp64One<kOne> one, const JobDesc* __restrict__ jobs, int njobs,
+fp64_ranges_reduce_kernel(const __grid_constant__ Fp64One<kOne> one, const JobDesc* jobs, int njobs,
                           Fp64Ranges ranges) {
   asm volatile("griddepcontrol.wait;" ::: "memory");
   const int64_t tile = blockIdx.x >> 2;

@@ -10,7 +10,11 @@ namespace hmat {
 // may be scheduled from here on, not only when this one ends (it still waits for
 // this one's results); wait_for_previous_kernel: returns when the previous kernel
 // has finished and its writes are visible.  Every kernel launched this way waits,
-// so a kernel's finish implies that all earlier ones have finished.  Only the
+// so a kernel's finish implies that all earlier ones have finished.  Such a kernel
+// is resident while memory that it will read is still being written, so its
+// parameters are not __restrict__ and nothing goes through __ldg: either would tell
+// the compiler that the memory does not change while the kernel runs, and let it move
+// a load above the wait or take it from the read-only cache.  Only the
 // exponents allow the next one early: the encoder doing so let residue-GEMM CTAs
 // settle while its last blocks ran, and a 512-product batch took 22.7 ms against
 // 21.3 (n = 4096: 20.9 against 19.9); from the GEMM it makes no difference, since
@@ -63,11 +67,28 @@ __device__ __forceinline__ int find_split_job(const SplitJob* jobs, int njobs, i
   return lo;
 }
 
+// A load before wait_for_previous_kernel() of data that an earlier kernel than the
+// previous one wrote (which the previous one has waited for): performed at the GPU's
+// point of coherence, since this SM's L1 may still hold a line from before that write.
+__device__ __forceinline__ unsigned long long load_coherent(const double* p) {
+  unsigned long long v;
+  asm volatile("ld.relaxed.gpu.global.b64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
+  return v;
+}
+
+// p itself, as a value that exists only from here on: loads through it, of whatever
+// kind, cannot move above an earlier wait_for_previous_kernel().
+template <class T>
+__device__ __forceinline__ T* known_from_here(T* p) {
+  asm volatile("" : "+l"(p)::"memory");
+  return p;
+}
+
 __device__ __forceinline__ float2 f2(float v) { return make_float2(v, v); }
 
 // The job of unit u of a stage: the one in the arguments, or the table's.
 template <bool kOne>
-__device__ __forceinline__ const SplitJob& unit_job(const JobParam<kOne>& one, const SplitJob* __restrict__ jobs,
+__device__ __forceinline__ const SplitJob& unit_job(const JobParam<kOne>& one, const SplitJob* jobs,
                                                     int njobs, int64_t u, int which) {
   if constexpr (kOne) return one.job;
   else return jobs[find_split_job(jobs, njobs, u, which)];

@@ -206,12 +206,12 @@ __device__ __forceinline__ int find_item_job(const SplitJob* jobs, int njobs, in
 // forward (one load per job boundary passed) instead of searching the whole
 // table for every item.
 __device__ __forceinline__ int advance_job(const SplitJob* jobs, int njobs, int64_t item, int cur) {
-  while (cur + 1 < njobs && __ldg(&jobs[cur + 1].item_begin) <= item) ++cur;
+  while (cur + 1 < njobs && jobs[cur + 1].item_begin <= item) ++cur;
   return cur;
 }
 
 template <bool kOne>
-__device__ __forceinline__ const SplitJob& item_job(const JobParam<kOne>& one, const SplitJob* __restrict__ jobs,
+__device__ __forceinline__ const SplitJob& item_job(const JobParam<kOne>& one, const SplitJob* jobs,
                                                     int job) {
   if constexpr (kOne) return one.job;
   else return jobs[job];
@@ -313,7 +313,7 @@ __constant__ GemmModConst c_gmod[2 * kModTable];   // the plans' moduli, then th
 // kOne: one job, in the arguments, instead of the table.
 template <bool kOneChunk, bool kOne>
 __global__ void __launch_bounds__(kThreads, 1)
-split_residue_gemm_kernel(const __grid_constant__ JobParam<kOne> one, const SplitJob* __restrict__ jobs, int njobs,
+split_residue_gemm_kernel(const __grid_constant__ JobParam<kOne> one, const SplitJob* jobs, int njobs,
                           int64_t total_items, uint8_t* ws, uint32_t* err) {
   extern __shared__ uint8_t smem_dyn[];
   // 1024-byte alignment for the swizzled operand tiles

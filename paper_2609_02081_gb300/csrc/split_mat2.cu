@@ -190,10 +190,14 @@ __device__ __forceinline__ void encode_pair(const longlong2* E, int l0, int l1, 
 // 10.2 ms at n = 8192, 0.94 of the copy bandwidth).
 template <int ND, bool kOne>
 __global__ void __launch_bounds__(kThreads, 4)
-    mat2_encode_kernel(const __grid_constant__ JobParam<kOne> one, const SplitJob* __restrict__ jobs, int njobs,
-                       unsigned char* __restrict__ ws, int64_t first) {
+    mat2_encode_kernel(const __grid_constant__ JobParam<kOne> one, const SplitJob* jobs, int njobs,
+                       unsigned char* ws, int64_t first) {
   __shared__ __align__(16) long long ent[8][kRows][kPitch];
   __shared__ int s_row[kRows];
+  // One job, in the arguments: the operands are read before the wait for the exponents,
+  // whose kernel has itself waited for whatever wrote the operands before it let this
+  // one start.  A table on the device is memory like any other: wait first.
+  if constexpr (!kOne) wait_for_previous_kernel();
   const int64_t blk = first + blockIdx.x;
   const SplitJob& sj = unit_job(one, jobs, njobs, blk, 5);
   const JobDesc& d = sj.d;
@@ -232,10 +236,11 @@ __global__ void __launch_bounds__(kThreads, 4)
     for (int c = 0; c < 8; ++c) {
       raw[u][c] = 0ull;
       if (in && ((flags >> c) & 1u))
-        raw[u][c] = (unsigned long long)__double_as_longlong(__ldcs(src + (int64_t)c * cs));
+        raw[u][c] = kOne ? load_coherent(src + (int64_t)c * cs)
+                         : (unsigned long long)__double_as_longlong(__ldcs(src + (int64_t)c * cs));
     }
   }
-  wait_for_previous_kernel();                    // the exponents
+  if constexpr (kOne) wait_for_previous_kernel();   // the exponents
   if (t < kRows) {
     const int r = r0 + t;
     s_row[t] = (r < nout) ? reinterpret_cast<const int32_t*>(ws + (side ? sj.off_texp : sj.off_sexp))[r] : 0;
@@ -459,8 +464,8 @@ __device__ __forceinline__ Mat2Pair turn(Mat2Pair x, int rot) {
 }
 
 // The block's work for a job of kind KIND; L: limbs of the sums, KS: k steps (of 16 moduli).
-template <int L, int KS, int KIND>
-__device__ __forceinline__ void crt_block(const SplitJob& sj, uint32_t local, const unsigned char* __restrict__ ws,
+template <int L, int KS, int KIND, bool kOne>
+__device__ __forceinline__ void crt_block(const SplitJob& sj, uint32_t local, const unsigned char* ws,
                                           uint8_t* ring, uint32_t (*tr)[8][kTrStride]) {
   constexpr int NP = KIND == kMat2Full ? 14 : KIND == kMat2Quat ? 7 : KIND == kMat2Scaled ? 8 : 2;
   constexpr int kStride = mod_stride(NP);
@@ -485,7 +490,7 @@ __device__ __forceinline__ void crt_block(const SplitJob& sj, uint32_t local, co
       for (int nt = 0; nt < 2; ++nt)
 #pragma unroll
         for (int v = 0; v < 2; ++v) b[h][ks][nt][v] = __ldg(&g_m2digits[nm][h][ks][nt][v][lane]);
-  wait_for_previous_kernel();                              // the residues
+  if constexpr (kOne) wait_for_previous_kernel();          // the residues
   // copy: thread tid takes 16-byte chunk tid % 8 of one product's planes, of every
   // 16 / NP-th modulus (constant steps in both addresses)
   {
@@ -707,19 +712,20 @@ __device__ __forceinline__ void crt_block(const SplitJob& sj, uint32_t local, co
 
 template <int L, int KS, bool kOne>
 __global__ void __launch_bounds__(kCrtThreads, 4)
-    mat2_crt_kernel(const __grid_constant__ JobParam<kOne> one, const SplitJob* __restrict__ jobs, int njobs,
-                    const unsigned char* __restrict__ ws) {
+    mat2_crt_kernel(const __grid_constant__ JobParam<kOne> one, const SplitJob* jobs, int njobs,
+                    const unsigned char* ws) {
   __shared__ __align__(16) uint8_t ring[(KS == 1 ? 16 : kMat2MaxModuli + 1) * mod_stride(kMat2MaxPlanes)];
   __shared__ __align__(16) uint32_t tr[kCrtThreads / 32][2][8][kTrStride];
+  if constexpr (!kOne) wait_for_previous_kernel();         // before anything is read from the table
   const int64_t blk = blockIdx.x;
   const SplitJob& sj = unit_job(one, jobs, njobs, blk, 6);
   const uint32_t local = (uint32_t)(blk - sj.crt2_begin);
   auto* mine = tr[threadIdx.x >> 5];
   switch (sj.mat2) {                                       // block-uniform
-    case kMat2Full: crt_block<L, KS, kMat2Full>(sj, local, ws, ring, mine); break;
-    case kMat2Quat: crt_block<L, KS, kMat2Quat>(sj, local, ws, ring, mine); break;
-    case kMat2Scaled: crt_block<L, KS, kMat2Scaled>(sj, local, ws, ring, mine); break;
-    default: crt_block<L, KS, kMat2Complex>(sj, local, ws, ring, mine); break;
+    case kMat2Full: crt_block<L, KS, kMat2Full, kOne>(sj, local, ws, ring, mine); break;
+    case kMat2Quat: crt_block<L, KS, kMat2Quat, kOne>(sj, local, ws, ring, mine); break;
+    case kMat2Scaled: crt_block<L, KS, kMat2Scaled, kOne>(sj, local, ws, ring, mine); break;
+    default: crt_block<L, KS, kMat2Complex, kOne>(sj, local, ws, ring, mine); break;
   }
 }
 
