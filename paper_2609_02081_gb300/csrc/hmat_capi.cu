@@ -710,12 +710,13 @@ hmat_status run_graph(hmat_context* h, int32_t count, const hmat_gemm_desc* desc
     return run(h, count, descs, mode, tol, workspace, ws_bytes, stream_ptr, SplitReuse{}, modes);
   std::lock_guard<std::mutex> lock(h->mu);
   h->last_bad = -1;
-  // key: descriptors + mode (or the per-product modes) + tol + workspace + algorithm + complex form + tile table
+  // key: descriptors + mode (or the per-product modes) + tol + workspace + algorithm + complex form + tile tables +
+  // FP64 split-k table
   const size_t tbl = sizeof(h->split.tile_table);
   const size_t ftbl = (size_t)h->split.n_flag_tables * (sizeof(uint16_t) + sizeof(h->split.flag_tables[0]));
   const size_t nmodes = modes ? (size_t)std::max(count, 0) : 0;
   std::vector<unsigned char> key(sizeof(int32_t) * 4 + sizeof(double) + sizeof(void*) + sizeof(size_t) + 1 + tbl +
-                                 sizeof(int32_t) + ftbl +
+                                 sizeof(int32_t) + ftbl + 1 + sizeof(h->fp64_splitk) +
                                  (size_t)std::max(count, 0) * sizeof(hmat_gemm_desc) + nmodes * sizeof(int32_t));
   {
     unsigned char* k = key.data();
@@ -733,6 +734,8 @@ hmat_status run_graph(hmat_context* h, int32_t count, const hmat_gemm_desc* desc
       std::memcpy(k, &h->split.flag_keys[f], sizeof(uint16_t)); k += sizeof(uint16_t);
       std::memcpy(k, h->split.flag_tables[f], sizeof(h->split.flag_tables[f])); k += sizeof(h->split.flag_tables[f]);
     }
+    *k++ = h->has_fp64_splitk ? 1 : 0;
+    std::memcpy(k, h->fp64_splitk, sizeof(h->fp64_splitk)); k += sizeof(h->fp64_splitk);
     if (count > 0 && descs) std::memcpy(k, descs, (size_t)count * sizeof(hmat_gemm_desc));
     k += (size_t)std::max(count, 0) * sizeof(hmat_gemm_desc);
     if (nmodes) std::memcpy(k, modes, nmodes * sizeof(int32_t));
