@@ -1043,21 +1043,24 @@ hmat_status workspace_bytes(int algo, const TileTables& tables, int32_t count, c
     // pass (every bilinear plan has at most 24 products), as fp64_layout places
     // them (a split-mode call leaves its few trivial products unsplit)
     const int tm = fp64_tile_m(), tn = fp64_tile_n(), tk = fp64_tile_k();
-    const int64_t sc = algo == HMAT_ALGO_ISOMORPH ? 2 : 1;
+    // (a product without an inner dimension is not mapped to its complex image, and its
+    // plan is empty)
+    auto iso_job = [&](const hmat_gemm_desc& d) { return algo == HMAT_ALGO_ISOMORPH && d.k > 0; };
+    auto scale = [&](const hmat_gemm_desc& d) -> int64_t { return iso_job(d) ? 2 : 1; };
+    auto flags = [&](const hmat_gemm_desc& d, uint32_t f) { return iso_job(d) ? (uint32_t)HMAT_COMPLEX : d.k > 0 ? f : 0u; };
     int64_t tiles = 0;
     for (int32_t i = 0; i < count; ++i) {
       if (!fp64[i]) continue;
-      const int64_t m = sc * descs[i].m, n = sc * descs[i].n;
+      const int64_t sc = scale(descs[i]), m = sc * descs[i].m, n = sc * descs[i].n;
       tiles += ((m + tm - 1) / tm) * ((n + tn - 1) / tn);
     }
     int64_t off = (int64_t)align_up256((int64_t)*bytes);
     std::vector<Fp64Shape> fshapes;
     for (int32_t i = 0; i < count && 2 * tiles <= h->sm_count; ++i) {
       if (!fp64[i]) continue;
-      const int64_t m = sc * descs[i].m, n = sc * descs[i].n;
+      const int64_t sc = scale(descs[i]), m = sc * descs[i].m, n = sc * descs[i].n;
       KPlan p;
-      const bool iso_job = algo == HMAT_ALGO_ISOMORPH;
-      if (!build_plan(iso_job ? HMAT_COMPLEX : descs[i].flagsA, iso_job ? HMAT_COMPLEX : descs[i].flagsB, &p))
+      if (!build_plan(flags(descs[i], descs[i].flagsA), flags(descs[i], descs[i].flagsB), &p))
         return HMAT_STATUS_INTERNAL;
       fshapes.push_back({((m + tm - 1) / tm) * ((n + tn - 1) / tn), sc * descs[i].k, p.np});
     }
@@ -1069,7 +1072,7 @@ hmat_status workspace_bytes(int algo, const TileTables& tables, int32_t count, c
     }
     for (int32_t i = 0; i < count; ++i) {
       if (!fp64[i]) continue;
-      const int64_t m = sc * descs[i].m, n = sc * descs[i].n, k = sc * descs[i].k;
+      const int64_t sc = scale(descs[i]), m = sc * descs[i].m, n = sc * descs[i].n, k = sc * descs[i].k;
       if (k <= 0) continue;
       const int s = fp64_kslices(h, tiles, k);
       if (s <= 1) continue;

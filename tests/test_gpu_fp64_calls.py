@@ -49,3 +49,16 @@ def test_graph_follows_the_split_k_table(handle):
             assert torch.equal(grouped(handle, probs, ws, True)[0], eager[0])
         seen.append(eager[0])
     assert torch.equal(seen[0], seen[2]) and not torch.equal(seen[0], seen[1])
+
+
+@pytest.mark.parametrize("algo", ["bilinear", "isomorph"])
+@pytest.mark.parametrize("m0", [32, 200])
+def test_reported_workspace_holds_the_cut(handle, algo, m0):
+    """Beside a product without an inner dimension (which no algorithm enlarges, and whose plan
+    is empty) the reported workspace is what the call's cut needs: more changes nothing."""
+    handle.set_algorithm(algo)
+    probs = [problem(910, 64, 64, 256), problem(920, m0, m0, 0)]
+    need = hm.hmat_workspace_size(handle, [hm.make_desc(*p) for p in probs], "fp64")
+    big = torch.empty(need + (64 << 20), dtype=torch.uint8, device="cuda")
+    first = grouped(handle, probs, big[:need], False)
+    assert torch.equal(grouped(handle, probs, big, False)[0], first[0])
