@@ -816,9 +816,10 @@ cudaError_t mat2_configure(const int* moduli, const int* root, int n, const int3
         }
     }
     const uint32_t* P = crt_P + m * kLimbs;
-    if (!crt_estimate_constants(P, 2.0 * m * kMat2WeightSum * kMat2HalfMax, m <= kMat2FourLimbs ? 4 : 5, &pb[m],
-                                &pinv[m]))
-      return cudaErrorInvalidValue;
+    // both limb counts that can run m moduli (a call's deepest job picks its kernel's)
+    for (int limbs = m <= kMat2FourLimbs ? 4 : kLimbs; limbs <= kLimbs; ++limbs)
+      if (!crt_estimate_constants(P, 2.0 * m * kMat2WeightSum * kMat2HalfMax, limbs, &pb[m], &pinv[m]))
+        return cudaErrorInvalidValue;
     unsigned long long carry = 1;                    // 2^128 - P
     uint32_t w[4];
     for (int q = 0; q < 4; ++q) {
