@@ -553,8 +553,8 @@ split_residue_gemm_kernel(const __grid_constant__ JobParam<kOne> one, const Spli
         ok = false;
         break;
       } else {
-      // running sum of chunk residues (each |r| <= 129, at most 127 chunks:
-      // exact in float)
+      // running sum of chunk residues (each |r| <= 129; at most 254 chunks, of the
+      // four-multiplication form, whose depth is 2 k: exact in float)
       float acc[kBnMax / 2];
 #pragma unroll
       for (int i = 0; i < kBnMax / 2; ++i) acc[i] = 0.f;
@@ -591,8 +591,8 @@ split_residue_gemm_kernel(const __grid_constant__ JobParam<kOne> one, const Spli
       }
       if (!ok) break;
       // reduce mod p to [-(p-1)/2, (p-1)/2] and store this row's residues
-      // (16-byte stores); rows and columns of padding are not stored.  |acc| <=
-      // 129 * 127 < 2^14, where acc * (1/p) is within 2^-9 of acc / p, which
+      // (32-byte stores); rows and columns of padding are not stored.  |acc| <=
+      // 129 * 254 < 2^15, where acc * (1/p) is within 2^-9 / p of acc / p, which
       // is at least 1/(2p) from a half-integer: the rounding is exact.
       if (row < it.rows) {
         int8_t* dst = it.out + (int64_t)row * it.row_bytes + (int64_t)(col0 >> 5) * it.group_bytes;

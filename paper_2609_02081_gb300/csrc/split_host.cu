@@ -34,7 +34,8 @@ static constexpr int kBitsMargin = 6;
 hmat_status split_params(int64_t k, double tol, SplitParams* out) {
   if (tol == 0.0) tol = 1e-12;
   if (!(tol > 0.0) || !std::isfinite(tol)) return HMAT_STATUS_INVALID_VALUE;
-  // drained int32 accumulators hold up to 127 chunks of 1024
+  // k of up to 127 chunks of 1024: the running sums of the chunks' residues (twice as
+  // many chunks in the four-multiplication form) stay exact
   if (k > (int64_t)127 * kChunkK) return HMAT_STATUS_UNSUPPORTED;
   SplitParams sp;
   const int want = (int)std::ceil(-std::log2(tol));

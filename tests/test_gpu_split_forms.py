@@ -1,5 +1,5 @@
 """Split mode's forms where the tests of one form do not reach the others: modulus counts
-that mix in one launch, the largest outputs of each form's own moduli, the
+that mix in one launch, the largest outputs of each form's own moduli, the deepest products, the
 no-allocation entry point."""
 import math
 from fractions import Fraction
@@ -100,6 +100,20 @@ def test_largest_outputs_of_each_forms_moduli(handles, form, tol, k, count):
         C = torch.full((8, m, n), float("nan"), dtype=torch.float64, device="cuda")
         hm.hmat_bq_gemm(handles[form], sign * A, B, C, mode="split", tol=tol)
         np.testing.assert_array_equal(C.cpu().numpy(), np.broadcast_to((sign * want)[:, None, None], (8, m, n)))
+
+
+def test_deepest_four_multiplication_products(handles):
+    """The forced four-multiplication form runs over 2 k: at the largest k 254 accumulation chunks,
+    whose running sums stay below 2^15: Gauss's and the default form's bits."""
+    k, m, n = 127 * 1024, 20, 40
+    A, B = bi.uniform(530, m, k).cuda(), bi.uniform(531, k, n).cuda()
+    outs = []
+    for form in ("four_m", "gauss", "auto"):
+        C = torch.full((8, m, n), float("nan"), dtype=torch.float64, device="cuda")
+        hm.hmat_bq_gemm(handles[form], A, B, C, mode="split", tol=1e-12)
+        outs.append(C)
+    torch.cuda.synchronize()
+    assert torch.equal(outs[0], outs[1]) and torch.equal(outs[2], outs[1])
 
 
 @pytest.mark.parametrize("m,n,k", [(96, 112, 200), (33, 20, 600)])

@@ -395,3 +395,21 @@ def test_narrow_products_beside_deep_ones():
             hm.hmat_bq_gemm(h, A, B, C, mode="split", tol=TOL)
             assert torch.equal(C, want)
         assert h.device_error() == 0
+
+
+def test_running_sums_of_chunk_residues():
+    """The GEMM's accumulation chunks: 1088-deep sums of products of the matrix form's residues (up to 121) are exact in
+    FP32, and so are the running sums of the chunks' residues (up to 129), 254 of them at the largest k in the
+    four-multiplication form, whose depth is 2 k."""
+    assert 1088 * 121 ** 2 < 2 ** 24
+    kmax = max(k for k in (127 * 1024, 127 * 1024 + 1) if _served(k))
+    assert kmax == 127 * 1024
+    assert 129 * (2 * kmax // 1024) < 2 ** 15
+
+
+def _served(k):
+    try:
+        hm.split_info(k, TOL)
+    except hm.HmatError:
+        return False
+    return True
