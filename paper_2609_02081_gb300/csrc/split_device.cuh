@@ -145,7 +145,6 @@ __device__ __forceinline__ void cp_async16(void* smem, const void* gmem) {
 }
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
 __device__ __forceinline__ void cp_async_wait2() { asm volatile("cp.async.wait_group 2;\n" ::: "memory"); }
-__device__ __forceinline__ void cp_async_wait4() { asm volatile("cp.async.wait_group 4;\n" ::: "memory"); }
 __device__ __forceinline__ void cp_async_wait6() { asm volatile("cp.async.wait_group 6;\n" ::: "memory"); }
 
 // |X| = [x3 x2 x1 x0] (below 2^127) times 2^scale_exp as a double, rounded

@@ -23,7 +23,6 @@ struct ModConst {
   float c18;    // 2^18 mod p, centred
   float c36;    // 2^36 mod p, centred
   float c23;    // 2^23 mod p, in [0, p)
-  unsigned long long fm;  // floor(2^64 / p) + 1 (fast exact 32-bit mod)
 };
 
 __constant__ ModConst c_mod[kModTable];
@@ -34,43 +33,6 @@ __constant__ uint32_t c_P[kMaxModuli + 1][kLimbs];                // product of 
 __constant__ uint32_t c_off[kMaxModuli + 1][kLimbs];              // N P with N = nmod * kMaxWeightSum * 127
 __constant__ float c_Pinv[kMaxModuli + 1];                        // 2^(32 Pbase) / P as float
 __constant__ int c_Pbase[kMaxModuli + 1];                         // limb index one below P's top limb
-
-// ------------------------------------------------------------------ small exact modular helpers
-// Centred residue of an integer-valued float |v| < 2^24: v - p*round(v/p),
-// |result| <= (p+1)/2.  round() by the 1.5 * 2^23 shift: for |t| < 2^22 the
-// sum t + 1.5*2^23 rounds t to an integer in round-to-nearest; v/p < 2^17.
-__device__ __forceinline__ float fmod_c(float v, const ModConst& mc) {
-  const float shifted = fmaf(v, mc.inv, 12582912.0f);
-  const float q = shifted - 12582912.0f;
-  return fmaf(-q, mc.pf, v);
-}
-
-// Residue in [0, p) of a 32-bit unsigned value (Lemire's fast modulus, exact).
-__device__ __forceinline__ uint32_t fastmod_u32(uint32_t x, const ModConst& mc) {
-  const unsigned long long low = mc.fm * (unsigned long long)x;
-  return (uint32_t)__umul64hi(low, (unsigned long long)mc.p);
-}
-
-// Centred residue of a signed 32-bit value (any magnitude), result in [-(p-1)/2, (p-1)/2].
-__device__ __forceinline__ int cmod_i32(int x, const ModConst& mc) {
-  // x = hi * 2^16 + lo with lo in [0, 2^16); hi in [-2^15, 2^15)
-  const uint32_t lo = (uint32_t)x & 0xFFFFu;
-  const int hi = x >> 16;
-  const uint32_t rhi = fastmod_u32((uint32_t)(hi + 256 * mc.p), mc);   // hi + 256p > 0 for p >= 129
-  const uint32_t c16 = fastmod_u32(65536u, mc);
-  const uint32_t r = fastmod_u32(rhi * c16 + fastmod_u32(lo, mc), mc);
-  const int half = (mc.p - 1) >> 1;
-  return (int)r > half ? (int)r - mc.p : (int)r;
-}
-
-// Centred residue (as float) of a scaled integer |X| <= 2^52.
-__device__ __forceinline__ float residue_i64(long long X, const ModConst& mc) {
-  const float x0 = (float)(int)(X & 0x3FFFF);
-  const float x1 = (float)(int)((X >> 18) & 0x3FFFF);
-  const float x2 = (float)(int)(X >> 36);        // |x2| <= 2^16
-  const float r2 = fmod_c(x2, mc), r1 = fmod_c(x1, mc), r0 = fmod_c(x0, mc);
-  return fmod_c(fmaf(r2, mc.c36, fmaf(r1, mc.c18, r0)), mc);
-}
 
 // ------------------------------------------------------------------ 1. exponents
 // Blocks of outputs: rows of op(A) or columns of op(B).
@@ -197,7 +159,7 @@ __global__ void __launch_bounds__(kThr)
 }
 
 // ------------------------------------------------------------------ 2. encode
-// One block per tile of 32 rows x 32 k of one side (op(A) rows, or op(B)
+// One block per tile of 16 rows x 32 k of one side (op(A) rows, or op(B)
 // columns); every modulus is handled by the same block.
 //   phase 1: the eight present components of the tile are read (coalesced
 //            along whichever index is contiguous in memory), scaled to
@@ -212,12 +174,6 @@ __global__ void __launch_bounds__(kThr)
 // (17.1 -> 20.0 ms at n = 8192: spills).
 constexpr int kEncRows = 16, kEncK = 32, kEncThreads = 128;
 
-__device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
-  uint32_t r;
-  asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(hi), "f"(lo));
-  return r;
-}
-
 // Centred residue (as float) of a scaled integer given by its float limbs:
 // X = hi 2^23 + lo for |X| <= 2^47 (LIMBS == 2), else X = x2 2^36 + x1 2^18 + x0
 // (|X| <= 2^52); every limb and partial sum stays below 2^24 (exact floats).
@@ -226,6 +182,7 @@ __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
 // resident blocks.)
 // The encoder works on two k positions at once with paired FP32 instructions
 // (__ffma2_rn / __fadd2_rn), each lane rounding exactly as the scalar form.
+// v - p round(v / p), |result| <= (p + 1) / 2: adding 1.5 * 2^23 rounds to an integer.
 __device__ __forceinline__ float2 fmod_c2(float2 v, const ModConst& mc) {
   const float2 q = __fadd2_rn(__ffma2_rn(v, f2(mc.inv), f2(12582912.0f)), f2(-12582912.0f));
   return __ffma2_rn(q, f2(-mc.pf), v);
@@ -984,7 +941,6 @@ cudaError_t split_upload_constants(const int* moduli, int nmod_table, const int3
     m.c18 = centred(1ll << 18);
     m.c36 = centred(1ll << 36);
     m.c23 = (float)((1ll << 23) % p);
-    m.fm = ~0ull / (unsigned long long)p + 1ull;
   }
   cudaError_t e = cudaMemcpyToSymbol(c_mod, mc, sizeof(mc));
   if (e != cudaSuccess) return e;
