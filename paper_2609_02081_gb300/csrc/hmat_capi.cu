@@ -1189,9 +1189,9 @@ hmat_status hmat_bq_gemm_split_noalloc(hmat_handle h, int32_t opA, int32_t opB, 
   noalloc_store_job_kernel<<<1, 1, 0, stream>>>(sj);
   e = cudaGetLastError();
   const SplitJobs jobs{a.job, 1, nullptr};
-  if (e == cudaSuccess) e = launch_split_exponents(jobs, u.exp, 0, stream, a.scratch);
+  if (e == cudaSuccess) e = launch_split_exponents(jobs, u.exp, 0, stream, a.scratch, h->sm_count);
   if (sj.mat2) {
-    if (e == cudaSuccess) e = launch_mat2_encode(jobs, u.encA + u.encB, 0, stream, a.scratch, u.max_bits);
+    if (e == cudaSuccess) e = launch_mat2_encode(jobs, u.encA + u.encB, 0, stream, a.scratch, u.max_bits, h->sm_count);
   } else {
     if (e == cudaSuccess) e = launch_split_encode(jobs, h->d_plans, 0, u.encA, stream, a.scratch, u.max_bits);
     if (e == cudaSuccess) e = launch_split_encode(jobs, h->d_plans, 1, u.encB, stream, a.scratch, u.max_bits);

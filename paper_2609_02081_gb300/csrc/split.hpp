@@ -292,7 +292,7 @@ SplitState& handle_split(hmat_context* h);
 
 // Device-side kernel launchers (split_kernels.cu).
 cudaError_t launch_split_exponents(const SplitJobs& jobs, int64_t units, int64_t first_unit,
-                                   cudaStream_t s, unsigned char* ws);
+                                   cudaStream_t s, unsigned char* ws, int sm_count);
 // units are blocks: encode tiles of 32 rows x 32 k, CRT blocks of 256 elements
 cudaError_t launch_split_encode(const SplitJobs& jobs, const KPlan* d_plans, int side, int64_t units,
                                 cudaStream_t s, unsigned char* ws, int max_bits);
@@ -311,7 +311,7 @@ cudaError_t launch_split_crt(const SplitJobs& jobs, const KPlan* d_plans, int64_
 // Matrix form (split_mat2.cu).  Encode blocks [first, first + units) of the
 // A and B sides of its jobs; jobs of other forms have no blocks.
 cudaError_t launch_mat2_encode(const SplitJobs& jobs, int64_t units, int64_t first, cudaStream_t s,
-                               unsigned char* ws, int max_bits);
+                               unsigned char* ws, int max_bits, int sm_count);
 cudaError_t launch_mat2_crt(const SplitJobs& jobs, int64_t units, cudaStream_t s, unsigned char* ws,
                             int max_nmod);
 // n (kMat2MaxModuli) moduli, root[l]^2 = -1 mod moduli[l], and by modulus count

@@ -590,7 +590,7 @@ hmat_status split_launch(hmat_context* h, const SplitPrep& sp, const SplitJob* d
     ProfScope ps(h, 1, stream);
     const int64_t a_units = njobs == 1 ? (sp.jobs[0].d.m + 31) / 32 : 0;
     const int64_t first = skip_a ? a_units : 0, end = skip_b ? a_units : sp.exp_units;
-    e = launch_split_exponents(jobs, end, first, stream, ws);
+    e = launch_split_exponents(jobs, end, first, stream, ws, handle_sm_count(h));
   }
   if (e != cudaSuccess) return split_cuda_error(e);
   {
@@ -602,7 +602,7 @@ hmat_status split_launch(hmat_context* h, const SplitPrep& sp, const SplitJob* d
     const int64_t a_blocks = njobs == 1 ? mat2_enc_blocks(sp.jobs[0].d.m, sp.jobs[0].d.k) : 0;
     const int64_t first = skip_a ? a_blocks : 0, end = skip_b ? std::min(a_blocks, sp.enc2_units) : sp.enc2_units;
     if (e == cudaSuccess && end > first)
-      e = launch_mat2_encode(jobs, end - first, first, stream, ws, sp.max_bits2);
+      e = launch_mat2_encode(jobs, end - first, first, stream, ws, sp.max_bits2, handle_sm_count(h));
   }
   if (e != cudaSuccess) return split_cuda_error(e);
   {

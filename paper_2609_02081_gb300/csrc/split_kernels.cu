@@ -962,7 +962,7 @@ cudaError_t split_upload_constants(const int* moduli, int nmod_table, const int3
 }
 
 cudaError_t launch_split_exponents(const SplitJobs& jobs, int64_t units, int64_t first_unit,
-                                   cudaStream_t s, unsigned char* ws) {
+                                   cudaStream_t s, unsigned char* ws, int sm_count) {
   if (units <= first_unit) return cudaSuccess;
   return with_jobs(jobs, [&](const auto& one) {
     constexpr bool kOne = std::is_same_v<std::decay_t<decltype(one)>, JobParam<true>>;
@@ -971,7 +971,7 @@ cudaError_t launch_split_exponents(const SplitJobs& jobs, int64_t units, int64_t
     // few groups: four blocks to each, so that more SMs share the reads (n = 256,
     // 16 groups: 14.3 us -> 8; a whole product 46.9 -> 41.1)
     const int64_t blocks = units - first_unit;
-    if (blocks < 152)
+    if (blocks < sm_count)
       return launch_dependent(split_exponents_kernel<kOne, 4, 1024>, dim3((unsigned)(4 * blocks)), dim3(1024), 0, s,
                               one, jobs.table, jobs.n, ws, device_error_ptr(), first_unit);
     return launch_dependent(split_exponents_kernel<kOne, 2, 512>, dim3((unsigned)(2 * blocks)), dim3(512), 0, s, one,

@@ -855,12 +855,12 @@ cudaError_t mat2_configure(const int* moduli, const int* root, int n, const int3
 }
 
 cudaError_t launch_mat2_encode(const SplitJobs& jobs, int64_t units, int64_t first, cudaStream_t s,
-                               unsigned char* ws, int max_bits) {
+                               unsigned char* ws, int max_bits, int sm_count) {
   if (units <= 0) return cudaSuccess;
-  // A launch whose tiles do not fill the GPU (152 SMs x 4 blocks) splits each
+  // A launch whose tiles do not fill the GPU (four blocks an SM) splits each
   // tile's moduli over up to four blocks, which repeat phase 1: a whole product
   // at n = 256 (256 tiles) 43.1 -> 41.0 us, at n = 64 24.6 -> 20.5.
-  const int64_t fill = 608;
+  const int64_t fill = 4 * (int64_t)sm_count;
   const unsigned groups = (unsigned)(units * 4 <= fill ? 4 : units * 2 <= fill ? 2 : 1);
   // the matrix entries are sums of two b-bit integers: three digits hold 2^47
   return with_jobs(jobs, [&](const auto& one) {

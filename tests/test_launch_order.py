@@ -78,3 +78,10 @@ def test_programmatic_kernels_wait_before_the_job_table():
         wait = re.search(WAIT, body).start()
         for use in re.finditer(r"\bunit_job\(|\bfind_item_job\(|\bfind_job\(|\bjobs\[", body):
             assert wait < use.start(), (u, n, use.group(0))
+
+
+def test_launch_rules_use_the_devices_sm_count():
+    """No rule of a launch compares with one chip's SM count (152) or its multiples."""
+    for u in sorted(os.listdir(CSRC)):
+        text = re.sub(r"/\*.*?\*/", "", source(u), flags=re.S)
+        assert not re.findall(r"\b(?:152|304|608|1216)\b", text), u
