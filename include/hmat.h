@@ -190,7 +190,8 @@ HMAT_API
 hmat_status hmat_destroy(hmat_handle handle);
 
 /* Workspace bytes that hmat_bq_gemm / hmat_bq_gemm_grouped need for these
- * problems in this mode (0 for FP64).  descs is a HOST array of `count`
+ * problems in this mode; for FP64 the partial outputs of a split inner dimension
+ * (0 when none would be split; the call runs without).  descs is a HOST array of `count`
  * descriptors (only op, flags, m, n, k are read).  tol: as for the call. */
 HMAT_API
 hmat_status hmat_workspace_size(hmat_handle handle, int32_t count,
@@ -468,7 +469,8 @@ hmat_status hmat_debug_wait_selftest(hmat_handle handle, int64_t limit_cycles, v
  * blocks return on a copy-out stream, so copies overlap the products.
  * Operands already in device memory are read in place.  With kb = k every
  * block is the same computation as the corresponding part of hmat_bq_gemm,
- * bit for bit, in both modes; with kb < k, C accumulates the chunks with
+ * bit for bit, in both modes (in FP64 mode of a call that does not split its
+ * inner dimension, as one without workspace); with kb < k, C accumulates the chunks with
  * beta = 1 (rounding differs; split-mode error is bounded per chunk).
  * ------------------------------------------------------------------------- */
 

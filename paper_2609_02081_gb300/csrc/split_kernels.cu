@@ -48,7 +48,7 @@ __device__ __forceinline__ int exp_field(double x, bool& bad) {
 // kSub: blocks per group of 32 outputs (2 or 4, each 32 / kSub of them); kThr: threads of
 // a block.  The registers allow 1024 threads an SM: as two blocks of 512, so that one's
 // reduction and start run beside the other's loads (one block of 1024 and 32 outputs: the
-// 512-product batch 1.09 ms, now 1.00; n = 4096 374 -> 349 us; n = 8192 1.34 -> 1.30 ms).
+// 512-product batch 1.09 ms, now 1.01; n = 4096 374 -> 356 us; n = 8192 1.34 -> 1.31 ms).
 template <bool kOne, int kSub, int kThr>
 __global__ void __launch_bounds__(kThr)
     split_exponents_kernel(const __grid_constant__ JobParam<kOne> one, const SplitJob* jobs, int njobs,

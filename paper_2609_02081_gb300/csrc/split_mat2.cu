@@ -355,7 +355,7 @@ __global__ void __launch_bounds__(kThreads, 4)
 // Bound by instruction issue (2.6 of 4 per cycle, 54 instructions per element and
 // warp lane; 64-bit multiply-adds per modulus, output and limb took 113): 1.2 ms
 // for 4096 x 4096 (2.35 ms with those), 0.68 ms of which its 4.6 GB would take at
-// the copy bandwidth; the 512-product batch 3.27 ms (6.1 ms).
+// the copy bandwidth; the 512-product batch 3.34 ms (6.1 ms).
 constexpr int kCrtThreads = 128;
 constexpr int mod_stride(int planes) {                // bytes; the four moduli pairs of a read fall on different banks
   return planes * kCrtCols + 16;
